@@ -1907,6 +1907,7 @@ __device__ __forceinline__ void iter_segments(const DecideArgs& a, uint64_t firs
 
 static_assert(kIterThreads == kGiantThreads && kIterThreads == kCommitThreads,
               "the part blocks and the commit sweep their lists in tiles of one block");
+static_assert(kIterThreads == kListThreads, "the list builder's tiles are one block's");
 static_assert(kIterDynWords >= 2 * kBlockSlots && 8 * 2 * kWarpSlots <= 2 * kBlockSlots &&
                   2 * kGiantSlots + 2 * kGiantChunk <= 2 * kBlockSlots,
               "the dynamic tables hold every unit kind");
@@ -2021,8 +2022,7 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
     if (!grid_barrier(ctrl, ia.bar_extra, ia.bar_polls)) return;
   }
   // 5. the next frontier's lists; clear the processed frontier's bitmap
-  lists_bits_body(ia.a.fbits_next, ia.words, ia.a.g.nv, ia.a.g.deg, ia.a.next_lists, ia.a.seg, ctrl,
-                  ia.a.next_buf, ia.k);
+  lists_body<true>(ia.a.fbits_next, ia.a.g.nv, ia.a.g.deg, ia.a.next_lists, ia.a.seg, ctrl, ia.a.next_buf, ia.k);
   for (uint64_t w = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; w < ia.words;
        w += uint64_t(gridDim.x) * blockDim.x)
     ia.fbits_cur[w] = 0;
@@ -2195,11 +2195,10 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
   }
   // the next frontier's lists, from its bitmap
   {
-    const uint32_t words = (a.g.nv + 31) / 32;
     LaunchScope ls(h, DFL_PROF_MARK, spine);
     // (the processed frontier's bitmap, cleared alongside, becomes the next-next target)
-    launch_pdl(k_lists_bits, grid_for(words, 256, 152 * 8), 256, 0, spine, a.fbits_next, words, a.g.nv,
-               a.g.deg, a.next_lists, a.seg, h->ctrl, nxt, k, h->fbits[cur], h->words);
+    launch_pdl(k_lists_bits, lists_grid(a.g.nv), kListThreads, 0, spine, a.fbits_next, a.g.nv, a.g.deg, a.next_lists,
+               a.seg, h->ctrl, nxt, k, h->fbits[cur], h->words);
     DFL_TRY(check_launch(h, "next frontier lists"));
   }
   if (par) {  // the handle's stream continues after the spine

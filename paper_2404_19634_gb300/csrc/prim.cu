@@ -249,39 +249,14 @@ __global__ void k_copy_i64(long long* d, const long long* s, uint64_t n) {
 // ---------------------------------------------------------------------------
 // Frontier lists
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_lists_all(uint32_t nv, const uint32_t* __restrict__ deg, uint32_t* lists,
-                                                   Segs seg, Ctrl* ctrl, int buf, uint32_t k) {
-  // every vertex with arcs, thread per vertex, counted per list key in shared
-  // memory and reserved once per block and key
-  __shared__ uint32_t s_cnt[kMaxSubsteps * kBins];
-  __shared__ uint32_t s_base[kMaxSubsteps * kBins];
-  const uint32_t nkeys = k * kBins;
-  for (uint64_t i0 = blockIdx.x * uint64_t(blockDim.x); i0 < nv; i0 += uint64_t(gridDim.x) * blockDim.x) {
-    const uint64_t i = i0 + threadIdx.x;
-    // a vertex without arcs has no neighbour community: it is processed
-    // (counted) but never queued
-    const uint32_t d = i < nv ? deg[i] : 0u;
-    const bool valid = i < nv && d > 0;
-    const unsigned idle = __ballot_sync(0xFFFFFFFFu, i < nv && d == 0);
-    if ((threadIdx.x & 31u) == 0 && idle) atomicAdd(&ctrl->skipped, (unsigned long long)__popc(idle));
-    const uint32_t key = valid ? vertex_class(uint32_t(i), k, seg) * kBins + degree_bin(d, seg) : 0u;
-    if (threadIdx.x < nkeys) s_cnt[threadIdx.x] = 0;
-    __syncthreads();
-    if (valid) atomicAdd(&s_cnt[key], 1u);
-    __syncthreads();
-    if (threadIdx.x < nkeys) {
-      const uint32_t c = s_cnt[threadIdx.x];
-      s_base[threadIdx.x] = c ? atomicAdd(&ctrl->count[buf][threadIdx.x / kBins][threadIdx.x % kBins], c) : 0u;
-      s_cnt[threadIdx.x] = 0;
-    }
-    __syncthreads();
-    if (valid) {
-      const uint32_t r = s_base[key] + atomicAdd(&s_cnt[key], 1u);
-      if (r < seg.cap[key]) lists[seg.off[key] + r] = uint32_t(i);
-      else atomicOr(&ctrl->err, kErrInternal);
-    }
-    __syncthreads();
-  }
+// Every vertex with arcs; one without has no neighbour community: it is
+// processed (counted) but never queued.
+__global__ void __launch_bounds__(kListThreads) k_lists_all(uint32_t nv, const uint32_t* __restrict__ deg,
+                                                            uint32_t* lists, Segs seg, Ctrl* ctrl, int buf,
+                                                            uint32_t k) {
+  uint32_t idle = lists_body<false>(nullptr, nv, deg, lists, seg, ctrl, buf, k);
+  idle = __reduce_add_sync(0xFFFFFFFFu, idle);
+  if ((threadIdx.x & 31u) == 0 && idle) atomicAdd(&ctrl->skipped, (unsigned long long)idle);
 }
 
 __global__ void k_bits_to_bytes(const uint32_t* bits, uint8_t* out, uint32_t n) {
@@ -313,16 +288,15 @@ __global__ void k_popcount(const uint32_t* bits, uint32_t words, unsigned long l
 
 }  // namespace
 
-__global__ void __launch_bounds__(256) k_lists_bits(const uint32_t* __restrict__ bits, uint32_t words,
-                                                    uint32_t nv, const uint32_t* __restrict__ deg,
-                                                    uint32_t* lists, Segs seg, Ctrl* ctrl, int buf,
-                                                    uint32_t k, uint32_t* __restrict__ clear,
-                                                    uint32_t clear_words) {
+__global__ void __launch_bounds__(kListThreads) k_lists_bits(const uint32_t* __restrict__ bits, uint32_t nv,
+                                                             const uint32_t* __restrict__ deg, uint32_t* lists,
+                                                             Segs seg, Ctrl* ctrl, int buf, uint32_t k,
+                                                             uint32_t* __restrict__ clear, uint32_t clear_words) {
   pdl_wait_only();
   for (uint64_t q = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; q < clear_words;
        q += uint64_t(gridDim.x) * blockDim.x)
     clear[q] = 0u;
-  lists_bits_body(bits, words, nv, deg, lists, seg, ctrl, buf, k);
+  lists_body<true>(bits, nv, deg, lists, seg, ctrl, buf, k);
 }
 
 // Segment layout for k sub-step classes: class s gets kBins segments, each
@@ -454,8 +428,7 @@ int lists_all(Handle* h, uint32_t nv, const uint32_t* deg, int buf, uint32_t k) 
   make_segs(h, k);
   const Segs& seg = h->segs;
   LaunchScope ls(h, DFL_PROF_MARK);
-  k_lists_all<<<grid_for(nv, 256, 152 * 8), 256, 0, h->stream>>>(nv, deg, h->lists[buf], seg, h->ctrl, buf,
-                                                        k);
+  k_lists_all<<<lists_grid(nv), kListThreads, 0, h->stream>>>(nv, deg, h->lists[buf], seg, h->ctrl, buf, k);
   return check_launch(h, "lists_all");
 }
 
@@ -463,10 +436,9 @@ int lists_from_bits(Handle* h, const uint32_t* bits, uint32_t nv, const uint32_t
                     uint32_t k) {
   make_segs(h, k);
   const Segs& seg = h->segs;
-  uint32_t words = (nv + 31) / 32;
   LaunchScope ls(h, DFL_PROF_MARK);
-  k_lists_bits<<<grid_for(words, 256, 152 * 8), 256, 0, h->stream>>>(bits, words, nv, deg, h->lists[buf],
-                                                                     seg, h->ctrl, buf, k, nullptr, 0u);
+  k_lists_bits<<<lists_grid(nv), kListThreads, 0, h->stream>>>(bits, nv, deg, h->lists[buf], seg, h->ctrl, buf, k,
+                                                               nullptr, 0u);
   return check_launch(h, "lists_from_bits");
 }
 

@@ -1,0 +1,81 @@
+"""Edges of the kernels' tiles and dispatch limits, bit for bit against the
+CPU oracle (every compared value is an integer, so nothing has a tolerance).
+"""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dfl():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2404_19634_gb300 as mod
+    mod.build()
+    mod.load()
+    return mod
+
+
+@pytest.fixture(scope="module")
+def orc():
+    import oracle
+    oracle.build()
+    return oracle
+
+
+_STREAMS = []
+
+
+def pair(dfl, orc, g, **kw):
+    import torch
+    off, idx, w = synth.to_csr(g)
+    s = torch.cuda.Stream()
+    _STREAMS.append(s)
+    a = dfl.Dfl(g.n, off, idx, w, options=dfl.default_options(**kw), stream=s)
+    b = orc.Oracle(g.n, off, idx, w)
+    b.set_options(**{k: v for k, v in kw.items() if k != "flags"})
+    return a, b
+
+
+def same(a, b):
+    assert np.array_equal(a.membership(), b.membership())
+    for x, y in zip(a.weights(), b.weights()):
+        assert np.array_equal(x, y)
+    assert a.modularity()[1:] == b.modularity()[1:]
+
+
+def random_graph(n, m, seed, w_max=9):
+    """n vertices and about m random weighted edges."""
+    rng = np.random.default_rng(seed)
+    if n < 2:
+        return synth.EdgeList(n, *(np.zeros(0, np.uint32),) * 3)
+    u, v = rng.integers(0, n, m), rng.integers(0, n, m)
+    key = np.unique(np.minimum(u, v)[u != v] * np.int64(n) + np.maximum(u, v)[u != v])
+    return synth.EdgeList(n, (key // n).astype(np.uint32), (key % n).astype(np.uint32),
+                          rng.integers(1, w_max + 1, key.size).astype(np.uint32))
+
+
+@pytest.mark.parametrize("n", [1, 31, 2047, 2049, 8191, 8200, 20_011])
+@pytest.mark.parametrize("density", [0.002, 0.2, 1.0])
+def test_frontier_lists_at_tile_edges(dfl, orc, n, density):
+    """A frontier given as a bitmap (sparse: its tiles compacted together;
+    dense: tile by tile) reaches exactly the vertices it names."""
+    g = random_graph(n, 3 * n, n)
+    rng = np.random.default_rng(7)
+    F = (rng.random(n) < density).astype(np.uint8)
+    F[-1] = 1
+    R = np.ones(n, np.uint8)
+    a, b = pair(dfl, orc, g)
+    C = rng.integers(0, max(1, n // 3), n).astype(np.uint32)
+    a.set_membership(C)
+    b.set_membership(C)
+    Fa, ma, Sa = a.move_iteration(F, R)
+    Fb, mb, Sb = b.move_iteration(F, R)
+    assert np.array_equal(Fa, Fb) and np.array_equal(ma, mb) and Sa == Sb
+    a.static()
+    b.static()
+    same(a, b)
