@@ -538,7 +538,7 @@ int dfl_modularity(dfl_handle* h, double* q, int64_t* parts) {
   if (h->ngraphs) return dfl::set_error(h, DFL_ERR_STATE, "a group handle takes the dfl_group_* calls");
   if (!h->have_communities) return set_error(h, DFL_ERR_STATE, "no communities yet");
   i128 num = 0, den = 0;
-  DFL_TRY(modularity_parts(h, &num, &den));
+  DFL_TRY(modularity_range(h, 0, h->n, h->m2, &num, &den));
   *q = den == 0 ? 0.0 : double(num) / double(den);
   if (parts) {
     parts[0] = int64_t(uint64_t((u128)num >> 64));

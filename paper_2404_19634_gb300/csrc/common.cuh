@@ -90,6 +90,7 @@ struct Ctrl {
   unsigned long long red_a;
   unsigned long long red_b;
   unsigned long long red_c;
+  unsigned long long long_rows;      // a queue of long rows: rows << 32 | pieces (push_row)
   unsigned int red_u;
   unsigned int apply_go;             // the batch apply's gate: the batch is written (1) or nothing is (0)
   unsigned int apply_defer;          // ... with rows to rebuild (by the multi-block rebuild kernel)
@@ -420,6 +421,10 @@ inline cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t
   return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
 }
 
+// A queue of at most n long rows (push_row) for passes over the base graph:
+// Sigma of the super-vertex levels is idle outside a Louvain run.
+inline uint2* row_queue(Handle* h) { return reinterpret_cast<uint2*>(h->Ss); }
+
 // ---------------------------------------------------------------------------
 // Device helpers
 // ---------------------------------------------------------------------------
@@ -663,6 +668,32 @@ __device__ __forceinline__ uint32_t lists_body(const uint32_t* __restrict__ bits
   }
 }
 
+// Queue of long rows, cut into pieces that the warps of a later kernel share.
+// One 64-bit counter holds (rows << 32 | pieces), so an entry's slot and its
+// first piece come from one atomic and the entries are in piece order: a warp
+// then finds the row of piece p with a 32-way search (three dependent loads
+// for 32,000 rows) instead of every block sweeping the whole queue through a
+// prefix sum (about 3 us per 256 rows).
+__device__ __forceinline__ void push_row(uint2* queue, unsigned long long* counter, uint32_t row, uint32_t pieces) {
+  const unsigned long long at = atomicAdd(counter, (1ull << 32) | pieces);
+  queue[at >> 32] = make_uint2(row, uint32_t(at));
+}
+
+// The queue entry (slot) that holds piece p, p < the queue's pieces.  Every
+// lane of the warp calls it with the same arguments.
+__device__ __forceinline__ uint32_t find_row(const uint2* queue, uint32_t rows, uint32_t p) {
+  uint32_t lo = 0, len = rows;  // the last entry of [lo, lo + len) with first piece <= p
+  while (len > 1) {
+    const uint32_t step = (len + 31) / 32;
+    const uint32_t k = (threadIdx.x & 31u) * step;
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, k < len && queue[lo + k].y <= p);
+    const uint32_t j = (__popc(m) - 1) * step;  // lane 0's entry always qualifies
+    lo += j;
+    len = len - j < step ? len - j : step;
+  }
+  return lo;
+}
+
 // ---------------------------------------------------------------------------
 // Host-side entry points of the other translation units
 // ---------------------------------------------------------------------------
@@ -700,7 +731,8 @@ int graph_build(Handle* h, const unsigned long long* off_in, const uint32_t* idx
 int weighted_degrees(Handle* h);  // K from scratch, m2 on host
 int compact_pool(Handle* h, uint64_t* before, uint64_t* after);  // dfl_compact
 int recompute_aux(Handle* h);      // K, 2m, Sigma, sizes from scratch (DFL_FLAG_RECOMPUTE_AUX)
-int modularity_parts(Handle* h, i128* num, i128* den);
+// Eq. 1's numerator and denominator over the rows and labels [v0, v1), with 2m = m2
+int modularity_range(Handle* h, uint32_t v0, uint32_t v1, long long m2, i128* num, i128* den);
 int graph_export(Handle* h, uint64_t* off, uint32_t* idx, uint32_t* w, bool device_out);
 int recompute_sigma_sizes(Handle* h, const uint32_t* C);
 

@@ -89,59 +89,170 @@ __global__ void k_fill_rows(uint32_t n, const unsigned long long* __restrict__ o
   }
 }
 
-// K_i = sum_j w_ij (Section 3), warp per row; 2m accumulated in ctrl->red_a.
-__global__ void k_weighted_degree(GraphView g, long long* __restrict__ K, Ctrl* ctrl) {
-  const uint32_t lane = threadIdx.x & 31u;
-  uint64_t warp = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) >> 5;
-  uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-  unsigned long long tot = 0;
-  for (uint64_t i = warp; i < g.nv; i += nwarps) {
-    unsigned long long s = 0;
-    unsigned long long o = g.off[i];
-    uint32_t d = g.deg[i];
-    for (uint32_t k = lane; k < d; k += 32) s += g.arcs[o + k].y;
-    for (int x = 16; x; x >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, x);
-    if (lane == 0) K[i] = (long long)s;
-    tot += s;
+// Sums over whole rows [v0, v1): K_i = sum_j w_ij (Section 3; 2m in red_a), or
+// with kInside the arc weights with both ends in one community (red_a) and,
+// for labels [v0, v1), sum_c Sigma_c^2 split into low (red_b) and high (red_c)
+// 32-bit parts.
+//
+// A chain of two or three dependent loads per row bounds it (offset ->
+// arcs -> communities), so a warp takes 32 rows: one load of their headers,
+// then four rows at a time with eight lanes each and four arcs a lane in
+// flight; rows longer than kRowShort take the whole warp, and those of more
+// than kRowHub arcs are queued for k_row_hubs, which spreads them over every
+// block.  One warp walking a hub's 100,000 arcs alone held the old kernels
+// up: K and 2m of the 2^22-vertex R-MAT graph (67 M arcs) took 541 us, now
+// 256 + 40; the modularity on 2^21 vertices (33 M arcs) 537 us, now 168 + 46.
+// Loading 16 rows' arcs at once instead of four was no faster (260 us; the
+// modularity 255): the rows' slack makes the pool twice the arcs' bytes.
+constexpr uint32_t kRowShort = 64, kRowHub = 1024, kRowPiece = 1024;
+constexpr int kRowThreads = 256;
+
+template <bool kInside>
+struct RowSums {
+  GraphView g;
+  const uint32_t* C;
+  const long long* Sigma;
+  long long* K;
+  uint32_t v0, v1;
+  uint2* hubs;  // queue of the rows longer than kRowHub (ctrl->long_rows)
+  Ctrl* ctrl;
+
+  // arcs [k0, k1) of row i, lanes striding by `step` from k0 + first: the weight
+  // this lane meets
+  __device__ __forceinline__ unsigned long long part(unsigned long long o, uint32_t ci, uint32_t k0, uint32_t k1,
+                                                     uint32_t first, uint32_t step) const {
+    unsigned long long sum = 0;
+    for (uint32_t b = k0 + first; b < k1; b += 4 * step) {
+      uint2 a[4];
+      uint32_t c[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t k = b + u * step;
+        a[u] = k < k1 ? g.arcs[o + k] : make_uint2(0u, 0u);
+      }
+      if constexpr (kInside) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c[u] = a[u].y ? C[a[u].x] : ci;  // (weight 0: deleted, or past the end)
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if constexpr (kInside) sum += c[u] == ci ? a[u].y : 0u;
+        else sum += a[u].y;
+      }
+    }
+    return sum;
   }
-  if (lane == 0 && tot) atomicAdd(&ctrl->red_a, tot);
+};
+
+__device__ __forceinline__ unsigned long long lanes_sum(unsigned long long x, int width) {
+  for (int o = width / 2; o; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
+  return x;
 }
 
-// sigma = sum of arc weights with both ends in one community (red_a);
-// sum_c Sigma_c^2 split into low (red_b) and high (red_c) 32-bit parts.
-__global__ void k_modularity(GraphView g, const uint32_t* __restrict__ C,
-                             const long long* __restrict__ Sigma, uint32_t n, Ctrl* ctrl) {
+template <bool kInside>
+__global__ void __launch_bounds__(kRowThreads) k_row_sums(RowSums<kInside> r) {
   const uint32_t lane = threadIdx.x & 31u;
-  uint64_t warp = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) >> 5;
-  uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-  unsigned long long sig = 0;
-  for (uint64_t i = warp; i < g.nv; i += nwarps) {
-    uint32_t ci = C[i];
-    unsigned long long o = g.off[i];
-    uint32_t d = g.deg[i];
-    for (uint32_t k = lane; k < d; k += 32) {
-      uint2 a = g.arcs[o + k];
-      if (C[a.x] == ci) sig += a.y;
+  const uint64_t warp = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) >> 5;
+  const uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
+  unsigned long long tot = 0;
+  for (uint64_t b = r.v0 + warp * 32; b < r.v1; b += nwarps * 32) {
+    const uint64_t i = b + lane;
+    const bool ok = i < r.v1;
+    const unsigned long long o = ok ? r.g.off[i] : 0ull;
+    uint32_t d = ok ? r.g.deg[i] : 0u;
+    const uint32_t ci = kInside && ok ? r.C[i] : 0u;
+    if (d > kRowHub) {
+      push_row(r.hubs, &r.ctrl->long_rows, uint32_t(i), (d + kRowPiece - 1) / kRowPiece);
+      d = 0;
+    }
+    unsigned long long mine = 0;  // row b + lane
+    for (uint32_t s = 0; s < 8; ++s) {
+      const int src = int(s * 4 + (lane >> 3));
+      const unsigned long long os = __shfl_sync(0xFFFFFFFFu, o, src);
+      const uint32_t ds = __shfl_sync(0xFFFFFFFFu, d, src), cs = __shfl_sync(0xFFFFFFFFu, ci, src);
+      unsigned long long sum = r.part(os, cs, 0, ds <= kRowShort ? ds : 0u, lane & 7u, 8);
+      if constexpr (kInside) {
+        tot += sum;
+      } else {
+        sum = lanes_sum(sum, 8);
+        sum = __shfl_sync(0xFFFFFFFFu, sum, int((lane & 3u) * 8));
+        if ((lane >> 2) == s) mine = sum;
+      }
+    }
+    for (unsigned m = __ballot_sync(0xFFFFFFFFu, d > kRowShort); m; m &= m - 1) {
+      const int src = __ffs(m) - 1;
+      const unsigned long long os = __shfl_sync(0xFFFFFFFFu, o, src);
+      const uint32_t ds = __shfl_sync(0xFFFFFFFFu, d, src), cs = __shfl_sync(0xFFFFFFFFu, ci, src);
+      unsigned long long sum = r.part(os, cs, 0, ds, lane, 32);
+      if constexpr (kInside) {
+        tot += sum;
+      } else {
+        sum = lanes_sum(sum, 32);
+        if (int(lane) == src) mine = sum;
+      }
+    }
+    if constexpr (!kInside) {
+      if (ok) r.K[i] = (long long)mine;  // (a queued hub's pieces are added by k_row_hubs)
+      tot += mine;
     }
   }
-  unsigned long long lo = 0, hi = 0;
-  for (uint64_t c = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; c < n;
-       c += uint64_t(gridDim.x) * blockDim.x) {
-    unsigned long long s = (unsigned long long)Sigma[c];
-    u128 sq = (u128)s * s;
-    lo += (unsigned long long)(sq & 0xFFFFFFFFull);
-    hi += (unsigned long long)(sq >> 32);
+  tot = lanes_sum(tot, 32);
+  if (lane == 0 && tot) atomicAdd(&r.ctrl->red_a, tot);
+  if constexpr (kInside) {
+    unsigned long long lo = 0, hi = 0;
+    for (uint64_t c = r.v0 + blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; c < r.v1;
+         c += uint64_t(gridDim.x) * blockDim.x) {
+      const unsigned long long s = (unsigned long long)r.Sigma[c];
+      const u128 sq = (u128)s * s;
+      lo += (unsigned long long)(sq & 0xFFFFFFFFull);
+      hi += (unsigned long long)(sq >> 32);
+    }
+    lo = lanes_sum(lo, 32);
+    hi = lanes_sum(hi, 32);
+    if (lane == 0) {
+      if (lo) atomicAdd(&r.ctrl->red_b, lo);
+      if (hi) atomicAdd(&r.ctrl->red_c, hi);
+    }
   }
-  for (int x = 16; x; x >>= 1) {
-    sig += __shfl_xor_sync(0xFFFFFFFFu, sig, x);
-    lo += __shfl_xor_sync(0xFFFFFFFFu, lo, x);
-    hi += __shfl_xor_sync(0xFFFFFFFFu, hi, x);
+}
+
+// The queued rows, a warp per piece of kRowPiece arcs.
+template <bool kInside>
+__global__ void __launch_bounds__(kRowThreads) k_row_hubs(RowSums<kInside> r) {
+  pdl_wait_only();
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t rows = uint32_t(r.ctrl->long_rows >> 32), pieces = uint32_t(r.ctrl->long_rows);
+  const uint32_t nwarps = gridDim.x * (kRowThreads / 32);
+  unsigned long long tot = 0;
+  for (uint64_t p = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5); p < pieces; p += nwarps) {
+    const uint2 e = r.hubs[find_row(r.hubs, rows, uint32_t(p))];
+    const uint32_t k0 = (uint32_t(p) - e.y) * kRowPiece, d = r.g.deg[e.x];
+    const uint32_t k1 = d - k0 < kRowPiece ? d : k0 + kRowPiece;
+    unsigned long long sum = r.part(r.g.off[e.x], kInside ? r.C[e.x] : 0u, k0, k1, lane, 32);
+    tot += sum;
+    if constexpr (!kInside) {
+      sum = lanes_sum(sum, 32);
+      if (lane == 0 && sum) atomicAdd((unsigned long long*)&r.K[e.x], sum);
+    }
   }
-  if (lane == 0) {
-    if (sig) atomicAdd(&ctrl->red_a, sig);
-    if (lo) atomicAdd(&ctrl->red_b, lo);
-    if (hi) atomicAdd(&ctrl->red_c, hi);
+  tot = lanes_sum(tot, 32);
+  if (lane == 0 && tot) atomicAdd(&r.ctrl->red_a, tot);
+}
+
+template <bool kInside>
+int row_sums(Handle* h, const RowSums<kInside>& r) {
+  // red_a, red_b, red_c and long_rows are adjacent
+  DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->red_a, 0, 4 * sizeof(unsigned long long), h->stream));
+  if (r.v1 <= r.v0) return DFL_OK;
+  {
+    LaunchScope ls(h, DFL_PROF_OTHER);
+    k_row_sums<kInside><<<grid_for(r.v1 - r.v0, kRowThreads, 152 * 8), kRowThreads, 0, h->stream>>>(r);
+    DFL_TRY(check_launch(h, "row sums"));
   }
+  if (h->max_deg <= kRowHub) return DFL_OK;  // (an upper bound: no row can have been queued)
+  LaunchScope ls(h, DFL_PROF_OTHER);
+  launch_pdl(k_row_hubs<kInside>, 152 * 6, kRowThreads, 0, h->stream, r);
+  return check_launch(h, "row sums of hubs");
 }
 
 __global__ void k_sigma_sizes(uint32_t n, const uint32_t* __restrict__ C,
@@ -221,31 +332,19 @@ int recompute_aux(Handle* h) {
 }
 
 int weighted_degrees(Handle* h) {
-  DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->red_a, 0, sizeof(unsigned long long), h->stream));
-  {
-    LaunchScope ls(h, DFL_PROF_OTHER);
-    k_weighted_degree<<<grid_for(uint64_t(h->n) * 32, 256), 256, 0, h->stream>>>(base_view(h), h->K,
-                                                                                  h->ctrl);
-    DFL_TRY(check_launch(h, "weighted degree"));
-  }
+  DFL_TRY(row_sums(h, RowSums<false>{base_view(h), nullptr, nullptr, h->K, 0u, h->n, row_queue(h), h->ctrl}));
   DFL_TRY(read_ctrl(h));
   h->m2 = (long long)h->hctrl->red_a;
   return DFL_OK;
 }
 
-int modularity_parts(Handle* h, i128* num, i128* den) {
-  DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->red_a, 0, 3 * sizeof(unsigned long long), h->stream));
-  {
-    LaunchScope ls(h, DFL_PROF_OTHER);
-    k_modularity<<<grid_for(uint64_t(h->n) * 32, 256), 256, 0, h->stream>>>(base_view(h), h->C,
-                                                                             h->Sigma, h->n, h->ctrl);
-    DFL_TRY(check_launch(h, "modularity"));
-  }
+int modularity_range(Handle* h, uint32_t v0, uint32_t v1, long long m2, i128* num, i128* den) {
+  DFL_TRY(row_sums(h, RowSums<true>{base_view(h), h->C, h->Sigma, nullptr, v0, v1, row_queue(h), h->ctrl}));
   DFL_TRY(read_ctrl(h));
-  i128 sig = (i128)h->hctrl->red_a;
-  i128 sq = ((i128)h->hctrl->red_c << 32) + (i128)h->hctrl->red_b;
-  *num = (i128)h->m2 * sig - sq;
-  *den = (i128)h->m2 * (i128)h->m2;
+  const i128 sig = (i128)h->hctrl->red_a;
+  const i128 sq = ((i128)h->hctrl->red_c << 32) + (i128)h->hctrl->red_b;
+  *num = (i128)m2 * sig - sq;
+  *den = (i128)m2 * (i128)m2;
   return DFL_OK;
 }
 

@@ -50,43 +50,6 @@ __global__ void k_group_m2_store(const unsigned long long* __restrict__ sum, lon
     gm2[g] = (long long)sum[g];
 }
 
-// sigma (arcs inside communities) over rows [v0, v1) and sum of Sigma_c^2
-// over labels [v0, v1): graph g's share of Eq. 1.
-__global__ void k_range_modularity(GraphView g, const uint32_t* __restrict__ C,
-                                   const long long* __restrict__ Sigma, uint32_t v0, uint32_t v1,
-                                   Ctrl* ctrl) {
-  const uint32_t lane = threadIdx.x & 31u;
-  uint64_t warp = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) >> 5;
-  uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-  unsigned long long sig = 0;
-  for (uint64_t i = v0 + warp; i < v1; i += nwarps) {
-    const uint32_t ci = C[i];
-    const unsigned long long o = g.off[i];
-    const uint32_t dg = g.deg[i];
-    for (uint32_t k = lane; k < dg; k += 32) {
-      uint2 arc = g.arcs[o + k];
-      if (arc.y && C[arc.x] == ci) sig += arc.y;
-    }
-  }
-  unsigned long long lo = 0, hi = 0;
-  for (uint64_t c = v0 + blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; c < v1;
-       c += uint64_t(gridDim.x) * blockDim.x) {
-    u128 sq = (u128)(unsigned long long)Sigma[c] * (unsigned long long)Sigma[c];
-    lo += (unsigned long long)(sq & 0xFFFFFFFFull);
-    hi += (unsigned long long)(sq >> 32);
-  }
-  for (int x = 16; x; x >>= 1) {
-    sig += __shfl_xor_sync(0xFFFFFFFFu, sig, x);
-    lo += __shfl_xor_sync(0xFFFFFFFFu, lo, x);
-    hi += __shfl_xor_sync(0xFFFFFFFFu, hi, x);
-  }
-  if (lane == 0) {
-    if (sig) atomicAdd(&ctrl->red_a, sig);
-    if (lo) atomicAdd(&ctrl->red_b, lo);
-    if (hi) atomicAdd(&ctrl->red_c, hi);
-  }
-}
-
 // next[g] = new id of the first label of graph g (the renumbering's
 // exclusive scan at the range start).
 __global__ void k_gather_starts(uint32_t ng, const uint32_t* __restrict__ goff,
@@ -181,22 +144,7 @@ int group_m2_take(Handle* h) {
 }
 
 int group_modularity(Handle* h, uint32_t g, i128* num, i128* den) {
-  const uint32_t v0 = h->goff0[g], v1 = h->goff0[g + 1];
-  DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->red_a, 0, 3 * sizeof(unsigned long long), h->stream));
-  if (v1 > v0) {
-    LaunchScope ls(h, DFL_PROF_OTHER);
-    k_range_modularity<<<grid_for(uint64_t(v1 - v0) * 32, 256), 256, 0, h->stream>>>(
-        base_view(h), h->C, h->Sigma, v0, v1, h->ctrl);
-    DFL_TRY(check_launch(h, "group modularity"));
-  }
-  DFL_CUDA(h, cudaMemcpyAsync(h->hctrl, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
-  DFL_CUDA(h, cudaStreamSynchronize(h->stream));
-  const i128 m2 = (i128)h->gm2[g];
-  const i128 sig = (i128)h->hctrl->red_a;
-  const i128 sq = ((i128)h->hctrl->red_c << 32) + (i128)h->hctrl->red_b;
-  *num = m2 * sig - sq;
-  *den = m2 * m2;
-  return DFL_OK;
+  return modularity_range(h, h->goff0[g], h->goff0[g + 1], h->gm2[g], num, den);
 }
 
 int louvain_group(Handle* h, bool all, bool use_range, uint64_t initial) {

@@ -59,6 +59,18 @@ def random_graph(n, m, seed, w_max=9):
                           rng.integers(1, w_max + 1, key.size).astype(np.uint32))
 
 
+def stars(degrees, leaves, seed):
+    """One centre per degree, joined to the first `degree` of a shared pool of
+    leaves, which are also joined in a ring (so that centres meet many
+    communities and leaves have choices)."""
+    rng = np.random.default_rng(seed)
+    c = len(degrees)
+    u = np.concatenate([np.full(d, k) for k, d in enumerate(degrees)] + [c + np.arange(leaves)])
+    v = np.concatenate([c + rng.permutation(leaves)[:d] for d in degrees] + [c + (np.arange(leaves) + 1) % leaves])
+    return synth.EdgeList(c + leaves, np.minimum(u, v).astype(np.uint32), np.maximum(u, v).astype(np.uint32),
+                          rng.integers(1, 20, u.size).astype(np.uint32))
+
+
 @pytest.mark.parametrize("n", [1, 31, 2047, 2049, 8191, 8200, 20_011])
 @pytest.mark.parametrize("density", [0.002, 0.2, 1.0])
 def test_frontier_lists_at_tile_edges(dfl, orc, n, density):
@@ -78,4 +90,16 @@ def test_frontier_lists_at_tile_edges(dfl, orc, n, density):
     assert np.array_equal(Fa, Fb) and np.array_equal(ma, mb) and Sa == Sb
     a.static()
     b.static()
+    same(a, b)
+
+
+@pytest.mark.parametrize("degrees", [(64, 65), (1023, 1024, 1025), (2048, 4097, 1), (1030,) * 40])
+def test_row_sums_of_hubs(dfl, orc, degrees):
+    """K, 2m and the modularity at the row lengths where a row takes the
+    whole warp, and where it is queued and cut into pieces."""
+    g = stars(degrees, 4100, 3)
+    a, b = pair(dfl, orc, g)
+    C = np.random.default_rng(1).integers(0, 50, g.n).astype(np.uint32)
+    a.set_membership(C)
+    b.set_membership(C)
     same(a, b)
