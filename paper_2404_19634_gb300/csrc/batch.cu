@@ -528,25 +528,63 @@ __global__ void k_ds_best(const unsigned long long* __restrict__ key, const uint
   }
 }
 
-// Alg. 3: neighbours of dE vertices join dV (warp per bitmap word).
-__global__ void k_ds_expand(const uint32_t* __restrict__ dE, uint32_t words, uint32_t n,
-                            GraphView g, uint32_t* dV) {
+// Alg. 3: neighbours of dE vertices join dV.  A warp takes a bitmap word and
+// walks the rows of its vertices; rows longer than kDsHub are queued (in
+// `hubs`, ctrl->long_rows) for k_ds_hubs, which spreads their arcs over
+// every block: a hub's tens of thousands of arcs walked by the one warp that
+// met it held up the kernel (161 us on a 2^20-vertex R-MAT graph with an
+// 839-edge batch; now 11 us, and 12 us for the hubs).
+constexpr uint32_t kDsHub = 512, kDsPiece = 512;
+constexpr int kDsThreads = 256;
+
+__device__ __forceinline__ void ds_mark(uint32_t* dV, uint2 a) {
+  // weight 0 = deleted arc; the bit is read first, so a vertex met often takes one atomic
+  if (a.y && !bit_test(dV, a.x)) bit_set(dV, a.x);
+}
+
+__global__ void __launch_bounds__(kDsThreads) k_ds_expand(const uint32_t* __restrict__ dE, uint32_t words, uint32_t n,
+                                                          GraphView g, uint32_t* dV, uint2* hubs, Ctrl* ctrl) {
   const uint32_t lane = threadIdx.x & 31u;
   uint64_t warp = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) >> 5;
   uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
   for (uint64_t wd = warp; wd < words; wd += nwarps) {
-    uint32_t x = dE[wd];
-    while (x) {
-      int b = __ffs(x) - 1;
-      x &= x - 1;
-      uint32_t i = uint32_t(wd * 32 + b);
-      if (i >= n) break;
-      unsigned long long o = g.off[i];
-      uint32_t d = g.deg[i];
-      for (uint32_t k = lane; k < d; k += 32) {
-        uint2 a = g.arcs[o + k];
-        if (a.y) bit_set(dV, a.x);  // weight 0 = deleted arc
-      }
+    const uint32_t x = dE[wd];
+    if (!x) continue;
+    // each lane's vertex of the word, if it is set: the headers at once
+    const uint32_t i = uint32_t(wd * 32 + lane);
+    const bool in = i < n && ((x >> lane) & 1u);
+    const unsigned long long o = in ? g.off[i] : 0ull;
+    uint32_t d = in ? g.deg[i] : 0u;
+    if (d > kDsHub) {
+      push_row(hubs, &ctrl->long_rows, i, (d + kDsPiece - 1) / kDsPiece);
+      d = 0;
+    }
+    for (unsigned m = __ballot_sync(0xFFFFFFFFu, d > 0); m; m &= m - 1) {
+      const int src = __ffs(m) - 1;
+      const unsigned long long os = __shfl_sync(0xFFFFFFFFu, o, src);
+      const uint32_t ds = __shfl_sync(0xFFFFFFFFu, d, src);
+      for (uint32_t k = lane; k < ds; k += 32) ds_mark(dV, g.arcs[os + k]);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kDsThreads) k_ds_hubs(GraphView g, uint32_t* dV, const uint2* __restrict__ hubs,
+                                                        const Ctrl* ctrl) {
+  pdl_wait_only();
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t rows = uint32_t(ctrl->long_rows >> 32), pieces = uint32_t(ctrl->long_rows);
+  const uint32_t nwarps = gridDim.x * (kDsThreads / 32);
+  for (uint64_t p = blockIdx.x * (kDsThreads / 32) + (threadIdx.x >> 5); p < pieces; p += nwarps) {
+    const uint2 e = hubs[find_row(hubs, rows, uint32_t(p))];
+    const uint32_t k0 = (uint32_t(p) - e.y) * kDsPiece, d = g.deg[e.x];
+    const uint32_t k1 = d - k0 < kDsPiece ? d : k0 + kDsPiece;
+    const unsigned long long o = g.off[e.x];
+    for (uint32_t b = k0 + lane; b < k1; b += 128) {
+      uint2 a[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] = b + u * 32 < k1 ? g.arcs[o + b + u * 32] : make_uint2(0u, 0u);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) ds_mark(dV, a[u]);
     }
   }
 }
@@ -1762,9 +1800,14 @@ int mark(Handle* h, int mode, bool* all, bool* use_range, uint64_t* initial) {
     }
     {
       LaunchScope ls(h, DFL_PROF_MARK);
-      k_ds_expand<<<grid_for(uint64_t(h->words) * 32, 256), 256, 0, h->stream>>>(
-          h->dsE, h->words, n, base_view(h), h->dsV);
+      k_ds_expand<<<grid_for(uint64_t(h->words) * 32, kDsThreads), kDsThreads, 0, h->stream>>>(
+          h->dsE, h->words, n, base_view(h), h->dsV, row_queue(h), h->ctrl);
       DFL_TRY(check_launch(h, "ds expand"));
+    }
+    if (h->max_deg > kDsHub) {  // (an upper bound: otherwise no row can have been queued)
+      LaunchScope ls(h, DFL_PROF_MARK);
+      launch_pdl(k_ds_hubs, 152 * 4, kDsThreads, 0, h->stream, base_view(h), h->dsV, row_queue(h), h->ctrl);
+      DFL_TRY(check_launch(h, "ds expand hubs"));
     }
     {
       LaunchScope ls(h, DFL_PROF_MARK);

@@ -103,3 +103,31 @@ def test_row_sums_of_hubs(dfl, orc, degrees):
     a.set_membership(C)
     b.set_membership(C)
     same(a, b)
+
+
+@pytest.mark.parametrize("degrees", [(512, 513), (1024, 1025, 3), (4000, 600, 511)])
+def test_delta_screening_marks_hub_neighbours(dfl, orc, degrees):
+    g = stars(degrees, 4100, 5)
+    a, b = pair(dfl, orc, g)
+    a.static()
+    b.static()
+    c = len(degrees)
+    C = a.membership()
+    # each centre loses an edge inside its community and gains one across
+    dels, ins = [], []
+    for k in range(c):
+        row = np.concatenate([g.v[g.u == k], g.u[g.v == k]])
+        inside = row[C[row] == C[k]]
+        if inside.size:
+            dels.append((k, inside[0], 0))
+        other = np.flatnonzero(C != C[k])
+        if other.size:
+            ins.append((k, other[-1 - k], 2))
+    dels, ins = np.array(dels, np.uint32).reshape(-1, 3), np.array(ins, np.uint32).reshape(-1, 3)
+    assert dels.size + ins.size
+    assert a.apply_batch(dels, ins) == 0 and b.apply_batch(dels, ins) == 0
+    for x, y in zip(a.mark(1), b.mark(1)):
+        assert np.array_equal(x, y)
+    a.update(1)
+    b.update(1)
+    same(a, b)
