@@ -31,8 +31,12 @@ typedef unsigned __int128 u128;
 // Compile-time configuration
 // ---------------------------------------------------------------------------
 constexpr int kWarp = 32;
-constexpr int kBins = 4;            // degree bins of the local-moving kernels
-constexpr uint32_t kBinWarp = 32;   // deg <= 32: registers only (largest bin-0 limit)
+// Degree bins of the local-moving kernels: registers (a few arcs), registers
+// (up to 32 arcs, one or two lanes a vertex), a warp's shared table, a block's
+// shared table, chunks summed in a global table.
+constexpr int kBins = 5;
+enum : int { kBinTiny = 0, kBinLanes = 1, kBinTable = 2, kBinWhole = 3, kBinHuge = 4 };
+constexpr uint32_t kBinWarp = 32;   // deg <= 32: registers only (largest bin-0 limit, and the lane bin's)
 constexpr uint32_t kBinWarpDefault = 8;  // default bin-0 limit: 8 lanes per vertex, 4 vertices a warp
 constexpr uint32_t kBinWarpHash = 256;   // deg <= 256: one warp, shared-memory table
 constexpr uint32_t kBinBlock = 4096;     // deg <= 4096: one block, shared-memory table
@@ -119,7 +123,7 @@ struct SuperGraph {
 struct Segs {
   uint32_t off[kMaxSubsteps * kBins];
   uint32_t cap[kMaxSubsteps * kBins];
-  uint32_t hi[kBins - 1];  // largest degree of bins 0..2 (tuning; bin 3 takes the rest)
+  uint32_t hi[kBins - 1];  // largest degree of every bin but the last, which takes the rest (tuning)
   // group: a vertex's sub-step class comes from its id within its own graph
   // (first vertex of each graph at the current level, device memory)
   const uint32_t* goff;
@@ -260,9 +264,9 @@ struct Handle {
   uint64_t g_lst_cap = 0;
 
   // auxiliary streams for the concurrent degree bins of a sub-step
-  cudaStream_t aux[kBins - 1] = {nullptr, nullptr, nullptr};
+  cudaStream_t aux[kBins - 1] = {};
   cudaEvent_t ev_fork = nullptr;
-  cudaEvent_t ev_join[kBins - 1] = {nullptr, nullptr, nullptr};
+  cudaEvent_t ev_join[kBins - 1] = {};
 
   // control
   Ctrl* ctrl = nullptr;       // device
@@ -450,7 +454,7 @@ __device__ __forceinline__ uint32_t vertex_class(uint32_t v, uint32_t k, const S
 }
 
 __host__ __device__ __forceinline__ uint32_t degree_bin(uint32_t d, const Segs& s) {
-  return d <= s.hi[0] ? 0u : d <= s.hi[1] ? 1u : d <= s.hi[2] ? 2u : 3u;
+  return d <= s.hi[0] ? 0u : d <= s.hi[1] ? 1u : d <= s.hi[2] ? 2u : d <= s.hi[3] ? 3u : 4u;
 }
 
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
@@ -779,12 +783,13 @@ struct MoveArgs {
   // batch arcs); chooses launch shapes for a replayed first iteration
   uint64_t frontier_hint = ~0ull;
 };
-// A frontier list of a sub-step class shorter than this is decided by the
-// per-vertex kernels of bin 0 (W lanes a vertex) instead of the
-// thread-per-vertex kernel: with few vertices the latter leaves the SMs to
+// A list of a sub-step class shorter than this is decided with several lanes
+// per vertex (W lanes in bin 0, a warp in the lane bin) instead of a lane per
+// vertex: with few vertices the latter leaves the SMs to
 // the largest-degree chain less well (R-MAT 2^22, DF at 1e-3|E|: 0.44 vs
 // 0.49-0.52 ms per batch), while on full frontiers it is the faster one.
 constexpr uint64_t kSmallList = 32768;
+constexpr uint64_t kSmallLanes = 8192;  // the lane bin's vertices weigh four of bin 0's
 // Below this many pending batch arcs a DF or DS update launches its
 // iterations from the host even when graph replay is allowed: a frontier of
 // a few vertices leaves most bins empty, and skipping them beats replaying

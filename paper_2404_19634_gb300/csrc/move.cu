@@ -173,7 +173,7 @@ __device__ __forceinline__ void mark_next(const DecideArgs& a, uint32_t j, bool 
 // warp decides 32 / W vertices at once, one arc per lane; aggregation by
 // community in registers inside each W-lane segment (W shuffles and
 // compares).  A long bin-0 list instead takes a vertex per thread
-// (k_decide_thread, below).
+// (k_decide_lanes, below).
 // ---------------------------------------------------------------------------
 
 // Argmax of (score, -c) over the aligned W-lane segment of each lane.
@@ -252,30 +252,45 @@ __device__ __forceinline__ bool decide_segment(const DecideArgs& a, bool active,
   return mv;
 }
 
+// Vertices [first, cnt) of the list, 32 / W of them per warp.
 template <int W>
-__global__ void __launch_bounds__(256, 5) k_decide_warp(DecideArgs a) {
+__device__ __forceinline__ void decide_segments(const DecideArgs& a, uint64_t first, uint32_t cnt, long long m2_one,
+                                                MoveSums& sums) {
+  const uint32_t lane = threadIdx.x & 31u, seg = lane / W, sl = lane % W;
+  const uint64_t t = first + seg;
+  bool active = t < cnt;
+  const uint32_t i = active ? a.list[t] : 0u;
+  long long m2 = m2_one;
+  uint32_t gi = 0;
+  if (active && !group_active(a, i, &m2, &gi)) active = false;
+  if (active && sl == 0) {
+    if (a.ever && bit_set(a.ever, i)) ++sums.ever;
+    ++sums.processed;
+  }
+  if (active && a.rbits && !bit_test(a.rbits, i)) active = false;  // processed, not in range
+  decide_segment<W>(a, active, i, m2, gi, sums);
+}
+
+// Short lists of small vertices: W lanes per vertex of the first list, then
+// (list2, if given) a warp per vertex of a second one, whose vertices are
+// dealt to the warps from the last one down.  One launch for both: each would
+// leave most of the GPU idle.
+template <int W>
+__global__ void __launch_bounds__(256, 5) k_decide_warp(DecideArgs a, const uint32_t* list2,
+                                                        const unsigned int* count2) {
   constexpr uint32_t kSegs = 32 / W;
   const long long m2_one = *a.m2p;
-  const uint32_t lane = threadIdx.x & 31u, seg = lane / W, sl = lane % W;
-  const uint32_t cnt = *a.count;
+  const uint32_t cnt = *a.count, cnt2 = count2 ? *count2 : 0u;
+  // a block without a vertex leaves at once (a replayed graph's grids are fixed)
+  const uint64_t bw = blockDim.x >> 5;
+  if (blockIdx.x * bw * kSegs >= cnt && (gridDim.x - 1 - blockIdx.x) * bw >= cnt2) return;
   const uint64_t warp = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) >> 5;
   const uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
   MoveSums sums;
-  for (uint64_t t0 = warp * kSegs; t0 < cnt; t0 += nwarps * kSegs) {
-    const uint64_t t = t0 + seg;
-    bool active = t < cnt;
-    const uint32_t i = active ? a.list[t] : 0u;
-    long long m2 = m2_one;
-    uint32_t gi = 0;
-    if (active && !group_active(a, i, &m2, &gi)) active = false;
-    if (active && sl == 0) {
-      if (a.ever && bit_set(a.ever, i)) ++sums.ever;
-      ++sums.processed;
-    }
-    if (active && a.rbits && !bit_test(a.rbits, i)) active = false;  // processed, not in range
-    decide_segment<W>(a, active, i, m2, gi, sums);
-  }
-  flush_sums(a, sums, sl == 0);
+  for (uint64_t t0 = warp * kSegs; t0 < cnt; t0 += nwarps * kSegs) decide_segments<W>(a, t0, cnt, m2_one, sums);
+  a.list = list2;
+  for (uint64_t t = nwarps - 1 - warp; t < cnt2; t += nwarps) decide_segments<32>(a, t, cnt2, m2_one, sums);
+  flush_sums(a, sums, (threadIdx.x & 31u) % W == 0);
 }
 
 // Open-addressing insert (linear probing) of weight w under key c; gives up
@@ -562,17 +577,6 @@ __device__ __forceinline__ bool decide64(const DecideArgs& a, const VHdr& v, boo
   return true;
 }
 
-// The same in 128 bits (vertices whose 2m * K_i reaches 2^63).
-__device__ __forceinline__ bool decide128(const DecideArgs& a, const VHdr& v, bool have, i128 best, uint32_t bc,
-                                          uint32_t Hd, i128* gain) {
-  if (!have) return false;
-  const i128 stay = gain_num(v.m2, Hd, v.Ki, v.Sd - v.Ki);
-  if (!(best > stay)) return false;
-  if (v.szd == 1 && bc > v.d && a.size[bc] == 1) return false;
-  *gain = best - stay;
-  return true;
-}
-
 // record_move for every mover lane of the warp with one slot reservation.
 // Every lane of the warp calls it.
 __device__ __forceinline__ void record_moves_warp(const DecideArgs& a, bool mv, uint32_t i, uint32_t c,
@@ -601,131 +605,167 @@ __device__ __forceinline__ void record_moves_warp(const DecideArgs& a, bool mv, 
 }
 
 // ---------------------------------------------------------------------------
-// Bin 0: one thread per vertex (degree <= D), its arcs, their communities and
-// the community weights in registers; the weight of a community is summed
-// by its first arc over the others (D x D compares, no table, no shuffles).
+// Long lists of small vertices (bins 0 and 1: at most 32 arcs): a lane per
+// vertex.  Issue slots bound these kernels (the gathers of 32 vertices are in
+// flight together), so the communities are grouped by a sorting network over
+// registers instead of comparing every pair: a key is (community << 5 | arc),
+// one 32-bit word, so a comparator is a min and a max, and the arcs' weights
+// wait in shared memory until their order is known.  A run of equal
+// communities is scored at its last key; runs come in ascending order, so the
+// first best wins the tie.
+// On 100,000 vertices of mean degree 16 (one sub-step of a 400,000-vertex
+// graph) a warp per vertex, with a shuffle and compare round per arc, issued
+// 354 instructions a vertex and took 65 us; a lane or two per vertex comparing
+// all pairs 165 and 60 us; this 91 and 40 us (492,000 vertices: 414 -> 226 us).
 // ---------------------------------------------------------------------------
+constexpr uint32_t kLaneLabels = (1u << 27) - 1;  // labels below this fit a key (and ~0 is none of theirs)
+constexpr int kLaneThreads = 128;
 
-// Best candidate over the thread's community weights (hw[k] > 0: arc k is the
-// first of a candidate community c[k]) and the move decision.
-template <int D, bool F64>
-__device__ __forceinline__ bool thread_decide(const DecideArgs& a, const VHdr& h, const uint32_t* c,
-                                              const uint32_t* hw, const uint32_t* sg, uint32_t Hd, uint32_t* bco,
-                                              i128* gain) {
-  bool have = false;
-  uint32_t bc = 0;
-  typename std::conditional<F64, unsigned long long, i128>::type best = 0;
+// Batcher's odd-even merge sort of N keys, ascending: the comparators of stage
+// (P, K) join i and i + K within blocks of 2P.
+template <int N, int P = 1, int K = 1>
+__device__ __forceinline__ void sort_keys(uint32_t (&x)[N]) {
 #pragma unroll
-  for (int k = 0; k < D; ++k) {
-    if (!hw[k]) continue;
-    decltype(best) sc;
-    if constexpr (F64) sc = score64(h.m2, hw[k], h.Ki, sg[k]);
-    else sc = gain_num(h.m2, hw[k], h.Ki, sg[k]);
-    if (!have || sc > best || (sc == best && c[k] < bc)) {
-      have = true;
-      best = sc;
-      bc = c[k];
+  for (int i = 0; i < N; ++i)
+    if (i >= K % P && (i - K % P) % (2 * K) < K && i + K < N && i / (2 * P) == (i + K) / (2 * P)) {
+      const uint32_t lo = min(x[i], x[i + K]), hi = max(x[i], x[i + K]);
+      x[i] = lo;
+      x[i + K] = hi;
+    }
+  if constexpr (K > 1) sort_keys<N, P, K / 2>(x);
+  else if constexpr (2 * P < N) sort_keys<N, 2 * P, 2 * P>(x);
+}
+
+// Decision of this lane's vertex v (if v.act; at most D arcs, scores in 64
+// bits).  `w`: this lane's column of the warp's weights, 32 words apart.  Rows
+// start 16-byte aligned and have an even capacity, so the pair of an odd last
+// arc is readable.
+template <int D>
+__device__ __forceinline__ bool lane_vertex(const DecideArgs& a, const VHdr& v, uint32_t* w, uint32_t* bco,
+                                            unsigned long long* gain, uint32_t* ncand) {
+  const uint4* row = reinterpret_cast<const uint4*>(a.g.arcs + v.o);
+  const uint32_t dg = v.act ? v.dg : 0u;
+  uint32_t key[D];
+#pragma unroll
+  for (int q = 0; q < D / 2; ++q) {
+    const uint4 x = 2 * q < dg ? row[q] : make_uint4(v.i, 0u, v.i, 0u);
+    // self-loops and deleted arcs (weight 0) are no arcs
+    key[2 * q] = x.y ? x.x : v.i;
+    key[2 * q + 1] = (x.w && 2 * q + 1 < dg) ? x.z : v.i;
+    w[(2 * q) * 32] = x.y;
+    w[(2 * q + 1) * 32] = x.w;
+  }
+#pragma unroll
+  for (int k = 0; k < D; ++k) key[k] = key[k] != v.i ? (a.C[key[k]] << 5) | uint32_t(k) : kEmpty;
+  sort_keys<D>(key);
+  uint32_t Hd = 0, nc = 0, run = 0, bc = kEmpty;
+  unsigned long long best = 0;  // (a candidate's score' is at least 1)
+#pragma unroll
+  for (int k0 = 0; k0 < D; k0 += 8) {  // eight runs' Sigma in flight
+    uint32_t sg[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = k0 + u;
+      const uint32_t c = key[k] >> 5;
+      const bool last = key[k] != kEmpty && (k + 1 == D || (key[k + 1 < D ? k + 1 : k] >> 5) != c);
+      sg[u] = (last && c != v.d) ? sigma32(a.Sigma, c) : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = k0 + u;
+      const uint32_t c = key[k] >> 5;
+      const bool last = key[k] != kEmpty && (k + 1 == D || (key[k + 1 < D ? k + 1 : k] >> 5) != c);
+      run += key[k] != kEmpty ? w[(key[k] & 31u) * 32] : 0u;
+      if (last) {
+        if (c == v.d) {
+          Hd = run;
+        } else {
+          ++nc;
+          const unsigned long long sc = score64(v.m2, run, v.Ki, sg[u]);
+          if (sc > best) {
+            best = sc;
+            bc = c;
+          }
+        }
+        run = 0;
+      }
     }
   }
   *bco = bc;
-  if constexpr (F64) return decide64(a, h, have, best, bc, Hd, gain);
-  else return decide128(a, h, have, best, bc, Hd, gain);
+  *ncand = nc;
+  i128 g = 0;
+  const bool mv = v.act && decide64(a, v, bc != kEmpty, best, bc, Hd, &g);
+  *gain = (unsigned long long)g;  // a gain is positive and below 2^64
+  return mv;
 }
 
+// The neighbours of a mover (its arcs again, cached), marked by one lane: four
+// arcs' bitmap words in flight.
+__device__ __forceinline__ void mark_row(const DecideArgs& a, uint32_t i, unsigned long long o, uint32_t dg) {
+  for (uint32_t k0 = 0; k0 < dg; k0 += 4) {
+    uint2 e[4];
+    bool on[4];
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) e[u] = k0 + u < dg ? a.g.arcs[o + k0 + u] : make_uint2(i, 0u);
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u)
+      on[u] = e[u].x != i && e[u].y != 0 && (!a.rbits || bit_test(a.rbits, e[u].x)) && !bit_test(a.fbits_next, e[u].x);
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u)
+      if (on[u]) bit_set(a.fbits_next, e[u].x);
+  }
+}
+
+// The rare vertices whose scores need 128 bits, a warp each, out of line.
+__device__ __noinline__ void lane_vertices_128(const DecideArgs& a, const VHdr& h, unsigned m, MoveSums& sums) {
+  for (; m; m &= m - 1) {
+    const VHdr v = shfl_header(h, __ffs(m) - 1);
+    decide_segment<32>(a, true, v.i, v.m2, v.gi, sums);
+  }
+}
+
+// Vertices of at most D arcs (D = 8, or 32: a warp with no vertex over 16 arcs
+// sorts 16 keys).  Labels must be below kLaneLabels.
 template <int D>
-__global__ void __launch_bounds__(256, 3) k_decide_thread(DecideArgs a) {
+__global__ void __launch_bounds__(kLaneThreads, D == 8 ? 8 : 5) k_decide_lanes(DecideArgs a) {
+  __shared__ uint32_t s_w[kLaneThreads / 32][D][32];
   const long long m2_one = *a.m2p;
   const uint32_t cnt = *a.count;
+  if (blockIdx.x * uint64_t(blockDim.x) >= cnt) return;  // no vertex for this block
   const uint32_t lane = threadIdx.x & 31u;
+  uint32_t* w = &s_w[threadIdx.x >> 5][0][lane];
   const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
   MoveSums sums;
   for (uint64_t t0 = blockIdx.x * uint64_t(blockDim.x) + (threadIdx.x & ~31u); t0 < cnt; t0 += stride) {
     const uint64_t t = t0 + lane;  // warp-uniform loop: the movers are recorded per warp
     VHdr h;
     load_header(a, t, t < cnt, m2_one, sums, h);
-    uint2 arc[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) arc[k] = (h.act && uint32_t(k) < h.dg) ? a.g.arcs[h.o + k] : make_uint2(h.i, 0u);
-    uint32_t c[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) c[k] = (arc[k].x != h.i && arc[k].y != 0) ? a.C[arc[k].x] : kEmpty;
-    // hw[k]: weight of candidate community c[k] if arc k is its first arc, else 0
-    uint32_t hw[D];
-    uint32_t Hd = 0, ncand = 0;
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-      uint32_t sum = 0;
-      bool lead = c[k] != kEmpty;
-#pragma unroll
-      for (int m = 0; m < D; ++m)
-        if (c[m] == c[k]) {
-          sum += arc[m].y;
-          if (m < k) lead = false;
-        }
-      if (lead && c[k] == h.d) Hd = sum;
-      hw[k] = lead && c[k] != h.d ? sum : 0u;  // a valid arc weighs at least 1
-      ncand += hw[k] ? 1u : 0u;
+    const unsigned wide = __ballot_sync(0xFFFFFFFFu, h.act && !fits64(h.m2, h.Ki));
+    if (wide) {
+      lane_vertices_128(a, h, wide, sums);
+      if ((wide >> lane) & 1u) h.act = false;
     }
-    uint32_t sg[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) sg[k] = hw[k] ? sigma32(a.Sigma, c[k]) : 0u;
-    uint32_t bc = 0;
-    i128 gain = 0;
-    bool mv = false;
-    if (h.act) {
-      mv = fits64(h.m2, h.Ki) ? thread_decide<D, true>(a, h, c, hw, sg, Hd, &bc, &gain)
-                              : thread_decide<D, false>(a, h, c, hw, sg, Hd, &bc, &gain);
-      sums.bytes += 24 + 12ull * h.dg + 12ull * ncand;
-    }
-    record_moves_warp(a, mv, h.i, bc, h.d, gain, h.gi, sums);
-    if (mv) {  // the arcs again (cached)
-      sums.bytes += 16 + 4ull * h.dg;
-      for (uint32_t k = 0; k < h.dg; ++k) {
-        const uint2 e = a.g.arcs[h.o + k];
-        mark_next(a, e.x, e.x != h.i && e.y != 0);
-      }
-    }
+    uint32_t bc = 0, ncand = 0;
+    unsigned long long gain = 0;
+    bool mv;
+    if (D == 8) mv = lane_vertex<8>(a, h, w, &bc, &gain, &ncand);
+    else if (__any_sync(0xFFFFFFFFu, h.act && h.dg > 16)) mv = lane_vertex<D>(a, h, w, &bc, &gain, &ncand);
+    else mv = lane_vertex<16>(a, h, w, &bc, &gain, &ncand);
+    if (h.act) sums.bytes += 24 + 12ull * h.dg + 12ull * ncand + (mv ? 16 + 4ull * h.dg : 0ull);
+    record_moves_warp(a, mv, h.i, bc, h.d, (i128)gain, h.gi, sums);
+    if (mv) mark_row(a, h.i, h.o, h.dg);
   }
   flush_sums_all(a, sums);
 }
 
 // ---------------------------------------------------------------------------
-// Bin 1: one warp per vertex, vertices taken in batches of up to 32 headers.
-// A vertex of at most 32 arcs is decided in registers (one arc per lane);
-// a larger one in the warp's shared table.  The table is empty at rest: the
+// Bin 2: one warp per vertex (more than 32 arcs), vertices taken in batches
+// of up to 32 headers, each decided in the warp's shared table.  The table is empty at rest: the
 // lane that creates a community's slot loads that community's Sigma at once,
 // and after the last arc is in, scores the slot and clears it, so the table
 // is neither cleared nor scanned as a whole.  Vertices whose scores need
 // 128 bits take the per-vertex path of the persistent kernel.
 // ---------------------------------------------------------------------------
-
-// Decision of vertex v (at most 32 arcs; `arc` = this lane's arc, lane < dg,
-// else (i, 0)), identical on every lane; *ncand on every lane.
-__device__ __forceinline__ bool reg_vertex(const DecideArgs& a, const VHdr& v, uint2 arc, uint32_t* bco,
-                                           i128* gain, uint32_t* ncand) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const bool valid = lane < v.dg && arc.x != v.i && arc.y != 0;
-  const uint32_t c = valid ? a.C[arc.x] : kEmpty;
-  const uint32_t wv = valid ? arc.y : 0u;
-  uint32_t hsum = 0;
-  bool leader = valid;
-  for (uint32_t k = 0; k < v.dg; ++k) {  // warp-uniform bound
-    const uint32_t ck = __shfl_sync(0xFFFFFFFFu, c, k);
-    const uint32_t wk = __shfl_sync(0xFFFFFFFFu, wv, k);
-    if (valid && ck == c) {
-      hsum += wk;
-      if (k < lane) leader = false;
-    }
-  }
-  const uint32_t Hd = __reduce_add_sync(0xFFFFFFFFu, (leader && c == v.d) ? hsum : 0u);
-  bool cand = leader && c != v.d;
-  *ncand = __popc(__ballot_sync(0xFFFFFFFFu, cand));
-  unsigned long long s = cand ? score64(v.m2, hsum, v.Ki, sigma32(a.Sigma, c)) : 0ull;
-  uint32_t bc = c;
-  warp_best64(cand, s, bc);
-  *bco = bc;
-  return decide64(a, v, cand, s, bc, Hd, gain);
-}
 
 // Decision of vertex v (32 < degree <= 32 U) in the warp's table (keys kEmpty
 // and values 0 at rest, and left so).  `a0` is this lane's first arc,
@@ -822,13 +862,6 @@ __global__ void __launch_bounds__(256, 3) k_decide_warp_hash(DecideArgs a) {
   __shared__ uint32_t skeys[kWarpHashWarps][kWarpSlots];
   __shared__ uint32_t svals[kWarpHashWarps][kWarpSlots];
   const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
-  uint32_t* keys = skeys[wib];
-  uint32_t* vals = svals[wib];
-  for (uint32_t s = lane; s < kWarpSlots; s += 32) {
-    keys[s] = kEmpty;
-    vals[s] = 0;
-  }
-  __syncwarp();
   const long long m2_one = *a.m2p;
   const uint32_t cnt = *a.count;
   const uint64_t warp = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) >> 5;
@@ -836,6 +869,14 @@ __global__ void __launch_bounds__(256, 3) k_decide_warp_hash(DecideArgs a) {
   // vertices per warp and round: up to 32, fewer when the list is short
   uint64_t B = (uint64_t(cnt) + nwarps - 1) / nwarps;
   B = B < 1 ? 1 : B > 32 ? 32 : B;
+  if (blockIdx.x * uint64_t(kWarpHashWarps) * B >= cnt) return;  // no vertex for this block
+  uint32_t* keys = skeys[wib];
+  uint32_t* vals = svals[wib];
+  for (uint32_t s = lane; s < kWarpSlots; s += 32) {
+    keys[s] = kEmpty;
+    vals[s] = 0;
+  }
+  __syncwarp();
   MoveSums sums;
   for (uint64_t t0 = warp * B; t0 < cnt; t0 += nwarps * B) {
     VHdr h;
@@ -875,10 +916,7 @@ __global__ void __launch_bounds__(256, 3) k_decide_warp_hash(DecideArgs a) {
       uint32_t bc = 0, ncand = 0;
       i128 gain = 0;
       bool mv;
-      if (v.dg <= 32) {
-        mv = reg_vertex(a, v, a0, &bc, &gain, &ncand);
-        if (mv) mark_next(a, a0.x, lane < v.dg && a0.x != v.i && a0.y != 0);
-      } else if (v.dg <= 64) {
+      if (v.dg <= 64) {
         mv = table_vertex<2>(a, v, a0, keys, vals, &bc, &gain, &ncand);
       } else if (v.dg <= 128) {
         mv = table_vertex<4>(a, v, a0, keys, vals, &bc, &gain, &ncand);
@@ -1030,6 +1068,10 @@ __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
   __shared__ int s_mv[32];
   constexpr uint32_t nthr = kThreads;
   const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
+  const long long m2_one = *a.m2p;
+  const uint32_t cnt = *a.count;
+  if (blockIdx.x >= cnt) return;  // no vertex for this block
+  const uint64_t G = gridDim.x;
   for (uint32_t s = threadIdx.x; s < kBlockSlots; s += nthr) {
     keys[s] = kEmpty;
     vals[s] = 0;
@@ -1038,9 +1080,6 @@ __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
     s_hd[threadIdx.x] = 0;
     s_nc[threadIdx.x] = 0;
   }
-  const long long m2_one = *a.m2p;
-  const uint32_t cnt = *a.count;
-  const uint64_t G = gridDim.x;
   MoveSums sums;
   __syncthreads();
   for (uint64_t t0 = blockIdx.x; t0 < cnt; t0 += 32 * G) {
@@ -1304,8 +1343,8 @@ __global__ void __launch_bounds__(1024) k_giant_prefix(DecideArgs a, GiantDecide
                                                        const uint32_t* lists, int cur) {
   pdl_wait_only();
   const uint32_t s = blockIdx.x;
-  a.list = lists + a.seg.off[s * kBins + 3];
-  a.count = &a.ctrl->count[cur][s][3];
+  a.list = lists + a.seg.off[s * kBins + kBinHuge];
+  a.count = &a.ctrl->count[cur][s][kBinHuge];
   giant_prefix_body(a, giant_class(gd, s, gstride, a.ctrl));
 }
 
@@ -1512,6 +1551,7 @@ __global__ void __launch_bounds__(kAccumThreads, 8) k_giant_accum(DecideArgs a, 
   const long long m2_one = *a.m2p;
   const uint32_t cnt = *a.count;
   const uint32_t nitems = *gd.nitems;
+  if (blockIdx.x >= nitems) return;  // no chunk for this block
   // the chunk prefix, cached in shared memory when it fits
   const uint32_t* cp = gd.cpre;
   if (cnt + 1 <= kGiantListSmem) {
@@ -1886,25 +1926,6 @@ __device__ __forceinline__ GiantDecide class_giant(const IterArgs& ia, uint32_t 
   return gd;
 }
 
-// Every lane of the warp calls it: bin-0 vertices of one warp (32 / W of them).
-template <int W>
-__device__ __forceinline__ void iter_segments(const DecideArgs& a, uint64_t first, uint32_t cnt, long long m2_one,
-                                              MoveSums& sums) {
-  const uint32_t lane = threadIdx.x & 31u, seg = lane / W, sl = lane % W;
-  const uint64_t t = first + seg;
-  bool active = t < cnt;
-  const uint32_t i = active ? a.list[t] : 0u;
-  long long m2 = m2_one;
-  uint32_t gi = 0;
-  if (active && !group_active(a, i, &m2, &gi)) active = false;
-  if (active && sl == 0) {
-    if (a.ever && bit_set(a.ever, i)) ++sums.ever;
-    ++sums.processed;
-  }
-  if (active && a.rbits && !bit_test(a.rbits, i)) active = false;
-  decide_segment<W>(a, active, i, m2, gi, sums);
-}
-
 static_assert(kIterThreads == kGiantThreads && kIterThreads == kCommitThreads,
               "the part blocks and the commit sweep their lists in tiles of one block");
 static_assert(kIterThreads == kListThreads, "the list builder's tiles are one block's");
@@ -1925,7 +1946,7 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
   MoveSums sums;
   // 1. the largest-degree lists of every class: chunk, table and list layouts
   if (blockIdx.x < ia.k) {
-    const DecideArgs a3 = bin_args(ia, blockIdx.x, 3);
+    const DecideArgs a3 = bin_args(ia, blockIdx.x, kBinHuge);
     giant_prefix_body(a3, class_giant(ia, blockIdx.x));
   }
   if (!grid_barrier(ctrl, ia.bar_extra, ia.bar_polls)) return;
@@ -1937,10 +1958,11 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
       ctrl->it_work[par ^ 1] = 0;
       ctrl->it_bignd[par ^ 1] = 0;
     }
-    const DecideArgs a0 = bin_args(ia, s, 0), a1 = bin_args(ia, s, 1), a2 = bin_args(ia, s, 2),
-                     a3 = bin_args(ia, s, 3);
+    // (the lane bin's vertices are warp units here too, in units of their own)
+    const DecideArgs a0 = bin_args(ia, s, kBinTiny), al = bin_args(ia, s, kBinLanes), a1 = bin_args(ia, s, kBinTable),
+                     a2 = bin_args(ia, s, kBinWhole), a3 = bin_args(ia, s, kBinHuge);
     const GiantDecide gd = class_giant(ia, s);
-    const uint32_t n0 = *a0.count, n1 = *a1.count, n2 = *a2.count, n3 = *a3.count;
+    const uint32_t n0 = *a0.count, nl = *al.count, n1 = *a1.count, n2 = *a2.count, n3 = *a3.count;
     const uint32_t G = *gd.nitems;
     // chunk prefix of the class, cached when it fits
     const uint32_t* cp = gd.cpre;
@@ -1952,7 +1974,8 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
     const uint32_t per_warp0 = 32 / ia.seg_lanes;
     const uint64_t U0 = (uint64_t(n0) + per_warp0 * 8 * kIterRounds0 - 1) / (per_warp0 * 8 * kIterRounds0);
     const uint64_t U1 = (uint64_t(n1) + 8 * kIterRounds1 - 1) / (8 * kIterRounds1);
-    const uint64_t total = uint64_t(G) + n2 + U1 + U0;
+    const uint64_t UL = (uint64_t(nl) + 8 * kIterRounds1 - 1) / (8 * kIterRounds1);
+    const uint64_t total = uint64_t(G) + n2 + U1 + UL + U0;
     // 2. decide: work units from the shared counter
     for (;;) {
       if (threadIdx.x == 0) s_unit = atomicAdd(&ctrl->it_work[par], 1u);
@@ -1980,33 +2003,36 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
         }
         if (a2.rbits && !bit_test(a2.rbits, i)) continue;
         block_vertex<kIterThreads>(a2, i, m2, gi, dyn, sc, sums);
-      } else if (u < uint64_t(G) + n2 + U1) {
-        // one bin-1 vertex per warp and round, in the warp's own table
+      } else if (u < uint64_t(G) + n2 + U1 + UL) {
+        // one table-bin or lane-bin vertex per warp and round, in the warp's own table
+        const bool table = u < uint64_t(G) + n2 + U1;
+        const uint64_t unit = table ? u - G - n2 : u - G - n2 - U1;
+        const DecideArgs& aw = table ? a1 : al;
         for (uint32_t r = 0; r < kIterRounds1; ++r) {
-          const uint64_t t = ((u - G - n2) * kIterRounds1 + r) * 8 + wib;
-          if (t >= n1) break;
-          const uint32_t i = a1.list[t];
+          const uint64_t t = (unit * kIterRounds1 + r) * 8 + wib;
+          if (t >= (table ? n1 : nl)) break;
+          const uint32_t i = aw.list[t];
           long long m2 = m2_one;
           uint32_t gi = 0;
-          if (!group_active(a1, i, &m2, &gi)) continue;
+          if (!group_active(aw, i, &m2, &gi)) continue;
           if (lane == 0) {
-            if (a1.ever && bit_set(a1.ever, i)) ++sums.ever;
+            if (aw.ever && bit_set(aw.ever, i)) ++sums.ever;
             ++sums.processed;
           }
-          if (!a1.rbits || bit_test(a1.rbits, i))
-            warp_table_vertex(a1, i, m2, gi, dyn + wib * 2 * kWarpSlots, dyn + wib * 2 * kWarpSlots + kWarpSlots,
+          if (!aw.rbits || bit_test(aw.rbits, i))
+            warp_table_vertex(aw, i, m2, gi, dyn + wib * 2 * kWarpSlots, dyn + wib * 2 * kWarpSlots + kWarpSlots,
                               sums);
         }
       } else {
         for (uint32_t r = 0; r < kIterRounds0; ++r) {
           const uint64_t first =
-              ((u - G - n2 - U1) * kIterRounds0 + r) * (per_warp0 * 8) + uint64_t(wib) * per_warp0;
+              ((u - G - n2 - U1 - UL) * kIterRounds0 + r) * (per_warp0 * 8) + uint64_t(wib) * per_warp0;
           if (first >= n0) break;  // warp-uniform
           switch (ia.seg_lanes) {
-            case 4: iter_segments<4>(a0, first, n0, m2_one, sums); break;
-            case 8: iter_segments<8>(a0, first, n0, m2_one, sums); break;
-            case 16: iter_segments<16>(a0, first, n0, m2_one, sums); break;
-            default: iter_segments<32>(a0, first, n0, m2_one, sums); break;
+            case 4: decide_segments<4>(a0, first, n0, m2_one, sums); break;
+            case 8: decide_segments<8>(a0, first, n0, m2_one, sums); break;
+            case 16: decide_segments<16>(a0, first, n0, m2_one, sums); break;
+            default: decide_segments<32>(a0, first, n0, m2_one, sums); break;
           }
         }
       }
@@ -2059,6 +2085,18 @@ __global__ void k_set_m2(Ctrl* ctrl, long long m2, const Ctrl* ap) {
 // slice of the global overflow table
 constexpr uint32_t kBlockGridMax = 3 * 152;
 
+// Profile class of each bin (the lane and table bins are one class).
+constexpr int kBinClass[kBins] = {DFL_PROF_BIN0, DFL_PROF_BIN1, DFL_PROF_BIN1, DFL_PROF_BIN2, DFL_PROF_BIN3};
+
+// k_decide_lanes for a list of c vertices (~0: its length is on the device) of
+// at most lim arcs.
+void launch_lanes(const DecideArgs& a, uint32_t lim, uint32_t c, cudaStream_t st) {
+  if (lim <= 8)
+    k_decide_lanes<8><<<c == ~0u ? 152 * 8 : grid_for(c, kLaneThreads, 152 * 64), kLaneThreads, 0, st>>>(a);
+  else
+    k_decide_lanes<32><<<c == ~0u ? 152 * 5 : grid_for(c, kLaneThreads, 152 * 64), kLaneThreads, 0, st>>>(a);
+}
+
 // Issue one local-moving iteration (all sub-steps) on h->stream.  With
 // `counts` (host-known list lengths) empty bins are skipped and grids are
 // sized to the work; without (graph capture) every bin is launched with a
@@ -2090,14 +2128,16 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
   // everything runs on the handle's stream.
   const bool par = !(h->opt.flags & DFL_FLAG_SERIAL_BINS);
   cudaStream_t spine = par ? h->aux[kBins - 2] : h->stream;
-  cudaStream_t bst[kBins] = {h->stream, par ? h->aux[0] : h->stream, par ? h->aux[1] : h->stream, spine};
+  cudaStream_t bst[kBins] = {h->stream, par ? h->aux[0] : h->stream, par ? h->aux[1] : h->stream,
+                             par ? h->aux[2] : h->stream, spine};
   if (par) {
     DFL_CUDA(h, cudaEventRecord(h->ev_fork, h->stream));
     DFL_CUDA(h, cudaStreamWaitEvent(spine, h->ev_fork, 0));
   }
-  bool any3 = !counts;
-  for (uint32_t s = 0; counts && s < k; ++s) any3 |= counts[s][3] != 0;
-  if (any3) {  // the largest-degree layouts of all classes, once
+  const bool wide_labels = a.g.nv >= kLaneLabels;  // labels that do not fit k_decide_lanes' keys
+  bool any_huge = !counts;
+  for (uint32_t s = 0; counts && s < k; ++s) any_huge |= counts[s][kBinHuge] != 0;
+  if (any_huge) {  // the largest-degree layouts of all classes, once
     LaunchScope ls(h, DFL_PROF_BIN3, spine);
     launch_pdl(k_giant_prefix, k, 1024, 0, spine, a, gd_base, gstride, h->lists[cur], cur);
     DFL_TRY(check_launch(h, "giant prefix"));
@@ -2107,9 +2147,20 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
     a.nbig = &h->ctrl->it_nbig[s & 1];
     a.clear_movers = s + 1 < k ? &h->ctrl->it_movers[(s + 1) & 1] : nullptr;
     a.clear_nbig = s + 1 < k ? &h->ctrl->it_nbig[(s + 1) & 1] : nullptr;
-    int nb = 0;
-    for (int b = 0; b < kBins; ++b) nb += (!counts || counts[s][b]) ? 1 : 0;
-    const bool any = nb > 0;
+    bool has[kBins], any = false;
+    for (int b = 0; b < kBins; ++b) {
+      has[b] = !counts || counts[s][b];
+      any |= has[b];
+    }
+    // short lists of the two register bins share a launch
+    const uint64_t n0 = counts ? counts[s][kBinTiny] : 0, n1 = counts ? counts[s][kBinLanes] : 0;
+    const bool short0 = wide_labels || (counts ? n0 < kSmallList : small_hint);
+    const bool short1 = wide_labels || (counts ? n1 < kSmallLanes : small_hint);
+    const bool merged = short0 && short1 && has[kBinLanes];
+    if (merged) {
+      has[kBinTiny] = true;
+      has[kBinLanes] = false;
+    }
     cudaEvent_t pa = nullptr, pb = nullptr;  // wall time of the decide phase (profiling)
     if (any && (h->opt.flags & (DFL_FLAG_PROFILE | DFL_FLAG_PROFILE_MOVE))) {
       pa = take_event(h);
@@ -2118,12 +2169,12 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
     }
     // the fork point is this sub-step's start on the spine, before its own kernels
     bool fork = false;
-    for (int b = 0; b < kBins; ++b) fork |= bst[b] != spine && (!counts || counts[s][b]);
+    for (int b = 0; b < kBins; ++b) fork |= bst[b] != spine && has[b];
     if (fork) DFL_CUDA(h, cudaEventRecord(h->ev_fork, spine));
-    bool joined[kBins - 1] = {false, false, false};
+    bool joined[kBins - 1] = {};
     for (int b = kBins - 1; b >= 0; --b) {
       const uint32_t c = counts ? counts[s][b] : 0u;
-      if (counts && !c) continue;
+      if (!has[b]) continue;
       cudaStream_t st = bst[b];
       if (st != spine) {
         DFL_CUDA(h, cudaStreamWaitEvent(st, h->ev_fork, 0));
@@ -2131,29 +2182,28 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
       }
       a.list = h->lists[cur] + h->segs.off[s * kBins + b];
       a.count = &h->ctrl->count[cur][s][b];
-      LaunchScope ls(h, DFL_PROF_BIN0 + b, st);
-      if (b == 0) {
+      LaunchScope ls(h, kBinClass[b], st);
+      if (b == kBinTiny) {
         const uint32_t lim = h->tune.bin_warp;
-        const bool small = counts ? c < kSmallList : small_hint;
-        if (lim <= 8 && small) {  // W = 4 or 8 lanes per vertex
-          const uint32_t segs = lim <= 4 ? 8 : 4;
-          const uint32_t grid = counts ? grid_for((uint64_t(c) + segs - 1) / segs * 32, 256, 152 * 64) : 152 * 8;
-          if (segs == 8) k_decide_warp<4><<<grid, 256, 0, st>>>(a);
-          else k_decide_warp<8><<<grid, 256, 0, st>>>(a);
-        } else if (lim <= 8) {  // a thread per vertex, its arcs in registers
-          const uint32_t grid = counts ? grid_for(c, 256, 152 * 16) : 152 * 4;
-          if (lim <= 4) k_decide_thread<4><<<grid, 256, 0, st>>>(a);
-          else k_decide_thread<8><<<grid, 256, 0, st>>>(a);
-        } else {  // W = 16 or 32 lanes per vertex
-          const uint32_t segs = lim <= 16 ? 2 : 1;
-          const uint32_t grid = counts ? grid_for((uint64_t(c) + segs - 1) / segs * 32, 256, 152 * 64) : 152 * 8;
-          if (segs == 2) k_decide_warp<16><<<grid, 256, 0, st>>>(a);
-          else k_decide_warp<32><<<grid, 256, 0, st>>>(a);
-        }
-      } else if (b == 1) {
+        const uint32_t segs = lim <= 4 ? 8 : lim <= 8 ? 4 : lim <= 16 ? 2 : 1;
+        const uint32_t grid = counts ? grid_for(((n0 + segs - 1) / segs + (merged ? n1 : 0)) * 32, 256, 152 * 64) : 152 * 8;
+        const uint32_t* l2 = merged ? h->lists[cur] + h->segs.off[s * kBins + kBinLanes] : nullptr;
+        const unsigned int* c2 = merged ? &h->ctrl->count[cur][s][kBinLanes] : nullptr;
+        if (!short0) launch_lanes(a, lim, counts ? c : ~0u, st);
+        else if (segs == 8) k_decide_warp<4><<<grid, 256, 0, st>>>(a, l2, c2);
+        else if (segs == 4) k_decide_warp<8><<<grid, 256, 0, st>>>(a, l2, c2);
+        else if (segs == 2) k_decide_warp<16><<<grid, 256, 0, st>>>(a, l2, c2);
+        else k_decide_warp<32><<<grid, 256, 0, st>>>(a, l2, c2);
+      } else if (b == kBinLanes) {
+        if (short1)  // a warp per vertex: the shorter chain
+          k_decide_warp<32><<<counts ? grid_for(uint64_t(c) * 32, 256, 152 * 64) : 152 * 8, 256, 0, st>>>(a, nullptr,
+                                                                                                       nullptr);
+        else
+          launch_lanes(a, h->segs.hi[kBinLanes], counts ? c : ~0u, st);
+      } else if (b == kBinTable) {
         // a warp per vertex, headers in batches of up to 32 (fewer when the list is short)
         k_decide_warp_hash<<<counts ? grid_for(uint64_t(c) * 32, 256, 152 * 6) : 152 * 3, 256, 0, st>>>(a);
-      } else if (b == 2) {
+      } else if (b == kBinWhole) {
         const size_t smem = sizeof(uint32_t) * 2 * kBlockSlots;
         const uint32_t bt = h->tune.block_threads;
         const uint32_t per_sm = bt == 512 ? 2 : 3;  // 64 KB table each; grid <= kBlockGridMax

@@ -304,9 +304,10 @@ __global__ void __launch_bounds__(kListThreads) k_lists_bits(const uint32_t* __r
 // one segment of a buffer, and a super-vertex graph has ids in [0, nv) with
 // nv <= n).
 void make_segs(Handle* h, uint32_t k) {
-  h->segs.hi[0] = h->tune.bin_warp;
-  h->segs.hi[1] = h->tune.bin_warp_hash;
-  h->segs.hi[2] = h->tune.bin_block;
+  h->segs.hi[kBinTiny] = h->tune.bin_warp;
+  h->segs.hi[kBinLanes] = h->tune.bin_warp_hash < kBinWarp ? h->tune.bin_warp_hash : kBinWarp;
+  h->segs.hi[kBinTable] = h->tune.bin_warp_hash;
+  h->segs.hi[kBinWhole] = h->tune.bin_block;
   h->segs.goff = h->ngraphs ? h->d_goff : nullptr;
   h->segs.ng = h->ngraphs;
   if (h->segs_k == k) return;

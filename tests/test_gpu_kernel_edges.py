@@ -131,3 +131,47 @@ def test_delta_screening_marks_hub_neighbours(dfl, orc, degrees):
     a.update(1)
     b.update(1)
     same(a, b)
+
+
+@pytest.mark.parametrize("mean_degree,n,flags", [
+    (16, 12_000, 4),    # a list above the lane bin's limit, host launches
+    (16, 33_000, 32),   # ... graph replay
+    (4, 33_000, 4),     # bin 0's long lists
+    (4, 33_000, 32),
+])
+def test_lane_per_vertex_lists(dfl, orc, mean_degree, n, flags):
+    """Long lists of vertices of up to 8, 16 and 32 arcs (a lane each), with
+    weights, deleted arcs and re-inserted ones in the rows."""
+    g = random_graph(n, n * mean_degree // 2, mean_degree)
+    a, b = pair(dfl, orc, g, substeps=1, flags=flags, max_iterations=3)
+    a.static()
+    b.static()
+    same(a, b)
+    stream = synth.BatchStream(g, 5)
+    for _ in range(2):
+        dels, ins = stream.next(2000, w_max=9)
+        assert a.apply_batch(dels, ins) == 0 and b.apply_batch(dels, ins) == 0
+        a.update(0)
+        b.update(0)
+        same(a, b)
+
+
+@pytest.mark.parametrize("flags", [4, 32])
+def test_lane_per_vertex_scores_beyond_64_bits(dfl, orc, flags):
+    """A community holding nearly all of 2m becomes a super-vertex (a
+    self-loop and a few arcs) whose K times 2m is above 2^63, in a second pass
+    over a long list of small super-vertices."""
+    n, heavy = 80_000, 105_000_000
+    g = random_graph(n - 21, (n - 21) * 5 // 4, 3, w_max=3)
+    hub = n - 21  # a star of 20 heavy edges, three of its leaves joined to the rest
+    u = np.concatenate([g.u, np.full(20, hub), np.array([5, 70, 900])]).astype(np.uint32)
+    v = np.concatenate([g.v, hub + 1 + np.arange(20), hub + 1 + np.arange(3)]).astype(np.uint32)
+    w = np.concatenate([g.w, np.full(20, heavy), np.ones(3)]).astype(np.uint32)
+    a, b = pair(dfl, orc, synth.EdgeList(n, u, v, w), substeps=1, flags=flags, max_iterations=3, tau_agg=1.0)
+    a.set_tuning(bin_warp=0)  # every vertex of up to 32 arcs in one list
+    a.static()
+    b.static()
+    same(a, b)
+    two_m = a.weights()[2]
+    assert two_m < 2**32 and (40 * heavy) * two_m > 2**63
+    assert a.stats()["num_communities"] > 12_000 and a.stats()["passes"] > 1
