@@ -62,8 +62,6 @@ struct Ctrl {
   unsigned long long processed;      // frontier vertices processed in the iteration
   unsigned long long moved;          // movers in the iteration
   unsigned long long move_bytes;     // algorithmic bytes of the decide kernels
-  unsigned int movers;               // movers of the current sub-step (list length)
-  unsigned int big_movers;           // ... of them listed for k_commit to mark the neighbours of
   unsigned int err;                  // kErr* bits
   unsigned int pad_err;
   unsigned int count[2][kMaxSubsteps][kBins];  // frontier list lengths [buffer][class][bin]
@@ -78,10 +76,12 @@ struct Ctrl {
   unsigned int pad2;
   unsigned long long skipped;        // frontier vertices without arcs (processed, not queued)
   unsigned long long ever_count;     // vertices newly added to the first-pass processed set
-  // persistent iteration kernel: per sub-step parity, movers, listed
-  // high-degree movers, work units taken, vertices left to the part blocks;
-  // chunk items of each class; grid barrier
-  unsigned int it_movers[2], it_nbig[2], it_work[2], it_bignd[2];
+  // per sub-step parity: the queue counter of the high-degree movers (rows <<
+  // 32 | pieces), the movers, and the persistent iteration kernel's work units
+  // taken and vertices left to the part blocks; chunk items of each class;
+  // grid barrier
+  unsigned long long it_nbig[2];
+  unsigned int it_movers[2], it_work[2], it_bignd[2];
   unsigned int it_items[kMaxSubsteps];
   unsigned int bar_count, bar_gen;
   long long m2v;                     // 2m of the current local-moving call
@@ -240,7 +240,7 @@ struct Handle {
   uint64_t tmp_cap = 0;
   uint2* gtable = nullptr;         // global hash tables of the largest bin
   uint64_t gtable_cap = 0;
-  uint32_t* bigmv = nullptr;       // high-degree movers of a sub-step (marked by k_mark_big)
+  uint2* bigmv = nullptr;          // queue of the high-degree movers of a sub-step
   uint64_t bigmv_cap = 0;
   uint2* aggq = nullptr;           // high-degree members of giant communities (aggregation)
   uint64_t aggq_cap = 0;

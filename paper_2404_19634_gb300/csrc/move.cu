@@ -45,11 +45,11 @@ struct DecideArgs {
   uint32_t k;
   uint2* gtable;          // bin 3: per-block global tables
   uint32_t gslots;        // slots per block (power of two)
-  uint32_t* bigmv;        // movers of degree > kMarkInline (neighbours marked by k_commit)
+  uint2* bigmv;           // queue of the movers of degree > kMarkInline (push_row)
   unsigned int* movers;   // movers of the sub-step (slot counter into mv_i/mv_c/mv_d)
-  unsigned int* nbig;     // ... of them in bigmv
+  unsigned long long* nbig;  // ... its counter
   unsigned int* clear_movers;  // the next sub-step's two counters, zeroed by this sub-step's
-  unsigned int* clear_nbig;    // commit (null: nothing to zero)
+  unsigned long long* clear_nbig;  // commit (null: nothing to zero)
   // group of graphs (ngraphs > 0): the vertex's graph gives its 2m, whether
   // it is still processed, and where its movers' dQ sum goes
   uint32_t ngraphs;
@@ -154,18 +154,42 @@ __device__ __forceinline__ void flush_sums_all(const DecideArgs& a, MoveSums v) 
   flush_sums(a, v, (threadIdx.x & 31u) == 0);
 }
 
-// A mover of more than kMarkInline arcs does not mark its neighbours itself
-// (one block would walk them all while the rest of the GPU idles): it is
-// listed, and k_commit spreads every listed mover's arcs over all blocks.
+// The commit marks the movers' neighbours for the next iteration (the decide
+// kernels only record the moves): of a mover of at most kMarkInline arcs from
+// the mover list, of a larger one from a queue cut into pieces of kMarkChunk
+// arcs, so that every mover's arcs are read coalesced and spread over the GPU.
 constexpr uint32_t kMarkInline = 512;
-constexpr uint32_t kMarkChunk = 1024;
+constexpr uint32_t kMarkChunk = 512;
 
-// Mark neighbour j of a mover for the next iteration: its bit in the next
-// frontier's bitmap (the lists are built from the bitmap once, at the end of
-// the iteration).  The bit is read first, so a vertex marked by many movers
+__device__ __forceinline__ void queue_marks(const DecideArgs& a, uint32_t i, uint32_t dg) {
+  push_row(a.bigmv, a.nbig, i, (dg + kMarkChunk - 1) / kMarkChunk);
+}
+
+// Mark arcs [k0, k1) of mover i's row at o, this lane's from k0 + first on in
+// steps of `step`, four arcs' bitmap words in flight: the neighbours' bits in
+// the next frontier's bitmap (the lists are built from it once, at the end of
+// the iteration).  The bits are read first, so a vertex marked by many movers
 // takes one atomic.
-__device__ __forceinline__ void mark_next(const DecideArgs& a, uint32_t j, bool valid) {
-  if (valid && (!a.rbits || bit_test(a.rbits, j)) && !bit_test(a.fbits_next, j)) bit_set(a.fbits_next, j);
+__device__ __forceinline__ void mark_arcs(const DecideArgs& a, uint32_t i, unsigned long long o, uint32_t k0,
+                                          uint32_t k1, uint32_t first, uint32_t step) {
+  for (uint32_t b = k0 + first; b < k1; b += 4 * step) {
+    uint2 e[4];
+    bool on[4];
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) e[u] = b + u * step < k1 ? a.g.arcs[o + b + u * step] : make_uint2(i, 0u);
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) {
+      on[u] = e[u].x != i && e[u].y != 0;  // not a self-loop, not a deleted arc
+      if (on[u]) on[u] = !bit_test(a.fbits_next, e[u].x);
+    }
+    if (a.rbits) {
+#pragma unroll
+      for (uint32_t u = 0; u < 4; ++u) on[u] = on[u] && bit_test(a.rbits, e[u].x);
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u)
+      if (on[u]) bit_set(a.fbits_next, e[u].x);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -248,7 +272,6 @@ __device__ __forceinline__ bool decide_segment(const DecideArgs& a, bool active,
       sums.bytes += 16 + 4ull * dg;
     }
   }
-  mark_next(a, arc.x, mv && valid);
   return mv;
 }
 
@@ -461,11 +484,6 @@ __device__ __forceinline__ void warp_table_vertex(const DecideArgs& a, uint32_t 
     if (lane == 0) {
       record_move(a, i, bc, d, gain, gi, sums);
       sums.bytes += 16 + 4ull * dg;
-    }
-    for (uint32_t k0 = 0; k0 < dg; k0 += 32) {
-      uint32_t k = k0 + lane;
-      uint2 arc = k < dg ? a.g.arcs[o + k] : make_uint2(i, 0u);
-      mark_next(a, arc.x, k < dg && arc.x != i && arc.y != 0);
     }
   }
   __syncwarp();
@@ -699,23 +717,6 @@ __device__ __forceinline__ bool lane_vertex(const DecideArgs& a, const VHdr& v, 
   return mv;
 }
 
-// The neighbours of a mover (its arcs again, cached), marked by one lane: four
-// arcs' bitmap words in flight.
-__device__ __forceinline__ void mark_row(const DecideArgs& a, uint32_t i, unsigned long long o, uint32_t dg) {
-  for (uint32_t k0 = 0; k0 < dg; k0 += 4) {
-    uint2 e[4];
-    bool on[4];
-#pragma unroll
-    for (uint32_t u = 0; u < 4; ++u) e[u] = k0 + u < dg ? a.g.arcs[o + k0 + u] : make_uint2(i, 0u);
-#pragma unroll
-    for (uint32_t u = 0; u < 4; ++u)
-      on[u] = e[u].x != i && e[u].y != 0 && (!a.rbits || bit_test(a.rbits, e[u].x)) && !bit_test(a.fbits_next, e[u].x);
-#pragma unroll
-    for (uint32_t u = 0; u < 4; ++u)
-      if (on[u]) bit_set(a.fbits_next, e[u].x);
-  }
-}
-
 // The rare vertices whose scores need 128 bits, a warp each, out of line.
 __device__ __noinline__ void lane_vertices_128(const DecideArgs& a, const VHdr& h, unsigned m, MoveSums& sums) {
   for (; m; m &= m - 1) {
@@ -753,7 +754,6 @@ __global__ void __launch_bounds__(kLaneThreads, D == 8 ? 8 : 5) k_decide_lanes(D
     else mv = lane_vertex<16>(a, h, w, &bc, &gain, &ncand);
     if (h.act) sums.bytes += 24 + 12ull * h.dg + 12ull * ncand + (mv ? 16 + 4ull * h.dg : 0ull);
     record_moves_warp(a, mv, h.i, bc, h.d, (i128)gain, h.gi, sums);
-    if (mv) mark_row(a, h.i, h.o, h.dg);
   }
   flush_sums_all(a, sums);
 }
@@ -769,8 +769,7 @@ __global__ void __launch_bounds__(kLaneThreads, D == 8 ? 8 : 5) k_decide_lanes(D
 
 // Decision of vertex v (32 < degree <= 32 U) in the warp's table (keys kEmpty
 // and values 0 at rest, and left so).  `a0` is this lane's first arc,
-// loaded ahead.  Returns the decision on every lane; a mover's arcs are read
-// again to mark the next frontier.
+// loaded ahead.  Returns the decision on every lane.
 template <int U>
 __device__ __forceinline__ bool table_vertex(const DecideArgs& a, const VHdr& v, uint2 a0, uint32_t* keys,
                                              uint32_t* vals, uint32_t* bco, i128* gain, uint32_t* ncand) {
@@ -841,14 +840,7 @@ __device__ __forceinline__ bool table_vertex(const DecideArgs& a, const VHdr& v,
   *ncand = __reduce_add_sync(0xFFFFFFFFu, nc);
   warp_best64(have, best, bc);
   *bco = bc;
-  const bool mv = decide64(a, v, have, best, bc, Hd, gain);
-  if (mv) {  // the arcs again (cached): holding them in registers costs occupancy
-    for (uint32_t k = lane; k < v.dg; k += 32) {
-      const uint2 e = a.g.arcs[v.o + k];
-      mark_next(a, e.x, e.x != v.i && e.y != 0);
-    }
-  }
-  return mv;
+  return decide64(a, v, have, best, bc, Hd, gain);
 }
 
 // The rare 128-bit vertices, out of line so that they do not cost the common
@@ -1017,19 +1009,10 @@ __device__ __forceinline__ void block_vertex(const DecideArgs& a, uint32_t i, lo
     i128 gain = 0;
     const bool mv = decide_move(a, m2, i, d, Ki, have, best, bc, sc.hd, &gain);
     sums.bytes += 24 + 12ull * dg + 12ull * sc.ncand;
-    sc.last = mv;
     if (mv) {
       record_move(a, i, bc, d, gain, gi, sums);
       sums.bytes += 16 + 4ull * dg;
-      if (dg > kMarkInline) a.bigmv[atomicAdd(a.nbig, 1u)] = i;
-    }
-  }
-  __syncthreads();
-  if (sc.last && dg <= kMarkInline) {
-    for (uint32_t k0 = wib * 32; k0 < dg; k0 += nthr) {
-      uint32_t k = k0 + lane;
-      uint2 arc = k < dg ? a.g.arcs[o + k] : make_uint2(i, 0u);
-      mark_next(a, arc.x, k < dg && arc.x != i && arc.y != 0);
+      if (dg > kMarkInline) queue_marks(a, i, dg);
     }
   }
   __syncthreads();
@@ -1175,17 +1158,11 @@ __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
       p ^= 1;
     }
     __syncthreads();  // every decision of the batch is made
-    if (wib == 0) {  // the batch's movers: one slot reservation, then the mover list for marking
+    if (wib == 0) {  // the batch's movers: one slot reservation
       const bool mv = lane < nv && s_mv[lane];
       const VHdr& v = s_hdr[lane];
       record_moves_warp(a, mv, v.i, s_mvc[lane], v.d, (i128)s_gain[lane], v.gi, sums);
-      const unsigned m = __ballot_sync(0xFFFFFFFFu, mv);
-      if (m) {
-        uint32_t base = 0;
-        if (lane == uint32_t(__ffs(m) - 1)) base = atomicAdd(a.nbig, uint32_t(__popc(m)));
-        base = __shfl_sync(0xFFFFFFFFu, base, __ffs(m) - 1);
-        if (mv) a.bigmv[base + __popc(m & ((1u << lane) - 1u))] = v.i;  // neighbours marked by k_commit
-      }
+      if (mv && v.dg > kMarkInline) queue_marks(a, v.i, v.dg);
     }
     __syncthreads();  // s_hdr and s_mv are rewritten by the next round
   }
@@ -1532,7 +1509,7 @@ __device__ __forceinline__ void giant_chunk(const DecideArgs& a, const GiantDeci
         sums.bytes += 24 + 12ull * dg + 12ull * sc.ncand;
         if (mv) {
           record_move(a, i, bc, d, gain, gi, sums);
-          a.bigmv[atomicAdd(a.nbig, 1u)] = i;  // neighbours marked by the commit
+          queue_marks(a, i, dg);
           sums.bytes += 16 + 4ull * dg;
         }
       }
@@ -1678,7 +1655,7 @@ __device__ __forceinline__ void giant_parts(const DecideArgs& a, const GiantDeci
           sums.bytes += 24 + 12ull * dg;
           if (mv) {
             record_move(a, i, bc, d, gain, gi, sums);
-            a.bigmv[atomicAdd(a.nbig, 1u)] = i;  // neighbours marked by k_commit
+            queue_marks(a, i, dg);
             sums.bytes += 16 + 4ull * dg;
           }
         }
@@ -1699,30 +1676,32 @@ __global__ void __launch_bounds__(kGiantThreads) k_giant_decide(DecideArgs a, Gi
 
 constexpr int kCommitThreads = 256;
 
-// Apply the moves of one sub-step, then mark the next frontier around the
-// listed high-degree movers: their arcs in kMarkChunk pieces spread over the
-// blocks.  The list is swept in tiles of one block's threads: a block-wide
-// prefix numbers the pieces of a tile, which are dealt round-robin over the
-// blocks, so a long list (the first iterations of a static run) costs every
-// block one parallel pass per tile instead of one dependent walk per mover.
+// Apply the moves of one sub-step and mark the movers' neighbours for the
+// next iteration.  Latency bounds it, so the two jobs go to different warps
+// where there are enough: the moves to the first warps, 32 a warp (movers of a
+// warp joining or leaving one community are summed first, so a popular
+// community takes one update per warp), the marks to the last, one mover a
+// warp while they last and up to 32 beyond, eight lanes a mover then.  The
+// decide kernels marked their own movers' rows before, at the end of each
+// vertex's chain: without it the lane kernel takes 27 us instead of 40 on
+// 100,000 vertices of mean degree 16 and the warp tables 45 instead of 55, the
+// commit 25 instead of 9; a small commit takes 4 us as before.
 // Blocks of kCommitThreads threads.
-__device__ __forceinline__ void commit_body(const DecideArgs& a, uint32_t m, uint32_t count) {
+__device__ __forceinline__ void commit_body(const DecideArgs& a, uint32_t m, unsigned long long big) {
   if (blockIdx.x == 0 && threadIdx.x == 0 && m) atomicAdd(&a.ctrl->moved, (unsigned long long)m);
   uint32_t* C = const_cast<uint32_t*>(a.C);
   long long* Sigma = const_cast<long long*>(a.Sigma);
   int* size = const_cast<int*>(a.size);
-  // warp-uniform loop; movers of one warp joining (or leaving) the same
-  // community are summed first, so a popular community takes one update
-  // per warp instead of one per mover
-  const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-  for (uint64_t t0 = blockIdx.x * uint64_t(blockDim.x) + (threadIdx.x & ~31u); t0 < m; t0 += stride) {
-    const uint64_t t = t0 + (threadIdx.x & 31u);
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t nwarps = gridDim.x * (kCommitThreads / 32);
+  const uint32_t warp = blockIdx.x * (kCommitThreads / 32) + (threadIdx.x >> 5);
+  for (uint64_t t0 = uint64_t(warp) * 32; t0 < m; t0 += uint64_t(nwarps) * 32) {
+    const uint64_t t = t0 + lane;
     const bool ok = t < m;
     const uint32_t i = ok ? a.mv_i[t] : 0u;
     const uint32_t c = ok ? a.mv_c[t] : kEmpty, d = ok ? a.mv_d[t] : kEmpty;
     const long long ki = ok ? a.K[i] : 0;
     if (ok) C[i] = c;
-    const uint32_t lane = threadIdx.x & 31u;
     for (int side = 0; side < 2; ++side) {
       const uint32_t key = side ? d : c;
       long long sk = 0;
@@ -1744,48 +1723,36 @@ __device__ __forceinline__ void commit_body(const DecideArgs& a, uint32_t m, uin
       }
     }
   }
-  const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
-  __shared__ uint32_t s_pre[kCommitThreads + 1];
-  __shared__ uint32_t s_w[kCommitThreads / 32];
-  uint64_t ibase = 0;  // pieces of the earlier tiles
-  for (uint32_t q0 = 0; q0 < count; q0 += kCommitThreads) {
-    const uint32_t q = q0 + threadIdx.x;
-    const uint32_t nch = q < count ? (a.g.deg[a.bigmv[q]] + kMarkChunk - 1) / kMarkChunk : 0u;
-    uint32_t x = nch;
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-      if (lane >= uint32_t(o)) x += y;
+  // marks, the warps counted from the last one down
+  const uint32_t rev = nwarps - 1 - warp;
+  uint32_t per = (m + nwarps - 1) / nwarps;
+  per = per < 32 ? per : 32;
+  for (uint64_t t0 = uint64_t(rev) * per; t0 < m; t0 += uint64_t(nwarps) * per) {
+    const bool ok = lane < per && t0 + lane < m;
+    const uint32_t i = ok ? a.mv_i[t0 + lane] : 0u;
+    const unsigned long long o = ok ? a.g.off[i] : 0ull;
+    uint32_t dg = ok ? a.g.deg[i] : 0u;
+    if (dg > kMarkInline) dg = 0;  // queued
+    // whole-warp rows: all of them while a warp has few movers, else the long ones
+    const uint32_t narrow = per > 4 ? 64u : 0u;
+    for (unsigned mk = __ballot_sync(0xFFFFFFFFu, dg > narrow); mk; mk &= mk - 1) {
+      const int src = __ffs(mk) - 1;
+      mark_arcs(a, __shfl_sync(0xFFFFFFFFu, i, src), __shfl_sync(0xFFFFFFFFu, o, src), 0,
+                __shfl_sync(0xFFFFFFFFu, dg, src), lane, 32);
     }
-    if (lane == 31) s_w[wib] = x;
-    __syncthreads();
-    uint32_t wbase = 0;
-    for (uint32_t k = 0; k < wib; ++k) wbase += s_w[k];
-    s_pre[threadIdx.x + 1] = wbase + x;
-    if (threadIdx.x == 0) s_pre[0] = 0;
-    __syncthreads();
-    const uint32_t tile_items = s_pre[kCommitThreads];
-    // piece `it` of the tile is item ibase + it, handled by block (ibase + it) mod grid
-    for (uint32_t it = uint32_t((blockIdx.x + gridDim.x - ibase % gridDim.x) % gridDim.x); it < tile_items;
-         it += gridDim.x) {
-      uint32_t lo = 0, hi = kCommitThreads;  // tile position owning piece `it`
-      while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (s_pre[mid] <= it) lo = mid;
-        else hi = mid;
-      }
-      const uint32_t i = a.bigmv[q0 + lo];
-      const uint32_t c = it - s_pre[lo];
-      const uint32_t dg = a.g.deg[i];
-      const unsigned long long o = a.g.off[i];
-      const uint32_t k1 = min(dg, (c + 1) * kMarkChunk);
-      for (uint32_t k0 = c * kMarkChunk + wib * 32; k0 < k1; k0 += kCommitThreads) {
-        const uint32_t k = k0 + lane;
-        const uint2 arc = k < k1 ? a.g.arcs[o + k] : make_uint2(i, 0u);
-        mark_next(a, arc.x, k < k1 && arc.x != i && arc.y != 0);
-      }
+    if (!narrow) continue;
+    if (dg > narrow) dg = 0;
+    for (uint32_t s = 0; s * 4 < per; ++s) {
+      const int src = int(s * 4 + (lane >> 3));
+      mark_arcs(a, __shfl_sync(0xFFFFFFFFu, i, src), __shfl_sync(0xFFFFFFFFu, o, src), 0,
+                __shfl_sync(0xFFFFFFFFu, dg, src), lane & 7u, 8);
     }
-    ibase += tile_items;
-    __syncthreads();  // s_pre and s_w are rewritten by the next tile
+  }
+  const uint32_t rows = uint32_t(big >> 32), pieces = uint32_t(big);
+  for (uint64_t p = rev; p < pieces; p += nwarps) {
+    const uint2 e = a.bigmv[find_row(a.bigmv, rows, uint32_t(p))];
+    const uint32_t k0 = (uint32_t(p) - e.y) * kMarkChunk, dg = a.g.deg[e.x];
+    mark_arcs(a, e.x, a.g.off[e.x], k0, dg - k0 < kMarkChunk ? dg : k0 + kMarkChunk, lane, 32);
   }
 }
 
@@ -2044,7 +2011,7 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
       if (!grid_barrier(ctrl, ia.bar_extra, ia.bar_polls)) return;
     }
     // 4. commit the sub-step's moves (and mark around high-degree movers)
-    commit_body(a0, *((volatile unsigned int*)a0.movers), *((volatile unsigned int*)a0.nbig));
+    commit_body(a0, *((volatile unsigned int*)a0.movers), *((volatile unsigned long long*)a0.nbig));
     if (!grid_barrier(ctrl, ia.bar_extra, ia.bar_polls)) return;
   }
   // 5. the next frontier's lists; clear the processed frontier's bitmap
@@ -2233,14 +2200,15 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
       if (pb) h->ev_free.push_back(pb);
     }
     if (any && decide_only) {
-      DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->it_movers[0], 0, 4 * sizeof(unsigned int), spine));
+      // (it_nbig and it_movers are adjacent)
+      DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->it_nbig[0], 0, sizeof(h->ctrl->it_nbig) + sizeof(h->ctrl->it_movers), spine));
     } else if (any) {
       LaunchScope ls(h, DFL_PROF_COMMIT, spine);
-      launch_pdl(k_commit, 152 * 2, kCommitThreads, 0, spine, a);
+      launch_pdl(k_commit, 152 * 4, kCommitThreads, 0, spine, a);
       DFL_TRY(check_launch(h, "commit"));
     } else if (a.clear_movers) {  // no commit ran: zero the next sub-step's counters here
       DFL_CUDA(h, cudaMemsetAsync(a.clear_movers, 0, sizeof(unsigned int), spine));
-      DFL_CUDA(h, cudaMemsetAsync(a.clear_nbig, 0, sizeof(unsigned int), spine));
+      DFL_CUDA(h, cudaMemsetAsync(a.clear_nbig, 0, sizeof(*a.clear_nbig), spine));
     }
   }
   // the next frontier's lists, from its bitmap
@@ -2285,9 +2253,8 @@ uint32_t persistent_grid() {
 int issue_persistent(Handle* h, const DecideArgs& a_base, int cur, const GiantDecide& gd, uint32_t grid) {
   const int nxt = cur ^ 1;
   DFL_CUDA(h, cudaMemsetAsync(h->ctrl, 0, offsetof(Ctrl, move_bytes), h->stream));
-  DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->movers, 0, 2 * sizeof(unsigned int), h->stream));
-  DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->it_movers[0], 0,
-                              offsetof(Ctrl, bar_gen) + sizeof(unsigned int) - offsetof(Ctrl, it_movers),
+  DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->it_nbig[0], 0,
+                              offsetof(Ctrl, bar_gen) + sizeof(unsigned int) - offsetof(Ctrl, it_nbig),
                               h->stream));
   DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->count[nxt][0][0], 0, sizeof(h->ctrl->count[0]), h->stream));
   if (a_base.ngraphs)
@@ -2496,19 +2463,18 @@ int prepare_move(Handle* h, const MoveArgs& ma, DecideArgs* out, GiantDecide* gd
     }
     DFL_TRY(regrow(&h->g_tlist, h->g_lst_cap, lst, sizeof(uint2), -1));
   }
-  {  // movers whose neighbours k_commit marks: at most one per vertex of degree
-     // > kMarkInline, or of the block-per-vertex bin (degree > bin_warp_hash)
+  {  // the queue of movers whose rows k_commit marks in pieces: at most one per
+     // vertex of degree > kMarkInline
     uint64_t arcs = pool_top_bound(h);
     for (int q = 0; q < 2; ++q) arcs = arcs > h->sg[q].arc_cap ? arcs : h->sg[q].arc_cap;
-    const uint64_t lo = h->tune.bin_warp_hash < kMarkInline ? h->tune.bin_warp_hash : kMarkInline;
-    uint64_t need = arcs / (lo + 1) + 64;
+    uint64_t need = arcs / (kMarkInline + 1) + 64;
     if (need > uint64_t(h->n) + 64) need = uint64_t(h->n) + 64;
     if (need > h->bigmv_cap) {
       cudaStreamSynchronize(h->stream);
       cudaFree(h->bigmv);
       h->bigmv = nullptr;
       h->bigmv_cap = 0;
-      DFL_CUDA(h, dev_malloc(&h->bigmv, sizeof(uint32_t) * (need + need / 2)));
+      DFL_CUDA(h, dev_malloc(&h->bigmv, sizeof(uint2) * (need + need / 2)));
       h->bigmv_cap = need + need / 2;
     }
   }
@@ -2549,8 +2515,8 @@ int prepare_move(Handle* h, const MoveArgs& ma, DecideArgs* out, GiantDecide* gd
   a.gtable = need_gtable ? h->gtable : nullptr;
   a.gslots = gslots;
   a.bigmv = h->bigmv;
-  a.movers = &h->ctrl->movers;
-  a.nbig = &h->ctrl->big_movers;
+  a.movers = &h->ctrl->it_movers[0];
+  a.nbig = &h->ctrl->it_nbig[0];
   if (h->ngraphs) {
     a.ngraphs = h->ngraphs;
     a.goff = h->d_goff;

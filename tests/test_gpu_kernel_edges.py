@@ -175,3 +175,23 @@ def test_lane_per_vertex_scores_beyond_64_bits(dfl, orc, flags):
     two_m = a.weights()[2]
     assert two_m < 2**32 and (40 * heavy) * two_m > 2**63
     assert a.stats()["num_communities"] > 12_000 and a.stats()["passes"] > 1
+
+
+@pytest.mark.parametrize("flags", [4, 16, 32])  # host launches, persistent kernel, graph replay
+@pytest.mark.parametrize("degrees", [(8, 9, 64, 65), (511, 512, 513), (1024, 1025, 2600), (520,) * 300])
+def test_movers_mark_their_neighbours(dfl, orc, degrees, flags):
+    """The next frontier around movers whose rows are marked by eight lanes,
+    a warp, or in queued pieces."""
+    g = stars(degrees, 2700, 9)
+    a, b = pair(dfl, orc, g, flags=flags)
+    rng = np.random.default_rng(2)
+    for _ in range(3):
+        C = rng.integers(0, g.n, g.n).astype(np.uint32)
+        a.set_membership(C)
+        b.set_membership(C)
+        F, R = (rng.random(g.n) < 0.7).astype(np.uint8), (rng.random(g.n) < 0.9).astype(np.uint8)
+        F[: len(degrees)] = 1
+        Fa, ma, Sa = a.move_iteration(F, R)
+        Fb, mb, Sb = b.move_iteration(F, R)
+        assert ma[: len(degrees)].any()
+        assert np.array_equal(Fa, Fb) and np.array_equal(ma, mb) and Sa == Sb
