@@ -104,7 +104,10 @@ enum {
                                  default stream).  Without this flag or DFL_FLAG_NO_GRAPH, replay
                                  is used except for group handles and for DF/DS updates of fewer
                                  than 256 batch edges, which launch from the host with the list
-                                 lengths read (empty bins skipped, grids fit to the work) */
+                                 lengths read (empty bins skipped, grids fit to the work).
+                                 Unless this flag forces replay, iterations whose frontier is
+                                 small (a few thousand vertices) run one after another in a
+                                 single launch of one thread-block cluster (same results) */
   DFL_FLAG_PROFILE_MOVE = 64u, /* time only the decide phase of each sub-step (two CUDA events per
                                  sub-step, the DFL_PROF_MOVE class of dfl_profile): the cheap
                                  subset of DFL_FLAG_PROFILE */

@@ -43,6 +43,7 @@ constexpr uint32_t kBinBlock = 4096;     // deg <= 4096: one block, shared-memor
                                           // larger: one block, global-memory table
 constexpr uint32_t kMaxSubsteps = 8;
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;  // empty hash-table key
+constexpr uint32_t kSmallIters = 20;      // iterations of one small-frontier launch
 
 // Error bits raised by kernels (ctrl.err)
 enum : uint32_t {
@@ -90,6 +91,11 @@ struct Ctrl {
   unsigned long long extra_top;      // new arcs of rebuilt rows
   unsigned long long pool_top;       // first free arc slot of the pool
   unsigned long long scratch_top;
+  // small-frontier kernel: iterations it ran, whether the pass is done, the
+  // initial frontier's length, and {processed, moved, S_hi, S_lo} per iteration
+  unsigned int sm_iters, sm_done;
+  unsigned long long sm_first;
+  unsigned long long sm_trace[kSmallIters][4];
   // misc reductions
   unsigned long long red_a;
   unsigned long long red_b;

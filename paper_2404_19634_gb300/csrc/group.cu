@@ -210,6 +210,7 @@ int louvain_group(Handle* h, bool all, bool use_range, uint64_t initial) {
     a.track_ever = pass == 0 && !all;
     a.prefer_host = true;
     a.graph_iters = git.data();
+    a.frontier_hint = (pass == 0 && !all && !use_range) ? h->pend_count : nv;
     uint32_t it = 0;
     uint64_t init0 = 0, ever0 = 0;
     DFL_TRY(local_move(h, a, pass, &it, false, &init0, &ever0));

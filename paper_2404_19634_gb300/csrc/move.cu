@@ -82,6 +82,11 @@ __device__ __forceinline__ i128 gain_num(long long m2, unsigned long long h, lon
   return (i128)p - (i128)q;
 }
 
+// Sigma_c as a 32-bit word (the low half of the int64: Sigma_c is in [0, 2m)).
+__device__ __forceinline__ uint32_t sigma32(const long long* Sigma, uint32_t c) {
+  return reinterpret_cast<const uint32_t*>(Sigma)[2ull * c];
+}
+
 // Outcome of one vertex's decision, identical on every lane / thread.
 __device__ __forceinline__ bool decide_move(const DecideArgs& a, long long m2, uint32_t i, uint32_t d,
                                             long long Ki, bool have, i128 best, uint32_t bc,
@@ -161,15 +166,26 @@ __device__ __forceinline__ void flush_sums_all(const DecideArgs& a, MoveSums v) 
 constexpr uint32_t kMarkInline = 512;
 constexpr uint32_t kMarkChunk = 512;
 
-__device__ __forceinline__ void queue_marks(const DecideArgs& a, uint32_t i, uint32_t dg) {
-  push_row(a.bigmv, a.nbig, i, (dg + kMarkChunk - 1) / kMarkChunk);
+__device__ __forceinline__ void queue_marks(const DecideArgs& a, unsigned long long* counter, uint32_t i,
+                                            uint32_t dg) {
+  push_row(a.bigmv, counter, i, (dg + kMarkChunk - 1) / kMarkChunk);
 }
 
 // Mark arcs [k0, k1) of mover i's row at o, this lane's from k0 + first on in
 // steps of `step`, four arcs' bitmap words in flight: the neighbours' bits in
 // the next frontier's bitmap (the lists are built from it once, at the end of
 // the iteration).  The bits are read first, so a vertex marked by many movers
-// takes one atomic.
+// takes one atomic.  kAppend: a vertex newly marked also goes straight onto its
+// list of the next frontier (the small-frontier kernel; the others build the
+// lists from the bitmap).
+__device__ __forceinline__ void append_next(const DecideArgs& a, uint32_t v) {
+  const uint32_t key = vertex_class(v, a.k, a.seg) * kBins + degree_bin(a.g.deg[v], a.seg);
+  const uint32_t r = atomicAdd(&a.ctrl->count[a.next_buf][key / kBins][key % kBins], 1u);
+  if (r < a.seg.cap[key]) a.next_lists[a.seg.off[key] + r] = v;
+  else atomicOr(&a.ctrl->err, kErrInternal);
+}
+
+template <bool kAppend>
 __device__ __forceinline__ void mark_arcs(const DecideArgs& a, uint32_t i, unsigned long long o, uint32_t k0,
                                           uint32_t k1, uint32_t first, uint32_t step) {
   for (uint32_t b = k0 + first; b < k1; b += 4 * step) {
@@ -188,7 +204,7 @@ __device__ __forceinline__ void mark_arcs(const DecideArgs& a, uint32_t i, unsig
     }
 #pragma unroll
     for (uint32_t u = 0; u < 4; ++u)
-      if (on[u]) bit_set(a.fbits_next, e[u].x);
+      if (on[u] && bit_set(a.fbits_next, e[u].x) && kAppend) append_next(a, e[u].x);
   }
 }
 
@@ -220,11 +236,21 @@ __device__ __forceinline__ void segment_argmax(bool& have, i128& score, uint32_t
   }
 }
 
-// One vertex per W-lane segment (`active` false: the segment idles).  Every
-// lane of the warp must call it.  Returns the segment's move decision.
+// A move: vertex i (row at o, dg arcs, weight K) from community d to c, whose
+// numerator 2m^2 * dQ is gain.
+struct Move {
+  unsigned long long o;
+  uint32_t i, d, c, dg, Ki;
+  i128 gain;
+};
+
+// Decision of one vertex per W-lane segment (`active` false: the segment
+// idles).  Every lane of the warp must call it; the move is returned on every
+// lane of the segment.  The chain list entry -> row header -> arcs (with
+// Sigma and size of the own community) -> communities -> their Sigma bounds it.
 template <int W>
-__device__ __forceinline__ bool decide_segment(const DecideArgs& a, bool active, uint32_t i, long long m2,
-                                               uint32_t gi, MoveSums& sums) {
+__device__ __forceinline__ bool decide_segment(const DecideArgs& a, bool active, uint32_t i, long long m2, Move* mvo,
+                                               MoveSums& sums) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t seg = lane / W, sl = lane % W;
   const unsigned segmask = W == 32 ? 0xFFFFFFFFu : (((1u << W) - 1u) << (seg * W));
@@ -232,6 +258,8 @@ __device__ __forceinline__ bool decide_segment(const DecideArgs& a, bool active,
   const long long Ki = active ? a.K[i] : 0;
   const unsigned long long o = active ? a.g.off[i] : 0ull;
   const uint32_t dg = active ? a.g.deg[i] : 0u;
+  const long long Sd = active ? a.Sigma[d] : 0;
+  const int szd = active ? a.size[d] : 0;
   uint2 arc = sl < dg ? a.g.arcs[o + sl] : make_uint2(i, 0u);
   const bool valid = sl < dg && arc.x != i && arc.y != 0;  // weight 0 = deleted arc
   const uint32_t c = valid ? a.C[arc.x] : kEmpty;
@@ -241,6 +269,7 @@ __device__ __forceinline__ bool decide_segment(const DecideArgs& a, bool active,
   uint32_t hsum = 0;
   bool leader = valid;
   const uint32_t wv = valid ? arc.y : 0u;
+  const uint32_t sg = (valid && c != d) ? sigma32(a.Sigma, c) : 0u;  // (in flight during the rounds)
 #pragma unroll
   for (int k = 0; k < W; ++k) {
     const uint32_t src = seg * W + k;
@@ -259,39 +288,49 @@ __device__ __forceinline__ bool decide_segment(const DecideArgs& a, bool active,
   const bool cand = leader && c != d;
   const unsigned cm = __ballot_sync(0xFFFFFFFFu, cand) & segmask;
   i128 score = 0;
-  if (cand) score = gain_num(m2, hsum, Ki, a.Sigma[c]);
+  if (cand) score = gain_num(m2, hsum, Ki, sg);
   bool have = cand;
   uint32_t bc = c;
   segment_argmax<W>(have, score, bc);
-  i128 gain = 0;
-  const bool mv = active && decide_move(a, m2, i, d, Ki, have, score, bc, Hd, &gain);
-  if (active && sl == 0) sums.bytes += 24 + 12ull * dg + 12ull * __popc(cm);
-  if (mv) {
-    if (sl == 0) {
-      record_move(a, i, bc, d, gain, gi, sums);
-      sums.bytes += 16 + 4ull * dg;
-    }
+  const i128 stay = gain_num(m2, Hd, Ki, Sd - Ki);
+  bool mv = active && have && score > stay;
+  if (mv && szd == 1 && bc > d && a.size[bc] == 1) mv = false;  // singleton-swap guard
+  if (active && sl == 0) sums.bytes += 24 + 12ull * dg + 12ull * __popc(cm) + (mv ? 16 + 4ull * dg : 0ull);
+  *mvo = Move{o, i, d, bc, dg, uint32_t(Ki), score - stay};
+  return mv;
+}
+
+// The same for list positions [first, first + 32 / W) below cnt; counted as
+// processed.  The ever-bit's old value is only looked at after the decision.
+template <int W>
+__device__ __forceinline__ bool decide_position(const DecideArgs& a, const uint32_t* list, uint64_t first, uint32_t cnt, long long m2_one,
+                                                uint32_t* gi, Move* mvo, MoveSums& sums) {
+  const uint32_t lane = threadIdx.x & 31u, seg = lane / W, sl = lane % W;
+  const uint64_t t = first + seg;
+  bool active = t < cnt;
+  const uint32_t i = active ? list[t] : 0u;
+  long long m2 = m2_one;
+  *gi = 0;
+  if (active && !group_active(a, i, &m2, gi)) active = false;
+  const bool head = active && sl == 0;
+  const uint32_t em = 1u << (i & 31u);
+  const uint32_t old = (head && a.ever) ? atomicOr(a.ever + (i >> 5), em) : em;
+  if (active && a.rbits && !bit_test(a.rbits, i)) active = false;  // processed, not in range
+  const bool mv = decide_segment<W>(a, active, i, m2, mvo, sums);
+  if (head) {
+    ++sums.processed;
+    if (!(old & em)) ++sums.ever;
   }
   return mv;
 }
 
-// Vertices [first, cnt) of the list, 32 / W of them per warp.
 template <int W>
 __device__ __forceinline__ void decide_segments(const DecideArgs& a, uint64_t first, uint32_t cnt, long long m2_one,
                                                 MoveSums& sums) {
-  const uint32_t lane = threadIdx.x & 31u, seg = lane / W, sl = lane % W;
-  const uint64_t t = first + seg;
-  bool active = t < cnt;
-  const uint32_t i = active ? a.list[t] : 0u;
-  long long m2 = m2_one;
-  uint32_t gi = 0;
-  if (active && !group_active(a, i, &m2, &gi)) active = false;
-  if (active && sl == 0) {
-    if (a.ever && bit_set(a.ever, i)) ++sums.ever;
-    ++sums.processed;
-  }
-  if (active && a.rbits && !bit_test(a.rbits, i)) active = false;  // processed, not in range
-  decide_segment<W>(a, active, i, m2, gi, sums);
+  uint32_t gi;
+  Move m;
+  const bool mv = decide_position<W>(a, a.list, first, cnt, m2_one, &gi, &m, sums);
+  if (mv && (threadIdx.x & 31u) % W == 0) record_move(a, m.i, m.c, m.d, m.gain, gi, sums);
 }
 
 // Short lists of small vertices: W lanes per vertex of the first list, then
@@ -411,7 +450,7 @@ __device__ __forceinline__ unsigned long long table_argmax(const DecideArgs& a, 
 
 // Reduce (have, score, c) of every thread of the block to thread 0 (larger
 // score wins, ties to the smaller c); every thread calls it.
-constexpr uint32_t kMaxBlockWarps = 16;  // blocks of up to 512 threads
+constexpr uint32_t kMaxBlockWarps = 32;  // blocks of up to 1024 threads
 
 __device__ __forceinline__ void block_argmax(bool& have, i128& best, uint32_t& bc) {
   __shared__ unsigned long long s_lo[kMaxBlockWarps], s_hi[kMaxBlockWarps];
@@ -445,14 +484,11 @@ static_assert(kBinWarpHash <= 8 * 32 && 2 * kBinWarpHash <= kWarpSlots, "a bin-1
 // One vertex of bin 1 by one warp (its degree up to kWarpSlots / 2): up to
 // 32 arcs by the register path, else a shared table of the warp.  Every lane
 // of the warp calls it.
-__device__ __forceinline__ void warp_table_vertex(const DecideArgs& a, uint32_t i, long long m2, uint32_t gi,
-                                                  uint32_t* keys, uint32_t* vals, MoveSums& sums) {
+__device__ __forceinline__ bool warp_table_vertex(const DecideArgs& a, uint32_t i, long long m2, uint32_t* keys,
+                                                  uint32_t* vals, Move* mvo, MoveSums& sums) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t dg = a.g.deg[i];
-  if (dg <= 32) {  // (when bin 0 takes fewer than 32 arcs) registers, not a table
-    decide_segment<32>(a, true, i, m2, gi, sums);
-    return;
-  }
+  if (dg <= 32) return decide_segment<32>(a, true, i, m2, mvo, sums);  // (the lane bin's) registers, not a table
   const uint32_t d = a.C[i];
   const long long Ki = a.K[i];
   const unsigned long long o = a.g.off[i];
@@ -478,15 +514,18 @@ __device__ __forceinline__ void warp_table_vertex(const DecideArgs& a, uint32_t 
   }
   warp_argmax(have, best, bc);
   i128 gain = 0;
-  bool mv = decide_move(a, m2, i, d, Ki, have, best, bc, Hd, &gain);
-  if (lane == 0) sums.bytes += 24 + 12ull * dg + 12ull * ncand;
-  if (mv) {
-    if (lane == 0) {
-      record_move(a, i, bc, d, gain, gi, sums);
-      sums.bytes += 16 + 4ull * dg;
-    }
-  }
+  const bool mv = decide_move(a, m2, i, d, Ki, have, best, bc, Hd, &gain);
+  if (lane == 0) sums.bytes += 24 + 12ull * dg + 12ull * ncand + (mv ? 16 + 4ull * dg : 0ull);
+  *mvo = Move{o, i, d, bc, dg, uint32_t(Ki), gain};
   __syncwarp();
+  return mv;
+}
+
+// A move decided by one thread (or the leader of a warp): recorded, and its
+// row queued for marking if it is long.
+__device__ __forceinline__ void record(const DecideArgs& a, const Move& m, uint32_t gi, MoveSums& sums) {
+  record_move(a, m.i, m.c, m.d, m.gain, gi, sums);
+  if (m.dg > kMarkInline) queue_marks(a, a.nbig, m.i, m.dg);
 }
 
 // ---------------------------------------------------------------------------
@@ -508,11 +547,6 @@ struct VHdr {
   int szd;               // size of d
   bool act;              // processed and in the affected range: decide it
 };
-
-// Sigma_c as a 32-bit word (the low half of the int64: Sigma_c is in [0, 2m)).
-__device__ __forceinline__ uint32_t sigma32(const long long* Sigma, uint32_t c) {
-  return reinterpret_cast<const uint32_t*>(Sigma)[2ull * c];
-}
 
 // Exact 64-bit form of Eq. 2's comparisons.  Adding K_i * 2m to every score
 // of vertex i shifts them all by the same amount:
@@ -721,7 +755,9 @@ __device__ __forceinline__ bool lane_vertex(const DecideArgs& a, const VHdr& v, 
 __device__ __noinline__ void lane_vertices_128(const DecideArgs& a, const VHdr& h, unsigned m, MoveSums& sums) {
   for (; m; m &= m - 1) {
     const VHdr v = shfl_header(h, __ffs(m) - 1);
-    decide_segment<32>(a, true, v.i, v.m2, v.gi, sums);
+    Move mv;
+    if (decide_segment<32>(a, true, v.i, v.m2, &mv, sums) && (threadIdx.x & 31u) == 0)
+      record_move(a, v.i, mv.c, mv.d, mv.gain, v.gi, sums);
   }
 }
 
@@ -847,7 +883,8 @@ __device__ __forceinline__ bool table_vertex(const DecideArgs& a, const VHdr& v,
 // path registers.
 __device__ __noinline__ void warp_vertex_128(const DecideArgs& a, const VHdr& v, uint32_t* keys, uint32_t* vals,
                                              MoveSums& sums) {
-  warp_table_vertex(a, v.i, v.m2, v.gi, keys, vals, sums);
+  Move m;
+  if (warp_table_vertex(a, v.i, v.m2, keys, vals, &m, sums) && (threadIdx.x & 31u) == 0) record(a, m, v.gi, sums);
 }
 
 __global__ void __launch_bounds__(256, 3) k_decide_warp_hash(DecideArgs a) {
@@ -947,9 +984,10 @@ struct BlockScratch {
 // 2 x degree slots at `dyn` (at most kBlockSlots keys + values); a vertex of
 // larger degree whose distinct communities overflow it is redone in the
 // block's slice of the global table.  Every thread of the block calls it.
+// The decision and its move are thread 0's.
 template <int kThreads>
-__device__ __forceinline__ void block_vertex(const DecideArgs& a, uint32_t i, long long m2, uint32_t gi,
-                                             uint32_t* dyn, BlockScratch& sc, MoveSums& sums) {
+__device__ __forceinline__ bool block_vertex(const DecideArgs& a, uint32_t i, long long m2, uint32_t* dyn,
+                                             BlockScratch& sc, Move* mvo, MoveSums& sums) {
   const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
   constexpr uint32_t nthr = kThreads;  // compile-time strides
   const uint32_t d = a.C[i];
@@ -1005,17 +1043,15 @@ __device__ __forceinline__ void block_vertex(const DecideArgs& a, uint32_t i, lo
   for (int x = 16; x; x >>= 1) ncand += __shfl_xor_sync(0xFFFFFFFFu, ncand, x);
   if (lane == 0 && ncand) atomicAdd(&sc.ncand, ncand);
   block_argmax(have, best, bc);
+  bool mv = false;
   if (threadIdx.x == 0) {
     i128 gain = 0;
-    const bool mv = decide_move(a, m2, i, d, Ki, have, best, bc, sc.hd, &gain);
-    sums.bytes += 24 + 12ull * dg + 12ull * sc.ncand;
-    if (mv) {
-      record_move(a, i, bc, d, gain, gi, sums);
-      sums.bytes += 16 + 4ull * dg;
-      if (dg > kMarkInline) queue_marks(a, i, dg);
-    }
+    mv = decide_move(a, m2, i, d, Ki, have, best, bc, sc.hd, &gain);
+    sums.bytes += 24 + 12ull * dg + 12ull * sc.ncand + (mv ? 16 + 4ull * dg : 0ull);
+    *mvo = Move{o, i, d, bc, dg, uint32_t(Ki), gain};
   }
   __syncthreads();
+  return mv;
 }
 
 // Bin 2 (and bin-3 degrees when the tuning sends them here): one block per
@@ -1033,7 +1069,8 @@ __device__ __forceinline__ void block_vertex(const DecideArgs& a, uint32_t i, lo
 template <int kThreads>
 __device__ __noinline__ void block_vertex_slow(const DecideArgs& a, const VHdr& v, uint32_t* dyn, BlockScratch& sc,
                                                MoveSums& sums) {
-  block_vertex<kThreads>(a, v.i, v.m2, v.gi, dyn, sc, sums);
+  Move m;
+  if (block_vertex<kThreads>(a, v.i, v.m2, dyn, sc, &m, sums)) record(a, m, v.gi, sums);
 }
 
 template <int kThreads>
@@ -1162,7 +1199,7 @@ __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
       const bool mv = lane < nv && s_mv[lane];
       const VHdr& v = s_hdr[lane];
       record_moves_warp(a, mv, v.i, s_mvc[lane], v.d, (i128)s_gain[lane], v.gi, sums);
-      if (mv && v.dg > kMarkInline) queue_marks(a, v.i, v.dg);
+      if (mv && v.dg > kMarkInline) queue_marks(a, a.nbig, v.i, v.dg);
     }
     __syncthreads();  // s_hdr and s_mv are rewritten by the next round
   }
@@ -1509,7 +1546,7 @@ __device__ __forceinline__ void giant_chunk(const DecideArgs& a, const GiantDeci
         sums.bytes += 24 + 12ull * dg + 12ull * sc.ncand;
         if (mv) {
           record_move(a, i, bc, d, gain, gi, sums);
-          queue_marks(a, i, dg);
+          queue_marks(a, a.nbig, i, dg);
           sums.bytes += 16 + 4ull * dg;
         }
       }
@@ -1655,7 +1692,7 @@ __device__ __forceinline__ void giant_parts(const DecideArgs& a, const GiantDeci
           sums.bytes += 24 + 12ull * dg;
           if (mv) {
             record_move(a, i, bc, d, gain, gi, sums);
-            queue_marks(a, i, dg);
+            queue_marks(a, a.nbig, i, dg);
             sums.bytes += 16 + 4ull * dg;
           }
         }
@@ -1674,6 +1711,18 @@ __global__ void __launch_bounds__(kGiantThreads) k_giant_decide(DecideArgs a, Gi
   flush_sums(a, sums, threadIdx.x == 0);
 }
 
+// Warp `warp` of `nwarps`' pieces of the queued movers' rows (`big`: the queue's counter).
+template <bool kAppend>
+__device__ __forceinline__ void mark_queued(const DecideArgs& a, unsigned long long big, uint32_t warp,
+                                            uint32_t nwarps) {
+  const uint32_t rows = uint32_t(big >> 32), pieces = uint32_t(big);
+  for (uint64_t p = warp; p < pieces; p += nwarps) {
+    const uint2 e = a.bigmv[find_row(a.bigmv, rows, uint32_t(p))];
+    const uint32_t k0 = (uint32_t(p) - e.y) * kMarkChunk, dg = a.g.deg[e.x];
+    mark_arcs<kAppend>(a, e.x, a.g.off[e.x], k0, dg - k0 < kMarkChunk ? dg : k0 + kMarkChunk, threadIdx.x & 31u, 32);
+  }
+}
+
 constexpr int kCommitThreads = 256;
 
 // Apply the moves of one sub-step and mark the movers' neighbours for the
@@ -1686,15 +1735,14 @@ constexpr int kCommitThreads = 256;
 // vertex's chain: without it the lane kernel takes 27 us instead of 40 on
 // 100,000 vertices of mean degree 16 and the warp tables 45 instead of 55, the
 // commit 25 instead of 9; a small commit takes 4 us as before.
-// Blocks of kCommitThreads threads.
-__device__ __forceinline__ void commit_body(const DecideArgs& a, uint32_t m, unsigned long long big) {
-  if (blockIdx.x == 0 && threadIdx.x == 0 && m) atomicAdd(&a.ctrl->moved, (unsigned long long)m);
+// Warp `warp` of `nwarps`; every lane of it calls this.
+__device__ __forceinline__ void commit_body(const DecideArgs& a, uint32_t m, unsigned long long big, uint32_t warp,
+                                            uint32_t nwarps) {
   uint32_t* C = const_cast<uint32_t*>(a.C);
   long long* Sigma = const_cast<long long*>(a.Sigma);
   int* size = const_cast<int*>(a.size);
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t nwarps = gridDim.x * (kCommitThreads / 32);
-  const uint32_t warp = blockIdx.x * (kCommitThreads / 32) + (threadIdx.x >> 5);
+  if (warp == 0 && lane == 0 && m) atomicAdd(&a.ctrl->moved, (unsigned long long)m);
   for (uint64_t t0 = uint64_t(warp) * 32; t0 < m; t0 += uint64_t(nwarps) * 32) {
     const uint64_t t = t0 + lane;
     const bool ok = t < m;
@@ -1737,23 +1785,18 @@ __device__ __forceinline__ void commit_body(const DecideArgs& a, uint32_t m, uns
     const uint32_t narrow = per > 4 ? 64u : 0u;
     for (unsigned mk = __ballot_sync(0xFFFFFFFFu, dg > narrow); mk; mk &= mk - 1) {
       const int src = __ffs(mk) - 1;
-      mark_arcs(a, __shfl_sync(0xFFFFFFFFu, i, src), __shfl_sync(0xFFFFFFFFu, o, src), 0,
+      mark_arcs<false>(a, __shfl_sync(0xFFFFFFFFu, i, src), __shfl_sync(0xFFFFFFFFu, o, src), 0,
                 __shfl_sync(0xFFFFFFFFu, dg, src), lane, 32);
     }
     if (!narrow) continue;
     if (dg > narrow) dg = 0;
     for (uint32_t s = 0; s * 4 < per; ++s) {
       const int src = int(s * 4 + (lane >> 3));
-      mark_arcs(a, __shfl_sync(0xFFFFFFFFu, i, src), __shfl_sync(0xFFFFFFFFu, o, src), 0,
+      mark_arcs<false>(a, __shfl_sync(0xFFFFFFFFu, i, src), __shfl_sync(0xFFFFFFFFu, o, src), 0,
                 __shfl_sync(0xFFFFFFFFu, dg, src), lane & 7u, 8);
     }
   }
-  const uint32_t rows = uint32_t(big >> 32), pieces = uint32_t(big);
-  for (uint64_t p = rev; p < pieces; p += nwarps) {
-    const uint2 e = a.bigmv[find_row(a.bigmv, rows, uint32_t(p))];
-    const uint32_t k0 = (uint32_t(p) - e.y) * kMarkChunk, dg = a.g.deg[e.x];
-    mark_arcs(a, e.x, a.g.off[e.x], k0, dg - k0 < kMarkChunk ? dg : k0 + kMarkChunk, lane, 32);
-  }
+  mark_queued<false>(a, big, rev, nwarps);
 }
 
 __global__ void __launch_bounds__(kCommitThreads) k_commit(DecideArgs a) {
@@ -1764,7 +1807,8 @@ __global__ void __launch_bounds__(kCommitThreads) k_commit(DecideArgs a) {
     *a.clear_movers = 0;
     *a.clear_nbig = 0;
   }
-  commit_body(a, *a.movers, *a.nbig);
+  commit_body(a, *a.movers, *a.nbig, blockIdx.x * (kCommitThreads / 32) + (threadIdx.x >> 5),
+                     gridDim.x * (kCommitThreads / 32));
 }
 
 int read_ctrl(Handle* h) {
@@ -1790,15 +1834,20 @@ int read_move_ctrl(Handle* h, bool* settled) {
 
 // floor(tau_num * m2^2 / (2 * tau_den * drop^pass)), the exact form of
 // "sum of dQ <= tau" (Alg. 5) with S = sum of the movers' 2m^2 * dQ.
-u128 tolerance_threshold(const dfl_options& o, long long m2, uint32_t pass) {
-  u128 num = (u128)o.tau_num * (u128)(uint64_t)m2 * (u128)(uint64_t)m2;
-  u128 den = (u128)2 * (u128)o.tau_den;
+__host__ __device__ inline u128 tolerance_threshold(uint64_t tau_num, uint64_t tau_den, uint64_t drop, long long m2,
+                                                    uint32_t pass) {
+  u128 num = (u128)tau_num * (u128)(uint64_t)m2 * (u128)(uint64_t)m2;
+  u128 den = (u128)2 * (u128)tau_den;
   for (uint32_t p = 0; p < pass; ++p) {
     if (den > num) return 0;
-    den *= (u128)o.tolerance_drop;
+    den *= (u128)drop;
   }
   if (den == 0) return ~(u128)0;
   return num / den;
+}
+
+u128 tolerance_threshold(const dfl_options& o, long long m2, uint32_t pass) {
+  return tolerance_threshold(o.tau_num, o.tau_den, o.tolerance_drop, m2, pass);
 }
 
 uint32_t next_pow2(uint64_t x) {
@@ -1969,7 +2018,8 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
           ++sums.processed;
         }
         if (a2.rbits && !bit_test(a2.rbits, i)) continue;
-        block_vertex<kIterThreads>(a2, i, m2, gi, dyn, sc, sums);
+        Move m;
+        if (block_vertex<kIterThreads>(a2, i, m2, dyn, sc, &m, sums)) record(a2, m, gi, sums);
       } else if (u < uint64_t(G) + n2 + U1 + UL) {
         // one table-bin or lane-bin vertex per warp and round, in the warp's own table
         const bool table = u < uint64_t(G) + n2 + U1;
@@ -1986,9 +2036,12 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
             if (aw.ever && bit_set(aw.ever, i)) ++sums.ever;
             ++sums.processed;
           }
+          Move m;
           if (!aw.rbits || bit_test(aw.rbits, i))
-            warp_table_vertex(aw, i, m2, gi, dyn + wib * 2 * kWarpSlots, dyn + wib * 2 * kWarpSlots + kWarpSlots,
-                              sums);
+            if (warp_table_vertex(aw, i, m2, dyn + wib * 2 * kWarpSlots, dyn + wib * 2 * kWarpSlots + kWarpSlots, &m,
+                                  sums) &&
+                lane == 0)
+              record(aw, m, gi, sums);
         }
       } else {
         for (uint32_t r = 0; r < kIterRounds0; ++r) {
@@ -2011,7 +2064,8 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
       if (!grid_barrier(ctrl, ia.bar_extra, ia.bar_polls)) return;
     }
     // 4. commit the sub-step's moves (and mark around high-degree movers)
-    commit_body(a0, *((volatile unsigned int*)a0.movers), *((volatile unsigned long long*)a0.nbig));
+    commit_body(a0, *((volatile unsigned int*)a0.movers), *((volatile unsigned long long*)a0.nbig),
+                       blockIdx.x * (kCommitThreads / 32) + wib, gridDim.x * (kCommitThreads / 32));
     if (!grid_barrier(ctrl, ia.bar_extra, ia.bar_polls)) return;
   }
   // 5. the next frontier's lists; clear the processed frontier's bitmap
@@ -2020,6 +2074,430 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
        w += uint64_t(gridDim.x) * blockDim.x)
     ia.fbits_cur[w] = 0;
   flush_sums_all(ia.a, sums);  // every thread holds counts (segment and warp leaders, block leaders)
+}
+
+// ---------------------------------------------------------------------------
+// Small frontiers: one thread-block cluster runs whole local-moving
+// iterations, one after another, in one launch.  A frontier of a few thousand
+// vertices leaves most of the GPU idle, and its iteration is a chain of about
+// a dozen kernels of 2-8 us each (launches, stream forks and joins, a control
+// read), so the chain itself bounds it.  Here the sub-steps' phases are
+// separated by hardware cluster barriers (no polling), newly marked vertices go
+// straight onto the next frontier's lists, and the tolerance test is made on
+// the device.  Vertices are dealt statically: a vertex of the last bin to the
+// whole cluster, over one table spread over the CTAs' shared memory; of the
+// block bin to a CTA, of the table and lane bins to a warp, of bin 0 to a few
+// lanes.  The kernel stops before an iteration whose estimated time is above
+// what the per-bin kernels need (small_cost), leaving its frontier to them.
+// A DF step's four sub-steps of 100 edges on 10,000 vertices take 34 us here
+// (30 + 15 us of decide and commit kernels, 4 us of lists, and the launches and
+// the control read between them before: 195 -> 136 us the whole step); an
+// iteration of the same graph's static run takes 49 us, 75 before.
+// ---------------------------------------------------------------------------
+constexpr int kSmallThreads = 512;
+constexpr uint32_t kSmallCtas = 16;
+constexpr uint32_t kSmallWarps = kSmallThreads / 32 * kSmallCtas;
+constexpr uint32_t kSmallSlots = 16384;                  // slots per CTA of the cluster's table
+constexpr uint32_t kSmallHuge = kSmallSlots * kSmallCtas / 2;  // largest degree it always holds
+constexpr size_t kSmallSmem = sizeof(uint32_t) * 2 * kSmallSlots;
+static_assert(2 * kSmallSlots >= 2 * kBlockSlots + kSmallThreads / 32 * 2 * kWarpSlots,
+              "the cluster table's memory also holds a block table and the warps' tables");
+
+// Estimated ns of one iteration's decisions over lists of the given lengths
+// (measured: a warp decides a vertex, or four of bin 0, in about 2.5 us, a CTA
+// one of the block bin in 6 us, the cluster one of the last bin in 10 us).
+__host__ __device__ inline uint64_t small_cost(const uint32_t* n) {
+  return (uint64_t(n[kBinTiny] / 4) + n[kBinLanes] + 2ull * n[kBinTable]) * 2500 / kSmallWarps +
+         uint64_t(n[kBinWhole]) * 6000 / kSmallCtas + uint64_t(n[kBinHuge]) * 10000;
+}
+constexpr uint64_t kSmallCostMax = 60000;
+
+struct SmallArgs {
+  DecideArgs a[2];         // by the processed frontier's buffer
+  int cur;                 // ... of the first iteration
+  uint32_t seg_lanes;      // W: lanes per bin-0 vertex
+  uint32_t* lists[2];
+  uint32_t* fbits[2];
+  uint32_t max_iters;      // iterations left to the pass
+  uint32_t single;         // stop after one iteration (a group: the host tests each graph's tolerance)
+  uint32_t pass;           // tolerance test
+  uint64_t tau_num, tau_den, drop;
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+// Barrier of the whole cluster: what any thread wrote before it is visible to
+// every thread after it.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Address of shared variable p in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(uint32_t(__cvta_generic_to_shared(p))), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_cas(uint32_t addr, uint32_t cmp, uint32_t val) {
+  uint32_t r;
+  asm volatile("atom.shared::cluster.cas.b32 %0, [%1], %2, %3;" : "=r"(r) : "r"(addr), "r"(cmp), "r"(val) : "memory");
+  return r;
+}
+__device__ __forceinline__ void cluster_add(uint32_t addr, uint32_t val) {
+  asm volatile("red.shared::cluster.add.u32 [%0], %1;" ::"r"(addr), "r"(val) : "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t addr, uint32_t val) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(val) : "memory");
+}
+
+// The cluster's parts of one vertex, gathered in CTA 0.
+struct SmallParts {
+  uint32_t lo[4][kSmallCtas];  // the best score's words
+  uint32_t c[kSmallCtas], have[kSmallCtas], ncand[kSmallCtas];
+  uint32_t hd;                 // weight to the own community
+};
+
+// One vertex by the whole cluster: its arcs' weights summed by community in an
+// open-addressing table of kSmallCtas x kSmallSlots slots (linear probing runs
+// on into the next CTA's slots), then each CTA scores its own slots.  Every
+// thread of the cluster calls it; the move is thread 0's of CTA 0.
+__device__ __forceinline__ bool cluster_vertex(const DecideArgs& a, uint32_t i, long long m2, uint32_t* dyn,
+                                               SmallParts& sp, BlockScratch& sc, Move* mvo, MoveSums& sums) {
+  constexpr uint32_t kMask = kSmallCtas * kSmallSlots - 1;
+  const uint32_t rank = cluster_rank();
+  uint32_t* keys = dyn;
+  uint32_t* vals = dyn + kSmallSlots;
+  const uint32_t d = a.C[i];
+  const long long Ki = a.K[i];
+  const unsigned long long o = a.g.off[i];
+  const uint32_t dg = a.g.deg[i];
+  for (uint32_t s = threadIdx.x; s < kSmallSlots; s += kSmallThreads) {
+    keys[s] = kEmpty;
+    vals[s] = 0;
+  }
+  if (threadIdx.x == 0) {
+    sp.hd = 0;
+    sc.ncand = 0;
+  }
+  cluster_sync();
+  constexpr uint32_t U = 4, kStep = kSmallCtas * kSmallThreads;
+  for (uint32_t b = rank * kSmallThreads + threadIdx.x; b < dg; b += U * kStep) {
+    uint2 e[U];
+    uint32_t c[U];
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) e[u] = b + u * kStep < dg ? a.g.arcs[o + b + u * kStep] : make_uint2(i, 0u);
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) c[u] = (e[u].x != i && e[u].y != 0) ? a.C[e[u].x] : kEmpty;
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      if (c[u] == kEmpty) continue;
+      uint32_t at = hash_move(c[u]) & kMask;
+      bool placed = false;
+      for (uint32_t probe = 0; probe <= kMask && !placed; ++probe) {  // load <= 1/2: the probe ends
+        const uint32_t owner = at / kSmallSlots, slot = at % kSmallSlots;
+        const uint32_t prev = cluster_cas(cluster_addr(keys + slot, owner), kEmpty, c[u]);
+        if (prev == kEmpty || prev == c[u]) {
+          cluster_add(cluster_addr(vals + slot, owner), e[u].y);
+          placed = true;
+        }
+        at = (at + 1) & kMask;
+      }
+      if (!placed) atomicOr(&a.ctrl->err, kErrInternal);
+    }
+  }
+  cluster_sync();
+  bool have = false;
+  i128 best = 0;
+  uint32_t bc = 0, ncand = 0;
+  const unsigned long long hd =
+      table_argmax<4>(a, keys, vals, kSmallSlots, threadIdx.x, kSmallThreads, d, m2, Ki, have, best, bc, ncand);
+  if (hd) cluster_store(cluster_addr(&sp.hd, 0), uint32_t(hd));  // exactly one slot of the table holds d
+  ncand = __reduce_add_sync(0xFFFFFFFFu, ncand);
+  if ((threadIdx.x & 31u) == 0 && ncand) atomicAdd(&sc.ncand, ncand);
+  block_argmax(have, best, bc);
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < 4; ++q) cluster_store(cluster_addr(&sp.lo[q][rank], 0), uint32_t((u128)best >> (32 * q)));
+    cluster_store(cluster_addr(&sp.c[rank], 0), bc);
+    cluster_store(cluster_addr(&sp.have[rank], 0), have ? 1u : 0u);
+    cluster_store(cluster_addr(&sp.ncand[rank], 0), sc.ncand);
+  }
+  cluster_sync();
+  bool mv = false;
+  if (rank == 0 && threadIdx.x == 0) {
+    have = false;
+    ncand = 0;
+    for (uint32_t r = 0; r < kSmallCtas; ++r) {
+      ncand += sp.ncand[r];
+      if (!sp.have[r]) continue;
+      u128 x = 0;
+      for (int q = 3; q >= 0; --q) x = (x << 32) | sp.lo[q][r];
+      if (!have || (i128)x > best || ((i128)x == best && sp.c[r] < bc)) {
+        have = true;
+        best = (i128)x;
+        bc = sp.c[r];
+      }
+    }
+    i128 gain = 0;
+    mv = decide_move(a, m2, i, d, Ki, have, best, bc, sp.hd, &gain);
+    sums.bytes += 24 + 12ull * dg + 12ull * ncand + (mv ? 16 + 4ull * dg : 0ull);
+    *mvo = Move{o, i, d, bc, dg, uint32_t(Ki), gain};
+  }
+  __syncthreads();  // (the parts are rewritten only after the next cluster barrier)
+  return mv;
+}
+
+// The moves a CTA decided in a sub-step, in its shared memory until they are
+// committed.
+struct SmallMove {
+  unsigned long long o;
+  uint32_t i, c, d, dg, Ki, pad;
+};
+constexpr uint32_t kSmallMoves = 1024;
+// Vertices of a sub-step class at most: a CTA then decides at most
+// kSmallClass / kSmallCtas + 8 a warp + 8 of them.
+constexpr uint32_t kSmallClass = 12000;
+static_assert(kSmallClass / kSmallCtas + 8 * kSmallThreads / 32 + kSmallThreads / 32 + 8 <= kSmallMoves,
+              "a CTA's moves fit");
+constexpr size_t kSmallSmemAll = kSmallSmem + sizeof(SmallMove) * kSmallMoves;
+
+__device__ __forceinline__ void small_record(const DecideArgs& a, const Move& m, uint32_t gi, SmallMove* moves,
+                                             uint32_t* count, unsigned long long* nbig, MoveSums& sums) {
+  const uint32_t at = atomicAdd(count, 1u);
+  moves[at] = SmallMove{m.o, m.i, m.c, m.d, m.dg, m.Ki, 0u};
+  const unsigned long long lo = (unsigned long long)((u128)m.gain & 0xFFFFFFFFull);
+  const unsigned long long hi = (unsigned long long)((u128)m.gain >> 32);
+  sums.s_lo += lo;
+  sums.s_hi += hi;
+  if (a.ngraphs) {
+    if (lo) atomicAdd(a.gS + 2 * gi, lo);
+    if (hi) atomicAdd(a.gS + 2 * gi + 1, hi);
+  }
+  if (m.dg > kMarkInline) queue_marks(a, nbig, m.i, m.dg);
+}
+
+__global__ void __launch_bounds__(kSmallThreads, 1) k_small_move(const __grid_constant__ SmallArgs q) {
+  pdl_wait_only();
+  // the warps' tables (empty at rest) and a block table, or the cluster's table; then the moves
+  extern __shared__ uint32_t dyn[];
+  __shared__ SmallParts sp;
+  __shared__ BlockScratch sc;
+  __shared__ uint32_t s_n[kMaxSubsteps][kBins];
+  __shared__ unsigned long long s_cost;
+  __shared__ uint32_t s_refuse, s_huge, s_nmv[2];
+  __shared__ int s_stop;
+  Ctrl* ctrl = q.a[0].ctrl;
+  const Segs& seg = q.a[0].seg;
+  const uint32_t k = q.a[0].k, rank = cluster_rank();
+  const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
+  const uint32_t warp = rank * (kSmallThreads / 32) + wib, rev = kSmallWarps - 1 - warp;
+  uint32_t* keys = dyn + wib * 2 * kWarpSlots;
+  uint32_t* vals = keys + kWarpSlots;
+  uint32_t* block_table = dyn + kSmallThreads / 32 * 2 * kWarpSlots;
+  SmallMove* moves = reinterpret_cast<SmallMove*>(dyn + 2 * kSmallSlots);
+  const long long m2_one = *q.a[0].m2p;
+  u128 threshold = 0;
+  if (threadIdx.x == 0 && !q.single) threshold = tolerance_threshold(q.tau_num, q.tau_den, q.drop, m2_one, q.pass);
+  if (threadIdx.x < 2) s_nmv[threadIdx.x] = 0;
+  auto empty_table = [&] {
+    for (uint32_t x = lane; x < kWarpSlots; x += 32) {
+      keys[x] = kEmpty;
+      vals[x] = 0;
+    }
+    __syncwarp();
+  };
+  empty_table();
+  int cur = q.cur;
+  uint32_t it = 0, step = 0;
+  MoveSums sums;
+  for (;;) {
+    // the frontier's lengths (every CTA reads them and decides alike)
+    if (threadIdx.x == 0) {
+      s_cost = 0;
+      s_refuse = s_huge = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x < k) {
+      uint32_t n[kBins], total = 0;
+      for (int b = 0; b < kBins; ++b) total += s_n[threadIdx.x][b] = n[b] = __ldcg(&ctrl->count[cur][threadIdx.x][b]);
+      atomicAdd(&s_cost, (unsigned long long)small_cost(n));
+      if (total > kSmallClass) s_refuse = 1;
+    }
+    __syncthreads();
+    if (s_cost > kSmallCostMax || s_refuse) break;  // left to the per-bin kernels
+    for (uint32_t s = 0; s < k; ++s)
+      for (uint32_t t = threadIdx.x; t < s_n[s][kBinHuge]; t += kSmallThreads)
+        if (q.a[0].g.deg[q.lists[cur][seg.off[s * kBins + kBinHuge] + t]] > kSmallHuge) s_huge = 1;
+    const int nxt = cur ^ 1;
+    const DecideArgs& a = q.a[cur];  // (marks and appends into the other buffer)
+    const uint32_t* base = q.lists[cur];
+    cluster_sync();  // every CTA has read what is reset here
+    if (s_huge) break;
+    if (rank == 0) {
+      if (threadIdx.x == 0) {
+        if (it == 0) {
+          unsigned long long first = 0;
+          for (uint32_t s = 0; s < k; ++s)
+            for (int b = 0; b < kBins; ++b) first += s_n[s][b];
+          ctrl->sm_first = first;
+        }
+        ctrl->s_lo = ctrl->s_hi = 0;
+        ctrl->processed = ctrl->moved = 0;
+      }
+      if (threadIdx.x < 2) ctrl->it_nbig[threadIdx.x] = 0;
+      for (uint32_t x = threadIdx.x; x < kMaxSubsteps * kBins; x += kSmallThreads) (&ctrl->count[nxt][0][0])[x] = 0;
+    }
+    cluster_sync();
+    for (uint32_t s = 0; s < k; ++s) {
+      const uint32_t n0 = s_n[s][kBinTiny], nl = s_n[s][kBinLanes], n1 = s_n[s][kBinTable], n2 = s_n[s][kBinWhole],
+                     n3 = s_n[s][kBinHuge];
+      if (!(n0 + nl + n1 + n2 + n3)) continue;
+      const uint32_t par = step++ & 1;  // the counters of this sub-step that is run
+      unsigned long long* nbig = &ctrl->it_nbig[par];
+      uint32_t gi;
+      Move m;
+      // 1. decide
+      for (uint32_t t = 0; t < n3; ++t) {
+        const uint32_t i = base[seg.off[s * kBins + kBinHuge] + t];
+        long long m2 = m2_one;
+        gi = 0;
+        if (!group_active(a, i, &m2, &gi)) continue;
+        if (rank == 0 && threadIdx.x == 0) {
+          if (a.ever && bit_set(a.ever, i)) ++sums.ever;
+          ++sums.processed;
+        }
+        if (a.rbits && !bit_test(a.rbits, i)) continue;
+        if (cluster_vertex(a, i, m2, dyn, sp, sc, &m, sums)) small_record(a, m, gi, moves, &s_nmv[par], nbig, sums);
+      }
+      if (n3) {
+        cluster_sync();  // the table's last reader is done: its memory is the warps' again
+        empty_table();
+      }
+      for (uint32_t t = rank; t < n2; t += kSmallCtas) {
+        const uint32_t i = base[seg.off[s * kBins + kBinWhole] + t];
+        long long m2 = m2_one;
+        gi = 0;
+        if (!group_active(a, i, &m2, &gi)) continue;
+        if (threadIdx.x == 0) {
+          if (a.ever && bit_set(a.ever, i)) ++sums.ever;
+          ++sums.processed;
+        }
+        if (a.rbits && !bit_test(a.rbits, i)) continue;
+        if (block_vertex<kSmallThreads>(a, i, m2, block_table, sc, &m, sums))
+          small_record(a, m, gi, moves, &s_nmv[par], nbig, sums);
+      }
+      for (uint32_t u = warp; u < n1; u += kSmallWarps) {
+        // (every lane loads the one header: broadcasts)
+        VHdr v;
+        v.i = base[seg.off[s * kBins + kBinTable] + u];
+        long long m2 = m2_one;
+        v.gi = 0;
+        if (!group_active(a, v.i, &m2, &v.gi)) continue;
+        v.m2 = uint32_t(m2);
+        v.d = a.C[v.i];
+        v.Ki = uint32_t(a.K[v.i]);
+        v.o = a.g.off[v.i];
+        v.dg = a.g.deg[v.i];
+        const uint32_t em = 1u << (v.i & 31u);
+        const uint32_t old = (lane == 0 && a.ever) ? atomicOr(a.ever + (v.i >> 5), em) : em;
+        if (!a.rbits || bit_test(a.rbits, v.i)) {
+          v.Sd = sigma32(a.Sigma, v.d);
+          v.szd = a.size[v.d];
+          v.act = true;
+          bool mv;
+          if (!fits64(v.m2, v.Ki)) {
+            mv = warp_table_vertex(a, v.i, m2, keys, vals, &m, sums);
+            empty_table();
+          } else {
+            const uint2 a0 = lane < v.dg ? a.g.arcs[v.o + lane] : make_uint2(v.i, 0u);
+            uint32_t bc = 0, ncand = 0;
+            i128 gain = 0;
+            mv = v.dg <= 64    ? table_vertex<2>(a, v, a0, keys, vals, &bc, &gain, &ncand)
+                 : v.dg <= 128 ? table_vertex<4>(a, v, a0, keys, vals, &bc, &gain, &ncand)
+                               : table_vertex<8>(a, v, a0, keys, vals, &bc, &gain, &ncand);
+            if (lane == 0) sums.bytes += 24 + 12ull * v.dg + 12ull * ncand + (mv ? 16 + 4ull * v.dg : 0ull);
+            m = Move{v.o, v.i, v.d, bc, v.dg, v.Ki, gain};
+          }
+          if (mv && lane == 0) small_record(a, m, v.gi, moves, &s_nmv[par], nbig, sums);
+        }
+        if (lane == 0) {
+          ++sums.processed;
+          if (!(old & em)) ++sums.ever;
+        }
+      }
+      for (uint32_t t = warp; t < nl; t += kSmallWarps)
+        if (decide_position<32>(a, base + seg.off[s * kBins + kBinLanes], t, nl, m2_one, &gi, &m, sums) && lane == 0)
+          small_record(a, m, gi, moves, &s_nmv[par], nbig, sums);
+      const uint32_t* tiny = base + seg.off[s * kBins + kBinTiny];
+      const uint32_t per = 32 / q.seg_lanes;
+      for (uint32_t first = rev * per; first < n0; first += kSmallWarps * per) {
+        bool mv;
+        switch (q.seg_lanes) {
+          case 4: mv = decide_position<4>(a, tiny, first, n0, m2_one, &gi, &m, sums); break;
+          case 8: mv = decide_position<8>(a, tiny, first, n0, m2_one, &gi, &m, sums); break;
+          case 16: mv = decide_position<16>(a, tiny, first, n0, m2_one, &gi, &m, sums); break;
+          default: mv = decide_position<32>(a, tiny, first, n0, m2_one, &gi, &m, sums); break;
+        }
+        if (mv && lane % q.seg_lanes == 0) small_record(a, m, gi, moves, &s_nmv[par], nbig, sums);
+      }
+      cluster_sync();
+      // 2. commit the CTA's own moves and mark around them; the other pair of counters is idle
+      const uint32_t nm = s_nmv[par];
+      if (threadIdx.x == 0) {
+        s_nmv[par ^ 1] = 0;
+        if (rank == 0) ctrl->it_nbig[par ^ 1] = 0;
+        if (nm) atomicAdd(&ctrl->moved, (unsigned long long)nm);
+      }
+      // a warp per move, or eight lanes when there are many
+      const uint32_t L = nm > 2 * kSmallThreads / 32 ? 8u : 32u, sl = lane & (L - 1);
+      for (uint32_t e0 = wib * (32 / L); e0 < nm; e0 += kSmallThreads / L) {
+        const uint32_t e = e0 + lane / L;
+        if (e >= nm) continue;
+        const SmallMove v = moves[e];
+        if (sl == 0) const_cast<uint32_t*>(a.C)[v.i] = v.c;
+        if (sl == 1 || sl == 2) {
+          const unsigned long long ki = v.Ki;
+          atomicAdd((unsigned long long*)const_cast<long long*>(a.Sigma) + (sl == 1 ? v.c : v.d), sl == 1 ? ki : 0ull - ki);
+        }
+        if (sl == 3 || sl == 4) atomicAdd(const_cast<int*>(a.size) + (sl == 3 ? v.c : v.d), sl == 3 ? 1 : -1);
+        if (v.dg <= kMarkInline) mark_arcs<true>(a, v.i, v.o, 0, v.dg, sl, L);
+      }
+      const unsigned long long big = __ldcg(nbig);
+      mark_queued<true>(a, big, rev, kSmallWarps);
+      cluster_sync();
+    }
+    // 3. the processed frontier's bits, the sums, the tolerance test
+    for (uint32_t s = 0; s < k; ++s)
+      for (int b = 0; b < kBins; ++b)
+        for (uint32_t t = rank * kSmallThreads + threadIdx.x; t < s_n[s][b]; t += kSmallCtas * kSmallThreads)
+          q.fbits[cur][base[seg.off[s * kBins + b] + t] >> 5] = 0u;
+    flush_sums_all(a, sums);
+    sums = MoveSums();
+    cluster_sync();
+    cur = nxt;
+    if (threadIdx.x == 0) {
+      const unsigned long long lo = __ldcg(&ctrl->s_lo), hi = __ldcg(&ctrl->s_hi);
+      const u128 S = ((u128)hi << 32) + (u128)lo;
+      if (rank == 0) {
+        unsigned long long* tr = ctrl->sm_trace[it];
+        tr[0] = __ldcg(&ctrl->processed);
+        tr[1] = __ldcg(&ctrl->moved);
+        tr[2] = (unsigned long long)(S >> 64);
+        tr[3] = (unsigned long long)S;
+      }
+      s_stop = (!q.single && S <= threshold) || it + 1 == q.max_iters ? 2 : (q.single || it + 1 == kSmallIters) ? 1 : 0;
+    }
+    __syncthreads();
+    ++it;
+    if (s_stop) break;
+  }
+  if (rank == 0 && threadIdx.x == 0) {
+    ctrl->sm_iters = it;
+    ctrl->sm_done = it && s_stop == 2;  // converged, or the pass is out of iterations
+  }
 }
 
 // The start of an iteration: its sums (s_lo .. moved), both pairs of mover
@@ -2226,6 +2704,60 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
   return DFL_OK;
 }
 
+// Launch configuration of the small-frontier kernel.
+struct SmallLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  explicit SmallLaunch(cudaStream_t s) {
+    cfg.gridDim = kSmallCtas;
+    cfg.blockDim = kSmallThreads;
+    cfg.dynamicSmemBytes = kSmallSmemAll;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kSmallCtas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+};
+
+// Whether lists of these lengths are a small frontier (the kernel's own rule).
+bool small_frontier(const unsigned int (*n)[kBins]) {
+  uint64_t cost = 0, longest = 0;
+  for (uint32_t s = 0; s < kMaxSubsteps; ++s) {
+    uint64_t total = 0;
+    for (int b = 0; b < kBins; ++b) total += n[s][b];
+    longest = longest > total ? longest : total;
+    cost += small_cost(n[s]);
+  }
+  return cost <= kSmallCostMax && longest <= kSmallClass;
+}
+
+// A frontier of at most this many vertices is tried without reading its
+// lengths first: the kernel checks them itself, and a refusal costs its empty
+// launch (the read it comes back with is needed either way).
+constexpr uint64_t kSmallTry = 16384;
+
+// Whether the GPU can hold the small-frontier kernel's cluster; queried once per process.
+bool small_available() {
+  static std::once_flag once;
+  static bool ok = false;
+  std::call_once(once, [] {
+    int n = 0;
+    if (cudaFuncSetAttribute(k_small_move, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(k_small_move, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmallSmemAll)) ==
+            cudaSuccess) {
+      SmallLaunch l(nullptr);
+      l.cfg.numAttrs = 1;
+      ok = cudaOccupancyMaxActiveClusters(&n, k_small_move, &l.cfg) == cudaSuccess && n >= 1;
+    }
+    if (!ok) cudaGetLastError();
+  });
+  return ok;
+}
+
 // Blocks of the cooperative iteration kernel that are resident at once
 // (0: it cannot run); queried once per process.
 uint32_t persistent_grid() {
@@ -2284,6 +2816,38 @@ int issue_persistent(Handle* h, const DecideArgs& a_base, int cur, const GiantDe
                                             sizeof(uint32_t) * kIterDynWords, h->stream));
   }
   return DFL_OK;
+}
+
+// Local-moving iterations of a small frontier (list buffer `cur`) in one
+// launch; how many ran, and whether the pass is done, is in the control block.
+int issue_small(Handle* h, const DecideArgs& a, int cur, uint32_t pass, uint32_t iters_left) {
+  if (a.ngraphs)
+    DFL_CUDA(h, cudaMemsetAsync(a.gS, 0, sizeof(unsigned long long) * 2 * a.ngraphs, h->stream));
+  SmallArgs q;
+  std::memset(&q, 0, sizeof(q));
+  for (int b = 0; b < 2; ++b) {
+    q.a[b] = a;
+    q.a[b].fbits_next = h->fbits[b ^ 1];
+    q.a[b].next_lists = h->lists[b ^ 1];
+    q.a[b].next_buf = b ^ 1;
+  }
+  q.cur = cur;
+  const uint32_t lim = h->tune.bin_warp;
+  q.seg_lanes = lim <= 4 ? 4 : lim <= 8 ? 8 : lim <= 16 ? 16 : 32;
+  for (int b = 0; b < 2; ++b) {
+    q.lists[b] = h->lists[b];
+    q.fbits[b] = h->fbits[b];
+  }
+  q.max_iters = iters_left;
+  q.single = a.ngraphs ? 1u : 0u;
+  q.pass = pass;
+  q.tau_num = h->opt.tau_num;
+  q.tau_den = h->opt.tau_den;
+  q.drop = h->opt.tolerance_drop;
+  LaunchScope ls(h, DFL_PROF_MOVE);
+  SmallLaunch l(h->stream);
+  cudaLaunchKernelEx(&l.cfg, k_small_move, q);
+  return check_launch(h, "small frontier");
 }
 
 // Everything an iteration graph bakes in; a different key means re-capture.
@@ -2561,10 +3125,16 @@ int local_move(Handle* h, const MoveArgs& ma, uint32_t pass, uint32_t* iteration
   const uint32_t fl = h->opt.flags;
   const bool want_graph = !(fl & DFL_FLAG_NO_GRAPH) && ((fl & DFL_FLAG_GRAPH) || !ma.prefer_host);
   const bool use_graph = !use_persistent && want_graph && ma.g.off == h->off && h->stream != nullptr;
+  // small frontiers: one launch for whole iterations, unless the launch form or
+  // the phases' times were asked for
+  bool can_small = !use_persistent && ma.g.nv && small_available() &&
+                   !(fl & (DFL_FLAG_SERIAL_BINS | DFL_FLAG_PROFILE | DFL_FLAG_PROFILE_MOVE)) &&
+                   !((fl & DFL_FLAG_GRAPH) && use_graph);
   unsigned int cur_count[kMaxSubsteps][kBins];
   unsigned long long skipped = 0;
-  bool have_counts = false;
-  if (!use_graph && !use_persistent) {
+  // a frontier that can only be small needs no read of its lengths first
+  bool small_next = can_small && !use_graph && ma.frontier_hint <= kSmallTry;
+  if (!use_graph && !use_persistent && !small_next) {
     DFL_TRY(read_move_ctrl(h, &settled));  // list lengths of the initial frontier (buffer 0)
     if (settled && !G) {
       threshold = tolerance_threshold(h->opt, h->m2, pass);
@@ -2574,7 +3144,7 @@ int local_move(Handle* h, const MoveArgs& ma, uint32_t pass, uint32_t* iteration
     for (uint32_t s = 0; s < kMaxSubsteps; ++s)
       for (int b = 0; b < kBins; ++b) cur_count[s][b] = h->hctrl->count[0][s][b];
     skipped = h->hctrl->skipped;
-    have_counts = true;
+    small_next = can_small && small_frontier(cur_count);
   }
   DecideArgs a;
   GiantDecide gd;
@@ -2583,7 +3153,60 @@ int local_move(Handle* h, const MoveArgs& ma, uint32_t pass, uint32_t* iteration
   uint32_t it = 0;
   uint64_t hint = ma.frontier_hint;  // upper bound of this iteration's frontier
   Handle::IterGraph* graph_used[2] = {nullptr, nullptr};
+  // the graphs that meet their own tolerance after iteration `it` stop being processed
+  auto group_converged = [&]() -> int {
+    bool changed = false;
+    for (uint32_t g = 0; g < G; ++g) {
+      if (!gactive[g]) continue;
+      if (ma.graph_iters) ma.graph_iters[g] = it;
+      const u128 Sg = ((u128)h->h_gS[2 * g + 1] << 32) + (u128)h->h_gS[2 * g];
+      if (Sg <= gthr[g]) {  // this graph converged: skip its vertices from now on
+        gactive[g] = 0;
+        h->h_gdone[g] = 1;
+        --nactive;
+        changed = true;
+      }
+    }
+    if (changed && nactive) DFL_TRY(group_upload_flags(h, h->d_gdone, h->h_gdone));
+    return DFL_OK;
+  };
+  auto take_counts = [&](int buf) {
+    hint = 0;
+    for (uint32_t s = 0; s < kMaxSubsteps; ++s)
+      for (int b = 0; b < kBins; ++b) hint += cur_count[s][b] = h->hctrl->count[buf][s][b];
+    small_next = can_small && small_frontier(cur_count);
+  };
   while (it < h->opt.max_iterations && (!G || nactive)) {
+    if (small_next) {
+      DFL_TRY(issue_small(h, a, cur, pass, h->opt.max_iterations - it));
+      if (G)
+        DFL_CUDA(h, cudaMemcpyAsync(h->h_gS, h->d_gS, sizeof(unsigned long long) * 2 * G,
+                                    cudaMemcpyDeviceToHost, h->stream));
+      DFL_TRY(read_move_ctrl(h, &settled));
+      if (settled && !G) threshold = tolerance_threshold(h->opt, h->m2, pass);
+      const Ctrl& c = *h->hctrl;
+      if (c.err) return set_error(h, DFL_ERR_CUDA, "internal error in local-moving (table overflow)");
+      if (it == 0) {
+        skipped = c.skipped;
+        if (initial && c.sm_iters) *initial = skipped + c.sm_first;
+      }
+      for (uint32_t r = 0; r < c.sm_iters && record_trace; ++r)
+        for (int q = 0; q < 4; ++q) h->trace.push_back(c.sm_trace[r][q] + (q == 0 && r == 0 ? skipped : 0));
+      if (c.sm_iters) skipped = 0;
+      it += c.sm_iters;
+      cur ^= int(c.sm_iters & 1);
+      const bool ran = c.sm_iters != 0, done = c.sm_done != 0;
+      take_counts(cur);
+      if (!ran) {  // it refused the frontier (above small_cost's limit, or a vertex too large)
+        if (small_next) can_small = false;
+        small_next = false;
+      } else if (G) {
+        DFL_TRY(group_converged());
+      } else if (done) {
+        break;
+      }
+      continue;
+    }
     ++it;
     const int nxt = cur ^ 1;
     if (use_graph) {
@@ -2641,31 +3264,14 @@ int local_move(Handle* h, const MoveArgs& ma, uint32_t pass, uint32_t* iteration
       h->trace.push_back(uint64_t(S >> 64));
       h->trace.push_back(uint64_t(S));
     }
-    if (have_counts)
-      for (uint32_t s = 0; s < kMaxSubsteps; ++s)
-        for (int b = 0; b < kBins; ++b) cur_count[s][b] = c.count[nxt][s][b];
-    hint = 0;
-    for (uint32_t s = 0; s < kMaxSubsteps; ++s)
-      for (int b = 0; b < kBins; ++b) hint += c.count[nxt][s][b];
     cur = nxt;
+    take_counts(cur);
     skipped = 0;
     if (!G) {
       if (S <= threshold) break;  // locally converged
       continue;
     }
-    bool changed = false;
-    for (uint32_t g = 0; g < G; ++g) {
-      if (!gactive[g]) continue;
-      if (ma.graph_iters) ma.graph_iters[g] = it;
-      const u128 Sg = ((u128)h->h_gS[2 * g + 1] << 32) + (u128)h->h_gS[2 * g];
-      if (Sg <= gthr[g]) {  // this graph converged: skip its vertices from now on
-        gactive[g] = 0;
-        h->h_gdone[g] = 1;
-        --nactive;
-        changed = true;
-      }
-    }
-    if (changed && nactive) DFL_TRY(group_upload_flags(h, h->d_gdone, h->h_gdone));
+    DFL_TRY(group_converged());
   }
   h->prof.bytes[DFL_PROF_MOVE] += h->hctrl->move_bytes;
   if (ever) *ever = h->hctrl->ever_count;

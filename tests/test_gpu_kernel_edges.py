@@ -195,3 +195,57 @@ def test_movers_mark_their_neighbours(dfl, orc, degrees, flags):
         Fb, mb, Sb = b.move_iteration(F, R)
         assert ma[: len(degrees)].any()
         assert np.array_equal(Fa, Fb) and np.array_equal(ma, mb) and Sa == Sb
+
+
+def hub_graph(degree, leaves, seed):
+    """A hub of the given degree among weighted leaves joined in a ring."""
+    return stars((degree, 300, 40, 12, 3), leaves, seed)
+
+
+@pytest.mark.parametrize("substeps", [1, 4, 8])
+@pytest.mark.parametrize("degree,leaves", [(4097, 4100), (5000, 6000), (60_000, 70_000), (131_072, 131_100),
+                                           (131_073, 131_100)])  # (the last one is left to the per-bin kernels)
+def test_small_frontier_with_a_hub(dfl, orc, degree, leaves, substeps):
+    """A frontier of a few vertices around a hub decided by the whole cluster:
+    a community of its own for every leaf, and a few communities."""
+    g = hub_graph(degree, leaves, 4)
+    a, b = pair(dfl, orc, g, flags=4, substeps=substeps)
+    rng = np.random.default_rng(8)
+    R = np.ones(g.n, np.uint8)
+    for communities in (g.n, 50, 3):
+        C = (np.arange(g.n) if communities == g.n else rng.integers(0, communities, g.n)).astype(np.uint32)
+        a.set_membership(C)
+        b.set_membership(C)
+        F = np.zeros(g.n, np.uint8)
+        F[:5] = 1
+        F[rng.integers(5, g.n, 200)] = 1
+        Fa, ma, Sa = a.move_iteration(F, R)
+        Fb, mb, Sb = b.move_iteration(F, R)
+        assert np.array_equal(Fa, Fb) and np.array_equal(ma, mb) and Sa == Sb
+        same(a, b)
+
+
+@pytest.mark.parametrize("n,m", [(40, 90), (700, 9000), (3000, 9000), (5000, 60_000)])
+@pytest.mark.parametrize("max_iterations", [1, 2, 20, 47])
+def test_small_frontier_runs_whole_passes(dfl, orc, n, m, max_iterations):
+    """Passes of several iterations in one launch: iteration counts, trace,
+    memberships; also when they take more than one launch's iterations, and
+    sub-steps without a vertex."""
+    g = random_graph(n, m, n + 1)
+    a, b = pair(dfl, orc, g, flags=4, substeps=8, max_iterations=max_iterations, tau_num=1, tau_den=10**12)
+    a.static()
+    b.static()
+    same(a, b)
+    assert a.stats()["iterations"] == b.stats()["iterations"] and a.trace() == b.trace()
+    stream = synth.BatchStream(g, 5)
+    for size in (1, 5, 100):
+        dels, ins = stream.next(size, w_max=9)
+        if size == 5:
+            assert a.apply_batch(dels, ins) == 0
+            a.update(2)
+        else:
+            assert a.step(dels, ins) == 0
+        assert b.apply_batch(dels, ins) == 0
+        b.update(2)
+        same(a, b)
+        assert a.stats()["affected_ever"] == b.stats()["affected_ever"] and a.trace() == b.trace()
