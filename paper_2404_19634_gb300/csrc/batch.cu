@@ -74,12 +74,21 @@ __global__ void k_expand(const dfl_edge* __restrict__ e, uint64_t nd, uint64_t n
   }
 }
 
-// Slot of neighbour v in row u: binary search of the sorted prefix, then a
-// scan of the tail.  Returns kEmpty if absent.
+// Slot of neighbour v in a row (rows start 16-byte aligned and have an even
+// capacity, so arcs are read in pairs): a search of the sorted prefix, whose
+// last step compares a window of 16 arcs at once, then a scan of the tail,
+// whose first eight arcs are loaded before the search (most rows end there).
+// Returns kEmpty if absent; *w: the arc's weight.
 __device__ __forceinline__ uint32_t find_slot(const uint2* __restrict__ row, uint32_t srt, uint32_t deg,
-                                              uint32_t v) {
-  // lower bound of v in the sorted prefix: nine-way splits with the eight
-  // probe loads in flight together (a hub row takes ~6 rounds, not ~20)
+                                              uint32_t v, uint32_t* w) {
+  const uint4* pairs = reinterpret_cast<const uint4*>(row);
+  const uint4 none = make_uint4(~v, 0u, ~v, 0u);
+  uint4 t0[4];
+  const uint32_t tb = srt / 2;  // the pair holding the tail's first arc
+#pragma unroll
+  for (uint32_t j = 0; j < 4; ++j) t0[j] = srt < deg && (tb + j) * 2 < deg ? pairs[tb + j] : none;
+  // bounds of v in the sorted prefix: nine-way splits with the eight probe
+  // loads in flight together (a hub row takes ~6 rounds, not ~20)
   uint32_t lo = 0, hi = srt;
   while (hi - lo > 16) {
     const uint32_t step = (hi - lo) / 9;
@@ -90,33 +99,42 @@ __device__ __forceinline__ uint32_t find_slot(const uint2* __restrict__ row, uin
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const uint32_t pos = lo + (j + 1) * step;
-      if (key[j] < v) nlo = pos + 1;
+      if (key[j] <= v) nlo = pos;
       else if (pos < nhi) nhi = pos;
     }
     lo = nlo;
     hi = nhi;
   }
+  uint32_t at = kEmpty, wt = 0;
+  const auto look = [&](const uint4& x, uint32_t k, uint32_t first, uint32_t end) {
+    if (x.x == v && k >= first && k < end) {
+      at = k;
+      wt = x.y;
+    }
+    if (x.z == v && k + 1 >= first && k + 1 < end) {
+      at = k + 1;
+      wt = x.w;
+    }
+  };
   {
-    uint32_t key[16];
+    uint4 x[9];
+    const uint32_t base = lo / 2;
 #pragma unroll
-    for (int j = 0; j < 16; ++j) key[j] = lo + j < hi ? row[lo + j].x : 0xFFFFFFFFu;
-    uint32_t lb = hi;
+    for (uint32_t j = 0; j < 9; ++j) x[j] = (base + j) * 2 < hi ? pairs[base + j] : none;
 #pragma unroll
-    for (int j = 15; j >= 0; --j)
-      if (lo + j < hi && key[j] >= v) lb = lo + j;
-    lo = lb;
+    for (uint32_t j = 0; j < 9; ++j) look(x[j], (base + j) * 2, lo, hi);
   }
-  if (lo < srt && row[lo].x == v) return lo;
-  // the unsorted tail (at most kTailMax arcs), eight loads in flight
-  for (uint32_t q0 = srt; q0 < deg; q0 += 8) {
-    uint32_t x[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = q0 + u < deg ? row[q0 + u].x : ~v;
+  for (uint32_t j = 0; j < 4; ++j) look(t0[j], (tb + j) * 2, srt, deg);
+  for (uint32_t q = tb + 4; at == kEmpty && q * 2 < deg; q += 4) {
+    uint4 x[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (x[u] == v) return q0 + u;
+    for (uint32_t j = 0; j < 4; ++j) x[j] = (q + j) * 2 < deg ? pairs[q + j] : none;
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) look(x[j], (q + j) * 2, srt, deg);
   }
-  return kEmpty;
+  *w = wt;
+  return at;
 }
 
 // Thread per sorted arc: each run head evaluates its (u, v) change against
@@ -156,8 +174,9 @@ __global__ void k_runs(const unsigned long long* __restrict__ key, const uint32_
     }
     if (ndel > 1) atomicOr(&ctrl->err, kErrInvalid);  // the same edge deleted twice
     const uint2* row = arcs + off[u];
-    uint32_t slot = find_slot(row, srt[u], deg[u], v);
-    unsigned long long wold = slot != kEmpty ? row[slot].y : 0ull;
+    uint32_t wrow = 0;
+    uint32_t slot = find_slot(row, srt[u], deg[u], v, &wrow);
+    unsigned long long wold = wrow;
     unsigned long long weff = 0;
     if (ndel) {
       if (wold == 0 || wdel > wold) atomicOr(&ctrl->err, kErrNotFound);  // absent edge
@@ -461,6 +480,24 @@ __global__ void k_mark_df(const unsigned long long* __restrict__ key, uint64_t n
   }
 }
 
+// The same into the bitmap alone, the lists built from it afterwards: for a
+// batch that touches a good part of the graph, where the appends' counters
+// would be what bounds it (2 million arcs on 2 million vertices: 235 us, now
+// 25 and 15 for the lists).
+__global__ void k_mark_df_bits(const unsigned long long* __restrict__ key, uint64_t na, KeyFmt f,
+                               const uint32_t* __restrict__ C, uint32_t* __restrict__ fbits,
+                               const unsigned int* go) {
+  pdl_wait();
+  if (go && *go == 0u) return;
+  const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
+  for (uint64_t p = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; p < na; p += stride) {
+    const unsigned long long kk = key[p];
+    const uint32_t u = f.u(kk), v = f.v(kk);
+    const bool ins = kk & 1ull;
+    if (ins != (C[u] == C[v]) && !bit_test(fbits, u)) bit_set(fbits, u);
+  }
+}
+
 // Alg. 3, deletions inside a community: dV[i], dE[i], dC[C[j]].
 __global__ void k_ds_del(const unsigned long long* __restrict__ key, uint64_t na, KeyFmt f,
                          const uint32_t* __restrict__ C, uint32_t* dV, uint32_t* dE, uint32_t* dC) {
@@ -605,30 +642,52 @@ __global__ void k_ds_comm(uint32_t n, const uint32_t* __restrict__ C, const uint
 // Hashed batch apply.  Arcs are grouped by (u, v) in an open-addressing table
 // (no sort); a new arc's tail position comes from a per-row counter (the tail
 // is unsorted, so the order does not matter); only rebuilt rows need their
-// new arcs sorted, which a block does in shared memory.  Per-vertex scratch
-// counters are zero at rest and reset for the touched rows at the end.
+// new arcs sorted, which a block does in shared memory.
+//
+// Random accesses bound it (the pair's record, its row's header, counters and
+// arcs), so all that is known of a pair, and all that is counted for a row, is
+// one 32-byte sector, and counters that every warp would update are summed or
+// claimed per block.  With an array per field (eight sectors a pair, five a
+// row) and per-warp updates of the shared counters, 2 million arcs on 2
+// million vertices took 2.75 ms of kernels (insert 258, pairs 1071, rows 62,
+// write 150, rebuild 575, weights 180, finish 103, pending list and reset 105
+// us); now 0.90 ms (insert 100, pairs 397, rows 48, write with the weights
+// 257, rebuild 13, finish with the reset 87).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kExtraMax = 4096;   // new arcs of one rebuilt row sorted in shared memory
 constexpr unsigned long long kNoKey = ~0ull;
 
+}  // namespace
+
+struct alignas(32) PairRec {
+  unsigned long long key;  // u << 32 | v, kNoKey = empty
+  unsigned long long acc;  // summed inserted weight; after validation, the change of the weight (0 at rest)
+  uint32_t nd;             // deletions of the pair; after validation, flags (0 at rest)
+  uint32_t wd;             // weight to delete (0 = all); after validation, row slot or append rank
+  uint32_t wnew;           // weight after the batch
+  uint32_t pad;
+};
+
+struct alignas(32) RowRec {        // zero at rest
+  unsigned long long touch;        // pairs of the row | appended arcs << 32
+  unsigned long long change;       // change of its live arcs + (change of its tombstones << 32), as one sum
+  uint32_t state;                  // 2: rebuilt
+  uint32_t reg;                    // rebuilt row: offset of its new arcs in `extra`
+  uint32_t pad[2];
+  __host__ __device__ uint32_t app() const { return uint32_t(touch >> 32); }
+  __host__ __device__ int live() const { return int(uint32_t(change)); }
+  __host__ __device__ int tomb() const { return int(uint32_t(change >> 32)) + (live() < 0 ? 1 : 0); }  // (its borrow)
+};
+
+namespace {
+
 struct HashApply {
-  unsigned long long* keys;   // (u << 32 | v), kNoKey = empty
-  uint32_t* ndel;             // deletions of the pair
-  uint32_t* wdel;             // their weight (0 = whole edge)
-  unsigned long long* wins;   // summed inserted weight
-  uint32_t* slot;             // row slot of the pair (found) or append rank
-  uint32_t* wnew;
-  uint32_t* flag;
-  long long* delta;
-  uint32_t* pairs;            // occupied table slots, in claim order
+  PairRec* tab;
   uint64_t mask;
-  // per-vertex scratch
-  uint32_t* r_app;            // appends of the row (then: rank counter)
-  int* r_tomb;                // tombstone change
-  int* r_live;                // live-arc change
-  uint32_t* r_state;          // 0 untouched, 1 touched, 2 rebuilt
-  uint32_t* r_reg;            // rebuilt row: offset of its new arcs in `extra`
+  uint32_t* pairs;            // occupied table slots, in claim order
+  RowRec* rec;                // per vertex
   uint32_t* rows;             // touched rows, in touch order
+  uint32_t* rebuild;          // rebuilt rows
   uint2* extra;               // new arcs of rebuilt rows
 };
 
@@ -641,19 +700,31 @@ __device__ __forceinline__ unsigned long long hash64(unsigned long long k) {
   return k;
 }
 
-// Thread per edge: both arcs into the table; arcs also staged (key format of
-// the pending list) for the frontier marking of the next update.
-// Claim `n` consecutive entries of a shared counter for the lanes with `want`
-// set (one atomic per warp); returns this lane's entry.  Every lane of the
-// warp must call it.
-__device__ __forceinline__ uint32_t warp_claim(unsigned int* counter, bool want) {
-  const unsigned m = __ballot_sync(0xFFFFFFFFu, want);
-  if (!m) return 0;
-  const uint32_t lane = threadIdx.x & 31u, leader = __ffs(m) - 1;
-  uint32_t base = 0;
-  if (lane == leader) base = atomicAdd(counter, uint32_t(__popc(m)));
-  base = __shfl_sync(0xFFFFFFFFu, base, leader);
-  return base + __popc(m & ((1u << lane) - 1u));
+// Consecutive entries of a shared counter for the block's threads, `want` (0
+// to 2) each, with one global atomic per block; returns this thread's first
+// entry.  Every thread of the block (at most 1024) must call it.
+__device__ __forceinline__ uint32_t block_claim(unsigned int* counter, uint32_t want) {
+  __shared__ uint32_t s_w[32], s_base;
+  const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const unsigned m1 = __ballot_sync(0xFFFFFFFFu, want & 1u), m2 = __ballot_sync(0xFFFFFFFFu, want & 2u);
+  if (lane == 0) s_w[wib] = __popc(m1) + 2 * __popc(m2);
+  __syncthreads();
+  if (wib == 0) {
+    const uint32_t v = lane < nw ? s_w[lane] : 0u;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+      if (lane >= uint32_t(o)) x += y;
+    }
+    if (lane == 31 && x) s_base = atomicAdd(counter, x);
+    if (lane < nw) s_w[lane] = x - v;
+  }
+  __syncthreads();
+  const unsigned below = (1u << lane) - 1u;
+  const uint32_t at = s_base + s_w[wib] + __popc(m1 & below) + 2 * __popc(m2 & below);
+  __syncthreads();  // s_w and s_base are rewritten by the next call
+  return at;
 }
 
 __device__ __forceinline__ long long warp_sum64(long long x) {
@@ -661,59 +732,58 @@ __device__ __forceinline__ long long warp_sum64(long long x) {
   return x;
 }
 
+// One edge per thread and round: both arcs into the table (the two probes in
+// flight together), and onto the pending list in the next update's key
+// format (they join it only if the batch is written).
 // del: the nd deletions, ins: the ne - nd insertions
 __device__ __forceinline__ void hash_insert_body(const dfl_edge* __restrict__ del, const dfl_edge* __restrict__ ins,
-                              uint64_t nd, uint64_t ne, uint32_t n,
-                              KeyFmt f, HashApply t, unsigned long long* __restrict__ key,
-                              uint32_t* __restrict__ w, Ctrl* ctrl, uint64_t base, uint64_t stride) {
-  // warp-uniform loop: the claims of new table slots are made per warp
-  const uint32_t lane = threadIdx.x & 31u;
-  for (uint64_t q0 = base + (threadIdx.x & ~31u); q0 < ne; q0 += stride) {
-    const uint64_t q = q0 + lane;
+                                                 uint64_t nd, uint64_t ne, uint32_t n, KeyFmt f, HashApply t,
+                                                 unsigned long long* __restrict__ key, uint32_t* __restrict__ w,
+                                                 Ctrl* ctrl, uint64_t base, uint64_t stride) {
+  for (uint64_t q0 = base; q0 < ne; q0 += stride) {  // block-uniform: claims are made per block
+    const uint64_t q = q0 + threadIdx.x;
     bool valid = q < ne;
     const bool is_ins = q >= nd;
-    dfl_edge x = valid ? (is_ins ? ins[q - nd] : del[q]) : dfl_edge{0, 0, 0};
+    const dfl_edge x = valid ? (is_ins ? ins[q - nd] : del[q]) : dfl_edge{0, 0, 0};
     if (valid && (x.u >= n || x.v >= n || x.u == x.v || (is_ins && x.w == 0))) {
       atomicOr(&ctrl->err, kErrInvalid);
       key[2 * q] = key[2 * q + 1] = 0;
       w[2 * q] = w[2 * q + 1] = 0;
       valid = false;
     }
-    for (int dir = 0; dir < 2; ++dir) {
-      bool claimed = false;
-      uint32_t cs = 0;
-      if (valid) {
+    uint32_t claimed = 0, cs[2] = {0, 0};
+    if (valid) {
+      unsigned long long k[2], prev[2];
+      uint64_t s[2];
+#pragma unroll
+      for (int dir = 0; dir < 2; ++dir) {
         const uint32_t a = dir ? x.v : x.u, b = dir ? x.u : x.v;
-        key[2 * q + dir] = ((unsigned long long)a << (f.b + 1)) | ((unsigned long long)b << 1) |
-                           (is_ins ? 1ull : 0ull);
+        key[2 * q + dir] = ((unsigned long long)a << (f.b + 1)) | ((unsigned long long)b << 1) | (is_ins ? 1ull : 0ull);
         w[2 * q + dir] = x.w;
-        const unsigned long long k = ((unsigned long long)a << 32) | b;
-        uint64_t s = hash64(k) & t.mask;
-        for (uint64_t probe = 0; probe <= t.mask; ++probe) {
-          unsigned long long prev = t.keys[s];
-          if (prev == kNoKey) {
-            prev = atomicCAS(&t.keys[s], kNoKey, k);
-            if (prev == kNoKey) {
-              claimed = true;
-              cs = uint32_t(s);
-              prev = k;
-            }
-          }
-          if (prev == k) {
-            if (is_ins) {
-              atomicAdd(&t.wins[s], (unsigned long long)x.w);
-            } else {
-              atomicAdd(&t.ndel[s], 1u);
-              t.wdel[s] = x.w;  // several deletions of one pair are an error anyway
-            }
-            break;
-          }
-          s = (s + 1) & t.mask;
+        k[dir] = ((unsigned long long)a << 32) | b;
+        s[dir] = hash64(k[dir]) & t.mask;
+      }
+#pragma unroll
+      for (int dir = 0; dir < 2; ++dir) prev[dir] = atomicCAS(&t.tab[s[dir]].key, kNoKey, k[dir]);
+#pragma unroll
+      for (int dir = 0; dir < 2; ++dir) {
+        for (uint64_t probe = 0; prev[dir] != kNoKey && prev[dir] != k[dir] && probe < t.mask; ++probe) {
+          s[dir] = (s[dir] + 1) & t.mask;
+          prev[dir] = atomicCAS(&t.tab[s[dir]].key, kNoKey, k[dir]);
+        }
+        if (prev[dir] == kNoKey) cs[claimed++] = uint32_t(s[dir]);
+        PairRec& r = t.tab[s[dir]];
+        if (is_ins) {
+          atomicAdd(&r.acc, (unsigned long long)x.w);
+        } else {
+          atomicAdd(&r.nd, 1u);
+          r.wd = x.w;  // several deletions of one pair are an error anyway
         }
       }
-      const uint32_t at = warp_claim(&ctrl->npairs, claimed);
-      if (claimed) t.pairs[at] = cs;
     }
+    const uint32_t at = block_claim(&ctrl->npairs, claimed);
+    if (claimed > 0) t.pairs[at] = cs[0];
+    if (claimed > 1) t.pairs[at + 1] = cs[1];
   }
 }
 
@@ -726,27 +796,25 @@ __global__ void k_hash_insert(const dfl_edge* __restrict__ del, const dfl_edge* 
 
 // Thread per pair: validate against the row, weights after the batch, and
 // per-row bookkeeping (append ranks, live and tombstone changes).
-__device__ __forceinline__ void hash_pairs_body(HashApply t, uint32_t n, const unsigned long long* __restrict__ off,
-                             const uint32_t* __restrict__ deg, const uint32_t* __restrict__ srt,
-                             const uint2* __restrict__ arcs, Ctrl* ctrl, uint64_t base, uint64_t stride) {
+__device__ __forceinline__ void hash_pairs_body(HashApply t, const unsigned long long* __restrict__ off,
+                                                const uint32_t* __restrict__ deg, const uint32_t* __restrict__ srt,
+                                                const uint2* __restrict__ arcs, Ctrl* ctrl, uint64_t base,
+                                                uint64_t stride) {
   const uint32_t np = ctrl->npairs;
-  const uint32_t lane = threadIdx.x & 31u;
-  // warp-uniform loop: 2m and arc-count changes are summed, new rows claimed, per warp
-  for (uint64_t p0 = base + (threadIdx.x & ~31u); p0 < np; p0 += stride) {
-    const uint64_t p = p0 + lane;
-    long long dm2 = 0, darcs = 0;
+  long long dm2 = 0, darcs = 0;
+  for (uint64_t p0 = base; p0 < np; p0 += stride) {  // block-uniform: new rows are claimed per block
+    const uint64_t p = p0 + threadIdx.x;
     bool new_row = false;
-    uint32_t row_u = 0;
+    uint32_t u = 0;
     if (p < np) {
-      const uint32_t s = t.pairs[p];
-      const unsigned long long k = t.keys[s];
-      const uint32_t u = uint32_t(k >> 32), v = uint32_t(k);
-      const uint32_t ndel = t.ndel[s], wdel = t.wdel[s];
-      const unsigned long long wins = t.wins[s];
+      PairRec& r = t.tab[t.pairs[p]];
+      const unsigned long long k = r.key, wins = r.acc;
+      u = uint32_t(k >> 32);
+      const uint32_t v = uint32_t(k), ndel = r.nd, wdel = r.wd;
       if (ndel > 1) atomicOr(&ctrl->err, kErrInvalid);  // the same edge deleted twice
-      const uint2* row = arcs + off[u];
-      const uint32_t slot = find_slot(row, srt[u], deg[u], v);
-      const unsigned long long wold = slot != kEmpty ? row[slot].y : 0ull;
+      uint32_t wrow = 0;
+      const uint32_t slot = find_slot(arcs + off[u], srt[u], deg[u], v, &wrow);
+      const unsigned long long wold = wrow;
       unsigned long long weff = 0;
       if (ndel) {
         if (wold == 0 || wdel > wold) atomicOr(&ctrl->err, kErrNotFound);
@@ -760,67 +828,63 @@ __device__ __forceinline__ void hash_pairs_body(HashApply t, uint32_t n, const u
       if (wn > 0) fl |= kLiveAfter;
       if (slot == kEmpty && wn > 0) fl |= kAppend;
       const long long dl = (long long)wins - (long long)weff;
-      t.wnew[s] = uint32_t(wn);
-      t.flag[s] = fl;
-      t.delta[s] = dl;
-      t.slot[s] = (fl & kAppend) ? atomicAdd(&t.r_app[u], 1u) : slot;
-      dm2 = dl;
+      RowRec& rr = t.rec[u];
+      const unsigned long long old = atomicAdd(&rr.touch, 1ull + ((fl & kAppend) ? 1ull << 32 : 0ull));
+      new_row = uint32_t(old) == 0u;
       const int live = (wn > 0 ? 1 : 0) - (wold > 0 ? 1 : 0);
-      if (live) {
-        atomicAdd(&t.r_live[u], live);
-        darcs = live;
-      }
-      if ((fl & kFound) && wold > 0 && wn == 0) atomicAdd(&t.r_tomb[u], 1);
-      if ((fl & kFound) && wold == 0 && wn > 0) atomicAdd(&t.r_tomb[u], -1);
-      new_row = atomicCAS(&t.r_state[u], 0u, 1u) == 0u;
-      row_u = u;
+      const int tomb = (fl & kFound) ? -live : 0;
+      if (live) atomicAdd(&rr.change, (unsigned long long)((long long)live + (long long)tomb * (1ll << 32)));
+      r.acc = (unsigned long long)dl;
+      r.nd = fl;
+      r.wd = (fl & kAppend) ? uint32_t(old >> 32) : slot;
+      r.wnew = uint32_t(wn);
+      dm2 += dl;
+      darcs += live;
     }
-    const uint32_t at = warp_claim(&ctrl->rows, new_row);
-    if (new_row) t.rows[at] = row_u;
-    dm2 = warp_sum64(dm2);
-    darcs = warp_sum64(darcs);
-    if (lane == 0) {
-      if (dm2) atomicAdd((unsigned long long*)&ctrl->m2_delta, (unsigned long long)dm2);
-      if (darcs) atomicAdd((unsigned long long*)&ctrl->arc_delta, (unsigned long long)darcs);
-    }
+    const uint32_t at = block_claim(&ctrl->rows, new_row ? 1u : 0u);
+    if (new_row) t.rows[at] = u;
+  }
+  dm2 = warp_sum64(dm2);
+  darcs = warp_sum64(darcs);
+  if ((threadIdx.x & 31u) == 0) {
+    if (dm2) atomicAdd((unsigned long long*)&ctrl->m2_delta, (unsigned long long)dm2);
+    if (darcs) atomicAdd((unsigned long long*)&ctrl->arc_delta, (unsigned long long)darcs);
   }
 }
 
-__global__ void k_hash_pairs(HashApply t, uint32_t n, const unsigned long long* __restrict__ off,
+__global__ void k_hash_pairs(HashApply t, const unsigned long long* __restrict__ off,
                              const uint32_t* __restrict__ deg, const uint32_t* __restrict__ srt,
                              const uint2* __restrict__ arcs, Ctrl* ctrl) {
   pdl_wait();
-  hash_pairs_body(t, n, off, deg, srt, arcs, ctrl, blockIdx.x * uint64_t(blockDim.x), uint64_t(gridDim.x) * blockDim.x);
+  hash_pairs_body(t, off, deg, srt, arcs, ctrl, blockIdx.x * uint64_t(blockDim.x), uint64_t(gridDim.x) * blockDim.x);
 }
 
 // Thread per touched row: keep (append in place) or rebuild.
 __device__ __forceinline__ void hash_rows_body(HashApply t, const uint32_t* __restrict__ deg, const uint32_t* __restrict__ cap,
                             const uint32_t* __restrict__ srt, const uint32_t* __restrict__ ntomb, Ctrl* ctrl, uint64_t base, uint64_t stride) {
   const uint32_t nr = ctrl->rows;
-  for (uint64_t q0 = base + (threadIdx.x & ~31u); q0 < nr; q0 += stride) {
-    const uint64_t q = q0 + (threadIdx.x & 31u);
-    uint32_t dmax = 0;
-    if (q < nr) {
-      const uint32_t u = t.rows[q];
-      const uint32_t d = deg[u], s = srt[u], app = t.r_app[u];
-      const long long tomb = (long long)ntomb[u] + t.r_tomb[u];
-      const long long live = (long long)d - ntomb[u] + t.r_live[u];
-      const uint32_t raw = d + app;
-      const uint32_t tomb_lim = raw / 4 > kTombMin ? raw / 4 : kTombMin;
-      const bool rebuild = raw > cap[u] || d - s + app > kTailMax || uint32_t(tomb) > tomb_lim;
-      if (rebuild) {
-        t.r_state[u] = 2u;
-        t.r_reg[u] = uint32_t(atomicAdd(&ctrl->extra_top, (unsigned long long)app));
-        atomicAdd(&ctrl->rebuild_rows, 1u);
-        atomicAdd(&ctrl->reloc_need, (unsigned long long)grow_cap(uint32_t(live)));
-        atomicAdd(&ctrl->scratch_need, (unsigned long long)s);
-        atomicMax(&ctrl->max_app, app);
-      }
-      dmax = rebuild ? uint32_t(live) : raw;
+  uint32_t dmax = 0;
+  for (uint64_t q = base + threadIdx.x; q < nr; q += stride) {
+    const uint32_t u = t.rows[q];
+    const RowRec rr = t.rec[u];
+    const uint32_t d = deg[u], s = srt[u], app = rr.app();
+    const long long tomb = (long long)ntomb[u] + rr.tomb();
+    const long long live = (long long)d - ntomb[u] + rr.live();
+    const uint32_t raw = d + app;
+    const uint32_t tomb_lim = raw / 4 > kTombMin ? raw / 4 : kTombMin;
+    const bool rebuild = raw > cap[u] || d - s + app > kTailMax || uint32_t(tomb) > tomb_lim;
+    if (rebuild) {
+      t.rec[u].state = 2u;
+      t.rec[u].reg = uint32_t(atomicAdd(&ctrl->extra_top, (unsigned long long)app));
+      t.rebuild[atomicAdd(&ctrl->rebuild_rows, 1u)] = u;
+      atomicAdd(&ctrl->reloc_need, (unsigned long long)grow_cap(uint32_t(live)));
+      atomicAdd(&ctrl->scratch_need, (unsigned long long)s);
+      atomicMax(&ctrl->max_app, app);
     }
-    dmax = __reduce_max_sync(0xFFFFFFFFu, dmax);  // one update per warp
-    if ((threadIdx.x & 31u) == 0 && dmax) atomicMax(&ctrl->max_deg, dmax);
+    dmax = max(dmax, rebuild ? uint32_t(live) : raw);
   }
+  dmax = __reduce_max_sync(0xFFFFFFFFu, dmax);  // one update per warp
+  if ((threadIdx.x & 31u) == 0 && dmax) atomicMax(&ctrl->max_deg, dmax);
 }
 
 __global__ void k_hash_rows(HashApply t, const uint32_t* __restrict__ deg, const uint32_t* __restrict__ cap,
@@ -829,24 +893,80 @@ __global__ void k_hash_rows(HashApply t, const uint32_t* __restrict__ deg, const
   hash_rows_body(t, deg, cap, srt, ntomb, ctrl, blockIdx.x * uint64_t(blockDim.x), uint64_t(gridDim.x) * blockDim.x);
 }
 
+// Changes of the communities' Sigma, summed per block in a small direct-mapped
+// shared cache before they go to memory: a large community takes an update per
+// block, not per arc.  Communities that meet an occupied entry go straight to
+// memory.  `sigma_flush` (after a block barrier) writes the sums back.
+// A change is kept as its low 16 bits and the rest, in two 32-bit sums (64-bit
+// shared adds retry under contention: 17 us for 12,000 arcs that mostly meet a
+// few communities, against 6.5), which hold the changes of kSigmaPairs pairs.
+constexpr uint32_t kSigmaCache = 512;
+constexpr uint64_t kSigmaPairs = 16384;
+struct SigmaCache {
+  uint32_t c[kSigmaCache], lo[kSigmaCache];
+  int hi[kSigmaCache];
+};
+
+__device__ __forceinline__ void sigma_init(SigmaCache& sc) {
+  for (uint32_t x = threadIdx.x; x < kSigmaCache; x += blockDim.x) {
+    sc.c[x] = kEmpty;
+    sc.lo[x] = 0;
+    sc.hi[x] = 0;
+  }
+}
+
+__device__ __forceinline__ void sigma_add(SigmaCache& sc, long long* Sigma, uint32_t c, long long dl) {
+  const uint32_t x = (c * 0x9E3779B1u) >> 23;  // 512 entries
+  uint32_t prev = sc.c[x];
+  if (prev == kEmpty) prev = atomicCAS(&sc.c[x], kEmpty, c);
+  if (prev == kEmpty || prev == c) {
+    const uint32_t lo = uint32_t(dl) & 0xFFFFu;
+    const int hi = int(dl >> 16);  // |dl| < 2^33
+    if (lo) atomicAdd(&sc.lo[x], lo);
+    if (hi) atomicAdd(&sc.hi[x], hi);
+  } else {
+    atomicAdd((unsigned long long*)&Sigma[c], (unsigned long long)dl);
+  }
+}
+
+__device__ __forceinline__ void sigma_flush(const SigmaCache& sc, long long* Sigma) {
+  for (uint32_t x = threadIdx.x; x < kSigmaCache; x += blockDim.x) {
+    const long long sum = (long long)sc.hi[x] * 65536 + (long long)sc.lo[x];
+    if (sum) atomicAdd((unsigned long long*)&Sigma[sc.c[x]], (unsigned long long)sum);
+  }
+}
+
 // Thread per pair: in-place weight changes; new arcs to the row's tail, or to
-// the rebuilt row's region of `extra`.
+// the rebuilt row's region of `extra`; K[u] and Sigma[C^{t-1}[u]] change by
+// the net weight (Alg. 7).  Every thread of the block calls it.
 __device__ __forceinline__ void hash_write_body(HashApply t, const unsigned long long* __restrict__ off,
-                             const uint32_t* __restrict__ deg, uint2* __restrict__ arcs, Ctrl* ctrl, uint64_t base, uint64_t stride) {
+                                                const uint32_t* __restrict__ deg, uint2* __restrict__ arcs,
+                                                const uint32_t* __restrict__ C, long long* __restrict__ K,
+                                                long long* __restrict__ Sigma, Ctrl* ctrl, uint64_t base,
+                                                uint64_t stride) {
+  __shared__ SigmaCache sc;
   const uint32_t np = ctrl->npairs;
-  for (uint64_t p = base + threadIdx.x; p < np;
-       p += stride) {
-    const uint32_t s = t.pairs[p];
-    const uint32_t fl = t.flag[s];
-    const unsigned long long k = t.keys[s];
-    const uint32_t u = uint32_t(k >> 32), v = uint32_t(k);
+  if (base >= np) return;  // block-uniform: no pair for this block
+  sigma_init(sc);
+  __syncthreads();
+  for (uint64_t p = base + threadIdx.x; p < np; p += stride) {
+    const PairRec r = t.tab[t.pairs[p]];
+    const uint32_t u = uint32_t(r.key >> 32), v = uint32_t(r.key), fl = r.nd;
     if (fl & kFound) {
-      arcs[off[u] + t.slot[s]].y = t.wnew[s];
+      arcs[off[u] + r.wd].y = r.wnew;
     } else if (fl & kAppend) {
-      if (t.r_state[u] == 2u) t.extra[t.r_reg[u] + t.slot[s]] = make_uint2(v, t.wnew[s]);
-      else arcs[off[u] + deg[u] + t.slot[s]] = make_uint2(v, t.wnew[s]);
+      const RowRec& rr = t.rec[u];
+      if (rr.state == 2u) t.extra[rr.reg + r.wd] = make_uint2(v, r.wnew);
+      else arcs[off[u] + deg[u] + r.wd] = make_uint2(v, r.wnew);
+    }
+    const long long dl = (long long)r.acc;
+    if (dl) {
+      atomicAdd((unsigned long long*)&K[u], (unsigned long long)dl);
+      sigma_add(sc, Sigma, C[u], dl);
     }
   }
+  __syncthreads();
+  sigma_flush(sc, Sigma);
 }
 
 // Whether a validated batch is written: no error, 2m stays below 2^32 (single
@@ -873,8 +993,9 @@ __device__ __forceinline__ bool gate_open(const Ctrl& c, const ApplyGate& g) {
 // ctrl->apply_go / apply_defer for the kernels after this one and the host),
 // and nothing is written if it is closed.
 __global__ void k_hash_write(HashApply t, const unsigned long long* __restrict__ off,
-                             const uint32_t* __restrict__ deg, uint2* __restrict__ arcs, Ctrl* ctrl,
-                             ApplyGate g) {
+                             const uint32_t* __restrict__ deg, uint2* __restrict__ arcs,
+                             const uint32_t* __restrict__ C, long long* __restrict__ K, long long* __restrict__ Sigma,
+                             Ctrl* ctrl, ApplyGate g) {
   pdl_wait();
   const bool go = gate_open(*ctrl, g);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -882,7 +1003,7 @@ __global__ void k_hash_write(HashApply t, const unsigned long long* __restrict__
     ctrl->apply_defer = go && ctrl->rebuild_rows ? 1u : 0u;
   }
   if (!go) return;
-  hash_write_body(t, off, deg, arcs, ctrl, blockIdx.x * uint64_t(blockDim.x), uint64_t(gridDim.x) * blockDim.x);
+  hash_write_body(t, off, deg, arcs, C, K, Sigma, ctrl, blockIdx.x * uint64_t(blockDim.x), uint64_t(gridDim.x) * blockDim.x);
 }
 
 constexpr int kHRebuildThreads = 256;
@@ -899,14 +1020,14 @@ __device__ __forceinline__ void hash_rebuild_body(HashApply t, unsigned long lon
   __shared__ uint2 sn[kExtraMax];
   __shared__ unsigned long long s_sbase, s_dst;
   __shared__ uint32_t s_nt, s_warp[kHRebuildThreads / 32], s_total;
-  const uint32_t nr = ctrl->rows;
+  const uint32_t nr = ctrl->rebuild_rows;
   const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
   for (uint32_t r = r0; r < nr; r += rstep) {
-    const uint32_t u = t.rows[r];
-    if (t.r_state[u] != 2u) continue;
+    const uint32_t u = t.rebuild[r];
+    const RowRec rr = t.rec[u];
     const uint2* old = arcs + off[u];
-    const uint32_t d = deg[u], s = srt[u], nnew = t.r_app[u];
-    const uint32_t live = uint32_t((long long)d - ntomb[u] + t.r_live[u]);
+    const uint32_t d = deg[u], s = srt[u], nnew = rr.app();
+    const uint32_t live = uint32_t((long long)d - ntomb[u] + rr.live());
     const uint32_t nc = grow_cap(live);
     if (threadIdx.x == 0) {
       s_sbase = atomicAdd(&ctrl->scratch_top, (unsigned long long)s);
@@ -952,7 +1073,7 @@ __device__ __forceinline__ void hash_rebuild_body(HashApply t, unsigned long lon
     uint32_t np2 = 1;
     while (np2 < nnew) np2 <<= 1;
     for (uint32_t k = threadIdx.x; k < np2; k += blockDim.x)
-      sn[k] = k < nnew ? t.extra[t.r_reg[u] + k] : make_uint2(0xFFFFFFFFu, 0u);
+      sn[k] = k < nnew ? t.extra[rr.reg + k] : make_uint2(0xFFFFFFFFu, 0u);
     __syncthreads();
     const uint32_t nt = s_nt;
     for (uint32_t k = threadIdx.x; k < nt; k += blockDim.x) {
@@ -1011,91 +1132,20 @@ k_hash_rebuild(HashApply t, unsigned long long* __restrict__ off, uint32_t* __re
   hash_rebuild_body(t, off, deg, cap, srt, ntomb, arcs, scratch, pool_base, pool_cap, scratch_cap, ctrl, blockIdx.x, gridDim.x);
 }
 
-// Thread per touched row: metadata of kept rows, then reset the scratch.
+// Thread per touched row: metadata of kept rows (if the batch was written),
+// then its record is zero again.
 __device__ __forceinline__ void hash_finish_body(HashApply t, uint32_t* __restrict__ deg, uint32_t* __restrict__ ntomb,
-                              Ctrl* ctrl, uint64_t base, uint64_t stride) {
+                                                 const Ctrl* ctrl, bool go, uint64_t base, uint64_t stride) {
   const uint32_t nr = ctrl->rows;
-  for (uint64_t q = base + threadIdx.x; q < nr;
-       q += stride) {
+  for (uint64_t q = base + threadIdx.x; q < nr; q += stride) {
     const uint32_t u = t.rows[q];
-    if (t.r_state[u] != 2u) {
-      deg[u] += t.r_app[u];
-      ntomb[u] = uint32_t((long long)ntomb[u] + t.r_tomb[u]);
+    const RowRec rr = t.rec[u];
+    if (go && rr.state != 2u) {
+      if (rr.app()) deg[u] += rr.app();
+      if (rr.tomb()) ntomb[u] = uint32_t((long long)ntomb[u] + rr.tomb());
     }
-    t.r_app[u] = 0;
-    t.r_tomb[u] = 0;
-    t.r_live[u] = 0;
-    t.r_state[u] = 0;
-    t.r_reg[u] = 0;
+    t.rec[u] = RowRec{};
   }
-}
-
-// need_defer: after the single-block path, which finished the rows itself
-// unless it left rebuilds to the multi-block kernels
-__global__ void k_hash_finish(HashApply t, uint32_t* __restrict__ deg, uint32_t* __restrict__ ntomb,
-                              Ctrl* ctrl, int need_defer) {
-  pdl_wait();
-  if (!ctrl->apply_go || (need_defer && !ctrl->apply_defer)) return;
-  hash_finish_body(t, deg, ntomb, ctrl, blockIdx.x * uint64_t(blockDim.x), uint64_t(gridDim.x) * blockDim.x);
-}
-
-// Alg. 7 per pair: K[u] and Sigma[C^{t-1}[u]] change by the net weight.
-__device__ __forceinline__ void hash_weights_body(HashApply t, const uint32_t* __restrict__ C, long long* __restrict__ K,
-                               long long* __restrict__ Sigma, Ctrl* ctrl, uint64_t base, uint64_t stride) {
-  const uint32_t np = ctrl->npairs;
-  const uint32_t lane = threadIdx.x & 31u;
-  // warp-uniform loop: changes to one community's Sigma are summed in the
-  // warp first (a large community takes one update per warp, not per arc)
-  for (uint64_t p0 = base + (threadIdx.x & ~31u); p0 < np; p0 += stride) {
-    const uint64_t p = p0 + lane;
-    long long dl = 0;
-    uint32_t c = kEmpty;
-    if (p < np) {
-      const uint32_t s = t.pairs[p];
-      dl = t.delta[s];
-      if (dl) {
-        const uint32_t u = uint32_t(t.keys[s] >> 32);
-        atomicAdd((unsigned long long*)&K[u], (unsigned long long)dl);
-        c = C[u];
-      }
-    }
-    long long sum = 0;
-    bool first = c != kEmpty;
-    for (int k = 0; k < 32; ++k) {
-      const uint32_t ck = __shfl_sync(0xFFFFFFFFu, c, k);
-      const long long dk = __shfl_sync(0xFFFFFFFFu, dl, k);
-      if (c != kEmpty && ck == c) {
-        sum += dk;
-        if (uint32_t(k) < lane) first = false;
-      }
-    }
-    if (first && sum) atomicAdd((unsigned long long*)&Sigma[c], (unsigned long long)sum);
-  }
-}
-
-__global__ void k_hash_weights(HashApply t, const uint32_t* __restrict__ C, long long* __restrict__ K,
-                               long long* __restrict__ Sigma, Ctrl* ctrl) {
-  pdl_wait();
-  if (!ctrl->apply_go) return;
-  hash_weights_body(t, C, K, Sigma, ctrl, blockIdx.x * uint64_t(blockDim.x), uint64_t(gridDim.x) * blockDim.x);
-}
-
-// Reset the per-vertex scratch of the touched rows after a failed validation.
-__device__ __forceinline__ void hash_reset_body(HashApply t, Ctrl* ctrl, uint64_t base, uint64_t stride) {
-  const uint32_t nr = ctrl->rows;
-  for (uint64_t q = base + threadIdx.x; q < nr;
-       q += stride) {
-    const uint32_t u = t.rows[q];
-    t.r_app[u] = 0;
-    t.r_tomb[u] = 0;
-    t.r_live[u] = 0;
-    t.r_state[u] = 0;
-    t.r_reg[u] = 0;
-  }
-}
-
-__global__ void k_hash_reset(HashApply t, Ctrl* ctrl) {
-  hash_reset_body(t, ctrl, blockIdx.x * uint64_t(blockDim.x), uint64_t(gridDim.x) * blockDim.x);
 }
 
 // Every slot a batch claimed in the pair table is emptied again after its
@@ -1104,44 +1154,38 @@ __global__ void k_hash_reset(HashApply t, Ctrl* ctrl) {
 __device__ __forceinline__ void apply_rest(HashApply t, const Ctrl* ctrl, Ctrl* next, uint64_t base,
                                            uint64_t stride) {
   const uint32_t np = ctrl->npairs;
-  for (uint64_t q = base; q < np; q += stride) {
-    const uint32_t s = t.pairs[q];
-    t.keys[s] = kNoKey;
-    t.ndel[s] = 0;
-    t.wins[s] = 0;
-  }
+  for (uint64_t q = base; q < np; q += stride) t.tab[t.pairs[q]] = PairRec{kNoKey, 0ull, 0u, 0u, 0u, 0u};
   if (base < sizeof(Ctrl) / sizeof(unsigned int)) {
     unsigned int* z = reinterpret_cast<unsigned int*>(next);
     for (uint64_t q = base; q < sizeof(Ctrl) / sizeof(unsigned int); q += stride) z[q] = 0u;
   }
 }
 
-// Last kernel of the multi-kernel apply: the batch's arcs join the pending
-// list of the next update if the batch was written; the table is emptied
-// either way.
-__global__ void k_apply_tail(const unsigned long long* __restrict__ key, const uint32_t* __restrict__ w,
-                             uint64_t na, unsigned long long* __restrict__ pend_key,
-                             uint32_t* __restrict__ pend_w, HashApply t, const Ctrl* ctrl, Ctrl* next) {
+// Last kernel of an apply: the rows' metadata and records, and (multi-kernel
+// path) the table.  After the single-block path, which finished the rows
+// itself unless it left rebuilds to the multi-block kernel, only the rest.
+__global__ void k_hash_finish(HashApply t, uint32_t* __restrict__ deg, uint32_t* __restrict__ ntomb,
+                              Ctrl* ctrl, Ctrl* next, int after_small) {
   pdl_wait();
-  const uint64_t base = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x;
-  const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-  if (ctrl->apply_go)
-    for (uint64_t q = base; q < na; q += stride) {
-      pend_key[q] = key[q];
-      pend_w[q] = w[q];
-    }
-  apply_rest(t, ctrl, next, base, stride);
+  if (after_small && !ctrl->apply_defer) return;
+  const uint64_t base = blockIdx.x * uint64_t(blockDim.x), stride = uint64_t(gridDim.x) * blockDim.x;
+  hash_finish_body(t, deg, ntomb, ctrl, ctrl->apply_go != 0u, base, stride);
+  if (!after_small) apply_rest(t, ctrl, next, base + threadIdx.x, stride);
+}
+
+__global__ void k_empty_table(PairRec* tab, uint64_t cap) {
+  for (uint64_t s = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; s < cap; s += uint64_t(gridDim.x) * blockDim.x)
+    tab[s] = PairRec{kNoKey, 0ull, 0u, 0u, 0u, 0u};
 }
 
 // Small batches (at most kSmallApplyEdges edges, one arc per thread) in one
 // block: the phases of the hashed apply above -- table insert, pair
 // validation, row decisions, then, if the batch is valid and fits, in-place
-// writes, K and Sigma, the pending list and the row metadata -- separated by
-// block barriers, so that a batch of a few edges costs one launch instead of
-// six kernels and three table clears.  The table is the first `t.mask + 1`
-// slots of the pair table, cleared here.  Nothing is written if the gate
-// (gate_open) is closed: the per-row scratch counters are cleared,
-// ctrl->apply_go stays 0 and the host reports the error or redoes the batch.
+// writes, K and Sigma, and the row metadata -- separated by block barriers, so
+// that a batch of a few edges costs one launch instead of six kernels.  The
+// table is the first `t.mask + 1` slots of the pair table.  Nothing is
+// written if the gate (gate_open) is closed: ctrl->apply_go stays 0 and the
+// host reports the error or redoes the batch.
 // Rows to rebuild (rare for small batches) are left to the multi-block
 // rebuild, one block per row, and the row metadata kernel after it, which
 // are enqueued behind this kernel and run only when it sets
@@ -1155,14 +1199,13 @@ k_apply_small(const dfl_edge* __restrict__ del, const dfl_edge* __restrict__ ins
               unsigned long long* __restrict__ key, uint32_t* __restrict__ w, const unsigned long long* __restrict__ off,
               uint32_t* __restrict__ deg, const uint32_t* __restrict__ cap, const uint32_t* __restrict__ srt,
               uint32_t* __restrict__ ntomb, uint2* __restrict__ arcs, const uint32_t* __restrict__ C,
-              long long* __restrict__ K, long long* __restrict__ Sigma, unsigned long long* __restrict__ pend_key,
-              uint32_t* __restrict__ pend_w, ApplyGate g, Ctrl* ctrl, Ctrl* next) {
+              long long* __restrict__ K, long long* __restrict__ Sigma, ApplyGate g, Ctrl* ctrl, Ctrl* next) {
   pdl_wait();
   __shared__ int s_go;
   const uint64_t nt = blockDim.x;
   hash_insert_body(del, ins, nd, ne, n, f, t, key, w, ctrl, 0, nt);
   __syncthreads();
-  hash_pairs_body(t, n, off, deg, srt, arcs, ctrl, 0, nt);
+  hash_pairs_body(t, off, deg, srt, arcs, ctrl, 0, nt);
   __syncthreads();
   hash_rows_body(t, deg, cap, srt, ntomb, ctrl, 0, nt);
   __syncthreads();
@@ -1175,21 +1218,10 @@ k_apply_small(const dfl_edge* __restrict__ del, const dfl_edge* __restrict__ ins
     ctrl->apply_defer = go && defer ? 1u : 0u;
   }
   __syncthreads();
-  if (!s_go) {
-    hash_reset_body(t, ctrl, 0, nt);
-  } else {
-    hash_write_body(t, off, deg, arcs, ctrl, 0, nt);
-    hash_weights_body(t, C, K, Sigma, ctrl, 0, nt);
-    for (uint64_t q = threadIdx.x; q < 2 * ne; q += nt) {
-      pend_key[q] = key[q];
-      pend_w[q] = w[q];
-    }
-    if (s_go == 1) {  // (rows to rebuild: the rebuild and metadata kernels enqueued behind this one)
-      __syncthreads();  // every write has read deg before the metadata changes it
-      hash_finish_body(t, deg, ntomb, ctrl, 0, nt);
-    }
-  }
-  __syncthreads();  // the table's last readers are done
+  if (s_go) hash_write_body(t, off, deg, arcs, C, K, Sigma, ctrl, 0, nt);
+  __syncthreads();  // every write has read deg before the metadata changes it; the table's last readers are done
+  // (rows to rebuild: the rebuild and metadata kernels enqueued behind this one)
+  if (s_go != 2) hash_finish_body(t, deg, ntomb, ctrl, s_go != 0, 0, nt);
   apply_rest(t, ctrl, next, threadIdx.x, nt);
 }
 
@@ -1254,58 +1286,38 @@ int ensure_hash_buffers(Handle* h, uint64_t na) {
     // freed and cleared together, so that an allocation failing below leaves
     // no member pointing at freed memory (destroy and the next growth free
     // every member)
-    void** old[] = {(void**)&h->h_keys, (void**)&h->h_ndel, (void**)&h->h_wdel, (void**)&h->h_wins,
-                    (void**)&h->h_slot, (void**)&h->h_wnew, (void**)&h->h_flag, (void**)&h->h_delta,
-                    (void**)&h->h_pairs};
+    void** old[] = {(void**)&h->h_tab, (void**)&h->h_pairs};
     for (void** q : old) {
       cudaFree(*q);
       *q = nullptr;
     }
     h->h_cap = 0;
-    DFL_CUDA(h, dev_malloc(&h->h_keys, sizeof(unsigned long long) * cap));
-    DFL_CUDA(h, dev_malloc(&h->h_ndel, sizeof(uint32_t) * cap));
-    DFL_CUDA(h, dev_malloc(&h->h_wdel, sizeof(uint32_t) * cap));
-    DFL_CUDA(h, dev_malloc(&h->h_wins, sizeof(unsigned long long) * cap));
-    DFL_CUDA(h, dev_malloc(&h->h_slot, sizeof(uint32_t) * cap));
-    DFL_CUDA(h, dev_malloc(&h->h_wnew, sizeof(uint32_t) * cap));
-    DFL_CUDA(h, dev_malloc(&h->h_flag, sizeof(uint32_t) * cap));
-    DFL_CUDA(h, dev_malloc(&h->h_delta, sizeof(long long) * cap));
+    DFL_CUDA(h, dev_malloc(&h->h_tab, sizeof(PairRec) * cap));
     DFL_CUDA(h, dev_malloc(&h->h_pairs, sizeof(uint32_t) * cap));
     // empty; every apply empties the slots it claimed again
-    DFL_CUDA(h, cudaMemsetAsync(h->h_keys, 0xFF, sizeof(unsigned long long) * cap, h->stream));
-    DFL_CUDA(h, cudaMemsetAsync(h->h_ndel, 0, sizeof(uint32_t) * cap, h->stream));
-    DFL_CUDA(h, cudaMemsetAsync(h->h_wins, 0, sizeof(unsigned long long) * cap, h->stream));
+    {
+      LaunchScope ls(h, DFL_PROF_APPLY);
+      k_empty_table<<<grid_for(cap, 256), 256, 0, h->stream>>>(h->h_tab, cap);
+      DFL_TRY(check_launch(h, "empty pair table"));
+    }
     h->h_cap = cap;
   }
-  if (!h->r_app || !h->r_tomb || !h->r_live || !h->r_state || !h->r_reg) {
-    // all five or none: what an earlier failed allocation left is freed first
-    void** rs[] = {(void**)&h->r_app, (void**)&h->r_tomb, (void**)&h->r_live, (void**)&h->r_state,
-                   (void**)&h->r_reg};
-    for (void** q : rs) {
-      cudaFree(*q);
-      *q = nullptr;
-    }
+  if (!h->h_rec) {
     const uint64_t n = h->n ? h->n : 1;
-    DFL_CUDA(h, dev_malloc(&h->r_app, sizeof(uint32_t) * n));
-    DFL_CUDA(h, dev_malloc(&h->r_tomb, sizeof(int) * n));
-    DFL_CUDA(h, dev_malloc(&h->r_live, sizeof(int) * n));
-    DFL_CUDA(h, dev_malloc(&h->r_state, sizeof(uint32_t) * n));
-    DFL_CUDA(h, dev_malloc(&h->r_reg, sizeof(uint32_t) * n));
-    DFL_CUDA(h, cudaMemsetAsync(h->r_app, 0, sizeof(uint32_t) * n, h->stream));
-    DFL_CUDA(h, cudaMemsetAsync(h->r_tomb, 0, sizeof(int) * n, h->stream));
-    DFL_CUDA(h, cudaMemsetAsync(h->r_live, 0, sizeof(int) * n, h->stream));
-    DFL_CUDA(h, cudaMemsetAsync(h->r_state, 0, sizeof(uint32_t) * n, h->stream));
-    DFL_CUDA(h, cudaMemsetAsync(h->r_reg, 0, sizeof(uint32_t) * n, h->stream));
+    DFL_CUDA(h, dev_malloc(&h->h_rec, sizeof(RowRec) * n));
+    DFL_CUDA(h, cudaMemsetAsync(h->h_rec, 0, sizeof(RowRec) * n, h->stream));
   }
   if (na > h->h_rows_cap) {
     cudaStreamSynchronize(h->stream);
-    cudaFree(h->h_rows);
-    cudaFree(h->h_extra);
-    h->h_rows = nullptr;
-    h->h_extra = nullptr;
+    void** old[] = {(void**)&h->h_rows, (void**)&h->h_rebuild, (void**)&h->h_extra};
+    for (void** q : old) {
+      cudaFree(*q);
+      *q = nullptr;
+    }
     h->h_rows_cap = 0;
     uint64_t want = na + na / 2 + 256;
     DFL_CUDA(h, dev_malloc(&h->h_rows, sizeof(uint32_t) * want));
+    DFL_CUDA(h, dev_malloc(&h->h_rebuild, sizeof(uint32_t) * want));
     DFL_CUDA(h, dev_malloc(&h->h_extra, sizeof(uint2) * want));
     h->h_rows_cap = want;
   }
@@ -1314,22 +1326,12 @@ int ensure_hash_buffers(Handle* h, uint64_t na) {
 
 HashApply hash_args(const Handle* h) {
   HashApply t;
-  t.keys = h->h_keys;
-  t.ndel = h->h_ndel;
-  t.wdel = h->h_wdel;
-  t.wins = h->h_wins;
-  t.slot = h->h_slot;
-  t.wnew = h->h_wnew;
-  t.flag = h->h_flag;
-  t.delta = h->h_delta;
-  t.pairs = h->h_pairs;
+  t.tab = h->h_tab;
   t.mask = h->h_cap - 1;
-  t.r_app = h->r_app;
-  t.r_tomb = h->r_tomb;
-  t.r_live = h->r_live;
-  t.r_state = h->r_state;
-  t.r_reg = h->r_reg;
+  t.pairs = h->h_pairs;
+  t.rec = h->h_rec;
   t.rows = h->h_rows;
+  t.rebuild = h->h_rebuild;
   t.extra = h->h_extra;
   return t;
 }
@@ -1340,14 +1342,6 @@ HashApply hash_args(const Handle* h) {
 // Batch apply (Section 3.4 and Alg. 7): validate, then change the graph, K,
 // Sigma and 2m, and append the batch to the pending list.
 namespace {
-
-int hash_reset(Handle* h, const HashApply& t, Ctrl* c) {
-  LaunchScope ls(h, DFL_PROF_APPLY);
-  k_hash_reset<<<grid_for(h->h_rows_cap, 256), 256, 0, h->stream>>>(t, c);
-  DFL_TRY(check_launch(h, "hash reset"));
-  DFL_CUDA(h, cudaStreamSynchronize(h->stream));
-  return DFL_OK;
-}
 
 ApplyGate apply_gate(const Handle* h, const unsigned int* pre_err) {
   return ApplyGate{h->pool_top, h->pool_cap, h->scratch_cap, h->m2, h->ngraphs ? 0 : 1, pre_err};
@@ -1375,26 +1369,27 @@ int enqueue_hashed(Handle* h, const dfl_edge* del, const dfl_edge* ins, uint64_t
   const ApplyGate gate = apply_gate(h, pre_err);
   const KeyFmt f = key_fmt(h);
   HashApply t = hash_args(h);
+  // the batch's arcs, behind the pending list: they join it if the batch is written
+  unsigned long long* key = h->pend_key + h->pend_count;
+  uint32_t* w = h->pend_w + h->pend_count;
   const bool small = ne <= kSmallApplyEdges;
   if (small) {
     uint64_t sc = 64;
     while (sc < 2 * na) sc <<= 1;
     t.mask = (sc < h->h_cap ? sc : h->h_cap) - 1;
     LaunchScope ls(h, DFL_PROF_APPLY);
-    launch_pdl(k_apply_small, 1, kSmallApplyThreads, 0, h->stream, del, ins, nd, ne, h->n, f, t, h->b_key, h->b_w, h->off, h->deg, h->cap, h->srt, h->ntomb, h->arcs,
-        h->C, h->K, h->Sigma, h->pend_key + h->pend_count, h->pend_w + h->pend_count, gate, c, next);
+    launch_pdl(k_apply_small, 1, kSmallApplyThreads, 0, h->stream, del, ins, nd, ne, h->n, f, t, key, w, h->off,
+               h->deg, h->cap, h->srt, h->ntomb, h->arcs, h->C, h->K, h->Sigma, gate, c, next);
     DFL_TRY(check_launch(h, "small batch apply"));
   } else {
     {
       LaunchScope ls(h, DFL_PROF_APPLY);
-      launch_pdl(k_hash_insert, grid_for(ne, 256), 256, 0, h->stream, del, ins, nd, ne, h->n, f, t,
-                 h->b_key, h->b_w, c);
+      launch_pdl(k_hash_insert, grid_for(ne, 256), 256, 0, h->stream, del, ins, nd, ne, h->n, f, t, key, w, c);
       DFL_TRY(check_launch(h, "hash insert"));
     }
     {
       LaunchScope ls(h, DFL_PROF_APPLY);
-      launch_pdl(k_hash_pairs, grid_for(na, 256), 256, 0, h->stream, t, h->n, h->off, h->deg, h->srt,
-                 h->arcs, c);
+      launch_pdl(k_hash_pairs, grid_for(na, 256), 256, 0, h->stream, t, h->off, h->deg, h->srt, h->arcs, c);
       DFL_TRY(check_launch(h, "hash pairs"));
     }
     {
@@ -1404,7 +1399,11 @@ int enqueue_hashed(Handle* h, const dfl_edge* del, const dfl_edge* ins, uint64_t
     }
     {
       LaunchScope ls(h, DFL_PROF_APPLY);
-      launch_pdl(k_hash_write, grid_for(na, 256), 256, 0, h->stream, t, h->off, h->deg, h->arcs, c, gate);
+      // (at most kSigmaPairs pairs a block)
+      const uint64_t least = na / kSigmaPairs + 1;
+      const uint32_t cap = uint32_t(least > 152 * 16 ? least : 152 * 16);
+      launch_pdl(k_hash_write, grid_for(na, 256, cap), 256, 0, h->stream, t, h->off, h->deg, h->arcs, h->C, h->K, h->Sigma,
+                 c, gate);
       DFL_TRY(check_launch(h, "hash write"));
     }
   }
@@ -1415,22 +1414,10 @@ int enqueue_hashed(Handle* h, const dfl_edge* del, const dfl_edge* ins, uint64_t
         h->scratch_cap, c);
     DFL_TRY(check_launch(h, "hash rebuild"));
   }
-  if (!small) {
-    LaunchScope ls(h, DFL_PROF_APPLY);
-    launch_pdl(k_hash_weights, grid_for(na, 256), 256, 0, h->stream, t, h->C, h->K, h->Sigma, c);
-    DFL_TRY(check_launch(h, "hash weights"));
-  }
   {
     LaunchScope ls(h, DFL_PROF_APPLY);
-    launch_pdl(k_hash_finish, grid_for(na, 256), 256, 0, h->stream, t, h->deg, h->ntomb, c,
-               small ? 1 : 0);
+    launch_pdl(k_hash_finish, grid_for(na, 256), 256, 0, h->stream, t, h->deg, h->ntomb, c, next, small ? 1 : 0);
     DFL_TRY(check_launch(h, "hash finish"));
-  }
-  if (!small) {
-    LaunchScope ls(h, DFL_PROF_APPLY);
-    launch_pdl(k_apply_tail, grid_for(na, 256), 256, 0, h->stream, h->b_key, h->b_w, na,
-               h->pend_key + h->pend_count, h->pend_w + h->pend_count, t, c, next);
-    DFL_TRY(check_launch(h, "pending list"));
   }
   h->apar = par ^ 1;
   h->papply.active = true;
@@ -1456,7 +1443,6 @@ int begin_hashed(Handle* h, const dfl_edge* del, uint64_t nd, const dfl_edge* in
     DFL_TRY(grow(h, &h->b_edges, ne, &cap, h->b_edges_cap));
     h->b_edges_cap = cap;
   }
-  DFL_TRY(ensure_batch_scratch(h, na));
   DFL_TRY(ensure_hash_buffers(h, na));
   if (mem_kind == DFL_MEM_DEVICE) {
     *ddel = del;
@@ -1495,9 +1481,8 @@ int settle_apply(Handle* h) {
     h->papply.rc = rc;
     return rc;
   }
-  // nothing was written; the per-row scratch counters are cleared again
-  rc = hash_reset(h, hash_args(h), h->actrl + par);
-  if (!rc) {
+  // nothing was written (the apply's last kernel cleared the scratch all the same)
+  {
     if (c.err & kErrInvalid) rc = set_error(h, DFL_ERR_INVALID, "invalid edge in batch");
     else if (c.err & kErrNotFound) rc = set_error(h, DFL_ERR_NOT_FOUND, "deleted edge not found");
     else if (c.err & kErrOverflow) rc = set_error(h, DFL_ERR_OVERFLOW, "edge weight overflow");
@@ -1758,11 +1743,18 @@ int mark(Handle* h, int mode, bool* all, bool* use_range, uint64_t* initial) {
     // apply's gate opened; its arcs follow the pending list's
     const bool pending = h->papply.active;
     const uint64_t np = h->pend_count + (pending ? h->papply.na : 0);
-    if (np) {
+    const unsigned int* go = pending ? &h->actrl[h->papply.par].apply_go : nullptr;
+    if (np >= n / 8 && np >= 65536) {
+      {
+        LaunchScope ls(h, DFL_PROF_MARK);
+        launch_pdl(k_mark_df_bits, grid_for(np, 256), 256, 0, h->stream, h->pend_key, np, f, h->C, h->fbits[0], go);
+        DFL_TRY(check_launch(h, "mark df"));
+      }
+      DFL_TRY(lists_from_bits(h, h->fbits[0], n, h->deg, 0, k));
+    } else if (np) {
       LaunchScope ls(h, DFL_PROF_MARK);
       launch_pdl(k_mark_df, grid_for(np, 256), 256, 0, h->stream, h->pend_key, np, f, h->C, h->deg,
-                 h->fbits[0], h->lists[0], h->segs, h->ctrl, k,
-                 pending ? &h->actrl[h->papply.par].apply_go : nullptr);
+                 h->fbits[0], h->lists[0], h->segs, h->ctrl, k, go);
       DFL_TRY(check_launch(h, "mark df"));
     }
     *initial = ~0ull;  // counted from the frontier lists when local-moving starts

@@ -136,6 +136,11 @@ struct Segs {
   uint32_t ng;
 };
 
+// One (u, v) pair of a batch, and one row it touches (batch.cu): a 32-byte
+// sector each, since every access to them is random.
+struct PairRec;
+struct RowRec;
+
 struct Handle {
   uint32_t n = 0;
   cudaStream_t stream = nullptr;
@@ -220,23 +225,14 @@ struct Handle {
   uint64_t b_edges_cap = 0;
   uint2* scratch = nullptr;        // merge scratch
   uint64_t scratch_cap = 0;
-  // hashed apply: pair table (capacity h_cap, a power of two), per-vertex
-  // scratch counters (zero at rest), touched rows, new arcs of rebuilt rows
-  unsigned long long* h_keys = nullptr;
-  uint32_t* h_ndel = nullptr;
-  uint32_t* h_wdel = nullptr;
-  unsigned long long* h_wins = nullptr;
-  uint32_t* h_slot = nullptr;
-  uint32_t* h_wnew = nullptr;
-  uint32_t* h_flag = nullptr;
-  long long* h_delta = nullptr;
+  // hashed apply: table of pair records (capacity h_cap, a power of two; empty
+  // at rest) and its occupied slots, per-vertex row records (zero at rest),
+  // touched and rebuilt rows, new arcs of rebuilt rows
+  PairRec* h_tab = nullptr;
   uint32_t* h_pairs = nullptr;
   uint64_t h_cap = 0;
-  uint32_t* r_app = nullptr;
-  int* r_tomb = nullptr;
-  int* r_live = nullptr;
-  uint32_t* r_state = nullptr;
-  uint32_t* r_reg = nullptr;
+  RowRec* h_rec = nullptr;
+  uint32_t* h_rebuild = nullptr;
   uint32_t* h_rows = nullptr;
   uint2* h_extra = nullptr;
   uint64_t h_rows_cap = 0;

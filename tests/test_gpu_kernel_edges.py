@@ -249,3 +249,80 @@ def test_small_frontier_runs_whole_passes(dfl, orc, n, m, max_iterations):
         b.update(2)
         same(a, b)
         assert a.stats()["affected_ever"] == b.stats()["affected_ever"] and a.trace() == b.trace()
+
+
+@pytest.mark.parametrize("two_calls", [True, False])
+def test_row_search_at_window_and_tail_edges(dfl, orc, two_calls):
+    """Batches that look up the first, last and middle arcs of rows of every
+    length around the search's windows and splits, then arcs of unsorted tails
+    of every length, tombstones among them; absent edges are refused."""
+    degrees = list(range(1, 40)) + [143, 144, 145, 146, 152, 153, 154, 161, 162, 1000, 1459, 4095, 4096]
+    g = stars(degrees, 4200, 6)
+    a, b = pair(dfl, orc, g)
+    a.static()
+    b.static()
+    c = len(degrees)
+    rows = [np.sort(np.concatenate([g.v[g.u == k], g.u[g.v == k]])) for k in range(c)]
+    rng = np.random.default_rng(3)
+
+    def both(dels, ins):
+        dels, ins = np.array(dels, np.uint32).reshape(-1, 3), np.array(ins, np.uint32).reshape(-1, 3)
+        if two_calls:
+            ra = a.apply_batch(dels, ins, check=False)
+            if ra == 0:
+                a.update(2)
+        else:
+            ra = a.step(dels, ins, check=False)
+        rb = b.apply_batch(dels, ins)
+        assert ra == rb
+        if rb == 0:
+            b.update(2)
+        return rb
+
+    added = [[] for _ in range(c)]
+    for t in range(6):
+        dels, ins = [], []
+        for k in range(c):
+            r = rows[k]
+            if t % 2 == 0 and r.size > 2:  # some arcs leave, some gain weight
+                for at in {0, r.size - 1, r.size // 2, int(rng.integers(r.size))}:
+                    (dels if rng.random() < 0.5 else ins).append((k, int(r[at]), 0 if len(dels) % 2 else 1))
+                ins = [(u, v, max(1, w)) for u, v, w in ins]
+            if added[k]:
+                v = added[k][int(rng.integers(len(added[k])))]
+                ins.append((k, v, 3))
+            free = np.setdiff1d(c + np.arange(4200), np.concatenate([r, np.array(added[k], np.int64)]))
+            if free.size:
+                new = rng.choice(free, min(1 + k % 7, free.size), replace=False)
+                ins += [(k, int(v), 2) for v in new]
+                added[k] += [int(v) for v in new]
+        assert both(dels, ins) in (0, -2)
+        for x, y in zip(a.graph(), b.graph()):
+            assert np.array_equal(x, y)
+        same(a, b)
+    absent = next(v for v in c + np.arange(4200) if v not in set(rows[20]) | set(added[20]))
+    assert both([(20, int(absent), 0)], []) == -2
+    same(a, b)
+
+
+def test_batch_touching_most_vertices(dfl, orc):
+    """A batch whose arcs outnumber an eighth of the vertices: marked through
+    the bitmap, and every row's record and pair's slot used and reset."""
+    g = random_graph(50_000, 150_000, 2)
+    a, b = pair(dfl, orc, g)
+    a.static()
+    b.static()
+    stream = synth.BatchStream(g, 6)
+    for t in range(3):
+        dels, ins = stream.next(60_000, w_max=5)
+        if t == 1:
+            assert a.apply_batch(dels, ins) == 0
+            a.update(2)
+        else:
+            assert a.step(dels, ins) == 0
+        assert b.apply_batch(dels, ins) == 0
+        b.update(2)
+        for x, y in zip(a.graph(), b.graph()):
+            assert np.array_equal(x, y)
+        same(a, b)
+        assert a.stats()["affected_initial"] == b.stats()["affected_initial"] and a.trace() == b.trace()
