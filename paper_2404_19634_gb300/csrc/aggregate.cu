@@ -9,11 +9,19 @@
 //      self = true); distinct keys are written as the super-vertex's row, and
 //      its weight K'' = Sigma'' is the row sum (Alg. 4, weight reset).
 // Communities are binned by total degree: one warp with a shared-memory
-// table (<= 256), one block with a shared-memory table (<= 4096); a larger
-// community is split into chunks of members, each chunk aggregated by one
-// block in shared memory and merged into the community's global table, which
-// is then emitted slot-parallel.  Every arc goes straight into a table with
-// a shared-memory (or, for a giant community's overflow, global) atomic.
+// table (<= 256), one block with a shared-memory table (<= 1024 and <= 4096); a
+// larger community is split into chunks of members, each chunk aggregated by
+// one block in shared memory and merged into the community's global table,
+// which is then emitted slot-parallel.  Every arc goes straight into a table
+// with a shared-memory (or, for a giant community's overflow, global) atomic.
+//
+// Latency bounds these kernels (member -> row -> arcs -> communities), and most
+// members have a few arcs, so a tile of members is flattened first: a prefix
+// sum over their degrees numbers the tile's arcs, which the lanes then take in
+// order, four in flight each.  A warp per member row, one member after another,
+// took 1.95 ms (block bin) and 1.79 ms (warp bin, which also took a warp per
+// isolated vertex) for the two levels of the 2^22-vertex R-MAT graph's static
+// run; this 0.61 and 0.57 ms.
 #include <mutex>
 #include <vector>
 
@@ -23,44 +31,103 @@ namespace dfl {
 
 namespace {
 
+// Lanes of the warp with this lane's community: its first lane, this lane's
+// rank among them and their number.  Every lane calls it (kEmpty: none).
+struct Peers {
+  unsigned mask;
+  bool first;
+  uint32_t rank;
+  __device__ __forceinline__ explicit Peers(uint32_t c) {
+    mask = __match_any_sync(0xFFFFFFFFu, c);
+    rank = __popc(mask & ((1u << (threadIdx.x & 31u)) - 1u));
+    first = rank == 0;
+  }
+};
+
+// (one update per warp and community: a giant community's counters are the
+// contended ones)
 __global__ void k_agg_count(GraphView g, const uint32_t* __restrict__ Cp, uint32_t* __restrict__ cnt,
                             unsigned long long* __restrict__ tdeg) {
-  for (uint64_t v = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; v < g.nv;
-       v += uint64_t(gridDim.x) * blockDim.x) {
-    uint32_t c = Cp[v];
-    atomicAdd(&cnt[c], 1u);
-    uint32_t d = g.deg[v];
-    if (d) atomicAdd(&tdeg[c], (unsigned long long)d);
+  const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
+  for (uint64_t v0 = blockIdx.x * uint64_t(blockDim.x); v0 < g.nv; v0 += stride) {
+    const uint64_t v = v0 + threadIdx.x;
+    const uint32_t c = v < g.nv ? Cp[v] : kEmpty;
+    const uint32_t d = v < g.nv ? g.deg[v] : 0u;
+    const Peers p(c);
+    unsigned long long sum = d;
+    if (p.mask & (p.mask - 1)) {  // (a lane alone needs no sum; the sums of 16-bit halves cannot wrap)
+      const uint32_t lo = __reduce_add_sync(p.mask, d & 0xFFFFu), hi = __reduce_add_sync(p.mask, d >> 16);
+      sum = ((unsigned long long)hi << 16) + lo;
+    }
+    if (c == kEmpty || !p.first) continue;
+    atomicAdd(&cnt[c], uint32_t(__popc(p.mask)));
+    if (sum) atomicAdd(&tdeg[c], sum);
   }
 }
 
+// Bins of communities by total degree.
+enum : int { kAggByWarp = 0, kAggByBlock = 1, kAggByBigBlock = 2, kAggGiant = 3, kAggBins = 4 };
+constexpr uint32_t kAggBlockDeg = 1024;
+
 // Round every community's total degree up to an even count (rows then start
-// 16-byte aligned), track the maximum, and bin the community.
-__global__ void k_agg_bins(uint32_t ncomm, unsigned long long* __restrict__ tdeg, uint32_t* lists,
-                           Segs seg, Ctrl* ctrl) {
-  uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-  for (uint64_t c0 = blockIdx.x * uint64_t(blockDim.x); c0 < ncomm; c0 += stride) {
-    uint64_t c = c0 + threadIdx.x;
-    bool valid = c < ncomm;
-    uint32_t key = 0;
-    if (valid) {
-      unsigned long long t = tdeg[c];
-      unsigned long long te = (t + 1) & ~1ull;
-      tdeg[c] = te;
-      uint32_t tc = t > 0xFFFFFFFFull ? 0xFFFFFFFFu : uint32_t(t);
-      key = tc <= kBinWarpHash ? 0u : tc <= kBinBlock ? 1u : 2u;
-      if (key == 2) atomicMax(&ctrl->red_u, tc);
+// 16-byte aligned) and bin the community; one without arcs (an isolated
+// vertex) is a finished empty row.
+__global__ void __launch_bounds__(256) k_agg_bins(uint32_t ncomm, unsigned long long* __restrict__ tdeg,
+                                                  uint32_t* lists, uint64_t lstride, uint32_t* __restrict__ deg_out,
+                                                  long long* __restrict__ Knew, Ctrl* ctrl) {
+  __shared__ uint32_t s_cnt[kAggBins], s_base[kAggBins];
+  constexpr uint32_t U = 4;
+  const uint64_t stride = uint64_t(gridDim.x) * blockDim.x * U;
+  for (uint64_t c0 = blockIdx.x * uint64_t(blockDim.x) * U; c0 < ncomm; c0 += stride) {
+    uint32_t key[U], rank[U];
+    if (threadIdx.x < kAggBins) s_cnt[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      const uint64_t c = c0 + u * blockDim.x + threadIdx.x;
+      key[u] = kAggBins;
+      if (c < ncomm) {
+        const unsigned long long t = tdeg[c];
+        if (t == 0) {
+          deg_out[c] = 0;
+          Knew[c] = 0;
+        } else {
+          if (t & 1ull) tdeg[c] = t + 1;
+          key[u] = t <= kBinWarpHash ? kAggByWarp : t <= kAggBlockDeg ? kAggByBlock : t <= kBinBlock ? kAggByBigBlock : kAggGiant;
+        }
+      }
     }
-    append_vertex(uint32_t(c), valid, key, lists, seg, ctrl, 1);
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      const Peers p(key[u]);
+      rank[u] = 0;
+      if (key[u] < kAggBins && p.first) rank[u] = atomicAdd(&s_cnt[key[u]], uint32_t(__popc(p.mask)));
+      rank[u] = __shfl_sync(0xFFFFFFFFu, rank[u], __ffs(p.mask) - 1) + p.rank;
+    }
+    __syncthreads();
+    if (threadIdx.x < kAggBins) {
+      const uint32_t n = s_cnt[threadIdx.x];
+      s_base[threadIdx.x] = n ? atomicAdd(&ctrl->count[1][0][threadIdx.x], n) : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u)
+      if (key[u] < kAggBins) lists[key[u] * lstride + s_base[key[u]] + rank[u]] = uint32_t(c0 + u * blockDim.x + threadIdx.x);
+    __syncthreads();
   }
 }
 
 __global__ void k_agg_fill(uint32_t nv, const uint32_t* __restrict__ Cp, const uint32_t* __restrict__ coff,
                            uint32_t* __restrict__ fillc, uint32_t* __restrict__ members) {
-  for (uint64_t v = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; v < nv;
-       v += uint64_t(gridDim.x) * blockDim.x) {
-    uint32_t c = Cp[v];
-    members[coff[c] + atomicAdd(&fillc[c], 1u)] = uint32_t(v);
+  const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
+  for (uint64_t v0 = blockIdx.x * uint64_t(blockDim.x); v0 < nv; v0 += stride) {
+    const uint64_t v = v0 + threadIdx.x;
+    const uint32_t c = v < nv ? Cp[v] : kEmpty;
+    const Peers p(c);
+    uint32_t at = 0;
+    if (c != kEmpty && p.first) at = coff[c] + atomicAdd(&fillc[c], uint32_t(__popc(p.mask)));
+    at = __shfl_sync(0xFFFFFFFFu, at, __ffs(p.mask) - 1) + p.rank;
+    if (c != kEmpty) members[at] = uint32_t(v);
   }
 }
 
@@ -75,62 +142,109 @@ struct AggArgs {
   long long* Knew;
   const uint32_t* list;
   const unsigned int* count;
-  uint32_t ncomm;
   Ctrl* ctrl;
-  uint2* gtable;
-  uint32_t gslots;
-  uint2* bigq;              // giant-community members of high degree: (member, giant index)
-  unsigned int* nbig;       // their count
 };
 
-__device__ __forceinline__ bool agg_add(uint32_t* keys, uint32_t* vals, uint32_t mask, uint32_t c,
-                                        uint32_t w, uint32_t limit) {
+// Open-addressing insert: 0 if no slot was found within `limit` probes, 2 if
+// it created its slot, else 1.
+__device__ __forceinline__ int agg_insert(uint32_t* keys, uint32_t* vals, uint32_t mask, uint32_t c, uint32_t w,
+                                          uint32_t limit) {
   uint32_t s = hash32(c) & mask;
   for (uint32_t probe = 0; probe < limit; ++probe) {
     uint32_t prev = keys[s];
     if (prev == kEmpty) prev = atomicCAS(&keys[s], kEmpty, c);
     if (prev == kEmpty || prev == c) {
       atomicAdd(&vals[s], w);
-      return true;
+      return prev == kEmpty ? 2 : 1;
     }
     s = (s + 1) & mask;
   }
-  return false;
+  return 0;
 }
 
-// Add arcs [0, d) of one vertex (warp-strided, two loads in flight per lane)
-// to the table by neighbour community; deleted arcs (weight 0) skipped.
-// Entries that do not fit are added to the fallback table if one is given.
-__device__ __forceinline__ bool agg_row(const AggArgs& a, unsigned long long o, uint32_t d,
-                                        uint32_t* keys, uint32_t* vals, uint32_t mask, uint32_t limit,
-                                        uint32_t* fkeys, uint32_t* fvals, uint32_t fmask) {
-  const uint32_t lane = threadIdx.x & 31u;
-  bool ok = true;
-  for (uint32_t k0 = 0; k0 < d; k0 += 64) {
-    uint2 arc0 = k0 + lane < d ? a.g.arcs[o + k0 + lane] : make_uint2(0u, 0u);
-    uint2 arc1 = k0 + 32 + lane < d ? a.g.arcs[o + k0 + 32 + lane] : make_uint2(0u, 0u);
-    uint32_t c0 = arc0.y ? a.Cp[arc0.x] : kEmpty;
-    uint32_t c1 = arc1.y ? a.Cp[arc1.x] : kEmpty;
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      uint32_t c = u ? c1 : c0;
-      uint32_t w = u ? arc1.y : arc0.y;
-      if (c != kEmpty && !agg_add(keys, vals, mask, c, w, limit)) {
-        if (fkeys) ok &= agg_add(fkeys, fvals, fmask, c, w, fmask + 1);
-        else ok = false;
-      }
-    }
-  }
-  return ok;
+__device__ __forceinline__ bool agg_add(uint32_t* keys, uint32_t* vals, uint32_t mask, uint32_t c, uint32_t w,
+                                        uint32_t limit) {
+  return agg_insert(keys, vals, mask, c, w, limit) != 0;
 }
 
 constexpr uint32_t kAggWarpSlots = 512;
 constexpr int kAggWarps = 8;
-constexpr uint32_t kAggBlockSlots = 2 * kBinBlock;  // 8192 keys + values = 64 KB
-constexpr uint32_t kChunkMembers = 256;             // members per block of a giant community
-constexpr uint32_t kAggBigMember = 512;             // larger member rows go to k_agg_big ...
-constexpr uint32_t kAggPiece = 2048;                // ... in pieces of this many arcs
+constexpr int kAggThreads = 256;
+constexpr uint32_t kChunkMembers = kAggThreads;     // members per block of a giant community
+constexpr uint32_t kAggBigMember = 128;             // larger member rows go to k_agg_big ...
+constexpr uint32_t kAggUnit = 64;                   // ... which deals their arcs in units of this many
 constexpr uint32_t kGiantSlots = 4096;              // shared table of a giant-community block
+constexpr uint32_t kGiantTile = 1024;               // global tables are multiples of this many slots
+
+// Arc `k` of a flattened tile of `rows` rows (a power of two): the row's
+// position by a binary search of the exclusive prefix `pre`, whose entry j is
+// the first arc of row j; base[j] + k is then the arc's index.
+template <int kRows>
+__device__ __forceinline__ uint32_t flat_row(const uint32_t* pre, uint32_t k) {
+  uint32_t j = 0;
+#pragma unroll
+  for (uint32_t s = kRows / 2; s; s >>= 1)
+    if (pre[j + s] <= k) j += s;
+  return j;
+}
+
+// A tile of up to kAggThreads rows, one per thread: d arcs from index o on.
+// Returns the tile's number of arcs.  Every thread of the block calls it; the
+// tile is rewritten by the next call, which a block barrier must separate.
+struct FlatTile {
+  unsigned long long base[kAggThreads];
+  uint32_t pre[kAggThreads];
+  uint32_t w[kAggThreads / 32];
+  __device__ __forceinline__ unsigned long long arc(uint32_t k) const { return base[flat_row<kAggThreads>(pre, k)] + k; }
+};
+__device__ __forceinline__ uint32_t flat_rows(FlatTile& ft, unsigned long long o, uint32_t d) {
+  const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
+  uint32_t x = d;
+#pragma unroll
+  for (int q = 1; q < 32; q <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, q);
+    if (lane >= uint32_t(q)) x += y;
+  }
+  if (lane == 31) ft.w[wib] = x;
+  __syncthreads();
+  uint32_t before = 0, total = 0;
+#pragma unroll
+  for (uint32_t q = 0; q < kAggThreads / 32; ++q) {
+    if (q == wib) before = total;
+    total += ft.w[q];
+  }
+  ft.pre[threadIdx.x] = before + x - d;
+  ft.base[threadIdx.x] = o - (before + x - d);
+  __syncthreads();
+  return total;
+}
+
+// This thread's member of [m0, m1): its row.
+__device__ __forceinline__ uint32_t member_row(const AggArgs& a, uint32_t m0, uint32_t m1, unsigned long long* o,
+                                               uint32_t* d) {
+  const uint32_t m = m0 + threadIdx.x;
+  const uint32_t v = m < m1 ? a.members[m] : 0u;
+  *o = m < m1 ? a.g.off[v] : 0ull;
+  *d = m < m1 ? a.g.deg[v] : 0u;
+  return v;
+}
+
+// This thread's arcs k0, k0 + kAggThreads, ... (four of them, below total) and
+// their neighbours' communities, all loads in flight; kEmpty where there is none.
+__device__ __forceinline__ void load_arcs(const AggArgs& a, const FlatTile& ft, uint32_t k0, uint32_t total,
+                                          uint32_t (&c)[4], uint32_t (&w)[4]) {
+  uint2 e[4];
+#pragma unroll
+  for (uint32_t u = 0; u < 4; ++u) {
+    const uint32_t k = k0 + u * kAggThreads;
+    e[u] = k < total ? a.g.arcs[ft.arc(k)] : make_uint2(0u, 0u);
+  }
+#pragma unroll
+  for (uint32_t u = 0; u < 4; ++u) {
+    c[u] = e[u].y ? a.Cp[e[u].x] : kEmpty;  // deleted arcs (weight 0) skipped
+    w[u] = e[u].y;
+  }
+}
 
 // Write the table's entries as the row of super-vertex c (ballot order).
 __device__ __forceinline__ void emit_warp(const AggArgs& a, uint32_t c, const uint32_t* keys,
@@ -181,9 +295,44 @@ __global__ void __launch_bounds__(256) k_agg_warp(AggArgs a) {
     }
     __syncwarp();
     bool ok = true;
-    for (uint32_t m = a.coff[c]; m < a.coff[c + 1]; ++m) {
-      uint32_t v = a.members[m];
-      ok &= agg_row(a, a.g.off[v], a.g.deg[v], keys, vals, slots - 1, slots, nullptr, nullptr, 0);
+    const uint32_t mend = a.coff[c + 1];
+    for (uint32_t m0 = a.coff[c]; m0 < mend; m0 += 32) {  // tiles of 32 members, flattened
+      uint32_t d = 0;
+      unsigned long long o = 0;
+      if (m0 + lane < mend) {
+        const uint32_t v = a.members[m0 + lane];
+        o = a.g.off[v];
+        d = a.g.deg[v];
+      }
+      uint32_t x = d;
+#pragma unroll
+      for (int q = 1; q < 32; q <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, q);
+        if (lane >= uint32_t(q)) x += y;
+      }
+      const uint32_t total = __shfl_sync(0xFFFFFFFFu, x, 31);
+      const uint32_t pre = x - d;
+      o -= pre;
+      constexpr uint32_t U = 4;
+      for (uint32_t k0 = 0; k0 < total; k0 += 32 * U) {
+        uint2 e[U];
+        uint32_t nc[U];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) {
+          const uint32_t k = k0 + u * 32 + lane;
+          uint32_t j = 0;  // the last row whose first arc is at or before k
+#pragma unroll
+          for (uint32_t s = 16; s; s >>= 1)
+            if (__shfl_sync(0xFFFFFFFFu, pre, j + s) <= k) j += s;
+          const unsigned long long ob = __shfl_sync(0xFFFFFFFFu, o, j);
+          e[u] = k < total ? a.g.arcs[ob + k] : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) nc[u] = e[u].y ? a.Cp[e[u].x] : kEmpty;
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u)
+          if (nc[u] != kEmpty) ok &= agg_add(keys, vals, slots - 1, nc[u], e[u].y, slots);
+      }
     }
     if (!__all_sync(0xFFFFFFFFu, ok) && lane == 0) atomicOr(&a.ctrl->err, kErrInternal);
     __syncwarp();
@@ -193,20 +342,23 @@ __global__ void __launch_bounds__(256) k_agg_warp(AggArgs a) {
   if (lane == 0 && maxd) atomicMax(&a.ctrl->max_deg, maxd);
 }
 
-// Bin 1: one block per community (total degree <= 4096); a warp per member.
-__global__ void __launch_bounds__(256) k_agg_block(AggArgs a) {
+// Bins 1 and 2: one block per community, its table of kSlots keys + values in
+// dynamic shared memory (kSlots >= 2 x total degree).
+template <uint32_t kSlots>
+__global__ void __launch_bounds__(kAggThreads) k_agg_block(AggArgs a) {
   extern __shared__ uint32_t dyn[];
+  __shared__ FlatTile ft;
   __shared__ unsigned int s_pos;
   __shared__ unsigned long long s_sum;
   __shared__ int s_ok;
-  const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
   const uint32_t cnt = *a.count;
   unsigned int maxd = 0;
   for (uint64_t t = blockIdx.x; t < cnt; t += gridDim.x) {
     const uint32_t c = a.list[t];
     const unsigned long long td = a.soff[c + 1] - a.soff[c];
-    uint32_t slots = 1024;
-    while (slots < 2 * td && slots < kAggBlockSlots) slots <<= 1;
+    uint32_t slots = 512;
+    while (slots < 2 * td && slots < kSlots) slots <<= 1;
     uint32_t* keys = dyn;
     uint32_t* vals = dyn + slots;
     for (uint32_t s = threadIdx.x; s < slots; s += blockDim.x) {
@@ -220,9 +372,20 @@ __global__ void __launch_bounds__(256) k_agg_block(AggArgs a) {
     }
     __syncthreads();
     bool ok = true;
-    for (uint32_t m = a.coff[c] + wib; m < a.coff[c + 1]; m += nw) {
-      uint32_t v = a.members[m];
-      ok &= agg_row(a, a.g.off[v], a.g.deg[v], keys, vals, slots - 1, slots, nullptr, nullptr, 0);
+    const uint32_t mend = a.coff[c + 1];
+    for (uint32_t m0 = a.coff[c]; m0 < mend; m0 += kAggThreads) {
+      unsigned long long o;
+      uint32_t d;
+      member_row(a, m0, mend, &o, &d);
+      const uint32_t total = flat_rows(ft, o, d);
+      for (uint32_t k0 = threadIdx.x; k0 < total; k0 += 4 * kAggThreads) {
+        uint32_t nc[4], w[4];
+        load_arcs(a, ft, k0, total, nc, w);
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u)
+          if (nc[u] != kEmpty) ok &= agg_add(keys, vals, slots - 1, nc[u], w[u], slots);
+      }
+      __syncthreads();  // the tile is rewritten
     }
     if (!ok) s_ok = 0;
     __syncthreads();
@@ -256,200 +419,355 @@ __global__ void __launch_bounds__(256) k_agg_block(AggArgs a) {
   if (threadIdx.x == 0 && maxd) atomicMax(&a.ctrl->max_deg, maxd);
 }
 
-// Giant communities (bin 2).  giant[g] = community, gtab[g] = offset of its
-// global table of gsize[g] slots (keys, then values, in uint2 units: the
-// table of g occupies gtable[gtab[g] .. gtab[g] + gsize[g]) as keys|values).
+// Giant communities (the last bin).  giant[g] = community, gtab[g] = offset of
+// its global table of gsize[g] slots in the key and value arrays.
 struct GiantArgs {
   const uint32_t* giant;
-  const unsigned long long* gtab;
-  const uint32_t* gsize;
-  const uint32_t* chunk0;  // first work item of each giant (exclusive scan of chunk counts)
+  unsigned long long* gtab;
+  uint32_t* gsize;
+  uint32_t* chunk0;        // first work item of each giant (exclusive scan of chunk counts)
   uint32_t ngiant;
   uint32_t nitems;         // total (giant, chunk) work items
+  uint32_t* keys;          // empty before the first kernel
+  uint32_t* vals;          // zero
+  uint32_t* units;         // per (work item, thread): units of a high-degree member; then their exclusive scan
 };
 
-// Block (g, chunk): aggregate members [chunk*256, +256) of giant g in shared
-// memory (overflow goes straight to the global table), then merge the shared
-// entries into the global table.
-__global__ void __launch_bounds__(256) k_agg_giant_accum(AggArgs a, GiantArgs gi) {
-  __shared__ uint32_t keys[kGiantSlots];
-  __shared__ uint32_t vals[kGiantSlots];
-  const uint32_t wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  bool ok = true;
-  for (uint32_t item = blockIdx.x; item < gi.nitems; item += gridDim.x) {
-    // giant owning this work item
-    uint32_t lo = 0, hi = gi.ngiant;
-    while (hi - lo > 1) {
-      uint32_t mid = (lo + hi) >> 1;
-      if (gi.chunk0[mid] <= item) lo = mid;
-      else hi = mid;
+// Giant owning work item `item`.
+__device__ __forceinline__ uint32_t giant_of(const GiantArgs& gi, uint32_t item) {
+  uint32_t lo = 0, hi = gi.ngiant;
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (gi.chunk0[mid] <= item) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// One block: the giants' tables and chunks laid out (a table holds twice the
+// distinct communities a row can have: at most its arcs, and at most the
+// communities that have arcs), their totals into red_a and red_b and the super
+// graph's row slots into red_c, so that the host reads one control block.
+__global__ void __launch_bounds__(1024) k_giant_layout(uint32_t ncomm, const unsigned long long* __restrict__ soff,
+                                                       const uint32_t* __restrict__ coff, GiantArgs gi,
+                                                       uint32_t* __restrict__ deg_out, long long* __restrict__ Knew,
+                                                       Ctrl* ctrl) {
+  __shared__ unsigned long long s_t[32], s_tbase;
+  __shared__ uint32_t s_c[32], s_cbase;
+  const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+  const uint32_t ng = ctrl->count[1][0][kAggGiant];
+  unsigned long long live = 0;
+  for (int b = 0; b < kAggBins; ++b) live += ctrl->count[1][0][b];
+  if (threadIdx.x == 0) {
+    s_tbase = 0;
+    s_cbase = 0;
+  }
+  __syncthreads();
+  for (uint32_t t0 = 0; t0 < ng; t0 += blockDim.x) {
+    const uint32_t t = t0 + threadIdx.x;
+    unsigned long long size = 0;
+    uint32_t chunks = 0;
+    if (t < ng) {
+      const uint32_t c = gi.giant[t];
+      const unsigned long long td = soff[c + 1] - soff[c], distinct = td < live ? td : live;
+      size = kGiantTile;
+      while (size < 2 * distinct) size <<= 1;
+      chunks = (coff[c + 1] - coff[c] + kChunkMembers - 1) / kChunkMembers;
+      deg_out[c] = 0;
+      Knew[c] = 0;
     }
-    const uint32_t g = lo;
-    const uint32_t chunk = item - gi.chunk0[g];
-    const uint32_t c = gi.giant[g];
-    const uint32_t gs = gi.gsize[g];
-    uint32_t* gkeys = reinterpret_cast<uint32_t*>(a.gtable + gi.gtab[g]);
-    uint32_t* gvals = gkeys + gs;
-    const uint64_t m0 = a.coff[c] + uint64_t(chunk) * kChunkMembers;
-    const uint64_t mend = m0 + kChunkMembers;
-    const uint32_t m1 = a.coff[c + 1] < mend ? a.coff[c + 1] : uint32_t(mend);
-    for (uint32_t s = threadIdx.x; s < kGiantSlots; s += blockDim.x) {
-      keys[s] = kEmpty;
-      vals[s] = 0;
-    }
-    __syncthreads();
-    for (uint32_t m = uint32_t(m0) + wib; m < m1; m += nw) {
-      const uint32_t v = a.members[m];
-      const uint32_t dv = a.g.deg[v];
-      if (dv > kAggBigMember) {  // spread over many blocks by k_agg_big
-        if ((threadIdx.x & 31u) == 0) a.bigq[atomicAdd(a.nbig, 1u)] = make_uint2(v, g);
-        continue;
+    unsigned long long xt = size;
+    uint32_t xc = chunks;
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long yt = __shfl_up_sync(0xFFFFFFFFu, xt, o);
+      const uint32_t yc = __shfl_up_sync(0xFFFFFFFFu, xc, o);
+      if (lane >= uint32_t(o)) {
+        xt += yt;
+        xc += yc;
       }
-      ok &= agg_row(a, a.g.off[v], dv, keys, vals, kGiantSlots - 1, 32, gkeys, gvals, gs - 1);
+    }
+    if (lane == 31) {
+      s_t[w] = xt;
+      s_c[w] = xc;
     }
     __syncthreads();
-    for (uint32_t s = threadIdx.x; s < kGiantSlots; s += blockDim.x) {
-      uint32_t k = keys[s];
-      if (k != kEmpty) ok &= agg_add(gkeys, gvals, gs - 1, k, vals[s], gs);
+    if (threadIdx.x == 0) {
+      for (uint32_t k = 0; k < blockDim.x / 32; ++k) {
+        const unsigned long long tt = s_t[k];
+        const uint32_t tc = s_c[k];
+        s_t[k] = s_tbase;
+        s_c[k] = s_cbase;
+        s_tbase += tt;
+        s_cbase += tc;
+      }
     }
     __syncthreads();
+    if (t < ng) {
+      gi.gtab[t] = s_t[w] + xt - size;
+      gi.gsize[t] = uint32_t(size);
+      gi.chunk0[t] = s_c[w] + xc - chunks;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    ctrl->red_a = s_tbase;
+    ctrl->red_b = s_cbase;
+    ctrl->red_c = soff[ncomm];
+  }
+}
+
+// Shared table of a giant's block (empty at rest): when a round of arcs could
+// overfill it, its entries move to the giant's global table.  Rows of
+// converged communities meet few distinct communities, so most chunks flush once.
+struct GiantTable {
+  uint32_t keys[kGiantSlots], vals[kGiantSlots];
+  uint16_t list[kGiantSlots];  // occupied slots, compacted for the flush
+  uint32_t claimed, n;
+};
+// Entries before a round of 4 x kAggThreads arcs: the table stays half empty
+// at the worst (long probes cost more than flushes: 1,754 us for both kernels
+// on the 2^22-vertex R-MAT graph's two levels, 1,787 with 2,048, 1,822 with
+// 512, 2,150 with 3,072 of 8,192 slots; 2,355 for a warp per member row, with
+// one merge per 256 members or per 2,048 arcs of a larger one).
+constexpr uint32_t kGiantFlush = 1024;
+
+__device__ __forceinline__ void giant_table_init(GiantTable& t) {
+  for (uint32_t s = threadIdx.x; s < kGiantSlots; s += kAggThreads) {
+    t.keys[s] = kEmpty;
+    t.vals[s] = 0;
+  }
+  if (threadIdx.x == 0) t.claimed = t.n = 0;
+  __syncthreads();
+}
+
+// Every entry into the global table, four per thread in flight; the shared
+// table is empty again.  Returns false if one found no slot.
+__device__ __forceinline__ bool giant_flush(GiantTable& t, uint32_t* gkeys, uint32_t* gvals, uint32_t gmask) {
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t s0 = threadIdx.x & ~31u; s0 < kGiantSlots; s0 += kAggThreads) {
+    const bool has = t.keys[s0 + lane] != kEmpty;
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, has);
+    if (!m) continue;
+    uint32_t at = 0;
+    if (lane == 0) at = atomicAdd(&t.n, uint32_t(__popc(m)));
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    if (has) t.list[at + __popc(m & ((1u << lane) - 1u))] = uint16_t(s0 + lane);
+  }
+  __syncthreads();
+  const uint32_t n = t.n;
+  bool ok = true;
+  for (uint32_t e0 = threadIdx.x; e0 < n; e0 += 4 * kAggThreads) {
+    uint32_t c[4], w[4], at[4], prev[4];
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) {
+      const uint32_t e = e0 + u * kAggThreads;
+      c[u] = kEmpty;
+      if (e >= n) continue;
+      const uint32_t s = t.list[e];
+      c[u] = t.keys[s];
+      w[u] = t.vals[s];
+      t.keys[s] = kEmpty;
+      t.vals[s] = 0;
+      at[u] = hash32(c[u]) & gmask;
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) prev[u] = c[u] != kEmpty ? atomicCAS(&gkeys[at[u]], kEmpty, c[u]) : kEmpty;
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) {
+      if (c[u] == kEmpty) continue;
+      for (uint32_t probe = 0; prev[u] != kEmpty && prev[u] != c[u] && probe < gmask; ++probe) {
+        at[u] = (at[u] + 1) & gmask;
+        prev[u] = atomicCAS(&gkeys[at[u]], kEmpty, c[u]);
+      }
+      if (prev[u] == kEmpty || prev[u] == c[u]) atomicAdd(&gvals[at[u]], w[u]);
+      else ok = false;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) t.claimed = t.n = 0;
+  __syncthreads();
+  return ok;
+}
+
+// The tile's arcs into the shared table, flushed when a further round could
+// overfill it.  Every thread of the block calls it.
+__device__ __forceinline__ bool giant_arcs(const AggArgs& a, GiantTable& t, const FlatTile& ft, uint32_t total,
+                                           uint32_t* gkeys, uint32_t* gvals, uint32_t gmask) {
+  bool ok = true;
+  for (uint32_t b = 0; b < total; b += 4 * kAggThreads) {  // block-uniform
+    uint32_t c[4], w[4], made = 0;
+    load_arcs(a, ft, b + threadIdx.x, total, c, w);
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) {
+      if (c[u] == kEmpty) continue;
+      const int r = agg_insert(t.keys, t.vals, kGiantSlots - 1, c[u], w[u], kGiantSlots);
+      ok &= r != 0;
+      made += r == 2 ? 1u : 0u;
+    }
+    made = __reduce_add_sync(0xFFFFFFFFu, made);
+    if ((threadIdx.x & 31u) == 0 && made) atomicAdd(&t.claimed, made);
+    __syncthreads();
+    if (t.claimed > kGiantFlush) ok &= giant_flush(t, gkeys, gvals, gmask);
+    else __syncthreads();  // (everyone has read the count)
+  }
+  return ok;
+}
+
+// Work item (g, chunk): members [chunk*256, +256) of giant g.  A block takes a
+// run of items and flushes its table when the giant changes.  The units of
+// rows of more than kAggBigMember arcs are noted for k_agg_big.
+__global__ void __launch_bounds__(kAggThreads) k_agg_giant_accum(AggArgs a, GiantArgs gi) {
+  extern __shared__ uint32_t dyn[];
+  GiantTable& t = *reinterpret_cast<GiantTable*>(dyn);
+  __shared__ FlatTile ft;
+  const uint32_t i0 = uint32_t(uint64_t(gi.nitems) * blockIdx.x / gridDim.x);
+  const uint32_t i1 = uint32_t(uint64_t(gi.nitems) * (blockIdx.x + 1) / gridDim.x);
+  if (i0 == i1) return;  // block-uniform
+  bool ok = true;
+  giant_table_init(t);
+  uint32_t g = giant_of(gi, i0);
+  for (uint32_t item = i0; item < i1; ++item) {
+    const uint32_t c = gi.giant[g], gmask = gi.gsize[g] - 1;
+    unsigned long long o;
+    uint32_t d;
+    member_row(a, a.coff[c] + (item - gi.chunk0[g]) * kChunkMembers, a.coff[c + 1], &o, &d);
+    const bool big = d > kAggBigMember;
+    gi.units[uint64_t(item) * kAggThreads + threadIdx.x] = big ? (d + kAggUnit - 1) / kAggUnit : 0u;
+    const uint32_t total = flat_rows(ft, o, big ? 0u : d);
+    uint32_t* gkeys = gi.keys + gi.gtab[g];
+    uint32_t* gvals = gi.vals + gi.gtab[g];
+    ok &= giant_arcs(a, t, ft, total, gkeys, gvals, gmask);
+    const bool next = g + 1 < gi.ngiant && gi.chunk0[g + 1] == item + 1;  // the next item is another giant's
+    if (next || item + 1 == i1) ok &= giant_flush(t, gkeys, gvals, gmask);
+    else __syncthreads();  // the tile is rewritten
+    g += next ? 1u : 0u;
   }
   if (!ok) atomicOr(&a.ctrl->err, kErrInternal);
 }
 
-// The queued high-degree members of giant communities: their rows in pieces
-// of kAggPiece arcs dealt over the blocks; a piece is aggregated in shared
-// memory and added to the community's global table.  The queue is swept in
-// tiles of one block's threads (a block-wide prefix numbers the pieces of a
-// tile, dealt round-robin), so a long queue costs each block one parallel
-// pass per tile rather than a dependent walk over every entry.
-constexpr int kAggBigThreads = 256;
+// The giant communities' high-degree members: every block takes an equal share
+// of their arcs (a run of units, which may begin and end inside a row), work
+// item by work item.
+__global__ void __launch_bounds__(kAggThreads) k_agg_big(AggArgs a, GiantArgs gi) {
+  extern __shared__ uint32_t dyn[];
+  GiantTable& t = *reinterpret_cast<GiantTable*>(dyn);
+  __shared__ FlatTile ft;
+  const uint32_t units = gi.units[uint64_t(gi.nitems) * kAggThreads];
+  const uint32_t u0 = uint32_t(uint64_t(units) * blockIdx.x / gridDim.x);
+  const uint32_t u1 = uint32_t(uint64_t(units) * (blockIdx.x + 1) / gridDim.x);
+  if (u0 == u1) return;  // block-uniform
+  bool ok = true, filled = false;
+  giant_table_init(t);
+  uint32_t lo = 0, hi = gi.nitems;  // the last item whose first unit is at or before u0
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (gi.units[uint64_t(mid) * kAggThreads] <= u0) lo = mid;
+    else hi = mid;
+  }
+  uint32_t g = giant_of(gi, lo);
+  for (uint32_t item = lo; item < gi.nitems; ++item) {
+    const uint32_t* un = gi.units + uint64_t(item) * kAggThreads;
+    const uint32_t first = un[0], end = un[kAggThreads];
+    if (first >= u1) break;  // block-uniform, as the branches below
+    uint32_t* gkeys = gi.keys + gi.gtab[g];
+    uint32_t* gvals = gi.vals + gi.gtab[g];
+    const uint32_t gmask = gi.gsize[g] - 1;
+    if (end > first && end > u0) {
+      // this thread's row, if it is a high-degree one with arcs in the share
+      const uint32_t ue = un[threadIdx.x], ux = un[threadIdx.x + 1];
+      unsigned long long o = 0;
+      uint32_t d = 0;
+      if (ux > ue && ux > u0 && ue < u1) {
+        const uint32_t c = gi.giant[g];
+        const uint32_t v = a.members[a.coff[c] + (item - gi.chunk0[g]) * kChunkMembers + threadIdx.x];
+        const uint32_t dv = a.g.deg[v], k0 = ue < u0 ? (u0 - ue) * kAggUnit : 0u;
+        const uint64_t k1 = uint64_t(u1 - ue) * kAggUnit;
+        o = a.g.off[v] + k0;
+        d = (k1 < dv ? uint32_t(k1) : dv) - k0;
+      }
+      const uint32_t total = flat_rows(ft, o, d);
+      ok &= giant_arcs(a, t, ft, total, gkeys, gvals, gmask);
+      __syncthreads();  // the tile is rewritten
+      filled = true;
+    }
+    const bool next = g + 1 < gi.ngiant && gi.chunk0[g + 1] == item + 1;  // the next item is another giant's
+    if (filled && (next || item + 1 == gi.nitems || end >= u1)) {
+      ok &= giant_flush(t, gkeys, gvals, gmask);
+      filled = false;
+    }
+    g += next ? 1u : 0u;
+  }
+  if (!ok) atomicOr(&a.ctrl->err, kErrInternal);
+}
 
-__global__ void __launch_bounds__(kAggBigThreads) k_agg_big(AggArgs a, GiantArgs gi) {
-  __shared__ uint32_t keys[kGiantSlots];
-  __shared__ uint32_t vals[kGiantSlots];
-  __shared__ uint32_t s_pre[kAggBigThreads + 1];
-  __shared__ uint32_t s_w[kAggBigThreads / 32];
+// The giants' tables as super arcs, a block per tile of kGiantTile slots (all
+// of one giant): the tile's row positions are claimed with one atomic (one per
+// entry took 1,053 us for the two levels above, this 135).
+__global__ void __launch_bounds__(kAggThreads) k_agg_giant_emit(AggArgs a, GiantArgs gi, unsigned long long total) {
+  pdl_wait_only();
+  __shared__ uint32_t s_w[kAggThreads / 32], s_base;
+  __shared__ unsigned long long s_k[kAggThreads / 32];
+  constexpr uint32_t U = kGiantTile / kAggThreads;
   const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
-  const uint32_t count = *a.nbig;
-  bool ok = true;
-  uint64_t ibase = 0;  // pieces of the earlier tiles
-  for (uint32_t q0 = 0; q0 < count; q0 += kAggBigThreads) {
-    const uint32_t q = q0 + threadIdx.x;
-    const uint32_t npc = q < count ? (a.g.deg[a.bigq[q].x] + kAggPiece - 1) / kAggPiece : 0u;
-    uint32_t x = npc;
+  uint32_t maxd = 0;
+  for (unsigned long long t0 = blockIdx.x * (unsigned long long)kGiantTile; t0 < total;
+       t0 += gridDim.x * (unsigned long long)kGiantTile) {
+    uint32_t key[U], val[U], n = 0;
+    unsigned long long ksum = 0;
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      key[u] = gi.keys[t0 + u * kAggThreads + threadIdx.x];
+      val[u] = gi.vals[t0 + u * kAggThreads + threadIdx.x];
+      n += key[u] != kEmpty ? 1u : 0u;
+      ksum += val[u];  // (0 in an empty slot)
+    }
+    // giant owning the tile (tables are laid out in giant order)
+    uint32_t lo = 0, hi = gi.ngiant;
+    while (hi - lo > 1) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if (gi.gtab[mid] <= t0) lo = mid;
+      else hi = mid;
+    }
+    const uint32_t c = gi.giant[lo];
+    uint32_t x = n;
+#pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
       if (lane >= uint32_t(o)) x += y;
     }
+    for (int o = 16; o; o >>= 1) ksum += __shfl_xor_sync(0xFFFFFFFFu, ksum, o);
     if (lane == 31) s_w[wib] = x;
+    if (lane == 0) s_k[wib] = ksum;
     __syncthreads();
-    uint32_t wbase = 0;
-    for (uint32_t k = 0; k < wib; ++k) wbase += s_w[k];
-    s_pre[threadIdx.x + 1] = wbase + x;
-    if (threadIdx.x == 0) s_pre[0] = 0;
+    if (threadIdx.x == 0) {
+      uint32_t run = 0;
+      unsigned long long kt = 0;
+      for (uint32_t q = 0; q < kAggThreads / 32; ++q) {
+        const uint32_t y = s_w[q];
+        s_w[q] = run;
+        run += y;
+        kt += s_k[q];
+      }
+      if (run) {
+        s_base = atomicAdd(&a.deg_out[c], run);
+        maxd = max(maxd, s_base + run);
+        atomicAdd((unsigned long long*)&a.Knew[c], kt);
+      }
+    }
     __syncthreads();
-    const uint32_t tile_items = s_pre[kAggBigThreads];
-    // piece `it` of the tile is item ibase + it, handled by block (ibase + it) mod grid
-    for (uint32_t it = uint32_t((blockIdx.x + gridDim.x - ibase % gridDim.x) % gridDim.x); it < tile_items;
-         it += gridDim.x) {
-      uint32_t lo = 0, hi = kAggBigThreads;  // tile position owning piece `it`
-      while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (s_pre[mid] <= it) lo = mid;
-        else hi = mid;
-      }
-      const uint2 e = a.bigq[q0 + lo];
-      const uint32_t v = e.x, g = e.y;
-      const uint32_t dv = a.g.deg[v];
-      const unsigned long long o = a.g.off[v];
-      const uint32_t gs = gi.gsize[g];
-      uint32_t* gkeys = reinterpret_cast<uint32_t*>(a.gtable + gi.gtab[g]);
-      uint32_t* gvals = gkeys + gs;
-      const uint32_t k0 = (it - s_pre[lo]) * kAggPiece, k1 = min(dv, k0 + kAggPiece);
-      for (uint32_t s = threadIdx.x; s < kGiantSlots; s += kAggBigThreads) {
-        keys[s] = kEmpty;
-        vals[s] = 0;
-      }
-      __syncthreads();
-      for (uint32_t k = k0 + threadIdx.x; k < k1; k += kAggBigThreads) {
-        const uint2 arc = a.g.arcs[o + k];
-        if (!arc.y) continue;  // deleted arc
-        const uint32_t c = a.Cp[arc.x];
-        if (!agg_add(keys, vals, kGiantSlots - 1, c, arc.y, 32)) ok &= agg_add(gkeys, gvals, gs - 1, c, arc.y, gs);
-      }
-      __syncthreads();
-      for (uint32_t s = threadIdx.x; s < kGiantSlots; s += kAggBigThreads) {
-        const uint32_t c = keys[s];
-        if (c != kEmpty) ok &= agg_add(gkeys, gvals, gs - 1, c, vals[s], gs);
-      }
-      __syncthreads();
-    }
-    ibase += tile_items;
-    __syncthreads();  // s_pre and s_w are rewritten by the next tile
+    unsigned long long at = a.soff[c] + s_base + s_w[wib] + x - n;
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u)
+      if (key[u] != kEmpty) a.arcs_out[at++] = make_uint2(key[u], val[u]);
+    __syncthreads();  // s_w, s_k and s_base are rewritten by the next tile
   }
-  if (!ok) atomicOr(&a.ctrl->err, kErrInternal);
-}
-
-// Thread per global-table slot of every giant: emit the super arcs.
-__global__ void k_agg_giant_emit(AggArgs a, GiantArgs gi, unsigned long long total) {
-  uint32_t maxd = 0;
-  for (unsigned long long t = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; t < total;
-       t += uint64_t(gridDim.x) * blockDim.x) {
-    // giant owning slot t (tables are laid out in giant order)
-    uint32_t lo = 0, hi = gi.ngiant;
-    while (hi - lo > 1) {
-      uint32_t mid = (lo + hi) >> 1;
-      if (gi.gtab[mid] <= t) lo = mid;
-      else hi = mid;
-    }
-    const uint32_t g = lo;
-    const unsigned long long s = t - gi.gtab[g];
-    if (s >= gi.gsize[g]) continue;
-    const uint32_t* gkeys = reinterpret_cast<const uint32_t*>(a.gtable + gi.gtab[g]);
-    uint32_t key = gkeys[s];
-    if (key == kEmpty) continue;
-    uint32_t val = gkeys[gi.gsize[g] + s];
-    uint32_t c = gi.giant[g];
-    uint32_t pos = atomicAdd(&a.deg_out[c], 1u);
-    a.arcs_out[a.soff[c] + pos] = make_uint2(key, val);
-    atomicAdd((unsigned long long*)&a.Knew[c], (unsigned long long)val);
-    maxd = max(maxd, pos + 1);
-  }
-  if (maxd) atomicMax(&a.ctrl->max_deg, maxd);
-}
-
-__global__ void k_giant_init(AggArgs a, GiantArgs gi, unsigned long long total) {
-  for (unsigned long long t = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; t < total;
-       t += uint64_t(gridDim.x) * blockDim.x) {
-    uint32_t* w = reinterpret_cast<uint32_t*>(a.gtable);
-    uint32_t lo = 0, hi = gi.ngiant;
-    while (hi - lo > 1) {
-      uint32_t mid = (lo + hi) >> 1;
-      if (gi.gtab[mid] <= t) lo = mid;
-      else hi = mid;
-    }
-    unsigned long long s = t - gi.gtab[lo];
-    // keys (first gsize words of the table) empty, values zero
-    w[2 * gi.gtab[lo] + s] = kEmpty;
-    w[2 * gi.gtab[lo] + gi.gsize[lo] + s] = 0;
-  }
-  for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < gi.ngiant; g += gridDim.x * blockDim.x) {
-    a.deg_out[gi.giant[g]] = 0;
-    a.Knew[gi.giant[g]] = 0;
-  }
+  if (threadIdx.x == 0 && maxd) atomicMax(&a.ctrl->max_deg, maxd);
 }
 
 int read_ctrl(Handle* h) {
   DFL_CUDA(h, cudaMemcpyAsync(h->hctrl, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
   DFL_CUDA(h, cudaStreamSynchronize(h->stream));
   return DFL_OK;
-}
-
-uint32_t next_pow2(uint64_t x) {
-  uint64_t p = 1;
-  while (p < x) p <<= 1;
-  return uint32_t(p);
 }
 
 }  // namespace
@@ -481,14 +799,10 @@ int aggregate(Handle* h, const GraphView& g, const uint32_t* Cp, uint32_t ncomm,
     k_agg_count<<<grid_for(g.nv, 256), 256, 0, h->stream>>>(g, Cp, h->cnt, sg.off);
     DFL_TRY(check_launch(h, "agg count"));
   }
-  Segs seg;
-  for (int b = 0; b < kMaxSubsteps * kBins; ++b) {
-    seg.off[b] = b < 3 ? uint32_t(b) * h->n : 0;
-    seg.cap[b] = b < 3 ? h->n : 0;
-  }
+  uint32_t* lists = h->lists[1];  // kAggBins lists of up to n communities
   {
     LaunchScope ls(h, DFL_PROF_AGG);
-    k_agg_bins<<<grid_for(ncomm, 256), 256, 0, h->stream>>>(ncomm, sg.off, h->lists[1], seg, h->ctrl);
+    k_agg_bins<<<grid_for(ncomm, 1024, 152 * 8), 256, 0, h->stream>>>(ncomm, sg.off, lists, h->n, sg.deg, Knew, h->ctrl);
     DFL_TRY(check_launch(h, "agg bins"));
   }
   DFL_TRY(scan_u32(h, h->cnt, h->cnt, ncomm));
@@ -498,16 +812,25 @@ int aggregate(Handle* h, const GraphView& g, const uint32_t* Cp, uint32_t ncomm,
     k_agg_fill<<<grid_for(g.nv, 256), 256, 0, h->stream>>>(g.nv, Cp, h->cnt, h->fillc, h->members);
     DFL_TRY(check_launch(h, "agg fill"));
   }
-  unsigned long long total = 0;
-  DFL_CUDA(h, cudaMemcpyAsync(&total, sg.off + ncomm, sizeof(total), cudaMemcpyDeviceToHost, h->stream));
+  // the giants' layout (in the idle frontier lists), then one control read
+  GiantArgs gi;
+  gi.giant = lists + uint64_t(kAggGiant) * h->n;
+  gi.gtab = reinterpret_cast<unsigned long long*>(h->lists[0]);
+  gi.gsize = h->lists[0] + 2ull * h->n;
+  gi.chunk0 = gi.gsize + h->n;
+  {
+    LaunchScope ls(h, DFL_PROF_AGG);
+    k_giant_layout<<<1, 1024, 0, h->stream>>>(ncomm, sg.off, h->cnt, gi, sg.deg, Knew, h->ctrl);
+    DFL_TRY(check_launch(h, "giant layout"));
+  }
   DFL_TRY(read_ctrl(h));
   const Ctrl c = *h->hctrl;
   if (c.err) return set_error(h, DFL_ERR_CUDA, "internal error in aggregation lists");
-  if (total > sg.arc_cap) {
+  if (c.red_c > sg.arc_cap) {
     cudaFree(sg.arcs);
     sg.arcs = nullptr;
     sg.arc_cap = 0;
-    uint64_t want = total + total / 8 + 1024;
+    uint64_t want = c.red_c + c.red_c / 8 + 1024;
     DFL_CUDA(h, dev_malloc(&sg.arcs, sizeof(uint2) * want));
     sg.arc_cap = want;
   }
@@ -515,8 +838,8 @@ int aggregate(Handle* h, const GraphView& g, const uint32_t* Cp, uint32_t ncomm,
   static std::once_flag smem_once;
   static cudaError_t smem_rc = cudaSuccess;
   std::call_once(smem_once, [] {
-    smem_rc = cudaFuncSetAttribute(k_agg_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   int(sizeof(uint32_t) * 2 * kAggBlockSlots));
+    smem_rc = cudaFuncSetAttribute(k_agg_block<2 * kBinBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   int(sizeof(uint32_t) * 4 * kBinBlock));
   });
   DFL_CUDA(h, smem_rc);
   AggArgs a;
@@ -528,50 +851,27 @@ int aggregate(Handle* h, const GraphView& g, const uint32_t* Cp, uint32_t ncomm,
   a.deg_out = sg.deg;
   a.arcs_out = sg.arcs;
   a.Knew = Knew;
-  a.ncomm = ncomm;
   a.ctrl = h->ctrl;
-  a.gtable = h->gtable;
-  a.gslots = 0;
-  for (int b = 0; b < 2; ++b) {
-    uint32_t nc = c.count[1][0][b];
+  for (int b = 0; b < kAggGiant; ++b) {
+    const uint32_t nc = c.count[1][0][b];
     if (!nc) continue;
-    a.list = h->lists[1] + seg.off[b];
+    a.list = lists + uint64_t(b) * h->n;
     a.count = &h->ctrl->count[1][0][b];
     LaunchScope ls(h, DFL_PROF_AGG);
-    if (b == 0)
+    if (b == kAggByWarp)
       k_agg_warp<<<grid_for(uint64_t(nc) * 32, 256, 152 * 16), 256, 0, h->stream>>>(a);
+    else if (b == kAggByBlock)
+      k_agg_block<2 * kAggBlockDeg><<<grid_for(nc, 1, 152 * 8), kAggThreads, sizeof(uint32_t) * 4 * kAggBlockDeg,
+                                      h->stream>>>(a);
     else
-      k_agg_block<<<grid_for(nc, 1, 152 * 3), 256, sizeof(uint32_t) * 2 * kAggBlockSlots,
-                    h->stream>>>(a);
+      k_agg_block<2 * kBinBlock><<<grid_for(nc, 1, 152 * 3), kAggThreads, sizeof(uint32_t) * 4 * kBinBlock,
+                                   h->stream>>>(a);
     DFL_TRY(check_launch(h, "aggregate"));
   }
-  const uint32_t ngiant = c.count[1][0][2];
-  if (ngiant) {
-    // giant communities: their ids and sizes on the host to lay out the tables
-    std::vector<uint32_t> giant(ngiant);
-    DFL_CUDA(h, cudaMemcpy(giant.data(), h->lists[1] + seg.off[2], sizeof(uint32_t) * ngiant,
-                           cudaMemcpyDeviceToHost));
-    std::vector<unsigned long long> soff(ncomm + 1);
-    DFL_CUDA(h, cudaMemcpy(soff.data(), sg.off, sizeof(unsigned long long) * (ncomm + 1),
-                           cudaMemcpyDeviceToHost));
-    std::vector<uint32_t> cntv(ncomm + 1);
-    DFL_CUDA(h, cudaMemcpy(cntv.data(), h->cnt, sizeof(uint32_t) * (ncomm + 1), cudaMemcpyDeviceToHost));
-    std::vector<unsigned long long> gtab(ngiant);
-    std::vector<uint32_t> gsize(ngiant);
-    unsigned long long total = 0;
-    std::vector<uint32_t> chunk0(ngiant);
-    uint32_t nitems = 0;
-    for (uint32_t k = 0; k < ngiant; ++k) {
-      uint32_t cc = giant[k];
-      unsigned long long td = soff[cc + 1] - soff[cc];
-      unsigned long long distinct = td < ncomm ? td : ncomm;
-      gsize[k] = next_pow2(2 * distinct);
-      gtab[k] = total;
-      total += gsize[k];
-      uint32_t members = cntv[cc + 1] - cntv[cc];
-      chunk0[k] = nitems;
-      nitems += (members + kChunkMembers - 1) / kChunkMembers;
-    }
+  gi.ngiant = c.count[1][0][kAggGiant];
+  if (gi.ngiant) {
+    const uint64_t total = c.red_a;
+    gi.nitems = uint32_t(c.red_b);
     if (total > h->gtable_cap) {
       cudaFree(h->gtable);
       h->gtable = nullptr;
@@ -579,60 +879,37 @@ int aggregate(Handle* h, const GraphView& g, const uint32_t* Cp, uint32_t ncomm,
       DFL_CUDA(h, dev_malloc(&h->gtable, sizeof(uint2) * total));
       h->gtable_cap = total;
     }
-    // small device arrays for the giant layout (in the generic scratch)
-    DFL_TRY(ensure_tmp(h, ngiant * (sizeof(uint32_t) * 3 + sizeof(unsigned long long)) + 64));
-    unsigned long long* d_gtab = static_cast<unsigned long long*>(h->tmp);
-    uint32_t* d_giant = reinterpret_cast<uint32_t*>(d_gtab + ngiant);
-    uint32_t* d_gsize = d_giant + ngiant;
-    uint32_t* d_chunk0 = d_gsize + ngiant;
-    DFL_CUDA(h, cudaMemcpyAsync(d_chunk0, chunk0.data(), sizeof(uint32_t) * ngiant, cudaMemcpyHostToDevice,
-                                h->stream));
-    DFL_CUDA(h, cudaMemcpyAsync(d_gtab, gtab.data(), sizeof(unsigned long long) * ngiant,
-                                cudaMemcpyHostToDevice, h->stream));
-    DFL_CUDA(h, cudaMemcpyAsync(d_giant, giant.data(), sizeof(uint32_t) * ngiant, cudaMemcpyHostToDevice,
-                                h->stream));
-    DFL_CUDA(h, cudaMemcpyAsync(d_gsize, gsize.data(), sizeof(uint32_t) * ngiant, cudaMemcpyHostToDevice,
-                                h->stream));
-    a.gtable = h->gtable;
-    {  // queue of high-degree members: at most one per vertex of degree > kAggBigMember
-      uint64_t arcs = h->num_arcs;
-      for (int q = 0; q < 2; ++q) arcs = arcs > h->sg[q].arc_cap ? arcs : h->sg[q].arc_cap;
-      const uint64_t need = arcs / (kAggBigMember + 1) + 64;
-      if (need > h->aggq_cap) {
-        cudaStreamSynchronize(h->stream);
-        cudaFree(h->aggq);
-        h->aggq = nullptr;
-        h->aggq_cap = 0;
-        DFL_CUDA(h, dev_malloc(&h->aggq, sizeof(uint2) * need));
-        h->aggq_cap = need;
-      }
+    gi.keys = reinterpret_cast<uint32_t*>(h->gtable);
+    gi.vals = gi.keys + total;
+    const uint64_t entries = uint64_t(gi.nitems) * kAggThreads;
+    if (entries + 1 > h->aggq_cap) {
+      cudaStreamSynchronize(h->stream);
+      cudaFree(h->aggq);
+      h->aggq = nullptr;
+      h->aggq_cap = 0;
+      DFL_CUDA(h, dev_malloc(&h->aggq, sizeof(uint32_t) * (entries + 1)));
+      h->aggq_cap = entries + 1;
     }
-    a.bigq = h->aggq;
-    a.nbig = &h->ctrl->red_u;
-    DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->red_u, 0, sizeof(unsigned int), h->stream));
-    GiantArgs gi{d_giant, d_gtab, d_gsize, d_chunk0, ngiant, nitems};
+    gi.units = h->aggq;
+    DFL_CUDA(h, cudaMemsetAsync(gi.keys, 0xFF, sizeof(uint32_t) * total, h->stream));
+    DFL_CUDA(h, cudaMemsetAsync(gi.vals, 0, sizeof(uint32_t) * total, h->stream));
     {
       LaunchScope ls(h, DFL_PROF_AGG);
-      k_giant_init<<<grid_for(total, 256), 256, 0, h->stream>>>(a, gi, total);
-      DFL_TRY(check_launch(h, "giant init"));
-    }
-    {
-      LaunchScope ls(h, DFL_PROF_AGG);
-      k_agg_giant_accum<<<grid_for(nitems, 1, 152 * 8), 256, 0, h->stream>>>(a, gi);
+      k_agg_giant_accum<<<grid_for(gi.nitems, 1, 152 * 5), kAggThreads, sizeof(GiantTable), h->stream>>>(a, gi);
       DFL_TRY(check_launch(h, "giant accum"));
     }
+    DFL_TRY(scan_u32(h, gi.units, gi.units, entries));
     {
       LaunchScope ls(h, DFL_PROF_AGG);
-      k_agg_big<<<152 * 4, kAggBigThreads, 0, h->stream>>>(a, gi);
+      k_agg_big<<<152 * 5, kAggThreads, sizeof(GiantTable), h->stream>>>(a, gi);
       DFL_TRY(check_launch(h, "giant members"));
     }
     {
       LaunchScope ls(h, DFL_PROF_AGG);
-      k_agg_giant_emit<<<grid_for(total, 256), 256, 0, h->stream>>>(a, gi, total);
+      launch_pdl(k_agg_giant_emit, grid_for(total, kGiantTile, 152 * 8), kAggThreads, 0, h->stream, a, gi,
+                 (unsigned long long)total);
       DFL_TRY(check_launch(h, "giant emit"));
     }
-    // the layout arrays live in h->tmp: finish before anyone reuses it
-    DFL_CUDA(h, cudaStreamSynchronize(h->stream));
   }
   DFL_TRY(read_ctrl(h));
   if (h->hctrl->err) return set_error(h, DFL_ERR_CUDA, "internal error in aggregation (table overflow)");

@@ -244,7 +244,7 @@ struct Handle {
   uint64_t gtable_cap = 0;
   uint2* bigmv = nullptr;          // queue of the high-degree movers of a sub-step
   uint64_t bigmv_cap = 0;
-  uint2* aggq = nullptr;           // high-degree members of giant communities (aggregation)
+  uint32_t* aggq = nullptr;        // units of giant communities' high-degree members (aggregation)
   uint64_t aggq_cap = 0;
   // decisions of the largest bin: per list position its table and list
   // offsets, chunk prefix, occupied-slot count, finished part blocks and

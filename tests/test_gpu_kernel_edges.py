@@ -326,3 +326,38 @@ def test_batch_touching_most_vertices(dfl, orc):
             assert np.array_equal(x, y)
         same(a, b)
         assert a.stats()["affected_initial"] == b.stats()["affected_initial"] and a.trace() == b.trace()
+
+
+@pytest.mark.parametrize("members", [1, 31, 33, 255, 257, 700])
+@pytest.mark.parametrize("degree", [0, 1, 3, 128, 129, 600])
+def test_aggregation_of_flattened_rows(dfl, orc, members, degree):
+    """One community of `members` vertices with `degree` arcs each outside it
+    (bins by total degree, rows queued from 129 arcs on), among communities of
+    one vertex, isolated vertices included."""
+    rng = np.random.default_rng(members * 1000 + degree)
+    n = 3000 + members
+    u = np.repeat(np.arange(members), degree)
+    v = np.concatenate([members + rng.permutation(2900)[:degree] for _ in range(members)]) if degree else u
+    ring = np.arange(members - 1)  # arcs inside, so that the community has a self-loop
+    u, v = np.concatenate([u, ring]), np.concatenate([v, ring + 1])
+    g = synth.EdgeList(n, u.astype(np.uint32), v.astype(np.uint32), rng.integers(1, 9, u.size).astype(np.uint32))
+    a, b = pair(dfl, orc, g)
+    C = np.arange(n, dtype=np.uint32)
+    C[:members] = 7 if members > 7 else 0
+    a.set_membership(C)
+    b.set_membership(C)
+    for x, y in zip(a.aggregate(), b.aggregate()):
+        assert np.array_equal(x, y)
+
+
+def test_aggregation_of_several_giants(dfl, orc):
+    """Giant communities side by side, with rows longer than one block's share."""
+    g = stars((3000, 2500, 200, 130, 5000), 6000, 12)
+    a, b = pair(dfl, orc, g)
+    rng = np.random.default_rng(0)
+    for k in (2, 3, 40):
+        C = rng.integers(0, k, g.n).astype(np.uint32)
+        a.set_membership(C)
+        b.set_membership(C)
+        for x, y in zip(a.aggregate(), b.aggregate()):
+            assert np.array_equal(x, y)
