@@ -82,7 +82,7 @@ struct Ctrl {
   // taken and vertices left to the part blocks; chunk items of each class;
   // grid barrier
   unsigned long long it_nbig[2];
-  unsigned int it_movers[2], it_work[2], it_bignd[2];
+  unsigned int it_movers[2], it_bignd[2], it_work[2];
   unsigned int it_items[kMaxSubsteps];
   unsigned int bar_count, bar_gen;
   long long m2v;                     // 2m of the current local-moving call

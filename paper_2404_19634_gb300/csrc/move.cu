@@ -48,8 +48,9 @@ struct DecideArgs {
   uint2* bigmv;           // queue of the movers of degree > kMarkInline (push_row)
   unsigned int* movers;   // movers of the sub-step (slot counter into mv_i/mv_c/mv_d)
   unsigned long long* nbig;  // ... its counter
-  unsigned int* clear_movers;  // the next sub-step's two counters, zeroed by this sub-step's
+  unsigned int* clear_movers;  // the next sub-step's three counters, zeroed by this sub-step's
   unsigned long long* clear_nbig;  // commit (null: nothing to zero)
+  unsigned int* clear_bignd;
   // group of graphs (ngraphs > 0): the vertex's graph gives its 2m, whether
   // it is still processed, and where its movers' dQ sum goes
   uint32_t ngraphs;
@@ -1223,9 +1224,17 @@ __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
 //                   kept (and the weight to the own community, when met); the
 //                   vertex's last part block reduces the parts and decides.
 // ---------------------------------------------------------------------------
-constexpr uint32_t kGiantChunk = 1024;             // short per-block work: latency, not bandwidth, bounds it
-constexpr uint32_t kGiantSlots = 2 * kGiantChunk;  // shared chunk table: 2048 keys + values = 16 KB
-constexpr int kAccumThreads = 128;
+// Chunk sizes: a chunk's fixed chain (headers, flush, fence, last-block decision)
+// takes longer than a few more rounds of arcs, so chunks of 1,024 arcs lost
+// (R-MAT 2^22 vertices: DF at 1e-3|E| 425 us a step, ND 1.64 ms, static 22.0
+// ms) against these (374 us, 1.48 ms, 20.6 ms); larger ones (8,192 or a single
+// chunk up to 16,384) lose where hubs are few (temporal stream 254 -> 263 us).
+constexpr uint32_t kGiantSingle = 8192;  // a vertex of at most this degree is one chunk ...
+constexpr uint32_t kGiantChunk = 4096;   // ... a larger one has chunks of this many arcs
+constexpr int kAccumThreads = 256;
+constexpr uint32_t kGiantRound = 8 * kAccumThreads;  // arcs in flight
+constexpr uint32_t kGiantSlots = 4096;               // shared chunk table: keys + values = 32 KB
+constexpr uint32_t kGiantFlush = 512;                // entries before a round (see ChunkTable)
 constexpr uint32_t kGiantPart = 2048;               // occupied slots per decide block
 constexpr int kGiantThreads = 256;
 constexpr uint32_t kGiantListSmem = 2048;          // chunk prefix cached in shared memory
@@ -1258,6 +1267,9 @@ __device__ __forceinline__ uint32_t giant_deg(const DecideArgs& a, uint32_t t) {
   return d;
 }
 
+// Arcs per chunk of a vertex of degree d.
+__device__ __forceinline__ uint32_t giant_chunk_arcs(uint32_t d) { return d <= kGiantSingle ? kGiantSingle : kGiantChunk; }
+
 // Table of a vertex of degree d: a power of two >= 2d (at least 64 slots).
 __device__ __forceinline__ uint64_t giant_table_slots(uint32_t d) {
   if (!d) return 0;
@@ -1283,7 +1295,7 @@ __device__ __forceinline__ void giant_prefix_body(const DecideArgs& a, const Gia
   for (uint32_t t0 = 0; t0 < cnt; t0 += blockDim.x) {
     const uint32_t t = t0 + threadIdx.x;
     const uint32_t d = t < cnt ? giant_deg(a, t) : 0u;
-    const uint32_t ch = (d + kGiantChunk - 1) / kGiantChunk;
+    const uint32_t ch = (d + giant_chunk_arcs(d) - 1) / giant_chunk_arcs(d);
     const unsigned long long ts = giant_table_slots(d);
     unsigned long long xt = ts, xl = d;
     uint32_t xc = ch;
@@ -1410,65 +1422,61 @@ __device__ __forceinline__ uint32_t giant_scan_entries(const DecideArgs& a, cons
 
 constexpr uint32_t kSmallDecide = 4096;  // occupied slots the last chunk block decides alone
 
-// One chunk (arcs [chunk * kGiantChunk, +kGiantChunk)) of list position t
-// by the whole block: aggregated in the shared table (keys, vals:
-// kGiantSlots each), its distinct communities compacted (ek, ev: kGiantChunk
-// each) and added into the vertex's global table; the vertex's last chunk
-// block decides it when the table holds at most kSmallDecide communities.
-// `nch` is the vertex's chunk count.  Every thread of the block calls it.
-__device__ __forceinline__ void giant_chunk(const DecideArgs& a, const GiantDecide& gd, uint32_t t,
-                                            uint32_t chunk, uint32_t nch, long long m2_one, uint32_t* keys,
-                                            uint32_t* vals, uint32_t* ek, uint32_t* ev, BlockScratch& sc,
-                                            MoveSums& sums) {
-  const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5, nthr = blockDim.x;
-  const uint32_t i = a.list[t];
-  if (chunk == 0 && threadIdx.x == 0) {
-    if (a.ever && bit_set(a.ever, i)) ++sums.ever;
-    ++sums.processed;
+// Shared table of a chunk's block, empty at rest.  Its entries move to the
+// vertex's global table at the end of the chunk, or when a further round of
+// arcs could overfill it: the arcs of a converged hub meet a few dozen
+// communities, so a chunk of 4,096 arcs costs one flush, while a singleton
+// start flushes every round (the table is then 5/8 full at the worst).
+struct ChunkTable {
+  uint32_t keys[kGiantSlots], vals[kGiantSlots];
+  uint16_t list[kGiantFlush + kGiantRound];  // occupied slots, compacted for the flush
+  uint32_t claimed, n;
+};
+
+__device__ __forceinline__ void chunk_table_init(ChunkTable& t) {
+  for (uint32_t s = threadIdx.x; s < kGiantSlots; s += kAccumThreads) {
+    t.keys[s] = kEmpty;
+    t.vals[s] = 0;
   }
-  if (a.rbits && !bit_test(a.rbits, i)) return;  // processed, not in the affected range
-  const unsigned long long o = a.g.off[i];
-  const uint32_t dg = a.g.deg[i];
-  const uint32_t k0 = chunk * kGiantChunk;
-  const uint32_t k1 = min(dg, k0 + kGiantChunk);
-  for (uint32_t s = threadIdx.x; s < kGiantSlots; s += nthr) {
-    keys[s] = kEmpty;
-    vals[s] = 0;
-  }
-  if (threadIdx.x == 0) sc.ne = 0;
+  if (threadIdx.x == 0) t.claimed = t.n = 0;
   __syncthreads();
-  // a table of 2x the chunk's arcs cannot overflow
-  scan_row<8>(a, i, o, k1, k0 + wib * 32, nthr, keys, vals, kGiantSlots - 1, kGiantSlots);
-  __syncthreads();
-  // the chunk's distinct communities: compacted in shared memory, then
-  // added into the vertex's global table, four per thread in flight; new
-  // keys' slots go onto its occupied list (one counter update per warp)
-  for (uint32_t s0 = wib * 32; s0 < kGiantSlots; s0 += nthr) {
-    const uint32_t c = keys[s0 + lane];
-    const unsigned m = __ballot_sync(0xFFFFFFFFu, c != kEmpty);
+}
+
+// Every entry of the chunk table into list position t's global table, four per
+// thread in flight; new keys' slots go onto its occupied list (one counter
+// update per warp).  The chunk table is empty again.
+__device__ __forceinline__ void chunk_flush(const DecideArgs& a, const GiantDecide& gd, uint32_t t, uint32_t tmask,
+                                            ChunkTable& ct) {
+  const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
+  for (uint32_t s0 = wib * 32; s0 < kGiantSlots; s0 += kAccumThreads) {
+    const bool has = ct.keys[s0 + lane] != kEmpty;
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, has);
     if (!m) continue;
-    uint32_t base = 0;
-    if (lane == uint32_t(__ffs(m) - 1)) base = atomicAdd(&sc.ne, uint32_t(__popc(m)));
-    base = __shfl_sync(0xFFFFFFFFu, base, __ffs(m) - 1);
-    if (c != kEmpty) {
-      const uint32_t r = base + __popc(m & ((1u << lane) - 1u));
-      ek[r] = c;
-      ev[r] = vals[s0 + lane];
-    }
+    uint32_t at = 0;
+    if (lane == 0) at = atomicAdd(&ct.n, uint32_t(__popc(m)));
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    if (has) ct.list[at + __popc(m & ((1u << lane) - 1u))] = uint16_t(s0 + lane);
   }
   __syncthreads();
-  const uint32_t ne = sc.ne;
-  const uint32_t tmask = uint32_t(giant_table_slots(dg) - 1);
+  const uint32_t ne = ct.n;
   uint32_t* gk = gd.tkeys + gd.toff[t];
   uint32_t* gv = gd.tvals + gd.toff[t];
   uint2* gl = gd.tlist + gd.loff[t];
   constexpr int U = 4;
-  for (uint32_t b0 = wib * 32 * U; b0 < ne; b0 += nthr * U) {  // warp-uniform
-    uint32_t c[U], slot[U], prev[U];
+  for (uint32_t b0 = wib * 32 * U; b0 < ne; b0 += kAccumThreads * U) {  // warp-uniform
+    uint32_t c[U], w[U], slot[U], prev[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const uint32_t e = b0 + u * 32 + lane;
-      c[u] = e < ne ? ek[e] : kEmpty;
+      c[u] = kEmpty;
+      w[u] = 0;
+      if (e < ne) {
+        const uint32_t q = ct.list[e];
+        c[u] = ct.keys[q];
+        w[u] = ct.vals[q];
+        ct.keys[q] = kEmpty;
+        ct.vals[q] = 0;
+      }
       slot[u] = hash_move(c[u]) & tmask;
     }
 #pragma unroll
@@ -1476,7 +1484,6 @@ __device__ __forceinline__ void giant_chunk(const DecideArgs& a, const GiantDeci
     unsigned cm[U];  // lanes that created a slot, per group
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const uint32_t e = b0 + u * 32 + lane;
       bool created = false;
       if (c[u] != kEmpty) {
         // load <= 1/2: the probe ends within the table
@@ -1488,7 +1495,7 @@ __device__ __forceinline__ void giant_chunk(const DecideArgs& a, const GiantDeci
           atomicOr(&a.ctrl->err, kErrInternal);  // (cannot happen: the table is never full)
         } else {
           created = prev[u] == kEmpty;
-          atomicAdd(&gv[slot[u]], ev[e]);
+          atomicAdd(&gv[slot[u]], w[u]);
         }
       }
       cm[u] = __ballot_sync(0xFFFFFFFFu, created);
@@ -1509,6 +1516,103 @@ __device__ __forceinline__ void giant_chunk(const DecideArgs& a, const GiantDeci
       }
     }
   }
+  __syncthreads();
+  if (threadIdx.x == 0) ct.claimed = ct.n = 0;
+}
+
+// One chunk of list position t by the whole block (kAccumThreads threads):
+// aggregated in the chunk table and added into the vertex's global table; the
+// vertex's last chunk block decides it when the table holds at most
+// kSmallDecide communities.  A vertex of one chunk whose table was never
+// flushed is decided from the chunk table itself.  `nch` is the vertex's chunk
+// count.  Every thread of the block calls it.
+__device__ __forceinline__ void giant_chunk(const DecideArgs& a, const GiantDecide& gd, uint32_t t,
+                                            uint32_t chunk, uint32_t nch, long long m2_one, ChunkTable& ct,
+                                            BlockScratch& sc, MoveSums& sums) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t i = a.list[t];
+  if (chunk == 0 && threadIdx.x == 0) {
+    if (a.ever && bit_set(a.ever, i)) ++sums.ever;
+    ++sums.processed;
+  }
+  if (a.rbits && !bit_test(a.rbits, i)) return;  // processed, not in the affected range
+  const unsigned long long o = a.g.off[i];
+  const uint32_t dg = a.g.deg[i];
+  const uint32_t size = giant_chunk_arcs(dg);
+  const uint32_t k0 = chunk * size;
+  const uint32_t k1 = min(dg, k0 + size);
+  const uint32_t tmask = uint32_t(giant_table_slots(dg) - 1);
+  long long m2 = m2_one;
+  uint32_t gi = 0;
+  group_active(a, i, &m2, &gi);  // (a finished graph's vertices have no chunk)
+  const uint32_t d = a.C[i];
+  const long long Ki = a.K[i];
+  bool flushed = false, decided = false;
+  for (uint32_t b = k0; b < k1; b += kGiantRound) {  // block-uniform
+    constexpr int U = kGiantRound / kAccumThreads;
+    uint2 e[U];
+    uint32_t c[U], made = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t k = b + u * kAccumThreads + threadIdx.x;
+      e[u] = k < k1 ? a.g.arcs[o + k] : make_uint2(i, 0u);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) c[u] = (e[u].x != i && e[u].y != 0) ? a.C[e[u].x] : kEmpty;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (c[u] == kEmpty) continue;
+      uint32_t q = hash_move(c[u]) & (kGiantSlots - 1);
+      for (;;) {  // (the table is never full: the probe ends)
+        uint32_t prev = ct.keys[q];
+        if (prev == kEmpty) {
+          prev = atomicCAS(&ct.keys[q], kEmpty, c[u]);
+          if (prev == kEmpty) ++made;
+        }
+        if (prev == kEmpty || prev == c[u]) break;
+        q = (q + 1) & (kGiantSlots - 1);
+      }
+      atomicAdd(&ct.vals[q], e[u].y);
+    }
+    const bool last = b + kGiantRound >= k1;
+    if (!last) {
+      made = __reduce_add_sync(0xFFFFFFFFu, made);
+      if (lane == 0 && made) atomicAdd(&ct.claimed, made);
+    }
+    __syncthreads();
+    const bool full = !last && ct.claimed > kGiantFlush;
+    decided = last && nch == 1 && !flushed;
+    if (full || (last && !decided)) chunk_flush(a, gd, t, tmask, ct);
+    flushed |= full;
+    if (!last) __syncthreads();  // the count has been read, or reset
+  }
+  if (decided) {
+    if (threadIdx.x == 0) sc.ncand = 0;
+    bool have = false;
+    i128 best = 0;
+    uint32_t bc = 0, ncand = 0;
+    const unsigned long long hd = table_argmax<4>(a, ct.keys, ct.vals, kGiantSlots, threadIdx.x, kAccumThreads, d, m2,
+                                                  Ki, have, best, bc, ncand);
+    if (threadIdx.x == 0) sc.hd = 0;
+    ncand = __reduce_add_sync(0xFFFFFFFFu, ncand);
+    __syncthreads();  // the table has been read
+    if (hd) sc.hd = hd;  // exactly one slot holds d
+    if (lane == 0 && ncand) atomicAdd(&sc.ncand, ncand);
+    for (uint32_t s = threadIdx.x; s < kGiantSlots; s += kAccumThreads) {
+      ct.keys[s] = kEmpty;
+      ct.vals[s] = 0;
+    }
+    if (threadIdx.x == 0) ct.claimed = 0;
+    block_argmax(have, best, bc);
+    if (threadIdx.x == 0) {
+      i128 gain = 0;
+      const bool mv = decide_move(a, m2, i, d, Ki, have, best, bc, sc.hd, &gain);
+      sums.bytes += 24 + 12ull * dg + 12ull * sc.ncand + (mv ? 16 + 4ull * dg : 0ull);
+      if (mv) record(a, Move{o, i, d, bc, dg, uint32_t(Ki), gain}, gi, sums);
+    }
+    __syncthreads();
+    return;
+  }
   // the vertex's last chunk block decides it when its table holds few
   // communities; the part blocks take the rest
   __threadfence();
@@ -1522,13 +1626,8 @@ __device__ __forceinline__ void giant_chunk(const DecideArgs& a, const GiantDeci
       gd.done[t] = 0;  // the part blocks count from 0
       sc.ncand = 0;
     }
-    if (nd > kSmallDecide && gd.nbignd && threadIdx.x == 0) atomicAdd(gd.nbignd, 1u);
+    if (nd > kSmallDecide && threadIdx.x == 0) atomicAdd(gd.nbignd, 1u);
     if (nd <= kSmallDecide) {
-      long long m2 = m2_one;
-      uint32_t gi = 0;
-      group_active(a, i, &m2, &gi);
-      const uint32_t d = a.C[i];
-      const long long Ki = a.K[i];
       bool have = false;
       i128 best = 0;
       uint32_t bc = 0;
@@ -1555,17 +1654,16 @@ __device__ __forceinline__ void giant_chunk(const DecideArgs& a, const GiantDeci
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(kAccumThreads, 8) k_giant_accum(DecideArgs a, GiantDecide gd) {
+__global__ void __launch_bounds__(kAccumThreads, 4) k_giant_accum(DecideArgs a, GiantDecide gd) {
   pdl_wait_only();
-  __shared__ uint32_t keys[kGiantSlots];
-  __shared__ uint32_t vals[kGiantSlots];
+  __shared__ ChunkTable ct;
   __shared__ uint32_t s_pre[kGiantListSmem];
-  __shared__ uint32_t s_ek[kGiantChunk], s_ev[kGiantChunk];  // distinct communities of a chunk
   __shared__ BlockScratch sc;
   const long long m2_one = *a.m2p;
   const uint32_t cnt = *a.count;
   const uint32_t nitems = *gd.nitems;
   if (blockIdx.x >= nitems) return;  // no chunk for this block
+  chunk_table_init(ct);
   // the chunk prefix, cached in shared memory when it fits
   const uint32_t* cp = gd.cpre;
   if (cnt + 1 <= kGiantListSmem) {
@@ -1581,7 +1679,7 @@ __global__ void __launch_bounds__(kAccumThreads, 8) k_giant_accum(DecideArgs a, 
       if (cp[mid] <= item) lo = mid;
       else hi = mid;
     }
-    giant_chunk(a, gd, lo, item - cp[lo], cp[lo + 1] - cp[lo], m2_one, keys, vals, s_ek, s_ev, sc, sums);
+    giant_chunk(a, gd, lo, item - cp[lo], cp[lo + 1] - cp[lo], m2_one, ct, sc, sums);
   }
   flush_sums(a, sums, threadIdx.x == 0);
 }
@@ -1706,6 +1804,7 @@ __device__ __forceinline__ void giant_parts(const DecideArgs& a, const GiantDeci
 
 __global__ void __launch_bounds__(kGiantThreads) k_giant_decide(DecideArgs a, GiantDecide gd) {
   pdl_wait_only();
+  if (*gd.nbignd == 0) return;  // every vertex was decided by its last chunk block
   MoveSums sums;
   giant_parts(a, gd, *a.m2p, sums);
   flush_sums(a, sums, threadIdx.x == 0);
@@ -1806,6 +1905,7 @@ __global__ void __launch_bounds__(kCommitThreads) k_commit(DecideArgs a) {
   if (blockIdx.x == 0 && threadIdx.x == 0 && a.clear_movers) {
     *a.clear_movers = 0;
     *a.clear_nbig = 0;
+    *a.clear_bignd = 0;
   }
   commit_body(a, *a.movers, *a.nbig, blockIdx.x * (kCommitThreads / 32) + (threadIdx.x >> 5),
                      gridDim.x * (kCommitThreads / 32));
@@ -1946,7 +2046,7 @@ static_assert(kIterThreads == kGiantThreads && kIterThreads == kCommitThreads,
               "the part blocks and the commit sweep their lists in tiles of one block");
 static_assert(kIterThreads == kListThreads, "the list builder's tiles are one block's");
 static_assert(kIterDynWords >= 2 * kBlockSlots && 8 * 2 * kWarpSlots <= 2 * kBlockSlots &&
-                  2 * kGiantSlots + 2 * kGiantChunk <= 2 * kBlockSlots,
+                  sizeof(ChunkTable) <= sizeof(uint32_t) * 2 * kBlockSlots && kIterThreads == kAccumThreads,
               "the dynamic tables hold every unit kind");
 
 // two blocks per SM: 128 registers a thread (three blocks, at 80 registers,
@@ -2006,8 +2106,9 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
           if (cp[mid] <= u) lo = mid;
           else hi = mid;
         }
-        giant_chunk(a3, gd, lo, uint32_t(u) - cp[lo], cp[lo + 1] - cp[lo], m2_one, dyn, dyn + kGiantSlots,
-                    dyn + 2 * kGiantSlots, dyn + 2 * kGiantSlots + kGiantChunk, sc, sums);
+        ChunkTable& ct = *reinterpret_cast<ChunkTable*>(dyn);
+        chunk_table_init(ct);  // (other units used the memory)
+        giant_chunk(a3, gd, lo, uint32_t(u) - cp[lo], cp[lo + 1] - cp[lo], m2_one, ct, sc, sums);
       } else if (u < uint64_t(G) + n2) {
         const uint32_t i = a2.list[u - G];
         long long m2 = m2_one;
@@ -2512,6 +2613,7 @@ __global__ void k_iter_start(Ctrl* ctrl, int nxt) {
   if (threadIdx.x < 2) {
     ctrl->it_movers[threadIdx.x] = 0;
     ctrl->it_nbig[threadIdx.x] = 0;
+    ctrl->it_bignd[threadIdx.x] = 0;
   }
   unsigned int* c = &ctrl->count[nxt][0][0];
   for (uint32_t q = threadIdx.x; q < sizeof(ctrl->count[0]) / sizeof(unsigned int); q += blockDim.x) c[q] = 0u;
@@ -2592,6 +2694,7 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
     a.nbig = &h->ctrl->it_nbig[s & 1];
     a.clear_movers = s + 1 < k ? &h->ctrl->it_movers[(s + 1) & 1] : nullptr;
     a.clear_nbig = s + 1 < k ? &h->ctrl->it_nbig[(s + 1) & 1] : nullptr;
+    a.clear_bignd = s + 1 < k ? &h->ctrl->it_bignd[(s + 1) & 1] : nullptr;
     bool has[kBins], any = false;
     for (int b = 0; b < kBins; ++b) {
       has[b] = !counts || counts[s][b];
@@ -2657,8 +2760,9 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
         else if (bt == 512) k_decide_block<512><<<grid, 512, smem, st>>>(a);
         else k_decide_block<256><<<grid, 256, smem, st>>>(a);
       } else {
-        const GiantDecide gd = giant_class(gd_base, s, gstride, h->ctrl);  // laid out above
-        launch_pdl(k_giant_accum, 152 * 8, kAccumThreads, 0, st, a, gd);
+        GiantDecide gd = giant_class(gd_base, s, gstride, h->ctrl);  // laid out above
+        gd.nbignd = &h->ctrl->it_bignd[s & 1];
+        launch_pdl(k_giant_accum, 152 * 4, kAccumThreads, 0, st, a, gd);
         DFL_TRY(check_launch(h, "giant accumulate"));
         launch_pdl(k_giant_decide, 152 * 4, kGiantThreads, 0, st, a, gd);
       }
@@ -2678,8 +2782,8 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
       if (pb) h->ev_free.push_back(pb);
     }
     if (any && decide_only) {
-      // (it_nbig and it_movers are adjacent)
-      DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->it_nbig[0], 0, sizeof(h->ctrl->it_nbig) + sizeof(h->ctrl->it_movers), spine));
+      // (it_nbig, it_movers and it_bignd are adjacent)
+      DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->it_nbig[0], 0, sizeof(h->ctrl->it_nbig) + 2 * sizeof(h->ctrl->it_movers), spine));
     } else if (any) {
       LaunchScope ls(h, DFL_PROF_COMMIT, spine);
       launch_pdl(k_commit, 152 * 4, kCommitThreads, 0, spine, a);
@@ -2687,6 +2791,7 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
     } else if (a.clear_movers) {  // no commit ran: zero the next sub-step's counters here
       DFL_CUDA(h, cudaMemsetAsync(a.clear_movers, 0, sizeof(unsigned int), spine));
       DFL_CUDA(h, cudaMemsetAsync(a.clear_nbig, 0, sizeof(*a.clear_nbig), spine));
+      DFL_CUDA(h, cudaMemsetAsync(a.clear_bignd, 0, sizeof(*a.clear_bignd), spine));
     }
   }
   // the next frontier's lists, from its bitmap

@@ -361,3 +361,27 @@ def test_aggregation_of_several_giants(dfl, orc):
         b.set_membership(C)
         for x, y in zip(a.aggregate(), b.aggregate()):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("flags", [16, 32])  # persistent kernel, graph replay
+@pytest.mark.parametrize("degrees", [(4097, 6143, 6145), (8191, 8192, 8193), (12_287, 12_289, 4500), (16_400,)])
+def test_huge_vertices_in_chunks(dfl, orc, degrees, flags):
+    """Vertices of one chunk and of several, with few communities (the chunk
+    table is decided as it is, or flushed once) and with one per leaf (flushed
+    every round)."""
+    g = stars(degrees, 16_500, 21)
+    a, b = pair(dfl, orc, g, flags=flags)
+    rng = np.random.default_rng(2)
+    R = np.ones(g.n, np.uint8)
+    for communities in (g.n, 2000, 5):
+        C = (np.arange(g.n) if communities == g.n else rng.integers(0, communities, g.n)).astype(np.uint32)
+        a.set_membership(C)
+        b.set_membership(C)
+        for _ in range(2):  # (the second round finds every table empty again)
+            F = np.zeros(g.n, np.uint8)
+            F[: len(degrees)] = 1
+            F[rng.integers(0, g.n, 300)] = 1
+            Fa, ma, Sa = a.move_iteration(F, R)
+            Fb, mb, Sb = b.move_iteration(F, R)
+            assert np.array_equal(Fa, Fb) and np.array_equal(ma, mb) and Sa == Sb
+        same(a, b)
