@@ -33,9 +33,10 @@ typedef unsigned __int128 u128;
 constexpr int kWarp = 32;
 // Degree bins of the local-moving kernels: registers (a few arcs), registers
 // (up to 32 arcs, one or two lanes a vertex), a warp's shared table, a block's
-// shared table, chunks summed in a global table.
-constexpr int kBins = 5;
-enum : int { kBinTiny = 0, kBinLanes = 1, kBinTable = 2, kBinWhole = 3, kBinHuge = 4 };
+// shared table (two sizes), chunks summed in a global table.
+constexpr int kBins = 6;
+enum : int { kBinTiny = 0, kBinLanes = 1, kBinTable = 2, kBinMid = 3, kBinWhole = 4, kBinHuge = 5 };
+constexpr uint32_t kMidDeg = 1024;  // largest degree of the smaller block bin
 constexpr uint32_t kBinWarp = 32;   // deg <= 32: registers only (largest bin-0 limit, and the lane bin's)
 constexpr uint32_t kBinWarpDefault = 8;  // default bin-0 limit: 8 lanes per vertex, 4 vertices a warp
 constexpr uint32_t kBinWarpHash = 256;   // deg <= 256: one warp, shared-memory table
@@ -456,7 +457,7 @@ __device__ __forceinline__ uint32_t vertex_class(uint32_t v, uint32_t k, const S
 }
 
 __host__ __device__ __forceinline__ uint32_t degree_bin(uint32_t d, const Segs& s) {
-  return d <= s.hi[0] ? 0u : d <= s.hi[1] ? 1u : d <= s.hi[2] ? 2u : d <= s.hi[3] ? 3u : 4u;
+  return d <= s.hi[0] ? 0u : d <= s.hi[1] ? 1u : d <= s.hi[2] ? 2u : d <= s.hi[3] ? 3u : d <= s.hi[4] ? 4u : 5u;
 }
 
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }

@@ -966,11 +966,10 @@ __global__ void __launch_bounds__(256, 3) k_decide_warp_hash(DecideArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// Bins 2 and 3: one block per vertex with a shared table of kBlockSlots
-// (bin 2 fits by construction; a bin-3 vertex has so many neighbours that the
-// number of distinct neighbour communities, not the degree, sizes the table).
-// If a bin-3 vertex overflows the shared table, it is redone with a table in
-// a per-block slice of global memory sized from the maximum degree.
+// One block per vertex with a shared table of kBlockSlots (a degree above
+// kBinBlock, which only a tuning sends here, may overflow it: the vertex is then
+// redone with a table in a per-block slice of global memory sized from the
+// maximum degree).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kBlockSlots = 2 * kBinBlock;  // 8192 keys + 8192 values = 64 KB
 
@@ -982,11 +981,11 @@ struct BlockScratch {
 };
 
 // One vertex by the whole block (up to 512 threads): a shared table of
-// 2 x degree slots at `dyn` (at most kBlockSlots keys + values); a vertex of
+// 2 x degree slots at `dyn` (at most kSlots keys + values); a vertex of
 // larger degree whose distinct communities overflow it is redone in the
 // block's slice of the global table.  Every thread of the block calls it.
 // The decision and its move are thread 0's.
-template <int kThreads>
+template <int kThreads, uint32_t kSlots>
 __device__ __forceinline__ bool block_vertex(const DecideArgs& a, uint32_t i, long long m2, uint32_t* dyn,
                                              BlockScratch& sc, Move* mvo, MoveSums& sums) {
   const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
@@ -996,7 +995,7 @@ __device__ __forceinline__ bool block_vertex(const DecideArgs& a, uint32_t i, lo
   const unsigned long long o = a.g.off[i];
   const uint32_t dg = a.g.deg[i];
   uint32_t slots = 1024;
-  while (slots < 2 * dg && slots < kBlockSlots) slots <<= 1;
+  while (slots < 2 * dg && slots < kSlots) slots <<= 1;
   uint32_t* keys = dyn;
   uint32_t* vals = dyn + slots;
   bool global = false;
@@ -1055,9 +1054,12 @@ __device__ __forceinline__ bool block_vertex(const DecideArgs& a, uint32_t i, lo
   return mv;
 }
 
-// Bin 2 (and bin-3 degrees when the tuning sends them here): one block per
-// vertex.  Headers are loaded by warp 0 for up to 32 of the block's vertices
-// at once.  The shared table (kBlockSlots keys + values) is empty at rest: a
+// The block bins: one block per vertex, of 128 threads with a table of 2,048
+// slots up to kMidDeg arcs, else of block_threads with kBlockSlots slots.  The
+// barriers between a vertex's phases bound it, so the smaller bin's gain is
+// eight vertices in progress per SM instead of three (ND on the 2^22-vertex
+// R-MAT graph: 452 us of block kernels an iteration in one bin, 185 + 158 in two).  Headers are loaded by warp 0 for up to 32 of the block's vertices
+// at once.  The shared table (kSlots keys + values) is empty at rest: a
 // vertex uses the first power of two >= 2 x degree slots, and the scan that
 // scores the occupied slots also clears them.  Two block barriers per
 // vertex: after the inserts, and after the per-warp bests; warp 0 then
@@ -1067,18 +1069,18 @@ __device__ __forceinline__ bool block_vertex(const DecideArgs& a, uint32_t i, lo
 // list it spreads over all blocks).  Vertices of degree above kBinBlock, or
 // whose scores need 128 bits, take block_vertex (which may fall back to a
 // global table) and the table is emptied after it.
-template <int kThreads>
+template <int kThreads, uint32_t kSlots>
 __device__ __noinline__ void block_vertex_slow(const DecideArgs& a, const VHdr& v, uint32_t* dyn, BlockScratch& sc,
                                                MoveSums& sums) {
   Move m;
-  if (block_vertex<kThreads>(a, v.i, v.m2, dyn, sc, &m, sums)) record(a, m, v.gi, sums);
+  if (block_vertex<kThreads, kSlots>(a, v.i, v.m2, dyn, sc, &m, sums)) record(a, m, v.gi, sums);
 }
 
-template <int kThreads>
+template <int kThreads, uint32_t kSlots>
 __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
   extern __shared__ uint32_t dyn[];
   uint32_t* keys = dyn;
-  uint32_t* vals = dyn + kBlockSlots;
+  uint32_t* vals = dyn + kSlots;
   __shared__ BlockScratch sc;  // the 128-bit path's
   __shared__ VHdr s_hdr[32];
   __shared__ unsigned long long s_best[2][kMaxBlockWarps];
@@ -1093,7 +1095,7 @@ __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
   const uint32_t cnt = *a.count;
   if (blockIdx.x >= cnt) return;  // no vertex for this block
   const uint64_t G = gridDim.x;
-  for (uint32_t s = threadIdx.x; s < kBlockSlots; s += nthr) {
+  for (uint32_t s = threadIdx.x; s < kSlots; s += nthr) {
     keys[s] = kEmpty;
     vals[s] = 0;
   }
@@ -1118,10 +1120,10 @@ __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
     for (uint32_t k = 0; k < nv; ++k) {
       const VHdr v = s_hdr[k];
       if (!v.act) continue;  // block-uniform
-      if (v.dg > kBinBlock || !fits64(v.m2, v.Ki)) {
+      if (v.dg > kSlots / 2 || !fits64(v.m2, v.Ki)) {
         __syncthreads();  // warp 0 has finished the decisions before (it uses sc)
-        block_vertex_slow<kThreads>(a, v, dyn, sc, sums);
-        for (uint32_t s = threadIdx.x; s < kBlockSlots; s += nthr) {
+        block_vertex_slow<kThreads, kSlots>(a, v, dyn, sc, sums);
+        for (uint32_t s = threadIdx.x; s < kSlots; s += nthr) {
           keys[s] = kEmpty;
           vals[s] = 0;
         }
@@ -2076,9 +2078,9 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
     }
     // (the lane bin's vertices are warp units here too, in units of their own)
     const DecideArgs a0 = bin_args(ia, s, kBinTiny), al = bin_args(ia, s, kBinLanes), a1 = bin_args(ia, s, kBinTable),
-                     a2 = bin_args(ia, s, kBinWhole), a3 = bin_args(ia, s, kBinHuge);
+                     am = bin_args(ia, s, kBinMid), a2 = bin_args(ia, s, kBinWhole), a3 = bin_args(ia, s, kBinHuge);
     const GiantDecide gd = class_giant(ia, s);
-    const uint32_t n0 = *a0.count, nl = *al.count, n1 = *a1.count, n2 = *a2.count, n3 = *a3.count;
+    const uint32_t n0 = *a0.count, nl = *al.count, n1 = *a1.count, nm = *am.count, n2 = nm + *a2.count, n3 = *a3.count;
     const uint32_t G = *gd.nitems;
     // chunk prefix of the class, cached when it fits
     const uint32_t* cp = gd.cpre;
@@ -2110,7 +2112,7 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
         chunk_table_init(ct);  // (other units used the memory)
         giant_chunk(a3, gd, lo, uint32_t(u) - cp[lo], cp[lo + 1] - cp[lo], m2_one, ct, sc, sums);
       } else if (u < uint64_t(G) + n2) {
-        const uint32_t i = a2.list[u - G];
+        const uint32_t i = u - G < nm ? am.list[u - G] : a2.list[u - G - nm];
         long long m2 = m2_one;
         uint32_t gi = 0;
         if (!group_active(a2, i, &m2, &gi)) continue;
@@ -2120,7 +2122,7 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
         }
         if (a2.rbits && !bit_test(a2.rbits, i)) continue;
         Move m;
-        if (block_vertex<kIterThreads>(a2, i, m2, dyn, sc, &m, sums)) record(a2, m, gi, sums);
+        if (block_vertex<kIterThreads, kBlockSlots>(a2, i, m2, dyn, sc, &m, sums)) record(a2, m, gi, sums);
       } else if (u < uint64_t(G) + n2 + U1 + UL) {
         // one table-bin or lane-bin vertex per warp and round, in the warp's own table
         const bool table = u < uint64_t(G) + n2 + U1;
@@ -2206,10 +2208,10 @@ static_assert(2 * kSmallSlots >= 2 * kBlockSlots + kSmallThreads / 32 * 2 * kWar
 
 // Estimated ns of one iteration's decisions over lists of the given lengths
 // (measured: a warp decides a vertex, or four of bin 0, in about 2.5 us, a CTA
-// one of the block bin in 6 us, the cluster one of the last bin in 10 us).
+// one of the block bins in 3 or 6 us, the cluster one of the last bin in 10 us).
 __host__ __device__ inline uint64_t small_cost(const uint32_t* n) {
   return (uint64_t(n[kBinTiny] / 4) + n[kBinLanes] + 2ull * n[kBinTable]) * 2500 / kSmallWarps +
-         uint64_t(n[kBinWhole]) * 6000 / kSmallCtas + uint64_t(n[kBinHuge]) * 10000;
+         (3000ull * n[kBinMid] + 6000ull * n[kBinWhole]) / kSmallCtas + uint64_t(n[kBinHuge]) * 10000;
 }
 constexpr uint64_t kSmallCostMax = 60000;
 
@@ -2453,8 +2455,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_move(const __grid_co
     }
     cluster_sync();
     for (uint32_t s = 0; s < k; ++s) {
-      const uint32_t n0 = s_n[s][kBinTiny], nl = s_n[s][kBinLanes], n1 = s_n[s][kBinTable], n2 = s_n[s][kBinWhole],
-                     n3 = s_n[s][kBinHuge];
+      const uint32_t n0 = s_n[s][kBinTiny], nl = s_n[s][kBinLanes], n1 = s_n[s][kBinTable], nm = s_n[s][kBinMid],
+                     n2 = nm + s_n[s][kBinWhole], n3 = s_n[s][kBinHuge];
       if (!(n0 + nl + n1 + n2 + n3)) continue;
       const uint32_t par = step++ & 1;  // the counters of this sub-step that is run
       unsigned long long* nbig = &ctrl->it_nbig[par];
@@ -2478,7 +2480,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_move(const __grid_co
         empty_table();
       }
       for (uint32_t t = rank; t < n2; t += kSmallCtas) {
-        const uint32_t i = base[seg.off[s * kBins + kBinWhole] + t];
+        const uint32_t i = t < nm ? base[seg.off[s * kBins + kBinMid] + t] : base[seg.off[s * kBins + kBinWhole] + t - nm];
         long long m2 = m2_one;
         gi = 0;
         if (!group_active(a, i, &m2, &gi)) continue;
@@ -2487,7 +2489,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_move(const __grid_co
           ++sums.processed;
         }
         if (a.rbits && !bit_test(a.rbits, i)) continue;
-        if (block_vertex<kSmallThreads>(a, i, m2, block_table, sc, &m, sums))
+        if (block_vertex<kSmallThreads, kBlockSlots>(a, i, m2, block_table, sc, &m, sums))
           small_record(a, m, gi, moves, &s_nmv[par], nbig, sums);
       }
       for (uint32_t u = warp; u < n1; u += kSmallWarps) {
@@ -2546,17 +2548,17 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_move(const __grid_co
       }
       cluster_sync();
       // 2. commit the CTA's own moves and mark around them; the other pair of counters is idle
-      const uint32_t nm = s_nmv[par];
+      const uint32_t done = s_nmv[par];
       if (threadIdx.x == 0) {
         s_nmv[par ^ 1] = 0;
         if (rank == 0) ctrl->it_nbig[par ^ 1] = 0;
-        if (nm) atomicAdd(&ctrl->moved, (unsigned long long)nm);
+        if (done) atomicAdd(&ctrl->moved, (unsigned long long)done);
       }
       // a warp per move, or eight lanes when there are many
-      const uint32_t L = nm > 2 * kSmallThreads / 32 ? 8u : 32u, sl = lane & (L - 1);
-      for (uint32_t e0 = wib * (32 / L); e0 < nm; e0 += kSmallThreads / L) {
+      const uint32_t L = done > 2 * kSmallThreads / 32 ? 8u : 32u, sl = lane & (L - 1);
+      for (uint32_t e0 = wib * (32 / L); e0 < done; e0 += kSmallThreads / L) {
         const uint32_t e = e0 + lane / L;
-        if (e >= nm) continue;
+        if (e >= done) continue;
         const SmallMove v = moves[e];
         if (sl == 0) const_cast<uint32_t*>(a.C)[v.i] = v.c;
         if (sl == 1 || sl == 2) {
@@ -2632,8 +2634,8 @@ __global__ void k_set_m2(Ctrl* ctrl, long long m2, const Ctrl* ap) {
 // slice of the global overflow table
 constexpr uint32_t kBlockGridMax = 3 * 152;
 
-// Profile class of each bin (the lane and table bins are one class).
-constexpr int kBinClass[kBins] = {DFL_PROF_BIN0, DFL_PROF_BIN1, DFL_PROF_BIN1, DFL_PROF_BIN2, DFL_PROF_BIN3};
+// Profile class of each bin (the lane and table bins are one class, as are the block bins).
+constexpr int kBinClass[kBins] = {DFL_PROF_BIN0, DFL_PROF_BIN1, DFL_PROF_BIN1, DFL_PROF_BIN2, DFL_PROF_BIN2, DFL_PROF_BIN3};
 
 // k_decide_lanes for a list of c vertices (~0: its length is on the device) of
 // at most lim arcs.
@@ -2676,7 +2678,7 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
   const bool par = !(h->opt.flags & DFL_FLAG_SERIAL_BINS);
   cudaStream_t spine = par ? h->aux[kBins - 2] : h->stream;
   cudaStream_t bst[kBins] = {h->stream, par ? h->aux[0] : h->stream, par ? h->aux[1] : h->stream,
-                             par ? h->aux[2] : h->stream, spine};
+                             par ? h->aux[2] : h->stream, par ? h->aux[3] : h->stream, spine};
   if (par) {
     DFL_CUDA(h, cudaEventRecord(h->ev_fork, h->stream));
     DFL_CUDA(h, cudaStreamWaitEvent(spine, h->ev_fork, 0));
@@ -2751,14 +2753,16 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
       } else if (b == kBinTable) {
         // a warp per vertex, headers in batches of up to 32 (fewer when the list is short)
         k_decide_warp_hash<<<counts ? grid_for(uint64_t(c) * 32, 256, 152 * 6) : 152 * 3, 256, 0, st>>>(a);
+      } else if (b == kBinMid) {
+        k_decide_block<128, 2 * kMidDeg><<<counts ? grid_for(c, 1, 152 * 8) : 152 * 8, 128, sizeof(uint32_t) * 4 * kMidDeg, st>>>(a);
       } else if (b == kBinWhole) {
         const size_t smem = sizeof(uint32_t) * 2 * kBlockSlots;
         const uint32_t bt = h->tune.block_threads;
         const uint32_t per_sm = bt == 512 ? 2 : 3;  // 64 KB table each; grid <= kBlockGridMax
         const uint32_t grid = counts ? grid_for(c, 1, 152 * per_sm) : 152 * per_sm;
-        if (bt == 128) k_decide_block<128><<<grid, 128, smem, st>>>(a);
-        else if (bt == 512) k_decide_block<512><<<grid, 512, smem, st>>>(a);
-        else k_decide_block<256><<<grid, 256, smem, st>>>(a);
+        if (bt == 128) k_decide_block<128, kBlockSlots><<<grid, 128, smem, st>>>(a);
+        else if (bt == 512) k_decide_block<512, kBlockSlots><<<grid, 512, smem, st>>>(a);
+        else k_decide_block<256, kBlockSlots><<<grid, 256, smem, st>>>(a);
       } else {
         GiantDecide gd = giant_class(gd_base, s, gstride, h->ctrl);  // laid out above
         gd.nbignd = &h->ctrl->it_bignd[s & 1];
@@ -3070,11 +3074,11 @@ int prepare_move(Handle* h, const MoveArgs& ma, DecideArgs* out, GiantDecide* gd
   static cudaError_t smem_rc = cudaSuccess;
   std::call_once(smem_once, [] {
     const int tb = int(sizeof(uint32_t) * 2 * kBlockSlots);
-    smem_rc = cudaFuncSetAttribute(k_decide_block<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, tb);
+    smem_rc = cudaFuncSetAttribute(k_decide_block<128, kBlockSlots>, cudaFuncAttributeMaxDynamicSharedMemorySize, tb);
     if (smem_rc == cudaSuccess)
-      smem_rc = cudaFuncSetAttribute(k_decide_block<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, tb);
+      smem_rc = cudaFuncSetAttribute(k_decide_block<256, kBlockSlots>, cudaFuncAttributeMaxDynamicSharedMemorySize, tb);
     if (smem_rc == cudaSuccess)
-      smem_rc = cudaFuncSetAttribute(k_decide_block<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, tb);
+      smem_rc = cudaFuncSetAttribute(k_decide_block<512, kBlockSlots>, cudaFuncAttributeMaxDynamicSharedMemorySize, tb);
     if (smem_rc == cudaSuccess)
       smem_rc = cudaFuncSetAttribute(k_iterate, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      int(sizeof(uint32_t) * kIterDynWords));

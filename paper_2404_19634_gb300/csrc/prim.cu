@@ -307,6 +307,7 @@ void make_segs(Handle* h, uint32_t k) {
   h->segs.hi[kBinTiny] = h->tune.bin_warp;
   h->segs.hi[kBinLanes] = h->tune.bin_warp_hash < kBinWarp ? h->tune.bin_warp_hash : kBinWarp;
   h->segs.hi[kBinTable] = h->tune.bin_warp_hash;
+  h->segs.hi[kBinMid] = h->tune.bin_block < kMidDeg ? h->tune.bin_block : kMidDeg;
   h->segs.hi[kBinWhole] = h->tune.bin_block;
   h->segs.goff = h->ngraphs ? h->d_goff : nullptr;
   h->segs.ng = h->ngraphs;
