@@ -385,3 +385,38 @@ def test_huge_vertices_in_chunks(dfl, orc, degrees, flags):
             Fb, mb, Sb = b.move_iteration(F, R)
             assert np.array_equal(Fa, Fb) and np.array_equal(ma, mb) and Sa == Sb
         same(a, b)
+
+
+@pytest.mark.parametrize("sizes", [(1,), (255, 1, 256, 257, 2, 31, 33, 700), (1,) * 300, (513, 3, 767), (5000,)])
+def test_group_weights_at_slice_borders(dfl, orc, sizes):
+    """Each graph's 2m (and so the exact modularity) where graphs begin and
+    end at, next to and inside a 256-vertex slice, before and after a batch."""
+    import torch
+    gs = [random_graph(n, 3 * n, 60 + k) for k, n in enumerate(sizes)]
+    csrs = [(g.n, *synth.to_csr(g)) for g in gs]
+    s = torch.cuda.Stream()
+    _STREAMS.append(s)
+    grp = dfl.DflGroup(csrs, stream=s)
+    orcs = [orc.Oracle(n, off, idx, w) for n, off, idx, w in csrs]
+
+    def check():
+        K = grp.weights()[0]
+        start = 0
+        for k, o in enumerate(orcs):
+            assert np.array_equal(grp.graph_membership(k), o.membership())
+            assert np.array_equal(K[start:start + sizes[k]], o.weights()[0])
+            assert grp.graph_modularity(k)[1:] == o.modularity()[1:]
+            start += sizes[k]
+
+    grp.static()
+    for o in orcs:
+        o.static()
+    check()
+    none = np.zeros((0, 3), np.uint32)
+    ins = [np.array([[0, n - 1, 3 + k]], np.uint32) if n > 1 else none for k, n in enumerate(sizes)]
+    grp.apply_batches([none] * len(sizes), ins)
+    grp.update(2)
+    for o, i in zip(orcs, ins):
+        assert o.apply_batch(none, i) == 0
+        o.update(2)
+    check()
