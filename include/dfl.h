@@ -163,7 +163,7 @@ enum {
   DFL_PROF_COMMIT = 3,  /* local-moving move-apply kernels */
   DFL_PROF_AGG = 4,     /* renumbering and aggregation */
   DFL_PROF_OTHER = 5,
-  DFL_PROF_BIN0 = 6,    /* decide kernels by degree bin (<= 32, <= 256, <= 4096, larger); */
+  DFL_PROF_BIN0 = 6,    /* decide kernels by degree bin (default limits <= 8, <= 256, <= 4096, larger); */
   DFL_PROF_BIN1 = 7,    /* these run concurrently inside the DFL_PROF_MOVE wall time */
   DFL_PROF_BIN2 = 8,
   DFL_PROF_BIN3 = 9,
@@ -341,14 +341,18 @@ int dfl_aggregate(dfl_handle* h, uint32_t* nv, uint64_t* na, uint64_t* offsets,
  *   degree <= bin_warp:       W = bin_warp rounded up to a power of two (>= 4)
  *                             lanes per vertex, 32/W vertices per warp,
  *                             communities grouped in registers
- *   degree <= bin_warp_hash:  one warp (registers up to 32 arcs, else an
- *                             open-addressing table in shared memory)
- *   degree <= bin_block:      one block of block_threads, shared-memory table
+ *                             (long lists: a lane per vertex)
+ *   degree <= bin_warp_hash:  one warp (registers up to 32 arcs, a lane per
+ *                             vertex in long lists; else an open-addressing
+ *                             table in shared memory)
+ *   degree <= bin_block:      one block (128 threads up to 1024 arcs, else
+ *                             block_threads), shared-memory table
  *                             (global-memory slice when it overflows)
- *   larger:                   split into 1024-arc chunks, one block each,
- *                             summed in a global table of the vertex; its
- *                             last chunk block (or, for many distinct
- *                             communities, a block per 2048 of them) decides
+ *   larger:                   one chunk up to 8192 arcs, else chunks of 4096,
+ *                             one block each, summed in a global table of the
+ *                             vertex; its last chunk block (or, for many
+ *                             distinct communities, a block per 2048 of them)
+ *                             decides
  * Valid ranges: bin_warp <= 32, bin_warp <= bin_warp_hash <= 256,
  * bin_warp_hash <= bin_block, block_threads in {128, 256, 512}.
  * Defaults: 8, 256, 4096, 256. */

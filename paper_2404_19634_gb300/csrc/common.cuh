@@ -37,11 +37,11 @@ constexpr int kWarp = 32;
 constexpr int kBins = 6;
 enum : int { kBinTiny = 0, kBinLanes = 1, kBinTable = 2, kBinMid = 3, kBinWhole = 4, kBinHuge = 5 };
 constexpr uint32_t kMidDeg = 1024;  // largest degree of the smaller block bin
-constexpr uint32_t kBinWarp = 32;   // deg <= 32: registers only (largest bin-0 limit, and the lane bin's)
-constexpr uint32_t kBinWarpDefault = 8;  // default bin-0 limit: 8 lanes per vertex, 4 vertices a warp
+constexpr uint32_t kBinWarp = 32;   // deg <= 32: registers only (the tiny bin's largest limit, and the lane bin's)
+constexpr uint32_t kBinWarpDefault = 8;  // the tiny bin's default limit: 8 lanes per vertex, 4 vertices a warp
 constexpr uint32_t kBinWarpHash = 256;   // deg <= 256: one warp, shared-memory table
 constexpr uint32_t kBinBlock = 4096;     // deg <= 4096: one block, shared-memory table
-                                          // larger: one block, global-memory table
+                                          // larger: chunks, global-memory table
 constexpr uint32_t kMaxSubsteps = 8;
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;  // empty hash-table key
 constexpr uint32_t kSmallIters = 20;      // iterations of one small-frontier launch
@@ -102,10 +102,8 @@ struct Ctrl {
   unsigned long long red_b;
   unsigned long long red_c;
   unsigned long long long_rows;      // a queue of long rows: rows << 32 | pieces (push_row)
-  unsigned int red_u;
   unsigned int apply_go;             // the batch apply's gate: the batch is written (1) or nothing is (0)
   unsigned int apply_defer;          // ... with rows to rebuild (by the multi-block rebuild kernel)
-  unsigned int pad3;
 };
 
 // A CSR whose rows are addressed by (offset, degree): the slack CSR of G^t
@@ -538,7 +536,7 @@ __device__ __forceinline__ void append_vertex(uint32_t v, bool valid, uint32_t k
 // sparse frontier costs one chain too.  A thread per bitmap word, walking its
 // vertices one after another, took 37 us for the frontiers of a 2-million-
 // vertex group (now 11 us) and a thread per vertex with a reservation per 256
-// took 92 us for all of 4 million vertices (now 31 us); a DF step's sparse
+// took 92 us for all of 4 million vertices (now 37 us); a DF step's sparse
 // frontier on 4 million vertices takes 9 us (6.6 before).
 // Returns, per thread, the vertices without arcs it met (kBits false: they are
 // processed but never queued; a bitmap's vertices are queued whatever their
@@ -787,18 +785,22 @@ struct MoveArgs {
   uint64_t frontier_hint = ~0ull;
 };
 // A list of a sub-step class shorter than this is decided with several lanes
-// per vertex (W lanes in bin 0, a warp in the lane bin) instead of a lane per
-// vertex: with few vertices the latter leaves the SMs to
-// the largest-degree chain less well (R-MAT 2^22, DF at 1e-3|E|: 0.44 vs
-// 0.49-0.52 ms per batch), while on full frontiers it is the faster one.
+// per vertex (W lanes in the tiny bin, a warp in the lane bin) instead of a lane
+// per vertex: with few vertices the latter leaves most of the GPU idle behind
+// one long chain a lane, while on full frontiers it is the faster one (DF at
+// 1e-3|E| on the 2^22-vertex R-MAT graph: 0.44 ms a batch short, 0.49-0.52 with
+// a thread per vertex).  The line is flat: halving or quartering either limit
+// changed neither DF nor static times on four graphs.
 constexpr uint64_t kSmallList = 32768;
-constexpr uint64_t kSmallLanes = 8192;  // the lane bin's vertices weigh four of bin 0's
+constexpr uint64_t kSmallLanes = 8192;  // the lane bin's vertices weigh four of the tiny bin's
 // Below this many pending batch arcs a DF or DS update launches its
 // iterations from the host even when graph replay is allowed: a frontier of
 // a few vertices leaves most bins empty, and skipping them beats replaying
 // a graph that launches every bin (R-MAT 2^22: 0.19 vs 0.23 ms at 3 edges,
 // while replay won from about 300 edges up).  Groups prefer host launches
-// too (64 graphs: 0.600 vs 0.607 ms per DF step, static 267 vs 296 ms).
+// too (64 graphs: 0.600 vs 0.607 ms per DF step, static 267 vs 296 ms).  (Both
+// measured before small frontiers had a kernel of their own, which is tried
+// first in either mode.)
 constexpr uint64_t kGraphMinArcs = 512;
 void destroy_iteration_graph(Handle::IterGraph& g);
 int local_move(Handle* h, const MoveArgs& a, uint32_t pass, uint32_t* iterations,

@@ -43,7 +43,7 @@ struct DecideArgs {
   uint32_t* mv_d;
   Ctrl* ctrl;
   uint32_t k;
-  uint2* gtable;          // bin 3: per-block global tables
+  uint2* gtable;          // block bins: per-block global overflow tables
   uint32_t gslots;        // slots per block (power of two)
   uint2* bigmv;           // queue of the movers of degree > kMarkInline (push_row)
   unsigned int* movers;   // movers of the sub-step (slot counter into mv_i/mv_c/mv_d)
@@ -210,11 +210,11 @@ __device__ __forceinline__ void mark_arcs(const DecideArgs& a, uint32_t i, unsig
 }
 
 // ---------------------------------------------------------------------------
-// Bin 0: small degrees (at most W <= 32 arcs), W lanes per vertex, so one
+// The tiny bin (at most W <= 32 arcs), W lanes per vertex, so one
 // warp decides 32 / W vertices at once, one arc per lane; aggregation by
 // community in registers inside each W-lane segment (W shuffles and
-// compares).  A long bin-0 list instead takes a vertex per thread
-// (k_decide_lanes, below).
+// compares).  A long list instead takes a vertex per lane (k_decide_lanes,
+// below).
 // ---------------------------------------------------------------------------
 
 // Argmax of (score, -c) over the aligned W-lane segment of each lane.
@@ -476,13 +476,14 @@ __device__ __forceinline__ void block_argmax(bool& have, i128& best, uint32_t& b
 }
 
 // ---------------------------------------------------------------------------
-// Bin 1: 32 < deg <= 256, one warp per vertex with a shared table.
+// One warp per vertex with a shared table, a vertex at a time (the persistent
+// and small-frontier kernels, and scores of 128 bits).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kWarpSlots = 512;
 constexpr int kWarpHashWarps = 8;
-static_assert(kBinWarpHash <= 8 * 32 && 2 * kBinWarpHash <= kWarpSlots, "a bin-1 vertex fits 8 arcs a lane and its table");
+static_assert(kBinWarpHash <= 8 * 32 && 2 * kBinWarpHash <= kWarpSlots, "a table-bin vertex fits 8 arcs a lane and its table");
 
-// One vertex of bin 1 by one warp (its degree up to kWarpSlots / 2): up to
+// One vertex of the table bin by one warp (its degree up to kWarpSlots / 2): up to
 // 32 arcs by the register path, else a shared table of the warp.  Every lane
 // of the warp calls it.
 __device__ __forceinline__ bool warp_table_vertex(const DecideArgs& a, uint32_t i, long long m2, uint32_t* keys,
@@ -796,9 +797,9 @@ __global__ void __launch_bounds__(kLaneThreads, D == 8 ? 8 : 5) k_decide_lanes(D
 }
 
 // ---------------------------------------------------------------------------
-// Bin 2: one warp per vertex (more than 32 arcs), vertices taken in batches
-// of up to 32 headers, each decided in the warp's shared table.  The table is empty at rest: the
-// lane that creates a community's slot loads that community's Sigma at once,
+// The table bin: one warp per vertex (more than 32 arcs), vertices taken in
+// batches of up to 32 headers, each decided in the warp's shared table.  The
+// table is empty at rest: the lane that creates a community's slot loads that community's Sigma at once,
 // and after the last arc is in, scores the slot and clears it, so the table
 // is neither cleared nor scanned as a whole.  Vertices whose scores need
 // 128 bits take the per-vertex path of the persistent kernel.
@@ -1018,7 +1019,7 @@ __device__ __forceinline__ bool block_vertex(const DecideArgs& a, uint32_t i, lo
     }
     __syncthreads();
     // a table of >= 2 * deg slots cannot overflow: probe it to the end;
-    // a smaller shared table (bin 3) gives up early and falls back
+    // a smaller shared table gives up early and falls back
     const uint32_t limit = (global || slots >= 2 * dg) ? slots : 64;
     bool ok = scan_row<8>(a, i, o, dg, wib * 32, nthr, keys, vals, mask, limit);
     if (!ok) sc.ok = 0;
@@ -1058,9 +1059,9 @@ __device__ __forceinline__ bool block_vertex(const DecideArgs& a, uint32_t i, lo
 // slots up to kMidDeg arcs, else of block_threads with kBlockSlots slots.  The
 // barriers between a vertex's phases bound it, so the smaller bin's gain is
 // eight vertices in progress per SM instead of three (ND on the 2^22-vertex
-// R-MAT graph: 452 us of block kernels an iteration in one bin, 185 + 158 in two).  Headers are loaded by warp 0 for up to 32 of the block's vertices
-// at once.  The shared table (kSlots keys + values) is empty at rest: a
-// vertex uses the first power of two >= 2 x degree slots, and the scan that
+// R-MAT graph: 452 us of block kernels an iteration in one bin, 185 + 158 in two).
+// Headers are loaded by warp 0 for up to 32 of the block's vertices at once.
+// The shared table (kSlots keys + values) is empty at rest: a vertex uses the first power of two >= 2 x degree slots, and the scan that
 // scores the occupied slots also clears them.  Two block barriers per
 // vertex: after the inserts, and after the per-warp bests; warp 0 then
 // decides while the other warps start the next vertex (the per-vertex
@@ -1210,11 +1211,11 @@ __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// Bin 3 (the largest degrees): three kernels, every step parallel and
+// The largest degrees: three kernels, every step parallel and
 // proportional to the vertex's arcs or its distinct neighbour communities.
 //   k_giant_prefix  at the start of an iteration, for every sub-step class
 //                   (one block each), lays out per listed vertex its chunks
-//                   of kGiantChunk arcs, a global open-addressing table of a
+//                   (kGiantSingle, kGiantChunk), a global open-addressing table of a
 //                   power of two >= 2 x degree slots (empty at rest) and a
 //                   list of the table's occupied slots (capacity = degree);
 //   k_giant_accum   one block per chunk: the chunk's arcs are aggregated by
@@ -1280,7 +1281,7 @@ __device__ __forceinline__ uint64_t giant_table_slots(uint32_t d) {
   return p;
 }
 
-// One block: exclusive prefixes over the bin-3 list of chunks, table slots
+// One block: exclusive prefixes over the huge bin's list of chunks, table slots
 // and list capacities.
 __device__ __forceinline__ void giant_prefix_body(const DecideArgs& a, const GiantDecide& gd) {
   __shared__ unsigned long long s_t[32], s_l[32];
@@ -1349,7 +1350,7 @@ __device__ __forceinline__ void giant_prefix_body(const DecideArgs& a, const Gia
   }
 }
 
-// Class s's region of the bin-3 arrays: every sub-step class has its own
+// Class s's region of the huge bin's arrays: every sub-step class has its own
 // layout (at s * gstride), so all of an iteration's layouts are made at once.
 __host__ __device__ __forceinline__ GiantDecide giant_class(GiantDecide gd, uint32_t s, uint64_t gstride,
                                                           Ctrl* ctrl) {
@@ -1364,7 +1365,7 @@ __host__ __device__ __forceinline__ GiantDecide giant_class(GiantDecide gd, uint
   return gd;
 }
 
-// The bin-3 layouts of every sub-step class (block s: class s), at the start
+// The huge bin's layouts of every sub-step class (block s: class s), at the start
 // of an iteration, when all classes' lists are final; each sub-step's chain
 // of largest-degree kernels then starts with its chunks.
 __global__ void __launch_bounds__(1024) k_giant_prefix(DecideArgs a, GiantDecide gd, uint64_t gstride,
@@ -1986,7 +1987,7 @@ struct IterArgs {
   uint32_t gstride;
   uint32_t k;
   int cur;
-  uint32_t seg_lanes;      // W: lanes per bin-0 vertex
+  uint32_t seg_lanes;      // W: lanes per tiny-bin vertex
   const uint32_t* lists_cur;
   uint32_t* fbits_cur;     // cleared at the end (the processed frontier)
   uint32_t words;
@@ -2189,12 +2190,12 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
 // straight onto the next frontier's lists, and the tolerance test is made on
 // the device.  Vertices are dealt statically: a vertex of the last bin to the
 // whole cluster, over one table spread over the CTAs' shared memory; of the
-// block bin to a CTA, of the table and lane bins to a warp, of bin 0 to a few
+// block bins to a CTA, of the table and lane bins to a warp, of the tiny bin to a few
 // lanes.  The kernel stops before an iteration whose estimated time is above
 // what the per-bin kernels need (small_cost), leaving its frontier to them.
 // A DF step's four sub-steps of 100 edges on 10,000 vertices take 34 us here
 // (30 + 15 us of decide and commit kernels, 4 us of lists, and the launches and
-// the control read between them before: 195 -> 136 us the whole step); an
+// the control read between them before: 195 -> 130 us the whole step); an
 // iteration of the same graph's static run takes 49 us, 75 before.
 // ---------------------------------------------------------------------------
 constexpr int kSmallThreads = 512;
@@ -2207,18 +2208,22 @@ static_assert(2 * kSmallSlots >= 2 * kBlockSlots + kSmallThreads / 32 * 2 * kWar
               "the cluster table's memory also holds a block table and the warps' tables");
 
 // Estimated ns of one iteration's decisions over lists of the given lengths
-// (measured: a warp decides a vertex, or four of bin 0, in about 2.5 us, a CTA
+// (measured: a warp decides a vertex, or four tiny ones, in about 2.5 us, a CTA
 // one of the block bins in 3 or 6 us, the cluster one of the last bin in 10 us).
 __host__ __device__ inline uint64_t small_cost(const uint32_t* n) {
   return (uint64_t(n[kBinTiny] / 4) + n[kBinLanes] + 2ull * n[kBinTable]) * 2500 / kSmallWarps +
          (3000ull * n[kBinMid] + 6000ull * n[kBinWhole]) / kSmallCtas + uint64_t(n[kBinHuge]) * 10000;
 }
+// Flat down to 45 us.  At 30 us static Louvain on 10,000 vertices loses the
+// iterations that gain most (2.59 -> 2.75 ms); at 120 us the cluster keeps
+// iterations that the per-bin kernels do faster with the whole GPU (static on
+// 400,000 vertices 4.24 -> 4.90 ms, on 32 graphs 15.4 -> 16.2 ms).
 constexpr uint64_t kSmallCostMax = 60000;
 
 struct SmallArgs {
   DecideArgs a[2];         // by the processed frontier's buffer
   int cur;                 // ... of the first iteration
-  uint32_t seg_lanes;      // W: lanes per bin-0 vertex
+  uint32_t seg_lanes;      // W: lanes per tiny-bin vertex
   uint32_t* lists[2];
   uint32_t* fbits[2];
   uint32_t max_iters;      // iterations left to the pass
@@ -2671,8 +2676,8 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
   // chain that bounds a sub-step -- the largest-degree chunks, their
   // decisions, the commit -- runs on one stream (the spine, the highest-
   // priority auxiliary stream), so that each of its kernels is a dependent
-  // launch of the one before; the spine forks the other bins (bin 0 on the
-  // handle's stream, bins 1 and 2 on auxiliary streams) at the start of a
+  // launch of the one before; the spine forks the other bins (the tiny one on
+  // the handle's stream, the rest on auxiliary streams) at the start of a
   // sub-step and joins them before the commit.  With DFL_FLAG_SERIAL_BINS
   // everything runs on the handle's stream.
   const bool par = !(h->opt.flags & DFL_FLAG_SERIAL_BINS);
@@ -3085,7 +3090,7 @@ int prepare_move(Handle* h, const MoveArgs& ma, DecideArgs* out, GiantDecide* gd
 
   });
   DFL_CUDA(h, smem_rc);
-  // bin-3 buffers, sized by bounds: at most arcs / (bin_block + 1) listed
+  // the huge bin's buffers, sized by bounds: at most arcs / (bin_block + 1) listed
   // vertices; tables of at most 4 x degree (>= 64) slots each; occupied
   // lists of at most degree entries; at most arcs / kGiantPart + items parts
   {
