@@ -124,9 +124,10 @@ struct SuperGraph {
 };
 
 // Frontier list layout: segment (class s, bin b) starts at off[s*kBins+b]
-// and holds at most the number of ids in [0, n) of class s.
+// and holds at most the number of ids in [0, n) of class s.  The offsets run
+// up to kBins * n, which does not fit 32 bits for every n that dfl_create takes.
 struct Segs {
-  uint32_t off[kMaxSubsteps * kBins];
+  uint64_t off[kMaxSubsteps * kBins];
   uint32_t cap[kMaxSubsteps * kBins];
   uint32_t hi[kBins - 1];  // largest degree of every bin but the last, which takes the rest (tuning)
   // group: a vertex's sub-step class comes from its id within its own graph
@@ -134,6 +135,17 @@ struct Segs {
   const uint32_t* goff;
   uint32_t ng;
 };
+
+// The segments of k classes with counts[s] ids each, one after another.
+inline void layout_segs(Segs& seg, const uint64_t* counts, uint32_t k) {
+  uint64_t off = 0;
+  for (uint32_t s = 0; s < kMaxSubsteps; ++s)
+    for (int b = 0; b < kBins; ++b) {
+      seg.off[s * kBins + b] = off;
+      seg.cap[s * kBins + b] = s < k ? uint32_t(counts[s]) : 0u;
+      off += s < k ? counts[s] : 0;
+    }
+}
 
 // One (u, v) pair of a batch, and one row it touches (batch.cu): a 32-byte
 // sector each, since every access to them is random.

@@ -321,13 +321,7 @@ void make_segs(Handle* h, uint32_t k) {
   } else {
     for (uint32_t i = 0; i < h->n; ++i) counts[substep_class(i, k)]++;
   }
-  uint64_t off = 0;
-  for (uint32_t c = 0; c < kMaxSubsteps; ++c)
-    for (int b = 0; b < kBins; ++b) {
-      h->segs.off[c * kBins + b] = uint32_t(off);
-      h->segs.cap[c * kBins + b] = c < k ? uint32_t(counts[c]) : 0u;
-      off += c < k ? counts[c] : 0;
-    }
+  layout_segs(h->segs, counts, k);
   h->segs_k = k;
 }
 
