@@ -435,7 +435,7 @@ int static_body(dfl_handle* h) {
   DFL_CUDA(h, cudaMemsetAsync(h->fbits[0], 0, sizeof(uint32_t) * h->words, h->stream));
   DFL_CUDA(h, cudaMemsetAsync(h->fbits[1], 0, sizeof(uint32_t) * h->words, h->stream));
   DFL_TRY(lists_all(h, h->n, h->deg, 0, h->opt.substeps));
-  return louvain(h, true, false, h->n);
+  return louvain(h, true, false, h->n, true);
 }
 
 }  // namespace
@@ -894,7 +894,7 @@ int group_static_body(dfl_handle* h) {
   DFL_CUDA(h, cudaMemsetAsync(h->fbits[0], 0, sizeof(uint32_t) * h->words, h->stream));
   DFL_CUDA(h, cudaMemsetAsync(h->fbits[1], 0, sizeof(uint32_t) * h->words, h->stream));
   DFL_TRY(lists_all(h, h->n, h->deg, 0, h->opt.substeps));
-  return louvain_group(h, true, false, h->n);
+  return louvain_group(h, true, false, h->n, true);
 }
 
 }  // namespace

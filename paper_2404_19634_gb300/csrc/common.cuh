@@ -87,6 +87,7 @@ struct Ctrl {
   unsigned int it_items[kMaxSubsteps];
   unsigned int bar_count, bar_gen;
   long long m2v;                     // 2m of the current local-moving call
+  unsigned int from_singletons;      // it starts with a community per vertex (MoveArgs)
   unsigned int npairs;               // distinct (u, v) pairs of the batch (hashed apply)
   unsigned int max_app;              // most new arcs of one rebuilt row
   unsigned long long extra_top;      // new arcs of rebuilt rows
@@ -791,6 +792,7 @@ struct MoveArgs {
   uint32_t max_deg;  // upper bound of the degrees of g
   bool use_range;
   bool track_ever;
+  bool from_singletons = false;  // every vertex starts in a community of its own
   bool prefer_host = false;  // launch from the host unless DFL_FLAG_GRAPH asks for replay
   // upper bound of the initial frontier's vertex count (DF: the pending
   // batch arcs); chooses launch shapes for a replayed first iteration
@@ -824,10 +826,11 @@ int count_communities(Handle* h, const uint32_t* Cp, uint32_t nv, uint32_t* ncom
 int renumber(Handle* h, uint32_t* Cp, uint32_t nv, bool first_level);
 int aggregate(Handle* h, const GraphView& g, const uint32_t* Cp, uint32_t ncomm, int dst,
               long long* Knew);
-int louvain(Handle* h, bool all, bool use_range, uint64_t initial);
+// (singletons: the first pass starts from a community per vertex)
+int louvain(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons = false);
 
 // group.cu
-int louvain_group(Handle* h, bool all, bool use_range, uint64_t initial);
+int louvain_group(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons = false);
 int group_m2(Handle* h);  // 2m of every graph from K (checks each < 2^32)
 // group_m2 without a wait: each graph's 2m from K into d_gm2 and into pinned
 // host memory (h_gS[0, G)), queued on the handle's stream; group_m2_take

@@ -1234,6 +1234,17 @@ __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
 // chunk up to 16,384) lose where hubs are few (temporal stream 254 -> 263 us).
 constexpr uint32_t kGiantSingle = 8192;  // a vertex of at most this degree is one chunk ...
 constexpr uint32_t kGiantChunk = 4096;   // ... a larger one has chunks of this many arcs
+// From singletons a hub's arcs meet as many communities as there are arcs, so a
+// chunk's time is its flushes into the vertex's table, and a class with few
+// chunks needs more of them to fill the GPU: chunks of kGiantFine arcs where there
+// would be fewer than kGiantFew of the others.  Static Louvain on R-MAT graphs
+// of 2^16, 2^18 and 2^19 vertices 2.68, 4.39 and 4.61 ms with chunks of 4,096,
+// now 2.32, 3.20 and 4.37; on 2^20 to 2^22 the same.  The line is flat from 24
+// to 76 chunks; at 12 the run on 2^18 vertices loses 11%, at 152 the one on 2^20
+// 1.4%.  Updates start from communities, where a hub's arcs meet few, and lose
+// with finer chunks (DF of 4,000 edges on 2^20 vertices 425 -> 442 us).
+constexpr uint32_t kGiantFine = 1024;
+constexpr uint32_t kGiantFew = 76;
 constexpr int kAccumThreads = 256;
 constexpr uint32_t kGiantRound = 8 * kAccumThreads;  // arcs in flight
 constexpr uint32_t kGiantSlots = 4096;               // shared chunk table: keys + values = 32 KB
@@ -1263,15 +1274,22 @@ struct GiantDecide {
   unsigned int* nbignd;       // vertices left to the part blocks (counted)
 };
 
-__device__ __forceinline__ uint32_t giant_deg(const DecideArgs& a, uint32_t t) {
-  const uint32_t v = a.list[t];
+__device__ __forceinline__ uint32_t giant_deg(const DecideArgs& a, const uint32_t* list, uint32_t t) {
+  const uint32_t v = list[t];
   uint32_t d = a.g.deg[v];
   if (d && a.ngraphs && a.gdone[graph_of(a.goff, a.ngraphs, v)]) d = 0;  // finished graph: skipped
   return d;
 }
 
-// Arcs per chunk of a vertex of degree d.
-__device__ __forceinline__ uint32_t giant_chunk_arcs(uint32_t d) { return d <= kGiantSingle ? kGiantSingle : kGiantChunk; }
+// Arcs per chunk of a vertex of degree d in a class of coarse or fine chunks.
+__device__ __forceinline__ uint32_t giant_chunk_arcs(uint32_t d, bool fine) {
+  return fine ? kGiantFine : d <= kGiantSingle ? kGiantSingle : kGiantChunk;
+}
+// The same from the vertex's number of chunks (of several chunks, 1,024 arcs
+// each and 4,096 each are never the same number).
+__device__ __forceinline__ uint32_t giant_chunk_arcs_of(uint32_t d, uint32_t nch) {
+  return nch == 1 ? kGiantSingle : nch == (d + kGiantChunk - 1) / kGiantChunk ? kGiantChunk : kGiantFine;
+}
 
 // Table of a vertex of degree d: a power of two >= 2d (at least 64 slots).
 __device__ __forceinline__ uint64_t giant_table_slots(uint32_t d) {
@@ -1283,22 +1301,33 @@ __device__ __forceinline__ uint64_t giant_table_slots(uint32_t d) {
 
 // One block: exclusive prefixes over the huge bin's list of chunks, table slots
 // and list capacities.
-__device__ __forceinline__ void giant_prefix_body(const DecideArgs& a, const GiantDecide& gd) {
+__device__ __forceinline__ void giant_prefix_body(const DecideArgs& a, const uint32_t* list, uint32_t cnt,
+                                                  const GiantDecide& gd) {
   __shared__ unsigned long long s_t[32], s_l[32];
   __shared__ uint32_t s_c[32];
   __shared__ unsigned long long s_tbase, s_lbase;
   __shared__ uint32_t s_cbase;
-  const uint32_t cnt = *a.count;
+  __shared__ unsigned long long s_arcs;
   const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
-    s_tbase = s_lbase = 0;
+    s_tbase = s_lbase = s_arcs = 0;
     s_cbase = 0;
   }
   __syncthreads();
+  const uint32_t d0 = threadIdx.x < cnt ? giant_deg(a, list, threadIdx.x) : 0u;
+  bool fine = a.ctrl->from_singletons != 0;
+  if (fine) {  // (the same in every thread) and if the class has few arcs
+    unsigned long long x = d0;
+    for (uint32_t t = threadIdx.x + blockDim.x; t < cnt; t += blockDim.x) x += giant_deg(a, list, t);
+    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
+    if (lane == 0 && x) atomicAdd(&s_arcs, x);
+    __syncthreads();
+    fine = s_arcs < uint64_t(kGiantFew) * kGiantChunk;
+  }
   for (uint32_t t0 = 0; t0 < cnt; t0 += blockDim.x) {
     const uint32_t t = t0 + threadIdx.x;
-    const uint32_t d = t < cnt ? giant_deg(a, t) : 0u;
-    const uint32_t ch = (d + giant_chunk_arcs(d) - 1) / giant_chunk_arcs(d);
+    const uint32_t d = t0 == 0 ? d0 : t < cnt ? giant_deg(a, list, t) : 0u;
+    const uint32_t size = giant_chunk_arcs(d, fine), ch = (d + size - 1) / size;
     const unsigned long long ts = giant_table_slots(d);
     unsigned long long xt = ts, xl = d;
     uint32_t xc = ch;
@@ -1372,9 +1401,8 @@ __global__ void __launch_bounds__(1024) k_giant_prefix(DecideArgs a, GiantDecide
                                                        const uint32_t* lists, int cur) {
   pdl_wait_only();
   const uint32_t s = blockIdx.x;
-  a.list = lists + a.seg.off[s * kBins + kBinHuge];
-  a.count = &a.ctrl->count[cur][s][kBinHuge];
-  giant_prefix_body(a, giant_class(gd, s, gstride, a.ctrl));
+  giant_prefix_body(a, lists + a.seg.off[s * kBins + kBinHuge], a.ctrl->count[cur][s][kBinHuge],
+                    giant_class(gd, s, gstride, a.ctrl));
 }
 
 // Entries [e0, e1) of vertex t's occupied list: read and clear them, keep the
@@ -1541,7 +1569,7 @@ __device__ __forceinline__ void giant_chunk(const DecideArgs& a, const GiantDeci
   if (a.rbits && !bit_test(a.rbits, i)) return;  // processed, not in the affected range
   const unsigned long long o = a.g.off[i];
   const uint32_t dg = a.g.deg[i];
-  const uint32_t size = giant_chunk_arcs(dg);
+  const uint32_t size = giant_chunk_arcs_of(dg, nch);
   const uint32_t k0 = chunk * size;
   const uint32_t k1 = min(dg, k0 + size);
   const uint32_t tmask = uint32_t(giant_table_slots(dg) - 1);
@@ -2068,8 +2096,8 @@ __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
   MoveSums sums;
   // 1. the largest-degree lists of every class: chunk, table and list layouts
   if (blockIdx.x < ia.k) {
-    const DecideArgs a3 = bin_args(ia, blockIdx.x, kBinHuge);
-    giant_prefix_body(a3, class_giant(ia, blockIdx.x));
+    giant_prefix_body(ia.a, ia.lists_cur + ia.a.seg.off[blockIdx.x * kBins + kBinHuge],
+                      ctrl->count[ia.cur][blockIdx.x][kBinHuge], class_giant(ia, blockIdx.x));
   }
   if (!grid_barrier(ctrl, ia.bar_extra, ia.bar_polls)) return;
   for (uint32_t s = 0; s < ia.k; ++s) {
@@ -2629,10 +2657,12 @@ __global__ void k_iter_start(Ctrl* ctrl, int nxt) {
   for (uint32_t q = threadIdx.x; q < sizeof(ctrl->count[0]) / sizeof(unsigned int); q += blockDim.x) c[q] = 0u;
 }
 
-// 2m of this local-moving call; with a batch apply enqueued just before (ap),
+// What a local-moving call sets in its control block: whether it starts from
+// singletons, its counters, and its 2m; with a batch apply enqueued just before (ap),
 // the batch's change of 2m if its gate opened
-__global__ void k_set_m2(Ctrl* ctrl, long long m2, const Ctrl* ap) {
+__global__ void k_set_m2(Ctrl* ctrl, long long m2, const Ctrl* ap, uint32_t from_singletons) {
   pdl_wait();
+  ctrl->from_singletons = from_singletons;
   ctrl->m2v = m2 + (ap && ap->apply_go ? ap->m2_delta : 0ll);
   ctrl->move_bytes = 0;  // this call's counters
   ctrl->ever_count = 0;
@@ -3174,7 +3204,7 @@ int prepare_move(Handle* h, const MoveArgs& ma, DecideArgs* out, GiantDecide* gd
   {
     LaunchScope ls(h, DFL_PROF_OTHER);
     launch_pdl(k_set_m2, 1, 1, 0, h->stream, h->ctrl, ma.m2,
-               h->papply.active ? h->actrl + h->papply.par : nullptr);
+               h->papply.active ? h->actrl + h->papply.par : nullptr, ma.from_singletons ? 1u : 0u);
     DFL_TRY(check_launch(h, "set m2"));
   }
   DecideArgs& a = *out;

@@ -192,3 +192,20 @@ def test_small_frontier_where_nearly_every_vertex_moves(dfl, orc, n, cycles, bin
     b.static()
     same(a, b)
     assert a.trace() == b.trace()
+
+
+@pytest.mark.parametrize("flags", [NO_GRAPH | SERIAL, PERSISTENT, 32])  # (32: graph replay)
+@pytest.mark.parametrize("degrees", [(4097, 5120, 5121), (8191, 8192, 8193), (12_289, 16_400), (4100,) * 75, (4100,) * 76,
+                                     (4150,) * 77])
+def test_hubs_of_a_run_from_singletons(dfl, orc, degrees, flags):  # noqa: F811
+    """Static runs over few hub arcs (chunks of 1,024) and over more than the
+    line between the chunk sizes, every class in one sub-step."""
+    g = stars(degrees, max(4200, max(degrees)), 17)
+    a, b = pair(dfl, orc, g, flags=flags, substeps=1, max_iterations=3)
+    a.static()
+    b.static()
+    same(a, b)
+    assert a.trace() == b.trace() and a.stats()["iterations"] == b.stats()["iterations"]
+    a.update(0)  # from communities: chunks of 4,096
+    b.update(0)
+    same(a, b)
