@@ -95,16 +95,27 @@ __global__ void k_fill_rows(uint32_t n, const unsigned long long* __restrict__ o
 // 32-bit parts.
 //
 // A chain of two or three dependent loads per row bounds it (offset ->
-// arcs -> communities), so a warp takes 32 rows: one load of their headers,
+// arcs -> communities), so a warp takes kPer rows: one load of their headers,
 // then four rows at a time with eight lanes each and four arcs a lane in
 // flight; rows longer than kRowShort take the whole warp, and those of more
-// than kRowHub arcs are queued for k_row_hubs, which spreads them over every
-// block.  One warp walking a hub's 100,000 arcs alone held the old kernels
+// than row_hub(kPer) arcs are queued for k_row_hubs, which spreads them over
+// every block.  One warp walking a hub's 100,000 arcs alone held the old kernels
 // up: K and 2m of the 2^22-vertex R-MAT graph (67 M arcs) took 541 us, now
 // 256 + 40; the modularity on 2^21 vertices (33 M arcs) 537 us, now 168 + 46.
 // Loading 16 rows' arcs at once instead of four was no faster (260 us; the
 // modularity 255): the rows' slack makes the pool twice the arcs' bytes.
-constexpr uint32_t kRowShort = 64, kRowHub = 1024, kRowPiece = 1024;
+// kPer is the smallest of 4 to 32 that leaves a warp at most four rounds, or one
+// round if every row is short (then a round is short too, and the headers are
+// what counts: 200,000 vertices of degree 12 take 30 us with 32 rows a warp and
+// 33 with 8).  With 32 always, and rows of up to 1,024 arcs kept, a graph of 10^4
+// to 10^5 vertices fills a tenth of the GPU with warps that take their long rows
+// one after another, dozens of them where hubs have neighbouring ids: the
+// modularity call on temporal streams of 10,000, 60,000, 200,000 and 800,000
+// vertices took 53, 79, 105 and 252 us, now 30, 32, 45 and 175.  A warp per row took 28, 41,
+// 53 and 239 there, and 1,105 us on the 2^22-vertex R-MAT graph (now 425).
+constexpr uint32_t kRowShort = 64;
+constexpr uint32_t kRowWarps = 38912, kRowWarpsEven = 9728;  // 152 SMs x 64 warps, times four rounds or one
+constexpr __host__ __device__ uint32_t row_hub(uint32_t per) { return per == 4 ? 128u : per == 32 ? 512u : 256u; }
 constexpr int kRowThreads = 256;
 
 template <bool kInside>
@@ -114,8 +125,9 @@ struct RowSums {
   const long long* Sigma;
   long long* K;
   uint32_t v0, v1;
-  uint2* hubs;  // queue of the rows longer than kRowHub (ctrl->long_rows)
+  uint2* hubs;  // queue of the rows longer than `hub` (ctrl->long_rows)
   Ctrl* ctrl;
+  uint32_t hub;  // the longest row a warp keeps, and the arcs of a queued row's piece
 
   // arcs [k0, k1) of row i, lanes striding by `step` from k0 + first: the weight
   // this lane meets
@@ -149,24 +161,24 @@ __device__ __forceinline__ unsigned long long lanes_sum(unsigned long long x, in
   return x;
 }
 
-template <bool kInside>
+template <bool kInside, uint32_t kPer>
 __global__ void __launch_bounds__(kRowThreads) k_row_sums(RowSums<kInside> r) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t warp = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) >> 5;
   const uint64_t nwarps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
   unsigned long long tot = 0;
-  for (uint64_t b = r.v0 + warp * 32; b < r.v1; b += nwarps * 32) {
+  for (uint64_t b = r.v0 + warp * kPer; b < r.v1; b += nwarps * kPer) {
     const uint64_t i = b + lane;
-    const bool ok = i < r.v1;
+    const bool ok = lane < kPer && i < r.v1;
     const unsigned long long o = ok ? r.g.off[i] : 0ull;
     uint32_t d = ok ? r.g.deg[i] : 0u;
     const uint32_t ci = kInside && ok ? r.C[i] : 0u;
-    if (d > kRowHub) {
-      push_row(r.hubs, &r.ctrl->long_rows, uint32_t(i), (d + kRowPiece - 1) / kRowPiece);
+    if (d > row_hub(kPer)) {
+      push_row(r.hubs, &r.ctrl->long_rows, uint32_t(i), (d + row_hub(kPer) - 1) / row_hub(kPer));
       d = 0;
     }
     unsigned long long mine = 0;  // row b + lane
-    for (uint32_t s = 0; s < 8; ++s) {
+    for (uint32_t s = 0; s < kPer / 4; ++s) {
       const int src = int(s * 4 + (lane >> 3));
       const unsigned long long os = __shfl_sync(0xFFFFFFFFu, o, src);
       const uint32_t ds = __shfl_sync(0xFFFFFFFFu, d, src), cs = __shfl_sync(0xFFFFFFFFu, ci, src);
@@ -216,7 +228,7 @@ __global__ void __launch_bounds__(kRowThreads) k_row_sums(RowSums<kInside> r) {
   }
 }
 
-// The queued rows, a warp per piece of kRowPiece arcs.
+// The queued rows, a warp per piece of `hub` arcs.
 template <bool kInside>
 __global__ void __launch_bounds__(kRowThreads) k_row_hubs(RowSums<kInside> r) {
   pdl_wait_only();
@@ -226,8 +238,8 @@ __global__ void __launch_bounds__(kRowThreads) k_row_hubs(RowSums<kInside> r) {
   unsigned long long tot = 0;
   for (uint64_t p = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5); p < pieces; p += nwarps) {
     const uint2 e = r.hubs[find_row(r.hubs, rows, uint32_t(p))];
-    const uint32_t k0 = (uint32_t(p) - e.y) * kRowPiece, d = r.g.deg[e.x];
-    const uint32_t k1 = d - k0 < kRowPiece ? d : k0 + kRowPiece;
+    const uint32_t k0 = (uint32_t(p) - e.y) * r.hub, d = r.g.deg[e.x];
+    const uint32_t k1 = d - k0 < r.hub ? d : k0 + r.hub;
     unsigned long long sum = r.part(r.g.off[e.x], kInside ? r.C[e.x] : 0u, k0, k1, lane, 32);
     tot += sum;
     if constexpr (!kInside) {
@@ -239,19 +251,33 @@ __global__ void __launch_bounds__(kRowThreads) k_row_hubs(RowSums<kInside> r) {
   if (lane == 0 && tot) atomicAdd(&r.ctrl->red_a, tot);
 }
 
+template <bool kInside, uint32_t kPer>
+void launch_row_sums(Handle* h, const RowSums<kInside>& r) {
+  k_row_sums<kInside, kPer><<<grid_for(r.v1 - r.v0, kRowThreads / 32 * kPer, 152 * 8), kRowThreads, 0, h->stream>>>(r);
+}
+
 template <bool kInside>
-int row_sums(Handle* h, const RowSums<kInside>& r) {
+int row_sums(Handle* h, RowSums<kInside> r) {
   // red_a, red_b, red_c and long_rows are adjacent
   DFL_CUDA(h, cudaMemsetAsync(&h->ctrl->red_a, 0, 4 * sizeof(unsigned long long), h->stream));
   if (r.v1 <= r.v0) return DFL_OK;
+  const uint64_t rows = r.v1 - r.v0;
+  const uint64_t warps = h->max_deg <= kRowShort ? kRowWarpsEven : kRowWarps;
+  uint32_t per = 4;
+  while (per < 32 && rows > warps * per) per *= 2;
+  r.hub = row_hub(per);
   {
     LaunchScope ls(h, DFL_PROF_OTHER);
-    k_row_sums<kInside><<<grid_for(r.v1 - r.v0, kRowThreads, 152 * 8), kRowThreads, 0, h->stream>>>(r);
+    if (per == 4) launch_row_sums<kInside, 4>(h, r);
+    else if (per == 8) launch_row_sums<kInside, 8>(h, r);
+    else if (per == 16) launch_row_sums<kInside, 16>(h, r);
+    else launch_row_sums<kInside, 32>(h, r);
     DFL_TRY(check_launch(h, "row sums"));
   }
-  if (h->max_deg <= kRowHub) return DFL_OK;  // (an upper bound: no row can have been queued)
+  if (h->max_deg <= r.hub) return DFL_OK;  // (an upper bound: no row can have been queued)
   LaunchScope ls(h, DFL_PROF_OTHER);
-  launch_pdl(k_row_hubs<kInside>, 152 * 6, kRowThreads, 0, h->stream, r);
+  launch_pdl(k_row_hubs<kInside>, grid_for(pool_top_bound(h) / r.hub, kRowThreads / 32, 152 * 6), kRowThreads, 0,
+             h->stream, r);
   return check_launch(h, "row sums of hubs");
 }
 
@@ -344,14 +370,14 @@ int recompute_aux(Handle* h) {
 }
 
 int weighted_degrees(Handle* h) {
-  DFL_TRY(row_sums(h, RowSums<false>{base_view(h), nullptr, nullptr, h->K, 0u, h->n, row_queue(h), h->ctrl}));
+  DFL_TRY(row_sums(h, RowSums<false>{base_view(h), nullptr, nullptr, h->K, 0u, h->n, row_queue(h), h->ctrl, 0u}));
   DFL_TRY(read_ctrl(h));
   h->m2 = (long long)h->hctrl->red_a;
   return DFL_OK;
 }
 
 int modularity_range(Handle* h, uint32_t v0, uint32_t v1, long long m2, i128* num, i128* den) {
-  DFL_TRY(row_sums(h, RowSums<true>{base_view(h), h->C, h->Sigma, nullptr, v0, v1, row_queue(h), h->ctrl}));
+  DFL_TRY(row_sums(h, RowSums<true>{base_view(h), h->C, h->Sigma, nullptr, v0, v1, row_queue(h), h->ctrl, 0u}));
   DFL_TRY(read_ctrl(h));
   const i128 sig = (i128)h->hctrl->red_a;
   const i128 sq = ((i128)h->hctrl->red_c << 32) + (i128)h->hctrl->red_b;

@@ -209,3 +209,24 @@ def test_hubs_of_a_run_from_singletons(dfl, orc, degrees, flags):  # noqa: F811
     a.update(0)  # from communities: chunks of 4,096
     b.update(0)
     same(a, b)
+
+
+@pytest.mark.parametrize("n,degrees", [
+    (3000, (64, 65, 128, 129, 2900)),            # four rows a warp
+    (155_648, (127, 128, 129, 257)), (155_649, (255, 256, 257, 1000)),  # ... eight
+    (311_297, (256, 257, 700)),                  # ... sixteen
+    (622_592, (256, 257, 513)), (622_593, (511, 512, 513, 40_000)),     # ... thirty-two
+])
+def test_row_sums_at_the_lines_between_their_forms(dfl, orc, n, degrees):  # noqa: F811
+    """K, 2m and the modularity where a warp takes more rows, with rows at the
+    lengths that are queued, side by side at the first ids."""
+    c = len(degrees)
+    hubs = stars(degrees, n - c, 5)
+    rng = np.random.default_rng(n)
+    keep = (np.arange(hubs.u.size) < sum(degrees)) | (rng.random(hubs.u.size) < 0.5)  # half of the leaves' ring
+    g = synth.EdgeList(n, hubs.u[keep], hubs.v[keep], hubs.w[keep])
+    a, b = pair(dfl, orc, g)
+    C = rng.integers(0, 40, n).astype(np.uint32)
+    a.set_membership(C)
+    b.set_membership(C)
+    same(a, b)
