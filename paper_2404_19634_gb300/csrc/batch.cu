@@ -29,7 +29,6 @@ namespace {
 // tombstone).  A row is rebuilt (sorted, tombstones dropped, relocated) when
 // it would outgrow its capacity, its tail or its tombstone budget.
 constexpr uint32_t kTailMax = 64;
-constexpr uint32_t kTombMin = 8;
 
 // b_flag bits
 constexpr uint32_t kRunHead = 1u;     // first arc of a (u, v) run
@@ -1424,6 +1423,7 @@ int enqueue_hashed(Handle* h, const dfl_edge* del, const dfl_edge* ins, uint64_t
   h->papply.par = par;
   h->papply.small = small;
   h->papply.na = na;
+  h->papply.nd = 2 * nd;
   h->papply.rc = DFL_OK;
   return DFL_OK;
 }
@@ -1476,6 +1476,7 @@ int settle_apply(Handle* h) {
     h->m2 += c.m2_delta;
     h->pool_top += c.reloc_need;
     h->num_arcs = uint64_t((long long)h->num_arcs + c.arc_delta);
+    h->tombs += h->papply.nd;
     if (c.max_deg > h->max_deg) h->max_deg = c.max_deg;
     if (c.err) rc = set_error(h, DFL_ERR_CUDA, "internal error in batch apply");
     h->papply.rc = rc;
@@ -1516,6 +1517,8 @@ int settle_apply(Handle* h) {
 uint64_t live_arcs_bound(const Handle* h) {
   return h->num_arcs + (h->papply.active ? h->papply.na : 0);
 }
+
+uint64_t tombs_bound(const Handle* h) { return h->tombs + (h->papply.active ? h->papply.nd : 0); }
 
 uint64_t pool_top_bound(const Handle* h) { return h->papply.active ? h->pool_cap : h->pool_top; }
 
@@ -1710,6 +1713,7 @@ int apply_batch_sorted(Handle* h, const dfl_edge* del, uint64_t nd, const dfl_ed
   h->m2 += c.m2_delta;
   h->pool_top += c.reloc_need;
   h->num_arcs = uint64_t((long long)h->num_arcs + c.arc_delta);
+  h->tombs += 2 * nd;
   if (c.max_deg > h->max_deg) h->max_deg = c.max_deg;
   return DFL_OK;
 }

@@ -170,6 +170,7 @@ struct Handle {
   uint64_t pool_cap = 0;   // arc slots allocated
   uint64_t pool_top = 0;   // first free slot (host mirror)
   uint64_t num_arcs = 0;   // arcs in use
+  uint64_t tombs = 0;      // upper bound of the tombstones: arcs deleted since the pool was written densely
   uint32_t max_deg = 0;    // upper bound of the degrees of G^t
 
   // community state
@@ -302,6 +303,7 @@ struct Handle {
     bool small = false;  // the single-block path
     int par = 0;         // its control block: actrl[par]
     uint64_t na = 0;     // arcs of the batch (2 per edge)
+    uint64_t nd = 0;     // ... of its deletions
     int rc = 0;          // how it settled: DFL_OK, a DFL_ERR code or kApplyRetry*
   } papply;
   bool ever_clear = false;  // DF marking cleared `ever` for the update that follows
@@ -358,6 +360,21 @@ struct Handle {
   uint64_t gb_cap = 0;
   uint64_t* d_eoff = nullptr;          // per graph edge offsets of a group batch (2 x (ngraphs + 1))
 };
+
+// ---------------------------------------------------------------------------
+// Rows with tombstones
+// ---------------------------------------------------------------------------
+// A row of d slots keeps at most max(kTombMin, d / 4) tombstones (batch.cu).
+constexpr uint32_t kTombMin = 8;
+
+// Upper bound of the slots in use (live arcs and tombstones), over the rows of
+// more than `lim` slots, of a graph of `live` arcs and at most `tombs`
+// tombstones.  What is sized for the rows' degrees is sized by it: the degrees
+// count the tombstones too, which from 32 slots on are at most a third of the
+// row's live arcs.
+inline uint64_t slots_bound(uint64_t live, uint64_t tombs, uint32_t lim) {
+  return live + (lim >= 4 * kTombMin && live / 3 < tombs ? live / 3 : tombs);
+}
 
 // ---------------------------------------------------------------------------
 // Error handling
@@ -771,9 +788,11 @@ int apply_batch_begin(Handle* h, const dfl_edge* del, uint64_t nd, const dfl_edg
 // error or the retry is returned.
 int copy_apply_ctrl(Handle* h);
 int settle_apply(Handle* h);
-// Upper bounds of the live arc count, the pool top and the largest degree
-// while an enqueued apply has not settled (the exact values once it has).
+// Upper bounds of the live arc count, the tombstones, the pool top and the
+// largest degree while an enqueued apply has not settled (the handle's own
+// values once it has).
 uint64_t live_arcs_bound(const Handle* h);
+uint64_t tombs_bound(const Handle* h);
 uint64_t pool_top_bound(const Handle* h);
 uint32_t max_deg_bound(const Handle* h);
 int apply_batch(Handle* h, const dfl_edge* del, uint64_t nd, const dfl_edge* ins, uint64_t ni,

@@ -490,6 +490,7 @@ int compact_pool(Handle* h, uint64_t* before, uint64_t* after) {
   h->arcs = pool;
   h->pool_cap = cap;
   h->pool_top = total;
+  h->tombs = 0;
   if (after) *after = h->pool_cap;
   return DFL_OK;
 }

@@ -3123,11 +3123,12 @@ int prepare_move(Handle* h, const MoveArgs& ma, DecideArgs* out, GiantDecide* gd
 
   });
   DFL_CUDA(h, smem_rc);
-  // the huge bin's buffers, sized by bounds: at most arcs / (bin_block + 1) listed
-  // vertices; tables of at most 4 x degree (>= 64) slots each; occupied
-  // lists of at most degree entries; at most arcs / kGiantPart + items parts
+  // the huge bin's buffers, sized by bounds (arcs: of the listed vertices'
+  // degrees): at most arcs / (bin_block + 1) listed vertices; tables of at most
+  // 4 x degree (>= 64) slots each; occupied lists of at most degree entries; at
+  // most arcs / kGiantPart + items parts
   {
-    uint64_t arcs = live_arcs_bound(h);
+    uint64_t arcs = slots_bound(live_arcs_bound(h), tombs_bound(h), h->tune.bin_block);
     for (int q = 0; q < 2; ++q) arcs = arcs > h->sg[q].arc_cap ? arcs : h->sg[q].arc_cap;
     // (one region per sub-step class: the persistent kernel lays out all
     // classes at the start of an iteration)

@@ -46,3 +46,23 @@ def test_frontier_segments_do_not_overlap(tmp_path, n, k):
             assert off[s * bins + b] == at and cap[s * bins + b] == counts[s]
             at += counts[s]
     assert at == bins * n  # what the list buffers hold
+
+
+@pytest.mark.parametrize("lim,rows", [
+    (4096, [(4097, 1024)] * 4098),                       # every row as full of tombstones as a row can be
+    (4096, [(4097, 0), (9000, 2250), (131_073, 7)]),
+    (32, [(33, 8), (40, 10), (35, 8)] * 50),
+    (31, [(32, 8), (33, 8)] * 9),
+    (0, [(9, 8), (1, 1), (8, 8), (30, 8)] * 20),         # short rows: tombstones alone, or nearly
+])
+def test_slots_bound_covers_tombstones(tmp_path, lim, rows):
+    """Buffers sized for the degrees (slots in use) of the rows above a limit
+    hold them when the rows carry tombstones, which the live arcs leave out."""
+    assert all(d > lim and t <= max(8, d // 4) for d, t in rows)
+    slots, tombs = sum(d for d, _ in rows), sum(t for _, t in rows)
+    exact, loose = run_host(tmp_path, """
+  std::printf("%%" PRIu64 " %%" PRIu64 "\\n", slots_bound(%dull, %dull, %du), slots_bound(%dull, %dull, %du));
+""" % (slots - tombs, tombs, lim, slots - tombs, tombs * 1000, lim))
+    assert exact >= slots  # the tombstones are known exactly ...
+    if lim >= 32:          # ... or only by a bound far above them
+        assert slots <= loose <= slots * 4 // 3
