@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(256) k_agg_warp(AggArgs a) {
 // dynamic shared memory (kSlots >= 2 x total degree).
 template <uint32_t kSlots>
 __global__ void __launch_bounds__(kAggThreads) k_agg_block(AggArgs a) {
-  extern __shared__ uint32_t dyn[];
+  extern __shared__ __align__(16) uint32_t dyn[];
   __shared__ FlatTile ft;
   __shared__ unsigned int s_pos;
   __shared__ unsigned long long s_sum;
@@ -617,7 +617,7 @@ __device__ __forceinline__ bool giant_arcs(const AggArgs& a, GiantTable& t, cons
 // run of items and flushes its table when the giant changes.  The units of
 // rows of more than kAggBigMember arcs are noted for k_agg_big.
 __global__ void __launch_bounds__(kAggThreads) k_agg_giant_accum(AggArgs a, GiantArgs gi) {
-  extern __shared__ uint32_t dyn[];
+  extern __shared__ __align__(16) uint32_t dyn[];
   GiantTable& t = *reinterpret_cast<GiantTable*>(dyn);
   __shared__ FlatTile ft;
   const uint32_t i0 = uint32_t(uint64_t(gi.nitems) * blockIdx.x / gridDim.x);
@@ -649,7 +649,7 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_giant_accum(AggArgs a, Gian
 // of their arcs (a run of units, which may begin and end inside a row), work
 // item by work item.
 __global__ void __launch_bounds__(kAggThreads) k_agg_big(AggArgs a, GiantArgs gi) {
-  extern __shared__ uint32_t dyn[];
+  extern __shared__ __align__(16) uint32_t dyn[];
   GiantTable& t = *reinterpret_cast<GiantTable*>(dyn);
   __shared__ FlatTile ft;
   const uint32_t units = gi.units[uint64_t(gi.nitems) * kAggThreads];

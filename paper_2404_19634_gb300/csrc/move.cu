@@ -1079,7 +1079,7 @@ __device__ __noinline__ void block_vertex_slow(const DecideArgs& a, const VHdr& 
 
 template <int kThreads, uint32_t kSlots>
 __global__ void __launch_bounds__(kThreads) k_decide_block(DecideArgs a) {
-  extern __shared__ uint32_t dyn[];
+  extern __shared__ __align__(16) uint32_t dyn[];
   uint32_t* keys = dyn;
   uint32_t* vals = dyn + kSlots;
   __shared__ BlockScratch sc;  // the 128-bit path's
@@ -2086,7 +2086,7 @@ static_assert(kIterDynWords >= 2 * kBlockSlots && 8 * 2 * kWarpSlots <= 2 * kBlo
 // two blocks per SM: 128 registers a thread (three blocks, at 80 registers,
 // spilled and measured slower)
 __global__ void __launch_bounds__(kIterThreads, 2) k_iterate(IterArgs ia) {
-  extern __shared__ uint32_t dyn[];
+  extern __shared__ __align__(16) uint32_t dyn[];
   __shared__ BlockScratch sc;
   __shared__ uint32_t s_unit;
   Ctrl* ctrl = ia.a.ctrl;
@@ -2402,6 +2402,7 @@ constexpr uint32_t kSmallClass = 12000;
 static_assert(kSmallClass / kSmallCtas + 8 * kSmallThreads / 32 + kSmallThreads / 32 + 8 <= kSmallMoves,
               "a CTA's moves fit");
 constexpr size_t kSmallSmemAll = kSmallSmem + sizeof(SmallMove) * kSmallMoves;
+static_assert(alignof(SmallMove) <= 16 && kSmallSmem % alignof(SmallMove) == 0, "the moves are aligned behind the tables");
 
 __device__ __forceinline__ void small_record(const DecideArgs& a, const Move& m, uint32_t gi, SmallMove* moves,
                                              uint32_t* count, unsigned long long* nbig, MoveSums& sums) {
@@ -2421,7 +2422,7 @@ __device__ __forceinline__ void small_record(const DecideArgs& a, const Move& m,
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small_move(const __grid_constant__ SmallArgs q) {
   pdl_wait_only();
   // the warps' tables (empty at rest) and a block table, or the cluster's table; then the moves
-  extern __shared__ uint32_t dyn[];
+  extern __shared__ __align__(16) uint32_t dyn[];
   __shared__ SmallParts sp;
   __shared__ BlockScratch sc;
   __shared__ uint32_t s_n[kMaxSubsteps][kBins];
