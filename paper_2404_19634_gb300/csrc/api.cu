@@ -466,7 +466,7 @@ int dfl_update(dfl_handle* h, int mode) {
   int rc = DFL_OK;
   if (h->opt.flags & DFL_FLAG_RECOMPUTE_AUX) rc = recompute_aux(h);
   if (!rc) rc = mark(h, mode, &all, &use_range, &initial);
-  if (!rc) rc = louvain(h, all, use_range, initial);
+  if (!rc) rc = louvain(h, all, use_range, initial, false, mode == DFL_DS);
   h->pend_count = 0;
   return louvain_result(h, rc);
 }
@@ -969,7 +969,7 @@ int dfl_group_update(dfl_handle* h, int mode) {
   int rc = group_set_level(h, h->d_goff0);  // classes of the base graphs' vertices
   if (!rc && (h->opt.flags & DFL_FLAG_RECOMPUTE_AUX)) rc = recompute_aux(h);
   if (!rc) rc = mark(h, mode, &all, &use_range, &initial);
-  if (!rc) rc = louvain_group(h, all, use_range, initial);
+  if (!rc) rc = louvain_group(h, all, use_range, initial, false, mode == DFL_DS);
   h->pend_count = 0;
   return louvain_result(h, rc);
 }

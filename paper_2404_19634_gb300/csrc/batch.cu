@@ -1815,9 +1815,13 @@ int mark(Handle* h, int mode, bool* all, bool* use_range, uint64_t* initial) {
                               cudaMemcpyDeviceToDevice, h->stream));
   DFL_TRY(lists_from_bits(h, h->dsV, n, h->deg, 0, k));
   *use_range = true;
-  int rc = DFL_OK;
-  *initial = popcount_bits(h, h->dsV, h->words, &rc);
-  return rc;
+  // the marked vertices are those on the lists, whose lengths local-moving then
+  // finds on the host (MoveArgs::counted)
+  DFL_TRY(read_ctrl(h));
+  *initial = 0;
+  for (uint32_t s = 0; s < k; ++s)
+    for (int b = 0; b < kBins; ++b) *initial += h->hctrl->count[0][s][b];
+  return DFL_OK;
 }
 
 }  // namespace dfl

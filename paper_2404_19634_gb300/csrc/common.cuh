@@ -816,6 +816,10 @@ struct MoveArgs {
   // upper bound of the initial frontier's vertex count (DF: the pending
   // batch arcs); chooses launch shapes for a replayed first iteration
   uint64_t frontier_hint = ~0ull;
+  // the host mirror of the control block already holds the initial frontier's
+  // list lengths (DS: mark() counted them), so that neither a read nor a blind
+  // try of the small-frontier kernel is needed to learn them
+  bool counted = false;
 };
 // A list of a sub-step class shorter than this is decided with several lanes
 // per vertex (W lanes in the tiny bin, a warp in the lane bin) instead of a lane
@@ -845,11 +849,13 @@ int count_communities(Handle* h, const uint32_t* Cp, uint32_t nv, uint32_t* ncom
 int renumber(Handle* h, uint32_t* Cp, uint32_t nv, bool first_level);
 int aggregate(Handle* h, const GraphView& g, const uint32_t* Cp, uint32_t ncomm, int dst,
               long long* Knew);
-// (singletons: the first pass starts from a community per vertex)
-int louvain(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons = false);
+// (singletons: the first pass starts from a community per vertex; counted:
+// MoveArgs::counted of the first pass, true after a DS mark())
+int louvain(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons = false, bool counted = false);
 
 // group.cu
-int louvain_group(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons = false);
+int louvain_group(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons = false,
+                  bool counted = false);
 int group_m2(Handle* h);  // 2m of every graph from K (checks each < 2^32)
 // group_m2 without a wait: each graph's 2m from K into d_gm2 and into pinned
 // host memory (h_gS[0, G)), queued on the handle's stream; group_m2_take

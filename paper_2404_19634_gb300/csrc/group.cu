@@ -169,7 +169,7 @@ int group_modularity(Handle* h, uint32_t g, i128* num, i128* den) {
   return modularity_range(h, h->goff0[g], h->goff0[g + 1], h->gm2[g], num, den);
 }
 
-int louvain_group(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons) {
+int louvain_group(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons, bool counted) {
   const uint32_t n = h->n, G = h->ngraphs;
   h->trace.clear();
   dfl_stats_t& st = h->stats;
@@ -233,6 +233,7 @@ int louvain_group(Handle* h, bool all, bool use_range, uint64_t initial, bool si
     a.prefer_host = true;
     a.graph_iters = git.data();
     a.frontier_hint = (pass == 0 && !all && !use_range) ? h->pend_count : nv;
+    a.counted = counted && pass == 0;
     a.from_singletons = singletons || pass > 0;
     uint32_t it = 0;
     uint64_t init0 = 0, ever0 = 0;

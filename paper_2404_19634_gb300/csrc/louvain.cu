@@ -74,7 +74,7 @@ int renumber(Handle* h, uint32_t* Cp, uint32_t nv, bool first_level) {
   return check_launch(h, "lookup");
 }
 
-int louvain(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons) {
+int louvain(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons, bool counted) {
   const uint32_t n = h->n;
   h->trace.clear();
   dfl_stats_t& st = h->stats;
@@ -119,6 +119,7 @@ int louvain(Handle* h, bool all, bool use_range, uint64_t initial, bool singleto
     // DF marks at most one vertex per pending batch arc; ND, DS and later
     // passes may mark every vertex
     a.frontier_hint = (pass == 0 && !all && !use_range) ? pend : nv;
+    a.counted = counted && pass == 0;
     a.from_singletons = singletons || pass > 0;
     uint32_t it = 0;
     uint64_t init0 = 0, ever0 = 0;

@@ -2885,7 +2885,8 @@ bool small_frontier(const unsigned int (*n)[kBins]) {
 
 // A frontier of at most this many vertices is tried without reading its
 // lengths first: the kernel checks them itself, and a refusal costs its empty
-// launch (the read it comes back with is needed either way).
+// launch (the read it comes back with is needed either way; 12 us on a skewed
+// graph of 2^14 vertices, whose DS updates know the lengths instead).
 constexpr uint64_t kSmallTry = 16384;
 
 // Whether the GPU can hold the small-frontier kernel's cluster; queried once per process.
@@ -3282,9 +3283,9 @@ int local_move(Handle* h, const MoveArgs& ma, uint32_t pass, uint32_t* iteration
   unsigned int cur_count[kMaxSubsteps][kBins];
   unsigned long long skipped = 0;
   // a frontier that can only be small needs no read of its lengths first
-  bool small_next = can_small && !use_graph && ma.frontier_hint <= kSmallTry;
+  bool small_next = can_small && !use_graph && !ma.counted && ma.frontier_hint <= kSmallTry;
   if (!use_graph && !use_persistent && !small_next) {
-    DFL_TRY(read_move_ctrl(h, &settled));  // list lengths of the initial frontier (buffer 0)
+    if (!ma.counted) DFL_TRY(read_move_ctrl(h, &settled));  // list lengths of the initial frontier (buffer 0)
     if (settled && !G) {
       threshold = tolerance_threshold(h->opt, h->m2, pass);
       mv.m2 = h->m2;  // the batch's 2m, for the decide kernels

@@ -230,3 +230,25 @@ def test_row_sums_at_the_lines_between_their_forms(dfl, orc, n, degrees):  # noq
     a.set_membership(C)
     b.set_membership(C)
     same(a, b)
+
+
+@pytest.mark.parametrize("flags", [0, NO_GRAPH, PERSISTENT, 32])
+@pytest.mark.parametrize("degrees,leaves", [((30, 5), 600), ((3000, 700, 300) * 20, 3000), ((5000, 4200) * 6, 9000)])
+def test_delta_screening_frontier_counted_on_the_host(dfl, orc, degrees, leaves, flags):  # noqa: F811
+    """DS updates whose frontier is small, refused by the small-frontier kernel,
+    or replayed: the marked vertices' count and the whole run, also after a
+    marking that no update followed."""
+    g = stars(degrees, leaves, 11)
+    a, b = pair(dfl, orc, g, flags=flags)
+    a.static()
+    b.static()
+    stream = synth.BatchStream(g, 5)
+    for size in (8, 900, 40):
+        dels, ins = stream.next(size, w_max=9)
+        assert a.apply_batch(dels, ins) == 0 and b.apply_batch(dels, ins) == 0
+        for x, y in zip(a.mark(1), b.mark(1)):
+            assert np.array_equal(x, y)
+        a.update(1)
+        b.update(1)
+        same(a, b)
+        assert a.stats()["affected_initial"] == b.stats()["affected_initial"] and a.trace() == b.trace()
