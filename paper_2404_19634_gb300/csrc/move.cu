@@ -2793,7 +2793,11 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
         // a warp per vertex, headers in batches of up to 32 (fewer when the list is short)
         k_decide_warp_hash<<<counts ? grid_for(uint64_t(c) * 32, 256, 152 * 6) : 152 * 3, 256, 0, st>>>(a);
       } else if (b == kBinMid) {
-        k_decide_block<128, 2 * kMidDeg><<<counts ? grid_for(c, 1, 152 * 8) : 152 * 8, 128, sizeof(uint32_t) * 4 * kMidDeg, st>>>(a);
+        // (a replayed graph launches every bin at once: with all eight blocks an SM
+        // this one keeps the lane bin's blocks, of the lowest priority too, waiting;
+        // ND on 2^18 vertices 324 us so, 300 with four, 2^20 and 2^22 the same)
+        k_decide_block<128, 2 * kMidDeg>
+            <<<counts ? grid_for(c, 1, 152 * 8) : 152 * 4, 128, sizeof(uint32_t) * 4 * kMidDeg, st>>>(a);
       } else if (b == kBinWhole) {
         const size_t smem = sizeof(uint32_t) * 2 * kBlockSlots;
         const uint32_t bt = h->tune.block_threads;
