@@ -103,7 +103,8 @@ def parse():
                    help="measure DF on the temporal stream (sliding-window batches)")
     p.add_argument("--launch", default="auto", choices=["auto", "host", "graph", "persistent"],
                    help="how a local-moving iteration is launched: the library's choice (default: "
-                        "graph replay, host launches for updates below 256 batch edges), kernels "
+                        "graph replay, host launches for updates below 256 batch edges, one "
+                        "cluster launch for iterations of a small frontier), kernels "
                         "from the host (DFL_FLAG_NO_GRAPH), always a replayed CUDA graph "
                         "(DFL_FLAG_GRAPH) or one cooperative kernel (DFL_FLAG_PERSISTENT)")
     p.add_argument("--no-extras", action="store_true",
@@ -113,8 +114,9 @@ def parse():
     return p.parse_args()
 
 
-LAUNCH_DESC = {"auto": "per-bin kernels, graph replay (host launches below 256 batch edges)",
-               "host": "per-bin kernels launched from the host", "graph": "per-bin kernels, graph replay",
+LAUNCH_DESC = {"auto": "per-bin kernels, graph replay (host launches below 256 batch edges), a cluster launch for small frontiers",
+               "host": "per-bin kernels launched from the host, a cluster launch for small frontiers",
+               "graph": "per-bin kernels, graph replay",
                "persistent": "one cooperative kernel per iteration"}
 
 
@@ -488,7 +490,7 @@ def roofline_record(mv: dict, steps: int, peak: float, peak_kind: str, traffic_o
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": cold,
             "kernel": "local-move decide phase (one sub-step: the concurrent decide kernels of its "
-                      "four degree bins)",
+                      "six degree bins)",
             "timing": f"CUDA events around each decide phase, in {steps} further DF steps of the "
                       "same size (the timed steps carry no profiling events)",
             "peak_kind": peak_kind, "bytes_per_launch": bytes_launch, "ms_per_launch": ms_launch,

@@ -87,11 +87,16 @@ enum {
 
 /* Option flags. */
 enum {
-  DFL_FLAG_PROFILE = 1u, /* time every kernel class with CUDA events (dfl_profile) */
+  DFL_FLAG_PROFILE = 1u, /* time every kernel class with CUDA events (dfl_profile).  The
+                            small-frontier launch (see DFL_FLAG_GRAPH) has no such classes, so
+                            with this flag its iterations run in the per-bin kernels: a small
+                            call's profile shows those, not the launch it uses otherwise */
   DFL_FLAG_TRACE = 2u,   /* reserved */
-  DFL_FLAG_NO_GRAPH = 4u, /* launch every kernel from the host (overrides DFL_FLAG_GRAPH) */
+  DFL_FLAG_NO_GRAPH = 4u, /* no graph replay (overrides DFL_FLAG_GRAPH): iterations are launched
+                             from the host, those of a small frontier still in one launch */
   DFL_FLAG_SERIAL_BINS = 8u, /* run the degree bins of a sub-step one after another on the handle's
-                                stream instead of concurrently (for measuring each bin alone) */
+                                stream instead of concurrently (for measuring each bin alone; the
+                                small-frontier launch is not used) */
   DFL_FLAG_PERSISTENT = 16u,  /* run each local-moving iteration as one cooperative launch whose
                                  blocks meet at bounded grid barriers between sub-steps; a barrier
                                  that waits about a second gives up and the call returns
@@ -105,12 +110,14 @@ enum {
                                  is used except for group handles and for DF/DS updates of fewer
                                  than 256 batch edges, which launch from the host with the list
                                  lengths read (empty bins skipped, grids fit to the work).
-                                 Unless this flag forces replay, iterations whose frontier is
-                                 small (a few thousand vertices) run one after another in a
-                                 single launch of one thread-block cluster (same results) */
+                                 Unless this flag forces replay, or DFL_FLAG_PERSISTENT,
+                                 DFL_FLAG_SERIAL_BINS or one of the profiling flags asks for
+                                 other kernels, iterations whose frontier is small (a few
+                                 thousand vertices) run one after another in a single launch of
+                                 one thread-block cluster (same results) */
   DFL_FLAG_PROFILE_MOVE = 64u, /* time only the decide phase of each sub-step (two CUDA events per
                                  sub-step, the DFL_PROF_MOVE class of dfl_profile): the cheap
-                                 subset of DFL_FLAG_PROFILE */
+                                 subset of DFL_FLAG_PROFILE (per-bin kernels, as there) */
   DFL_FLAG_RECOMPUTE_AUX = 128u, /* the ablation of Section 4.2: every dfl_update / dfl_group_update
                                  first recomputes K from the graph and Sigma (and 2m) from K and
                                  the memberships, as a dynamic method without auxiliary
@@ -348,7 +355,8 @@ int dfl_aggregate(dfl_handle* h, uint32_t* nv, uint64_t* na, uint64_t* offsets,
  *   degree <= bin_block:      one block (128 threads up to 1024 arcs, else
  *                             block_threads), shared-memory table
  *                             (global-memory slice when it overflows)
- *   larger:                   one chunk up to 8192 arcs, else chunks of 4096,
+ *   larger:                   one chunk up to 8192 arcs, else chunks of 4096
+ *                             (1024 where a run from singletons has few),
  *                             one block each, summed in a global table of the
  *                             vertex; its last chunk block (or, for many
  *                             distinct communities, a block per 2048 of them)

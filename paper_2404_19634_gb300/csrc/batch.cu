@@ -1584,7 +1584,7 @@ int group_apply(Handle* h, const dfl_edge* sd, uint64_t nd, const dfl_edge* si, 
       return rc;
     }
     const unsigned int err = h->hctrl->err;
-    const int arc = settle_apply(h);  // (a closed gate: the row counters are cleared)
+    const int arc = settle_apply(h);  // (a closed gate: nothing was written)
     if (err & kErrInvalid) return set_error(h, DFL_ERR_INVALID, "vertex id >= the graph's size");
     if (err & kErrOverflow) return set_error(h, DFL_ERR_OVERFLOW, "a graph's 2m could reach 2^32");
     rc = arc;

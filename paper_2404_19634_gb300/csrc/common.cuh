@@ -31,9 +31,10 @@ typedef unsigned __int128 u128;
 // Compile-time configuration
 // ---------------------------------------------------------------------------
 constexpr int kWarp = 32;
-// Degree bins of the local-moving kernels: registers (a few arcs), registers
-// (up to 32 arcs, one or two lanes a vertex), a warp's shared table, a block's
-// shared table (two sizes), chunks summed in a global table.
+// Degree bins of the local-moving kernels: registers (a few arcs; a lane a
+// vertex in long lists, 4 to 32 lanes in short ones), registers (up to 32 arcs; a
+// lane a vertex, or a warp), a warp's shared table, a block's shared table (two
+// sizes), chunks summed in a global table.
 constexpr int kBins = 6;
 enum : int { kBinTiny = 0, kBinLanes = 1, kBinTable = 2, kBinMid = 3, kBinWhole = 4, kBinHuge = 5 };
 constexpr uint32_t kMidDeg = 1024;  // largest degree of the smaller block bin
@@ -197,7 +198,6 @@ struct Handle {
   int* sizes = nullptr;
   uint32_t* used = nullptr;     // n+1: flags, then exclusive scan = new ids
   uint32_t* cnt = nullptr;      // n+1: community vertex counts / offsets
-  unsigned long long* tdeg = nullptr;  // n+1: community total degree / super offsets
   uint32_t* fillc = nullptr;    // n
   uint32_t* members = nullptr;  // n
   SuperGraph sg[2];
@@ -496,8 +496,8 @@ __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 // use different multipliers: aggregation writes a super-vertex's row in its
 // table's slot order, and with the same multiplier a run of consecutive arcs
 // would fill a narrow window of a local-moving table densely (R-MAT 2^22,
-// second pass: probe runs of up to 1,000 slots in the 2,048-slot chunk
-// tables of the largest-degree vertices).
+// second pass: probe runs of up to 1,000 slots in chunk tables of 2,048
+// slots, half of today's, of the largest-degree vertices).
 __device__ __forceinline__ uint32_t hash32(uint32_t x) { return x * 0x9E3779B1u; }       // aggregation
 __device__ __forceinline__ uint32_t hash_move(uint32_t x) { return x * 0x85EBCA6Bu; }    // local-moving
 
@@ -784,8 +784,8 @@ int apply_batch_begin(Handle* h, const dfl_edge* del, uint64_t nd, const dfl_edg
 // Copy the apply's control block to the host (ordered on the handle's
 // stream, no wait) / settle it from that copy: on success the host mirrors
 // (2m, the pending count, the pool top, the arc count, the largest degree)
-// take the batch; otherwise the per-row scratch counters are cleared and the
-// error or the retry is returned.
+// take the batch; otherwise nothing was written (the apply's last kernel has
+// reset its records all the same) and the error or the retry is returned.
 int copy_apply_ctrl(Handle* h);
 int settle_apply(Handle* h);
 // Upper bounds of the live arc count, the tombstones, the pool top and the
@@ -827,7 +827,9 @@ struct MoveArgs {
 // one long chain a lane, while on full frontiers it is the faster one (DF at
 // 1e-3|E| on the 2^22-vertex R-MAT graph: 0.44 ms a batch short, 0.49-0.52 with
 // a thread per vertex).  The line is flat: halving or quartering either limit
-// changed neither DF nor static times on four graphs.
+// changed neither DF nor static times on four graphs.  A replayed graph, whose
+// lists' lengths are not known on the host, takes both lists as short if the
+// whole frontier's share of a sub-step is below kSmallList.
 constexpr uint64_t kSmallList = 32768;
 constexpr uint64_t kSmallLanes = 8192;  // the lane bin's vertices weigh four of the tiny bin's
 // Below this many pending batch arcs a DF or DS update launches its

@@ -977,7 +977,7 @@ constexpr uint32_t kBlockSlots = 2 * kBinBlock;  // 8192 keys + 8192 values = 64
 // Shared scalars of the block-level bodies.
 struct BlockScratch {
   unsigned long long hd;
-  uint32_t ncand, ne;
+  uint32_t ncand;
   int ok, last;
 };
 
