@@ -628,7 +628,7 @@ int dfl_set_membership(dfl_handle* h, const uint32_t* C, int mem_kind) {
   DFL_TRY(weighted_degrees(h));
   DFL_TRY(recompute_sigma_sizes(h, h->C));
   h->pend_count = 0;
-  h->have_communities = true;
+  h->have_communities = h->labels_given = true;
   DFL_CUDA(h, cudaStreamSynchronize(h->stream));
   return DFL_OK;
 }
@@ -692,6 +692,7 @@ int dfl_move_iteration(dfl_handle* h, uint8_t* F, const uint8_t* R, uint8_t* mov
   a.max_deg = h->max_deg;
   a.use_range = true;
   a.track_ever = false;
+  a.from_singletons = h->labels_given;
   uint32_t saved = h->opt.max_iterations;
   h->opt.max_iterations = 1;
   h->trace.clear();

@@ -88,7 +88,7 @@ struct Ctrl {
   unsigned int it_items[kMaxSubsteps];
   unsigned int bar_count, bar_gen;
   long long m2v;                     // 2m of the current local-moving call
-  unsigned int from_singletons;      // it starts with a community per vertex (MoveArgs)
+  unsigned int from_singletons;      // it may start with a community per vertex (MoveArgs)
   unsigned int npairs;               // distinct (u, v) pairs of the batch (hashed apply)
   unsigned int max_app;              // most new arcs of one rebuilt row
   unsigned long long extra_top;      // new arcs of rebuilt rows
@@ -181,6 +181,7 @@ struct Handle {
   uint32_t* C = nullptr;
   long long m2 = 0;
   bool have_communities = false;
+  bool labels_given = false;  // C is as the caller set it: no run has been made from it yet
 
   // pending batch arcs (sorted keys and weights of every dfl_apply_batch
   // since the last update)
@@ -811,7 +812,9 @@ struct MoveArgs {
   uint32_t max_deg;  // upper bound of the degrees of g
   bool use_range;
   bool track_ever;
-  bool from_singletons = false;  // every vertex starts in a community of its own
+  // every vertex starts in a community of its own, or the labels are the
+  // caller's and nothing is known of them
+  bool from_singletons = false;
   bool prefer_host = false;  // launch from the host unless DFL_FLAG_GRAPH asks for replay
   // upper bound of the initial frontier's vertex count (DF: the pending
   // batch arcs); chooses launch shapes for a replayed first iteration

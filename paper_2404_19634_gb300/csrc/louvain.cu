@@ -76,6 +76,8 @@ int renumber(Handle* h, uint32_t* Cp, uint32_t nv, bool first_level) {
 
 int louvain(Handle* h, bool all, bool use_range, uint64_t initial, bool singletons, bool counted) {
   const uint32_t n = h->n;
+  const bool given = h->labels_given;
+  h->labels_given = false;
   h->trace.clear();
   dfl_stats_t& st = h->stats;
   st.passes = 0;
@@ -120,7 +122,7 @@ int louvain(Handle* h, bool all, bool use_range, uint64_t initial, bool singleto
     // passes may mark every vertex
     a.frontier_hint = (pass == 0 && !all && !use_range) ? pend : nv;
     a.counted = counted && pass == 0;
-    a.from_singletons = singletons || pass > 0;
+    a.from_singletons = singletons || given || pass > 0;
     uint32_t it = 0;
     uint64_t init0 = 0, ever0 = 0;
     DFL_TRY(local_move(h, a, pass, &it, pass == 0, &init0, &ever0));

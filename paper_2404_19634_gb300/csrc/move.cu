@@ -1242,7 +1242,10 @@ constexpr uint32_t kGiantChunk = 4096;   // ... a larger one has chunks of this 
 // now 2.32, 3.20 and 4.37; on 2^20 to 2^22 the same.  The line is flat from 24
 // to 76 chunks; at 12 the run on 2^18 vertices loses 11%, at 152 the one on 2^20
 // 1.4%.  Updates start from communities, where a hub's arcs meet few, and lose
-// with finer chunks (DF of 4,000 edges on 2^20 vertices 425 -> 442 us).
+// with finer chunks (DF of 4,000 edges on 2^20 vertices 262 -> 275 us).  Labels
+// that the caller has set count as singletons, since nothing is known of them
+// (an iteration from communities of seven vertices, 2^18 in all, 950 us with the
+// larger chunks, now 692; 718 when every chunk was small).
 constexpr uint32_t kGiantFine = 1024;
 constexpr uint32_t kGiantFew = 76;
 constexpr int kAccumThreads = 256;

@@ -209,6 +209,17 @@ def test_hubs_of_a_run_from_singletons(dfl, orc, degrees, flags):  # noqa: F811
     a.update(0)  # from communities: chunks of 4,096
     b.update(0)
     same(a, b)
+    # ... and from the many communities that one iteration leaves
+    kw = dict(max_passes=1, max_iterations=1, substeps=1)
+    a.set_options(dfl.default_options(flags=flags, **kw))
+    b.set_options(**kw)
+    a.static()
+    b.static()
+    F = R = np.ones(g.n, np.uint8)
+    Fa, ma, Sa = a.move_iteration(F, R)
+    Fb, mb, Sb = b.move_iteration(F, R)
+    assert np.array_equal(Fa, Fb) and np.array_equal(ma, mb) and Sa == Sb
+    same(a, b)
 
 
 @pytest.mark.parametrize("n,degrees", [
