@@ -67,8 +67,8 @@ BATCH_FRAC = 1e-3
 # divided by their sub-steps: caches flushed before each launch (cold) and
 # kept (warm).  They belong to the kernel sources whose hash is recorded;
 # with other sources, or another workload, the line reports null.
-DECIDE_TRAFFIC = {"sources_sha256": "c9f3270124151e96ffa397b71f9861b44525eb09126feba9cb40985cd42e046b",
-                  "cold": 57_004_245, "warm": 17_056_939,
+DECIDE_TRAFFIC = {"sources_sha256": "a0fc632ea16a938a927870b811372beb29913a6681ec10ac306c30494aad3431",
+                  "cold": 57_006_208, "warm": 16_954_581,
                   "profile": "profiles/decide_traffic_rmat22_df.md"}
 SIZES = [1e-7, 1e-6, 1e-5, 1e-4, 1e-3]
 METRIC = "ms/batch DF update (R-MAT 2^22, 1e-3|E| batches)"

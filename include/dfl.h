@@ -356,7 +356,8 @@ int dfl_aggregate(dfl_handle* h, uint32_t* nv, uint64_t* na, uint64_t* offsets,
  *                             block_threads), shared-memory table
  *                             (global-memory slice when it overflows)
  *   larger:                   one chunk up to 8192 arcs, else chunks of 4096
- *                             (1024 where a run from singletons has few),
+ *                             (1024 where a run from singletons, or from
+ *                             dfl_set_membership's labels, has few),
  *                             one block each, summed in a global table of the
  *                             vertex; its last chunk block (or, for many
  *                             distinct communities, a block per 2048 of them)
