@@ -2797,10 +2797,11 @@ int issue_iteration(Handle* h, DecideArgs a, int cur, const unsigned int (*count
         k_decide_warp_hash<<<counts ? grid_for(uint64_t(c) * 32, 256, 152 * 6) : 152 * 3, 256, 0, st>>>(a);
       } else if (b == kBinMid) {
         // (a replayed graph launches every bin at once: with all eight blocks an SM
-        // this one keeps the lane bin's blocks, of the lowest priority too, waiting;
-        // ND on 2^18 vertices 324 us so, 300 with four, 2^20 and 2^22 the same)
+        // this one keeps the lane bin's blocks, of the lowest priority too, waiting:
+        // ND on 2^18, 2^20 and 2^22 vertices 315, 533 and 1,468 us so, 295, 514 and
+        // 1,475 with five, 301, 522 and 1,490 with four)
         k_decide_block<128, 2 * kMidDeg>
-            <<<counts ? grid_for(c, 1, 152 * 8) : 152 * 4, 128, sizeof(uint32_t) * 4 * kMidDeg, st>>>(a);
+            <<<counts ? grid_for(c, 1, 152 * 8) : 152 * 5, 128, sizeof(uint32_t) * 4 * kMidDeg, st>>>(a);
       } else if (b == kBinWhole) {
         const size_t smem = sizeof(uint32_t) * 2 * kBlockSlots;
         const uint32_t bt = h->tune.block_threads;
