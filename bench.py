@@ -67,8 +67,8 @@ BATCH_FRAC = 1e-3
 # divided by their sub-steps: caches flushed before each launch (cold) and
 # kept (warm).  They belong to the kernel sources whose hash is recorded;
 # with other sources, or another workload, the line reports null.
-DECIDE_TRAFFIC = {"sources_sha256": "a0fc632ea16a938a927870b811372beb29913a6681ec10ac306c30494aad3431",
-                  "cold": 57_006_208, "warm": 16_954_581,
+DECIDE_TRAFFIC = {"sources_sha256": "131034bdfb5e23590660e9107299e983274eed5e277d72e236c20d17c4918392",
+                  "cold": 57_003_179, "warm": 17_089_131,
                   "profile": "profiles/decide_traffic_rmat22_df.md"}
 SIZES = [1e-7, 1e-6, 1e-5, 1e-4, 1e-3]
 METRIC = "ms/batch DF update (R-MAT 2^22, 1e-3|E| batches)"
